@@ -16,6 +16,8 @@
 using namespace mvla;
 
 namespace {
+constexpr int kMaxBatch = 64;       // samples per call (mvla_prune_create refuses more)
+constexpr int kMapSlots = 16;       // tensor maps a context remembers
 constexpr int kSets = 6;            // scratch sets = prune steps that may be in flight at once
 #ifndef MVLA_TAIL_CTAS_PER_SM
 #define MVLA_TAIL_CTAS_PER_SM 2
@@ -118,10 +120,11 @@ struct mvla_ctx {
     int* status_dev;
     cudaError_t last_cuda;
     PFN_cuTensorMapEncodeTiled_v12000 encode;
-    // tensor maps are cached per (pointer, rows)
-    const void* tm_ptr[2];
-    int64_t tm_rows[2];
-    CUtensorMap tm[2];
+    // Tensor maps by (pointer, rows, which tensor): a server's calls cycle through a few buffers, and encoding one
+    // costs as much host time as the rest of the call's bookkeeping.  Replaced in turn.
+    struct MapSlot { const void* ptr; int64_t rows; int which; CUtensorMap map; };
+    MapSlot maps[kMapSlots];
+    unsigned next_map;
 };
 
 namespace {
@@ -179,7 +182,8 @@ int32_t validate_samples(const mvla_ctx* ctx, int32_t batch, const mvla_sample* 
 // Everything about a call that the host can decide: layout offsets, budgets, state addressing,
 // the smoothing weights of this action step.
 struct Plan {
-    std::vector<SampleDev> s;
+    SampleDev s[kMaxBatch];
+    int32_t n = 0;
     int32_t total_vis = 0;
     int32_t total_out = 0;
 };
@@ -187,7 +191,7 @@ struct Plan {
 int32_t make_plan(mvla_ctx* ctx, int32_t prune_point, int32_t batch, const mvla_sample* samples, int32_t mode,
                   uint32_t flags, bool with_state, Plan* plan)
 {
-    plan->s.resize(batch);
+    plan->n = batch;
     const mvla_config& c = ctx->cfg;
     if (with_state) {
         if (prune_point < 0 || prune_point >= c.n_prune_points) return MVLA_ERR_STATE;
@@ -198,7 +202,7 @@ int32_t make_plan(mvla_ctx* ctx, int32_t prune_point, int32_t batch, const mvla_
     int32_t vis_off = 0, out_off = 0, cap_off = 0;
     for (int b = 0; b < batch; ++b) {
         const mvla_sample& in = samples[b];
-        SampleDev d;
+        SampleDev& d = plan->s[b];
         std::memset(&d, 0, sizeof d);
         d.seq_off = in.seq_off; d.off_txt = in.off_txt; d.n_txt = in.n_txt;
         d.off_2d = in.off_2d; d.n_2d = in.n_2d; d.off_3d = in.off_3d; d.n_3d = in.n_3d;
@@ -251,7 +255,6 @@ int32_t make_plan(mvla_ctx* ctx, int32_t prune_point, int32_t batch, const mvla_
             d.out_off = out_off;
             out_off += d.n_out;
         }
-        plan->s[b] = d;
     }
     plan->total_vis = vis_off;
     plan->total_out = out_off;
@@ -260,16 +263,16 @@ int32_t make_plan(mvla_ctx* ctx, int32_t prune_point, int32_t batch, const mvla_
 
 void commit_steps(mvla_ctx* ctx, int32_t prune_point, const Plan& plan, const mvla_sample* samples)
 {
-    for (size_t b = 0; b < plan.s.size(); ++b)
+    for (int b = 0; b < plan.n; ++b)
         if (plan.s[b].update_state) ctx->t_host[prune_point * ctx->n_slots + samples[b].state_slot] = plan.s[b].t;
 }
 
+// (descriptors past the n-th are left as they are: no kernel looks at them)
 BatchDesc chunk_of(const Plan& plan, int first, int n)
 {
     BatchDesc bd;
-    std::memset(&bd, 0, sizeof bd);
     bd.n = n;
-    for (int i = 0; i < n; ++i) bd.s[i] = plan.s[first + i];
+    std::memcpy(bd.s, plan.s + first, static_cast<size_t>(n) * sizeof(SampleDev));
     return bd;
 }
 
@@ -282,10 +285,18 @@ int tiles_of(const SampleDev& s)
 // `box_rows` land in shared memory as `box_rows` rows of 128 bytes with the 128-byte swizzle.
 int32_t tensor_map(mvla_ctx* ctx, int which, const void* ptr, int64_t rows, int box_rows, const CUtensorMap** out)
 {
-    if (ctx->tm_ptr[which] == ptr && ctx->tm_rows[which] == rows) {
-        *out = &ctx->tm[which];
-        return MVLA_OK;
+    for (const mvla_ctx::MapSlot& m : ctx->maps)
+        if (m.ptr == ptr && m.rows == rows && m.which == which) {
+            *out = &m.map;
+            return MVLA_OK;
+        }
+    // the slot after the last one filled: never the one that the other map of this call was just found or put in
+    mvla_ctx::MapSlot* slot = &ctx->maps[ctx->next_map];
+    if (&slot->map == *out) {
+        ctx->next_map = (ctx->next_map + 1) % kMapSlots;
+        slot = &ctx->maps[ctx->next_map];
     }
+    ctx->next_map = (ctx->next_map + 1) % kMapSlots;
     const mvla_config& c = ctx->cfg;
     const cuuint64_t heads = static_cast<cuuint64_t>(which == 1 ? ctx->kv_heads : c.n_heads);   // map 1 is the key tensor
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(c.head_dim), heads, static_cast<cuuint64_t>(rows)};
@@ -294,16 +305,15 @@ int32_t tensor_map(mvla_ctx* ctx, int which, const void* ptr, int64_t rows, int 
     cuuint32_t box[3] = {static_cast<cuuint32_t>(128 / es), 1, static_cast<cuuint32_t>(box_rows)};
     cuuint32_t estr[3] = {1, 1, 1};
     const CUtensorMapDataType dt = es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    const CUresult r = ctx->encode(&ctx->tm[which], dt, 3, const_cast<void*>(ptr), dims,
+    slot->ptr = nullptr;
+    const CUresult r = ctx->encode(&slot->map, dt, 3, const_cast<void*>(ptr), dims,
                                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        ctx->tm_ptr[which] = nullptr;
-        return MVLA_ERR_CUDA;
-    }
-    ctx->tm_ptr[which] = ptr;
-    ctx->tm_rows[which] = rows;
-    *out = &ctx->tm[which];
+    if (r != CUDA_SUCCESS) return MVLA_ERR_CUDA;
+    slot->ptr = ptr;
+    slot->rows = rows;
+    slot->which = which;
+    *out = &slot->map;
     return MVLA_OK;
 }
 
@@ -335,6 +345,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     if (ctx->use_umma) {
         int32_t r = tensor_map(ctx, 0, q, rows, 16, &tq);
         if (r != MVLA_OK) return r;
+        tk = tq;                              // (the slot not to be reused)
         r = tensor_map(ctx, 1, k, rows, kKeyTile, &tk);
         if (r != MVLA_OK) return r;
     }
@@ -373,10 +384,10 @@ mvla_ctx::Range range_of(const void* p, size_t bytes)
     return {c, c ? c + bytes : c};
 }
 
-bool chunk_is_fast(const mvla_ctx* ctx, const BatchDesc& bd)
+bool chunk_is_fast(const mvla_ctx* ctx, const Plan& plan, int first, int n)
 {
     int max_tiles = 1;
-    for (int b = 0; b < bd.n; ++b) max_tiles = std::max(max_tiles, tiles_of(bd.s[b]));
+    for (int b = first; b < first + n; ++b) max_tiles = std::max(max_tiles, tiles_of(plan.s[b]));
     return ctx->use_umma && fast_salience_supported((max_tiles + kMaxCluster - 1) / kMaxCluster);
 }
 
@@ -614,7 +625,7 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
     bool forked = false;
     ForkPlan fp;
     if ((flags & MVLA_FLAG_INPUTS_STABLE) && ctx->patch_sets == kSets && batch <= kMaxChunk &&
-        chunk_is_fast(ctx, chunk_of(plan, 0, batch))) {
+        chunk_is_fast(ctx, plan, 0, batch)) {
         forked = true;
         const size_t nvis_b = static_cast<size_t>(plan.total_vis), npat_b = nvis_b / 2, in_rows = static_cast<size_t>(in->rows);
         const size_t hb = static_cast<size_t>(ctx->cfg.d_model) * ctx->elem, kb = static_cast<size_t>(kv_bytes);
@@ -640,7 +651,7 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
     float* attn = out->attn ? out->attn : ctx->patch_attn_ws + set * ctx->vis_all;
     float* x = out->patch_x ? out->patch_x : ctx->patch_x_ws + set * (ctx->vis_all / 2 + 1) * 4;
     const BatchDesc whole = chunk_of(plan, 0, std::min(batch, kMaxChunk));
-    if (!forked && batch <= kMaxChunk && chunk_is_fast(ctx, whole) && patch_tail_supported(whole)) {
+    if (!forked && batch <= kMaxChunk && chunk_is_fast(ctx, plan, 0, batch) && patch_tail_supported(whole)) {
         // two kernels: scoring (leaves the attention copy, re-arms the hand-over words), then indicators,
         // stages 1-4 and the row copy in one
         int32_t* list = ctx->tail_list + par * ctx->rows_all;
@@ -721,7 +732,7 @@ static int32_t mvla_prune_create_impl(const mvla_config* cfg, mvla_ctx** out)
     if (c.head_dim < 64 || c.head_dim > 256 || c.head_dim % 32 != 0) return MVLA_ERR_UNSUPPORTED;
     if (c.n_kv_heads < 0 || (c.n_kv_heads > 0 && (c.n_kv_heads > c.n_heads || c.n_heads % c.n_kv_heads != 0))) return MVLA_ERR_INVALID_ARG;
     if (c.patch_path && c.n_kv_heads > 0 && c.n_kv_heads != c.n_heads) return MVLA_ERR_UNSUPPORTED;   // the patch path is built for ungrouped keys
-    if (c.max_text > kMaxText || c.max_2d + c.max_3d > kMaxVis || c.max_batch > 64) return MVLA_ERR_UNSUPPORTED;
+    if (c.max_text > kMaxText || c.max_2d + c.max_3d > kMaxVis || c.max_batch > kMaxBatch) return MVLA_ERR_UNSUPPORTED;
     const size_t elem = c.dtype == MVLA_DTYPE_FP32 ? 4 : 2;       // hidden: fp32, or bf16 (also beside e4m3 q / k / v)
     if ((static_cast<size_t>(c.d_model) * elem) % 16 != 0) return MVLA_ERR_UNSUPPORTED;
 
@@ -774,8 +785,8 @@ static int32_t mvla_prune_create_impl(const mvla_config* cfg, mvla_ctx** out)
     ctx->hist_unknown = true;
     ctx->status_host = ctx->status_dev = nullptr;
     ctx->last_cuda = cudaSuccess;
-    ctx->tm_ptr[0] = ctx->tm_ptr[1] = nullptr;
-    ctx->tm_rows[0] = ctx->tm_rows[1] = -1;
+    for (mvla_ctx::MapSlot& m : ctx->maps) m.ptr = nullptr;
+    ctx->next_map = 0;
     ctx->encode = nullptr;
     ctx->t_host.assign(static_cast<size_t>(c.n_prune_points) * ctx->n_slots, 0);
 
@@ -1146,7 +1157,7 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
     const size_t nvis_b = static_cast<size_t>(plan.total_vis), nout_b = static_cast<size_t>(plan.total_out);
     const size_t hb = static_cast<size_t>(ctx->cfg.d_model) * ctx->elem, kb = static_cast<size_t>(kv_bytes);
     const size_t qb = static_cast<size_t>(ctx->cfg.n_heads) * ctx->cfg.head_dim * ctx->qk_elem;
-    if ((flags & MVLA_FLAG_INPUTS_STABLE) && batch <= kMaxChunk && chunk_is_fast(ctx, chunk_of(plan, 0, batch))) {
+    if ((flags & MVLA_FLAG_INPUTS_STABLE) && batch <= kMaxChunk && chunk_is_fast(ctx, plan, 0, batch)) {
         forked = true;
         // buffers the side-stream work touches: selection outputs, and the inputs of scoring
         const size_t in_rows = static_cast<size_t>(in->rows);
@@ -1203,9 +1214,7 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         if (!forked && used_acc64 && select_copy_supported(bd)) {
             // one kernel for selection and row copy: every CTA repeats its sample's selection, then copies
             ctx->sel_valid[par] = false;             // this set was used outside the event chain
-            const bool copying = (job.src[0] && job.dst[0]) || (job.src[1] && job.dst[1]) || (job.src[2] && job.dst[2]);
-            (void)copying;
-            ph.mark("mvla: selection + row copy");
+                ph.mark("mvla: selection + row copy");
             const cudaError_t e2 = launch_select_copy(bd, gp, io, job, ctx->tail_list + par * ctx->rows_all,
                                                       ctx->status_dev, ctx->sm_count * kTailCtasPerSm - n,
                                                       ctx->stamps ? ctx->stamps + 2 * kStampSlots : nullptr, st);

@@ -6,6 +6,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "mvla_prune.h"
 
 namespace mvla {
@@ -95,6 +97,16 @@ inline cudaLaunchAttribute pdl_attribute()
 
 // Multiprocessors of the current device (looked up once per device).
 int sm_count_of_current_device();
+
+// What has been set up for one kernel on one device: asking the runtime again on every launch costs host time that a
+// small step would see.  One object per kernel instantiation; host threads may share it.
+struct KernelSetup {
+    std::atomic<int> smem_set[64];       // dynamic shared memory the kernel may use (the largest asked for so far)
+    std::atomic<int> smem_checked[64];   // dynamic shared memory whose occupancy was last checked, + 1
+};
+// Lets `kern` use `smem` bytes of dynamic shared memory and, with `tmem_cols` > 0, makes sure that the CTAs of
+// `threads` threads that fit on a multiprocessor cannot ask for more tensor memory than it has.
+cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t smem, int tmem_cols);
 
 // ---- launchers (each enqueues on `stream` and returns the launch status) ----
 

@@ -5,8 +5,10 @@
 // 16-byte loads per lane are issued back to back (512 bytes per lane-round in flight per warp),
 // then four stores.  The loads bypass L1 (read once), the stores are streaming.
 #include "common.cuh"
+#include "tmem_plan.h"
 
 #include <algorithm>
+#include <mutex>
 
 namespace mvla {
 namespace {
@@ -94,6 +96,30 @@ int sm_count_of_current_device()
         cached[dev] = n;
     }
     return cached[dev];
+}
+
+cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t smem, int tmem_cols)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool known = dev >= 0 && dev < 64;
+    const int bytes = static_cast<int>(smem);
+    if (!known || ks.smem_set[dev].load(std::memory_order_acquire) < bytes) {
+        static std::mutex m;                 // the attribute only ever grows, whichever thread comes first
+        std::lock_guard<std::mutex> lock(m);
+        if (!known || ks.smem_set[dev].load(std::memory_order_relaxed) < bytes) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+        if (known && ks.smem_set[dev].load(std::memory_order_relaxed) < bytes) ks.smem_set[dev].store(bytes, std::memory_order_release);
+    }
+    if (tmem_cols > 0 && !(known && ks.smem_checked[dev].load(std::memory_order_relaxed) == bytes + 1)) {
+        int resident = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, threads, smem);
+        if (e != cudaSuccess) return e;
+        if (resident * tmem_cols > kTmemColsPerSm) return cudaErrorInvalidConfiguration;
+        if (known) ks.smem_checked[dev].store(bytes + 1, std::memory_order_relaxed);
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_compact(const BatchDesc& bd, const CompactJob& job, const int32_t* kept_idx,

@@ -361,14 +361,9 @@ cudaError_t launch_salience_t(const BatchDesc& bd, int n_heads, int kv_group, in
         smem = smem_for_tmem(smem, tmem_cols);
         if (smem == 0) return cudaErrorInvalidConfiguration;
     }
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    static KernelSetup ks;
+    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kThreads, smem, tmem_cols);
     if (e != cudaSuccess) return e;
-    if (UMMA) {
-        int resident = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, kThreads, smem);
-        if (e != cudaSuccess) return e;
-        if (resident * tmem_cols > kTmemColsPerSm) return cudaErrorInvalidConfiguration;
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster, n_heads, bd.n);
     cfg.blockDim = dim3(kThreads);

@@ -1,4 +1,5 @@
-"""Thin ctypes binding of ``libmvla_prune.so`` (see ``include/mvla_prune.h``).
+"""Thin binding of ``libmvla_prune.so`` (see ``include/mvla_prune.h``): ctypes for the calls a program makes once,
+the extension module ``_native`` (``csrc/binding.cpp``) for those it makes on every step.
 
 Argument marshalling only: every step of the prune path runs in the CUDA
 library.  PyTorch supplies device memory and streams.  There is no CPU
@@ -11,6 +12,7 @@ import os
 from dataclasses import dataclass
 from typing import Optional, Sequence
 
+import numpy as np
 import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
@@ -131,13 +133,26 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_nat = None
+
+
+def native():
+    """The extension module that marshals the per-step calls."""
+    global _nat
+    if _nat is None:
+        try:
+            from . import _native
+        except ImportError as e:
+            raise OSError(f"the extension module _native is missing: build it with `python -m paper_2604_09244_b200.build` "
+                          f"(there is no fallback path): {e}") from e
+        _nat = _native
+    return _nat
+
+
 def c_samples(samples: Sequence) -> "C.Array[CSample]":
     """From objects with the descriptor's field names (``workloads.Sample``)."""
     arr = (CSample * len(samples))()
-    for i, s in enumerate(samples):
-        arr[i] = CSample(int(s.seq_off), int(s.off_txt), int(s.n_txt), int(s.off_2d), int(s.n_2d),
-                         int(s.off_3d), int(s.n_3d), int(getattr(s, "state_slot", 0)),
-                         float(s.keep_2d), float(s.keep_3d), float(s.keep_total))
+    native().fill_samples(arr, samples)
     return arr
 
 
@@ -185,6 +200,7 @@ class PruneContext:
                  obj_2d_min: float = 0.5, kmeans_max_iter: int = 32, n_kv_heads: int = 0, logit_cache: int = 0):
         self._h = C.c_void_p()
         self._lib = lib()
+        self._nat = native()
         if device is None:
             device = torch.cuda.current_device()
         self.device = torch.device("cuda", device)
@@ -268,57 +284,44 @@ class PruneContext:
             patch_info=mk(npat, dtype=torch.int32) if patch else None,
             patch_diag=torch.zeros(len(samples), 16, dtype=torch.int32, device=dev) if patch else None)
 
-    # -- the six entry points ----------------------------------------------
+    # -- the six entry points (`samples`: a ctypes array from c_samples, or objects with the descriptor's field names) --
     def salience(self, samples, q, k, hidden=None, *, attn_out=None, l1_out=None, stream=None):
-        cs = samples if isinstance(samples, C.Array) else c_samples(samples)
-        nvis = sum(s.n_2d + s.n_3d for s in cs)
-        if attn_out is None:
-            attn_out = torch.empty(nvis, dtype=torch.float32, device=self.device)
-        if hidden is not None and l1_out is None:
-            l1_out = torch.empty(nvis, dtype=torch.float32, device=self.device)
-        rc = self._lib.mvla_salience(self._h, len(cs), cs, _ptr(q), _ptr(k), _ptr(hidden), q.shape[0],
-                                     _ptr(attn_out), _ptr(l1_out), _stream(stream))
+        rc, attn_out, l1_out = self._nat.salience(self._h.value or 0, samples, q, k, hidden, attn_out, l1_out, stream)
         if rc != OK:
             raise MvlaError(rc, "mvla_salience")
         return attn_out, l1_out
 
     def select(self, prune_point, samples, mode, attn, l1=None, *, flags=0, out: StepOutputs = None,
                stream=None) -> StepOutputs:
-        cs = samples if isinstance(samples, C.Array) else c_samples(samples)
         if out is None:
-            out = self.alloc_outputs(cs, hidden=False, kv=False, extras=True)
-        rc = self._lib.mvla_select(self._h, prune_point, len(cs), cs, mode, flags, _ptr(attn), _ptr(l1),
-                                   _ptr(out.kept_idx), _ptr(out.out_offsets), _ptr(out.budgets),
-                                   _ptr(out.ahat), _ptr(out.z), _ptr(out.diag), _stream(stream))
+            out = self.alloc_outputs(samples, hidden=False, kv=False, extras=True)
+        rc = self._nat.select(self._h.value or 0, prune_point, samples, mode, flags, attn, l1, out, stream)
         if rc != OK:
             raise MvlaError(rc, "mvla_select")
         return out
 
     def compact(self, samples, kept_idx, out_offsets, total_kept, hidden=None, k=None, v=None, *,
                 out_hidden=None, out_k=None, out_v=None, stream=None):
-        cs = samples if isinstance(samples, C.Array) else c_samples(samples)
         mk = lambda src: None if src is None else torch.empty((total_kept,) + tuple(src.shape[1:]),
                                                               dtype=src.dtype, device=src.device)
         out_hidden = mk(hidden) if out_hidden is None else out_hidden
         out_k = mk(k) if out_k is None else out_k
         out_v = mk(v) if out_v is None else out_v
-        rc = self._lib.mvla_compact(self._h, len(cs), cs, _ptr(kept_idx), _ptr(out_offsets), int(total_kept),
-                                    _ptr(hidden), _ptr(k), _ptr(v), _ptr(out_hidden), _ptr(out_k),
-                                    _ptr(out_v), _stream(stream))
+        rc = self._nat.compact(self._h.value or 0, samples, kept_idx, out_offsets, total_kept, hidden, k, v,
+                               out_hidden, out_k, out_v, stream)
         if rc != OK:
             raise MvlaError(rc, "mvla_compact")
         return out_hidden, out_k, out_v
 
     def patch_indicators(self, samples, q, k, hidden, *, attn_out=None, x_out=None, stream=None):
         """Per-token scores and the four per-patch indicators (``mvla_patch_indicators``)."""
-        cs = samples if isinstance(samples, C.Array) else c_samples(samples)
-        nvis = sum(s.n_2d + s.n_3d for s in cs)
-        if attn_out is None:
-            attn_out = torch.empty(nvis, dtype=torch.float32, device=self.device)
-        if x_out is None:
-            x_out = torch.empty(nvis // 2, 4, dtype=torch.float32, device=self.device)
-        rc = self._lib.mvla_patch_indicators(self._h, len(cs), cs, _ptr(q), _ptr(k), _ptr(hidden), q.shape[0],
-                                             _ptr(attn_out), _ptr(x_out), _stream(stream))
+        if attn_out is None or x_out is None:
+            nvis = sum(s.n_2d + s.n_3d for s in samples)
+            if attn_out is None:
+                attn_out = torch.empty(nvis, dtype=torch.float32, device=self.device)
+            if x_out is None:
+                x_out = torch.empty(nvis // 2, 4, dtype=torch.float32, device=self.device)
+        rc = self._nat.patch_indicators(self._h.value or 0, samples, q, k, hidden, attn_out, x_out, stream)
         if rc != OK:
             raise MvlaError(rc, "mvla_patch_indicators")
         return attn_out, x_out
@@ -326,40 +329,25 @@ class PruneContext:
     def patch_select(self, prune_point, samples, attn, x, rand_u, *, flags=0, out: StepOutputs = None,
                      stream=None) -> StepOutputs:
         """Alg. 1 stages 1-4 patch by patch (``mvla_patch_select``); kept counts land in ``out.budgets``."""
-        cs = samples if isinstance(samples, C.Array) else c_samples(samples)
         if out is None:
-            out = self.alloc_outputs(cs, hidden=False, kv=False, patch=True)
-        rc = self._lib.mvla_patch_select(self._h, prune_point, len(cs), cs, flags, _ptr(attn), _ptr(x), _ptr(rand_u),
-                                         _ptr(out.kept_idx), _ptr(out.out_offsets), _ptr(out.budgets),
-                                         _ptr(out.patch_xhat), _ptr(out.patch_info), _ptr(out.patch_diag),
-                                         _stream(stream))
+            out = self.alloc_outputs(samples, hidden=False, kv=False, patch=True)
+        rc = self._nat.patch_select(self._h.value or 0, prune_point, samples, flags, attn, x, rand_u, out, stream)
         if rc != OK:
             raise MvlaError(rc, "mvla_patch_select")
         return out
 
     def prune_step(self, prune_point, samples, mode, q, k, v, hidden, *, flags=0,
                    out: StepOutputs = None, stream=None, rand_u=None, changed_rows=None) -> StepOutputs:
-        cs = samples if isinstance(samples, C.Array) else c_samples(samples)
         if out is None:
-            out = self.alloc_outputs(cs, hidden=hidden is not None, kv=v is not None, extras=True,
+            out = self.alloc_outputs(samples, hidden=hidden is not None, kv=v is not None, extras=True,
                                      patch=mode == MODE_PATCH)
-        ch = None
         if changed_rows is not None:         # host bytes, read during the call
-            import numpy as np
             changed_rows = np.ascontiguousarray(changed_rows, dtype=np.uint8)
-            assert changed_rows.shape[0] == q.shape[0], "one byte per row of the packed tensors"
-            ch = changed_rows.ctypes.data
-        tin = CTensors(_ptr(q), _ptr(k), _ptr(v), _ptr(hidden), q.shape[0], _ptr(rand_u), ch)
-        tout = COutputs(_ptr(out.out_hidden), _ptr(out.out_k), _ptr(out.out_v), _ptr(out.kept_idx),
-                        _ptr(out.out_offsets), _ptr(out.budgets), _ptr(out.attn), _ptr(out.ahat),
-                        _ptr(out.z), _ptr(out.diag), _ptr(out.patch_x), _ptr(out.patch_xhat),
-                        _ptr(out.patch_info), _ptr(out.patch_diag))
-        total = C.c_int32(0)
-        rc = self._lib.mvla_prune_step(self._h, prune_point, len(cs), cs, mode, flags, C.byref(tin),
-                                       C.byref(tout), C.byref(total), _stream(stream))
-        if rc != OK:
+        rc = self._nat.prune_step(self._h.value or 0, prune_point, samples, mode, flags, q, k, v, hidden, rand_u,
+                                  changed_rows, out, stream)
+        if rc < 0:
             raise MvlaError(rc, "mvla_prune_step")
-        out.total_kept = total.value
+        out.total_kept = rc
         return out
 
 
