@@ -16,7 +16,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libmvla_prune.so")
 EXT = os.path.join(PKG, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
-SOURCES = ["api.cu", "salience.cu", "fused.cu", "select.cu", "compact.cu", "step.cu", "patch.cu", "patch_step.cu", "salience_noalloc.cu"]
+SOURCES = ["api.cu", "salience.cu", "fused.cu", "stream.cu", "select.cu", "compact.cu", "step.cu", "patch.cu", "patch_step.cu", "salience_noalloc.cu"]
 BINDING = "binding.cpp"
 HEADER = os.path.join(ROOT, "include", "mvla_prune.h")
 

@@ -19,10 +19,6 @@ namespace {
 constexpr int kMaxBatch = 64;       // samples per call (mvla_prune_create refuses more)
 constexpr int kMapSlots = 16;       // tensor maps a context remembers
 constexpr int kSets = 6;            // scratch sets = prune steps that may be in flight at once
-#ifndef MVLA_TAIL_CTAS_PER_SM
-#define MVLA_TAIL_CTAS_PER_SM 2
-#endif
-constexpr int kTailCtasPerSm = MVLA_TAIL_CTAS_PER_SM;   // grid of the selection + row copy kernel
 
 // Tracing and logging, both on the host and off the device's path: every public call is an NVTX range (a profiler
 // shows the call and, inside mvla_prune_step, its phases around the kernels they enqueue; without a profiler
@@ -322,6 +318,17 @@ int32_t check_sticky(mvla_ctx* ctx)
     return (ctx->status_host && *reinterpret_cast<volatile int*>(ctx->status_host) != 0) ? MVLA_ERR_TIMEOUT : MVLA_OK;
 }
 
+// Which of the two tensor-core scoring kernels.  The latency-shaped one of fused.cu covers up to 16 key tiles a sample
+// and is the faster one while its CTAs all run at once (three with one key tile to a multiprocessor, two with two tiles);
+// from the second wave on the streaming one is (stream.cu).  Measured at 32 heads, 256 + 512 tokens, whole step in us,
+// latency-shaped / streaming: 2 samples 16.1 / 17.1, 3 samples (576 CTAs) 22.0 / 20.8, 4 samples 27.5 / 23.9, 16
+// samples 120 / 97; 768 + 1023 tokens: 1 sample (224 CTAs) 18.5 / 20.9, 2 samples 33.9 / 30.8.
+bool stream_pays(const mvla_ctx* ctx, const BatchDesc& bd, int tiles_per_cta, int cluster)
+{
+    return !fast_salience_supported(tiles_per_cta) ||
+           bd.n * ctx->cfg.n_heads * cluster > ctx->sm_count * (tiles_per_cta == 1 ? 3 : 2);
+}
+
 // Salience of one chunk (+ L1 norms into `l1` when asked).  The per-head contributions land in
 // ctx->part, or, when `want_acc64` and the register-resident tensor-core kernel covers the shape, in the
 // fixed-point accumulators ctx->acc64 (*used_acc64 = true).
@@ -334,10 +341,13 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     if (used_acc64) *used_acc64 = false;
     const mvla_config& c = ctx->cfg;
     int max_tiles = 1, max_txt = 1;
+    bool cached = false;
     for (int b = 0; b < bd.n; ++b) {
         max_tiles = std::max(max_tiles, tiles_of(bd.s[b]));
         max_txt = std::max(max_txt, bd.s[b].n_txt);
+        cached |= bd.s[b].cache_state >= 0;
     }
+    with_cache = with_cache && cached;
     const int tiles_per_cta = (max_tiles + kMaxCluster - 1) / kMaxCluster;
     const int cluster = (max_tiles + tiles_per_cta - 1) / tiles_per_cta;
     const int npad = (max_txt + 15) / 16 * 16;
@@ -350,7 +360,8 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
         if (r != MVLA_OK) return r;
     }
     cudaError_t e;
-    const bool fast = ctx->use_umma && fast_salience_supported(tiles_per_cta);
+    const bool streaming = ctx->use_umma && acc64 && !alpha.ptr && !with_cache && stream_pays(ctx, bd, tiles_per_cta, cluster);
+    const bool fast = streaming || (ctx->use_umma && fast_salience_supported(tiles_per_cta));
     // The norms do not depend on the scores: with `norms_beside` (fast kernel only) they are launched AFTER
     // the scoring kernel and run beside it instead of in front of it.
     norms_beside = norms_beside && fast;
@@ -358,7 +369,11 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
         e = launch_l1norm(bd, ctx->hidden_dtype, c.d_model, hidden, l1, false, st);
         if (e != cudaSuccess) return fail_cuda(ctx, e);
     }
-    if (fast) {
+    if (streaming) {
+        e = launch_salience_stream(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk, acc64,
+                                   ctx->status_dev, free_running, rearm, stamps, st);
+        if (used_acc64) *used_acc64 = true;
+    } else if (fast) {
         e = launch_salience_fast(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk,
                                  tiles_per_cta, cluster, npad,
                                  alpha.ptr && !acc64 ? nullptr : ctx->part,     // the patch path reads the attention copy only
@@ -1157,7 +1172,7 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
     const size_t nvis_b = static_cast<size_t>(plan.total_vis), nout_b = static_cast<size_t>(plan.total_out);
     const size_t hb = static_cast<size_t>(ctx->cfg.d_model) * ctx->elem, kb = static_cast<size_t>(kv_bytes);
     const size_t qb = static_cast<size_t>(ctx->cfg.n_heads) * ctx->cfg.head_dim * ctx->qk_elem;
-    if ((flags & MVLA_FLAG_INPUTS_STABLE) && batch <= kMaxChunk && chunk_is_fast(ctx, plan, 0, batch)) {
+    if ((flags & MVLA_FLAG_INPUTS_STABLE) && batch <= kMaxChunk && ctx->use_umma) {
         forked = true;
         // buffers the side-stream work touches: selection outputs, and the inputs of scoring
         const size_t in_rows = static_cast<size_t>(in->rows);
@@ -1179,7 +1194,7 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         const BatchDesc bd = chunk_of(plan, first, n);
         bool used_acc64 = false;
         // the fused selection + copy kernel (below) wants its list words re-armed by the scoring kernel
-        const bool tail = !forked && select_copy_supported(bd);
+        const bool tail = !forked;
         ph.mark("mvla: scoring");
         rc = run_salience_chunk(ctx, bd, in->q, in->k, in->rows, adaptive ? in->hidden : nullptr, l1_ws, acc64,
                                 &used_acc64, false, forked ? ctx->aux[par] : st, AlphaOut{nullptr, 0, 0},
@@ -1211,12 +1226,12 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         io.attn_out = out->attn; io.ahat_out = out->ahat; io.z_out = out->z; io.diag = out->diag;
         io.chunk_first = first; io.total_out = plan.total_out; io.write_total = first + n == batch;
         io.n_in_launch = n;
-        if (!forked && used_acc64 && select_copy_supported(bd)) {
+        if (!forked && used_acc64) {
             // one kernel for selection and row copy: every CTA repeats its sample's selection, then copies
             ctx->sel_valid[par] = false;             // this set was used outside the event chain
                 ph.mark("mvla: selection + row copy");
             const cudaError_t e2 = launch_select_copy(bd, gp, io, job, ctx->tail_list + par * ctx->rows_all,
-                                                      ctx->status_dev, ctx->sm_count * kTailCtasPerSm - n,
+                                                      ctx->status_dev,
                                                       ctx->stamps ? ctx->stamps + 2 * kStampSlots : nullptr, st);
             if (e2 != cudaSuccess) {
                 clear_accumulators(acc64, bd, st);

@@ -143,6 +143,11 @@ cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group,
                                  bool free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                                  float* lcache, int cache_vis, int cache_cols, cudaStream_t stream);
 
+// The same scores into the same fixed-point accumulators by the streaming kernel (stream.cu): persistent CTAs, key
+// tiles through a shared-memory ring; for batches and for samples of any size.  `free_running`, `rearm`, `stamps` as above.
+cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
+                                   const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
+                                   bool free_running, int32_t* rearm, unsigned long long* stamps, cudaStream_t stream);
 
 // Salience: per-head partial scores part[h][vis] (already scaled by 1/(H n_t)).
 // `use_umma`: tensor-core path (bf16 only).  tmaps: device-usable tensor maps (passed by value).
@@ -203,18 +208,16 @@ cudaError_t launch_compact(const BatchDesc& bd, const CompactJob& job, const int
                            int32_t chunk_rows, int32_t chunk_row0, const int32_t* out_offsets,
                            int32_t chunk_first, int32_t batch_total, cudaStream_t stream);
 
-// Tail of the fused step for samples of up to 2048 visual tokens: carry-over + budget + top-k (as in
+// Tail of the fused step: carry-over + budget + top-k (as in
 // launch_select) AND the row copy in one kernel.  One CTA per sample selects; the other CTAs copy the
 // text rows at once, then take the kept rows word by word from `list` as the selecting CTA writes them
 // (bounded waits, MVLA_ERR_TIMEOUT into `status` when one runs out): no kernel boundary, fence or flag lies
 // between selection and copy.  `list`: one int per output row of the batch, all -1 when the kernel starts
 // (the scoring kernel before it re-arms them, see launch_salience_fast).
-// `ctas`: copying CTAs to aim for (every sample gets at least one); together with the selecting CTAs no more than
-// fit on the device at once, see the kernel.  `stamps`: as in launch_salience_fast
+// The CTAs are no more than fit on the device at once, see the kernel.  `stamps`: as in launch_salience_fast
 // (start: past the wait for the kernel before; the selecting CTA's end is when the list is written).
-bool select_copy_supported(const BatchDesc& bd);
 cudaError_t launch_select_copy(const BatchDesc& bd, const GateParams& gp, const SelectIO& io, const CompactJob& job,
-                               int32_t* list, int* status, int ctas, unsigned long long* stamps, cudaStream_t stream);
+                               int32_t* list, int* status, unsigned long long* stamps, cudaStream_t stream);
 
 // One warp runs the copying CTAs' bounded wait on `never_set` (a word that holds -1 and stays so) with the
 // given limit and reports MVLA_ERR_TIMEOUT into `status` when it runs out.

@@ -135,8 +135,6 @@ int max_vis_of(const BatchDesc& bd)
 
 }  // namespace
 
-bool select_copy_supported(const BatchDesc& bd) { return max_vis_of(bd) <= 2048; }
-
 cudaError_t launch_wait_probe(const int32_t* never_set, uint64_t limit_ns, int* status, cudaStream_t stream)
 {
     wait_probe_kernel<<<1, 32, 0, stream>>>(never_set, limit_ns, status);
@@ -144,10 +142,12 @@ cudaError_t launch_wait_probe(const int32_t* never_set, uint64_t limit_ns, int* 
 }
 
 cudaError_t launch_select_copy(const BatchDesc& bd, const GateParams& gp, const SelectIO& io, const CompactJob& job,
-                               int32_t* list, int* status, int ctas, unsigned long long* stamps, cudaStream_t stream)
+                               int32_t* list, int* status, unsigned long long* stamps, cudaStream_t stream)
 {
-    if (bd.n < 1 || !select_copy_supported(bd)) return cudaErrorInvalidConfiguration;
+    if (bd.n < 1) return cudaErrorInvalidConfiguration;
     const CompactArgs ca = compact_args(job);
+    // CTAs on the device at once: two of 512 threads to a multiprocessor, or one of 1024 (more than 2048 visual tokens)
+    int ctas = sm_count_of_current_device() * (max_vis_of(bd) > 2048 ? 1 : 2) - bd.n;
     TailPlan tp;
     int next = 0;
     if (ca.seg_begin[3] > 0) {
@@ -179,6 +179,7 @@ cudaError_t launch_select_copy(const BatchDesc& bd, const GateParams& gp, const 
     }
     for (int b = bd.n; b <= kMaxChunk; ++b) tp.cta0[b] = static_cast<int16_t>(next);
     if (max_vis_of(bd) <= 1024) return launch_t<512, 1024>(bd, tp, gp, io, ca, list, status, stamps, stream);
+    if (max_vis_of(bd) > 2048) return launch_t<1024, kMaxVis>(bd, tp, gp, io, ca, list, status, stamps, stream);
     return launch_t<512, 2048>(bd, tp, gp, io, ca, list, status, stamps, stream);
 }
 

@@ -1,0 +1,662 @@
+// Scoring kernel for many key tiles (Sec. 3.2.1 of the paper): batches, and samples with more visual tokens than the
+// latency-shaped kernel of fused.cu covers.
+//
+// A (sample, head) is a job: its keys (T tiles of 128) are read once, its logits have to stay somewhere until the
+// softmax denominators over all T tiles are known.  Here they stay in tensor memory (512 columns = 8 tiles at 64 text
+// queries, 32 at 16), so a job belongs to one CTA, or, when T tiles do not fit, to a cluster of 2, 4 or 8 CTAs that
+// exchange one (maximum, sum) pair per query.  CTAs are persistent, one per multiprocessor, and made of roles that
+// run ahead of one another across jobs:
+//   * one thread streams key tiles through a ring of shared-memory stages by TMA (the text queries of a job in one of
+//     two buffers of their own): 128-160 KB in flight per multiprocessor whatever the softmax is doing;
+//   * one thread issues the MMAs of a tile into the next free tensor-memory slot (slots are a ring too);
+//   * eight warps take the softmax: a warp reads its own 32 tensor-memory lanes of every other tile, against references of
+//     its own, so that a job has two block barriers in all.  Exponentials go back to tensor memory; per-key contributions are added into the 64-bit fixed-point
+//     accumulators (scale 2^60: the sum over heads is exact and independent of scheduling).
+// What bounds it: HBM (the keys are read once); softmax arithmetic comes second (16 exponentials per clock and
+// multiprocessor: half of the time of the key stream at 48 queries, nine tenths at 64).
+#include "common.cuh"
+#include "device_utils.cuh"
+#include "select_impl.cuh"
+#include "tmem_plan.h"
+
+#include <algorithm>
+
+namespace mvla {
+namespace {
+
+constexpr int kSoftWarps = 8;
+constexpr int kSoftThreads = kSoftWarps * 32;
+constexpr int kStreamThreads = kSoftThreads + 64;     // + the loading warp and the MMA warp
+constexpr int kMaxStages = 12;
+constexpr uint32_t kStageBytes = 16384;               // 128 keys x 128 bytes: one swizzled box of a key tile
+constexpr float kRescaleAt = 64.f;                    // exponents (log2) above this move a warp's reference
+constexpr int kMaxSlots = 32;
+// Pairs of job n go to buffer n mod 2: a CTA sends those of job n + 2 only after it has the pairs of job n + 1 of every
+// peer, which that peer sent when it was done with job n's.
+constexpr int kPairBufs = 2;
+
+struct StreamArgs {
+    int n_heads, kv_group, head_dim, esize;
+    int stages;                   // boxes in the shared-memory ring
+    int width, slots;             // columns of a tensor-memory slot (the padded text queries of the longest text), slots
+    int n_jobs;                   // samples x heads
+    unsigned long long* acc64;
+    int* status;
+    int free_running;
+    int32_t* rearm;               // see launch_salience_fast
+    unsigned long long* stamps;
+};
+
+struct StreamSmem {
+    alignas(8) uint64_t kfull[kMaxStages], kempty[kMaxStages];
+    uint64_t qfull[2], qempty[2];
+    uint64_t tfull[kMaxSlots], tempty[kMaxSlots];
+    uint64_t xbar[kPairBufs];                      // pairs of the cluster's CTAs have landed
+    alignas(16) float m[kSoftWarps][kMaxText];     // per warp and query: -reference (log2 domain; +inf: no key)
+    alignas(16) float w[kSoftWarps][kMaxText];     // ... its sum of exponentials, then its weight
+    float g[kMaxText], iz[kMaxText];               // common reference of the job's keys; 1 / (denominator H n_t)
+    float2 peer[kPairBufs][kMaxCluster][kMaxText];
+    uint32_t tmem;
+    int aborted;                                   // a bounded wait ran out: nobody waits any longer
+};
+
+// Bounded wait; gives up at once when another role has.
+template <bool CLUSTER>
+__device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatile int* aborted, int* status)
+{
+    uint64_t t0 = 0;
+    for (uint32_t it = 0; it < kSpinLimit; ++it) {
+        uint32_t ok;
+        if constexpr (CLUSTER)
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                         "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        else
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                         "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+        if ((it & 63u) == 63u) {
+            if (*aborted) return false;
+            const uint64_t now = global_ns();
+            if (t0 == 0) t0 = now;
+            if (now - t0 > 1000000000ull) break;
+        }
+    }
+    *aborted = 1;
+    *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
+    return false;
+}
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// Barrier of the softmax warps.
+__device__ __forceinline__ void soft_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kSoftThreads) : "memory"); }
+__device__ __forceinline__ float fast_ex2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                 ::"r"(taddr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+                   "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])),
+                   "r"(__float_as_uint(v[7])), "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])),
+                   "r"(__float_as_uint(v[11])), "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
+                   "r"(__float_as_uint(v[15])) : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void st_async_pair(uint32_t local_addr, uint32_t local_bar, uint32_t rank, float2 v)
+{
+    uint32_t raddr, rbar;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(raddr) : "r"(local_addr), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbar) : "r"(local_bar), "r"(rank));
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
+                 ::"r"(raddr), "f"(v.x), "f"(v.y), "r"(rbar) : "memory");
+}
+
+// Two fp32 operations per instruction.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+        "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+// 16 tensor-memory columns of this thread's lane, as a load that is issued here and waited for later (tmem_wait_ld
+// names the registers again, so that nothing that uses them can move in front of it).
+__device__ __forceinline__ void tmem_issue16(uint32_t taddr, float (&v)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+                   "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld(float (&v)[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]),
+                   "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]) :: "memory");
+}
+
+// A job's geometry in registers.  (The descriptors are kernel parameters: read with a run-time index a field costs some
+// hundred cycles each time, 700 per tile when the geometry was taken from there tile by tile.)
+struct JobTiles {
+    int n_2d, n_3d, t2;           // tokens per modality; key tiles of the 2D segment
+    int first, count;             // the tiles that fall to this CTA: [first, first + count)
+    __device__ __forceinline__ JobTiles() {}
+    __device__ __forceinline__ JobTiles(const SampleDev& s, int rank, int lg)     // rank of 2^lg CTAs
+    {
+        n_2d = s.n_2d; n_3d = s.n_3d;
+        t2 = (n_2d + kKeyTile - 1) / kKeyTile;
+        const int T = t2 + (n_3d + kKeyTile - 1) / kKeyTile;
+        first = (T * rank) >> lg;
+        count = ((T * (rank + 1)) >> lg) - first;
+    }
+    // tile t of the CTA's: keys that exist, index of its first key in visual order
+    __device__ __forceinline__ int valid(int t) const
+    {
+        const int g = first + t;
+        return min(kKeyTile, g < t2 ? n_2d - g * kKeyTile : n_3d - (g - t2) * kKeyTile);
+    }
+    __device__ __forceinline__ int vis0(int t) const
+    {
+        const int g = first + t;
+        return g < t2 ? g * kKeyTile : n_2d + (g - t2) * kKeyTile;
+    }
+};
+
+// What a softmax warp needs to know about a job.
+struct SoftJob {
+    JobTiles tr;
+    unsigned long long* acc;      // the sample's accumulators
+    int slot0, slots, width;      // slot of the job's first tile, slots in the ring, columns per slot
+    uint32_t parity0;             // parity of that slot's use
+    uint32_t lane_base;           // tensor-memory address of the warp's 32 lanes
+    float cscale;
+    __device__ __forceinline__ int slot(int t) const { const int u = slot0 + t; return u >= slots ? u - slots : u; }   // a job has at most `slots` tiles
+    __device__ __forceinline__ uint32_t parity(int t) const { return parity0 ^ (slot0 + t >= slots ? 1u : 0u); }
+    __device__ __forceinline__ uint32_t cols(int t) const { return lane_base + static_cast<uint32_t>(slot(t) * width); }
+};
+
+// The warp's references (`nm` = -reference per query) move up to what tile t asks for: an exponent could overflow.  Rare.
+// Leaves the factors for everything computed against the old ones in `w`, applied here to what earlier tiles left in
+// tensor memory and by the caller to its sums.
+// (By value: a job whose address is taken would live in local memory on the usual path, too.)
+__device__ __noinline__ void raise_references(uint32_t cols_t, uint32_t lane_base, int first_slot, int slots, int width, int t, int group,
+                                              int chunks, float cscale, bool live, float* nm, float* w)
+{
+    const int lane = threadIdx.x & 31;
+    tmem_wait_st();
+    for (int c = 0; c < chunks; ++c) {
+        float r[16];
+        tmem_issue16(cols_t + c * 16, r);
+        tmem_wait_ld(r);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) r[i] = live ? r[i] : -CUDART_INF_F;
+        const float red = warp_reduce16<true>(r, lane) * cscale;
+        const int col = c * 16 + col16(lane);
+        const float old = -nm[col], now = fmaxf(old, red);
+        __syncwarp();
+        if ((lane & 1) == 0) { nm[col] = -now; w[col] = fast_ex2(old - now); }
+        __syncwarp();
+        for (int u = group; u < t; u += 2) {
+            const int slot = first_slot + u;
+            const uint32_t at = lane_base + static_cast<uint32_t>((slot >= slots ? slot - slots : slot) * width + c * 16);
+            float e[16];
+            tmem_issue16(at, e);
+            tmem_wait_ld(e);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) e[i] *= w[c * 16 + i];
+            tmem_st16(at, e);
+        }
+    }
+    tmem_wait_st();
+}
+
+// A warp's exponentials and sums for its tiles of a job and N chunks of 16 text queries from chunk c0 on, tile by tile
+// (as they arrive, when c0 = 0): exponentials against a reference of the warp's own (the logits of its first key), back to
+// tensor memory.  The reference need not be the maximum -- fp32 is as precise at 2^40 as at 1 -- so no pass over the
+// tiles and no reduction comes before the exponentials; only an exponent that could overflow moves it.
+template <int N>
+__device__ __forceinline__ void soft_exps(const SoftJob& j, StreamSmem& sm, int c0, int warp, int lane, int* status)
+{
+    const int group = warp >> 2, first_key = (warp & 3) * 32;
+    float* const nm = sm.m[warp] + c0 * 16;
+    float* const my_w = sm.w[warp] + c0 * 16;
+    const float2 cs2 = make_float2(j.cscale, j.cscale);
+    float2 sum[N * 8];
+#pragma unroll
+    for (int i = 0; i < N * 8; ++i) sum[i] = make_float2(0.f, 0.f);
+    bool have_ref = false;
+#pragma unroll 1
+    for (int t = group; t < j.tr.count; t += 2) {
+        const int valid = j.tr.valid(t);
+        const bool live = first_key + lane < valid;
+        const uint32_t cols = j.cols(t) + c0 * 16;
+        if (c0 == 0) {
+            ring_wait<false>(smem_u32(&sm.tfull[j.slot(t)]), j.parity(t), &sm.aborted, status);
+            __syncwarp();
+            tc_fence_after();
+        }
+        if (first_key >= valid) continue;                      // no key of this warp in a ragged tile
+        float v[N][16];
+#pragma unroll 1
+        for (;;) {
+#pragma unroll
+            for (int c = 0; c < N; ++c) tmem_issue16(cols + c * 16, v[c]);
+#pragma unroll
+            for (int c = 0; c < N; ++c) tmem_wait_ld(v[c]);
+            if (valid < kKeyTile) {                            // a ragged tile (uniform; the empty statement keeps it a branch)
+                asm volatile("" ::: "memory");
+#pragma unroll
+                for (int c = 0; c < N; ++c)
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[c][i] = live ? v[c][i] : -CUDART_INF_F;
+            }
+            if (!have_ref) {                                   // warp-uniform
+                have_ref = true;
+                if (lane == 0)
+#pragma unroll
+                    for (int c = 0; c < N; ++c)
+#pragma unroll
+                        for (int i = 0; i < 16; i += 4)
+                            *reinterpret_cast<float4*>(&nm[c * 16 + i]) = make_float4(-v[c][i] * j.cscale, -v[c][i + 1] * j.cscale,
+                                                                                      -v[c][i + 2] * j.cscale, -v[c][i + 3] * j.cscale);
+                __syncwarp();
+            }
+            float top[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll
+            for (int c = 0; c < N; ++c)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 m4 = *reinterpret_cast<const float4*>(&nm[c * 16 + 4 * i]);
+                    const float2 y0 = fma2(make_float2(v[c][4 * i], v[c][4 * i + 1]), cs2, make_float2(m4.x, m4.y));
+                    const float2 y1 = fma2(make_float2(v[c][4 * i + 2], v[c][4 * i + 3]), cs2, make_float2(m4.z, m4.w));
+                    v[c][4 * i] = y0.x; v[c][4 * i + 1] = y0.y; v[c][4 * i + 2] = y1.x; v[c][4 * i + 3] = y1.y;
+                    top[i] = fmaxf(top[i], fmaxf(fmaxf(y0.x, y0.y), fmaxf(y1.x, y1.y)));
+                }
+            if (!__any_sync(0xffffffffu, fmaxf(fmaxf(top[0], top[1]), fmaxf(top[2], top[3])) > kRescaleAt)) break;
+            raise_references(cols, j.lane_base + c0 * 16, j.slot0, j.slots, j.width, t, group, N, j.cscale, live, nm, my_w);
+#pragma unroll
+            for (int i = 0; i < N * 8; ++i) { sum[i].x *= my_w[2 * i]; sum[i].y *= my_w[2 * i + 1]; }
+            __syncwarp();
+        }
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                v[c][2 * i] = fast_ex2(v[c][2 * i]);
+                v[c][2 * i + 1] = fast_ex2(v[c][2 * i + 1]);
+                sum[c * 8 + i] = add2(sum[c * 8 + i], make_float2(v[c][2 * i], v[c][2 * i + 1]));
+            }
+            tmem_st16(cols + c * 16, v[c]);
+        }
+    }
+    if (!have_ref && lane < N * 16) nm[lane] = CUDART_INF_F;   // no key of this warp in the whole job
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+        float r[16];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { r[2 * i] = sum[c * 8 + i].x; r[2 * i + 1] = sum[c * 8 + i].y; }
+        const float red = warp_reduce16<false>(r, lane);
+        if ((lane & 1) == 0) my_w[c * 16 + col16(lane)] = red;
+    }
+}
+
+// Per key, the sum of its exponentials weighted by sm.w[warp] (the normalised, head-averaged attention mass), added into
+// the accumulators; a tile's slot is free once the four warps of its group are done.
+__device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, int nch, int warp, int lane)
+{
+    const int key = (warp & 3) * 32 + lane;
+    const float* const my_w = sm.w[warp];
+#pragma unroll 1
+    for (int t = warp >> 2; t < j.tr.count; t += 2) {
+        const uint32_t cols = j.cols(t);
+        float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        auto add16 = [&](const float (&v)[16], int c) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 w4 = *reinterpret_cast<const float4*>(&my_w[c * 16 + 4 * i]);
+                acc[0] = fma2(make_float2(v[4 * i], v[4 * i + 1]), make_float2(w4.x, w4.y), acc[0]);
+                acc[1] = fma2(make_float2(v[4 * i + 2], v[4 * i + 3]), make_float2(w4.z, w4.w), acc[1]);
+            }
+        };
+        int c = 0;
+#pragma unroll 1
+        for (; c + 2 <= nch; c += 2) {
+            float v0[16], v1[16];
+            tmem_issue16(cols + c * 16, v0);
+            tmem_issue16(cols + c * 16 + 16, v1);
+            tmem_wait_ld(v0);
+            tmem_wait_ld(v1);
+            add16(v0, c);
+            add16(v1, c + 1);
+        }
+        if (c < nch) {
+            float v0[16];
+            tmem_issue16(cols + c * 16, v0);
+            tmem_wait_ld(v0);
+            add16(v0, c);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sm.tempty[j.slot(t)]));
+        const float a = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
+        if (key < j.tr.valid(t)) atomicAdd(j.acc + j.tr.vis0(t) + key, __float2ull_rn(a * kFixScale));
+    }
+    __syncwarp();
+}
+
+// grid = clusters x cluster size (1-D), kStreamThreads threads, one CTA per multiprocessor.
+__global__ void __launch_bounds__(kStreamThreads, 1)
+salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,
+                       const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ StreamArgs a)
+{
+    const int W = a.width;
+    extern __shared__ uint8_t dyn_smem_raw[];
+    uint8_t* dyn = dyn_smem_raw + ((1024u - (smem_u32(dyn_smem_raw) & 1023u)) & 1023u);   // swizzle atoms are 1 KB
+    __shared__ StreamSmem sm;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t csize, crank = cluster_ctarank();
+    asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(csize));
+    const int lg = 31 - __clz(csize);                    // cluster sizes are powers of two
+    const int first_job = blockIdx.x >> lg, job_step = gridDim.x >> lg;
+    const int b_step = job_step / a.n_heads, h_step = job_step - b_step * a.n_heads;
+    const int b_first = first_job / a.n_heads, h_first = first_job - b_first * a.n_heads;
+    // the next job's sample and head
+    auto advance = [&](int& b, int& h) {
+        b += b_step;
+        h += h_step;
+        if (h >= a.n_heads) { h -= a.n_heads; ++b; }
+    };
+    const int khalves = (a.head_dim * a.esize + 127) / 128;
+    uint8_t* const Qs = dyn + static_cast<size_t>(a.stages) * kStageBytes;      // two buffers of khalves x W rows x 128 B
+    const uint32_t q_bytes = static_cast<uint32_t>(khalves) * (W * 128);
+
+    if (tid == 0) {
+        for (int i = 0; i < a.stages; ++i) { mbar_init(smem_u32(&sm.kfull[i]), 1); mbar_init(smem_u32(&sm.kempty[i]), 1); }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_u32(&sm.qfull[i]), 1); mbar_init(smem_u32(&sm.qempty[i]), 1);
+        }
+        for (int i = 0; i < kPairBufs; ++i) mbar_init(smem_u32(&sm.xbar[i]), 1);
+        for (int i = 0; i < a.slots; ++i) { mbar_init(smem_u32(&sm.tfull[i]), 1); mbar_init(smem_u32(&sm.tempty[i]), 4); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        sm.aborted = 0;
+    }
+    // all 512 columns: the launcher's shared-memory footprint keeps every other user of tensor memory off this multiprocessor
+    if (warp == kSoftWarps + 1) tmem_alloc(smem_u32(&sm.tmem), kTmemColsPerSm);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (csize > 1) {                          // no pair may be sent to a CTA that has not set up its barriers
+        cluster_arrive_release();
+        cluster_wait_acquire();
+    }
+    const uint32_t tmem_base = sm.tmem;
+    volatile int* const aborted = &sm.aborted;
+
+    // The loading warp and the MMA warp run their loops as whole warps, all values the same in every lane, and one
+    // elected lane issues: coordinates and descriptors then stay in uniform registers.  (As a single-thread branch the
+    // same loops moved every operand there one by one: 1.0 us per key tile instead of 0.25.)
+    if (warp == kSoftWarps) {
+        // ---------------------------------------------------------------- loads
+        const bool one = elect_one();
+        if (one) {
+            prefetch_tensormap(&tmap_q);
+            prefetch_tensormap(&tmap_k);
+        }
+        if (!a.free_running) pdl_wait();
+        if (a.stamps && one && blockIdx.x < kStampSlots) a.stamps[2 * blockIdx.x] = global_ns();
+        pdl_trigger();                        // whatever the kernel before this one wrote is complete
+        const int box_elems = 128 / a.esize;
+        int stage = 0, n_live = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int job = first_job, b = b_first, h = h_first; ok && job < a.n_jobs; job += job_step, advance(b, h)) {
+            const SampleDev& s = bd.s[b];
+            const JobTiles tr(s, crank, lg);
+            if (tr.count == 0) continue;
+            const int npad = (s.n_txt + 15) & ~15, qb = n_live & 1;
+            const int row_2d = s.seq_off + s.off_2d, row_3d = s.seq_off + s.off_3d, row_q = s.seq_off + s.off_txt;
+            ok = ring_wait<false>(smem_u32(&sm.qempty[qb]), ((n_live >> 1) & 1) ^ 1, aborted, a.status);
+            if (!ok) break;
+            if (one) {
+                const uint32_t qbar = smem_u32(&sm.qfull[qb]);
+                mbar_expect_tx(qbar, static_cast<uint32_t>(khalves * npad) * 128u);
+                for (int kh = 0; kh < khalves; ++kh)
+                    for (int c = 0; c < npad / 16; ++c)
+                        tma_load_3d(smem_u32(Qs + qb * q_bytes + kh * npad * 128 + c * 2048), &tmap_q, kh * box_elems, h,
+                                    row_q + c * 16, qbar);
+            }
+            ++n_live;
+            const int hk = h / a.kv_group;
+            for (int t = 0; ok && t < tr.count; ++t) {
+                const int g = tr.first + t, row0 = g < tr.t2 ? row_2d + g * kKeyTile : row_3d + (g - tr.t2) * kKeyTile;
+                for (int kh = 0; kh < khalves; ++kh) {
+                    ok = ring_wait<false>(smem_u32(&sm.kempty[stage]), phase ^ 1, aborted, a.status);
+                    if (!ok) break;
+                    if (one) {
+                        const uint32_t bar = smem_u32(&sm.kfull[stage]);
+                        mbar_expect_tx(bar, kStageBytes);
+                        tma_load_3d(smem_u32(dyn) + static_cast<uint32_t>(stage) * kStageBytes, &tmap_k, kh * box_elems, hk, row0, bar);
+                    }
+                    if (++stage == a.stages) { stage = 0; phase ^= 1; }
+                }
+            }
+        }
+        if (!ok) {                            // gave up: let the copies in flight land before the CTA may end
+            const uint64_t t0 = global_ns();
+            while (global_ns() - t0 < 1000000ull) { }
+        }
+    } else if (warp == kSoftWarps + 1) {
+        // ---------------------------------------------------------------- MMAs
+        const bool one = elect_one();
+        const int ksteps = (a.head_dim * a.esize + 31) / 32;       // an instruction consumes 32 bytes of every row
+        const uint64_t k_desc0 = smem_desc_sw128(smem_u32(dyn)), q_desc0 = smem_desc_sw128(smem_u32(Qs));   // (addresses / 16 in the low bits)
+        int stage = 0, slot = 0, n_live = 0;
+        uint32_t phase = 0, sphase = 0;
+        bool ok = true;
+        for (int job = first_job, b = b_first, h = h_first; ok && job < a.n_jobs; job += job_step, advance(b, h)) {
+            const SampleDev& s = bd.s[b];
+            const JobTiles tr(s, crank, lg);
+            if (tr.count == 0) continue;
+            const int npad = (s.n_txt + 15) & ~15, qb = n_live & 1;
+            const uint32_t idesc = idesc_by_size(a.esize, npad);
+            ok = ring_wait<false>(smem_u32(&sm.qfull[qb]), (n_live >> 1) & 1, aborted, a.status);
+            ++n_live;
+            for (int t = 0; ok && t < tr.count; ++t) {
+                ok = ring_wait<false>(smem_u32(&sm.tempty[slot]), sphase ^ 1, aborted, a.status);
+                for (int kh = 0; ok && kh < khalves; ++kh) {
+                    ok = ring_wait<false>(smem_u32(&sm.kfull[stage]), phase, aborted, a.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t kd = k_desc0 + static_cast<uint64_t>(stage) * (kStageBytes >> 4);
+                    const uint64_t qd = q_desc0 + ((static_cast<uint64_t>(qb) * q_bytes + static_cast<uint64_t>(kh * npad) * 128) >> 4);
+                    if (one) {
+                        const int n = min(4, ksteps - kh * 4);
+                        if (a.esize == 2)
+                            for (int kb = 0; kb < n; ++kb) umma_bf16(tmem_base + slot * W, kd + 2 * kb, qd + 2 * kb, idesc, kh + kb > 0 ? 1u : 0u);
+                        else
+                            for (int kb = 0; kb < n; ++kb) umma_e4m3(tmem_base + slot * W, kd + 2 * kb, qd + 2 * kb, idesc, kh + kb > 0 ? 1u : 0u);
+                        umma_commit(smem_u32(&sm.kempty[stage]));
+                    }
+                    if (++stage == a.stages) { stage = 0; phase ^= 1; }
+                }
+                if (!ok) break;
+                if (one) umma_commit(smem_u32(&sm.tfull[slot]));
+                if (++slot == a.slots) { slot = 0; sphase ^= 1; }
+            }
+            if (ok && one) umma_commit(smem_u32(&sm.qempty[qb]));
+        }
+    } else {
+        // ---------------------------------------------------------------- softmax
+        SoftJob j;
+        j.slot0 = 0; j.slots = a.slots; j.width = W; j.parity0 = 0;
+        j.lane_base = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        j.cscale = 1.4426950408889634f * rsqrtf(static_cast<float>(a.head_dim));   // log2 domain
+        float* const my_w = sm.w[warp];
+        bool waited = a.free_running != 0;
+        int jn = 0;
+        for (int job = first_job, b = b_first, h = h_first; job < a.n_jobs; job += job_step, ++jn, advance(b, h)) {
+            const SampleDev& s = bd.s[b];
+            j.tr = JobTiles(s, crank, lg);
+            j.acc = a.acc64 + s.vis_off;
+            const int n_txt = s.n_txt, npad = (n_txt + 15) & ~15;
+            if (a.rearm && h == 0 && crank == 0)      // the tail kernel's hand-over words; their last users finished long ago
+                for (int i = tid; i < s.n_out; i += kSoftThreads) a.rearm[s.out_off + i] = -1;
+            const int nch = npad >> 4;
+            {
+                int c = 0;
+                for (; c + 2 <= nch; c += 2) soft_exps<2>(j, sm, c, warp, lane, a.status);
+                if (c < nch) soft_exps<1>(j, sm, c, warp, lane, a.status);
+                tmem_wait_st();
+            }
+            soft_barrier();
+            // ---- one thread per query: the pairs of the warps, then those of the cluster's CTAs
+            if (tid < npad) {
+                float mk[kSoftWarps], mx = -CUDART_INF_F, z = 0.f;
+#pragma unroll
+                for (int k = 0; k < kSoftWarps; ++k) { mk[k] = -sm.m[k][tid]; mx = fmaxf(mx, mk[k]); }
+#pragma unroll
+                for (int k = 0; k < kSoftWarps; ++k)
+                    if (mk[k] > -CUDART_INF_F) z += sm.w[k][tid] * fast_ex2(mk[k] - mx);
+                if (csize > 1) {
+                    const int xb = jn & (kPairBufs - 1);
+                    const uint32_t xbar = smem_u32(&sm.xbar[xb]);
+                    // (pairs may land before the count is armed: the phase cannot complete without this arrival)
+                    if (tid == 0) mbar_expect_tx(xbar, csize * static_cast<uint32_t>(npad) * 8u);
+                    for (uint32_t r = 0; r < csize; ++r) st_async_pair(smem_u32(&sm.peer[xb][crank][tid]), xbar, r, make_float2(mx, z));
+                    ring_wait<true>(xbar, (jn / kPairBufs) & 1, &sm.aborted, a.status);
+                    mx = -CUDART_INF_F;
+                    z = 0.f;
+                    for (uint32_t r = 0; r < csize; ++r) mx = fmaxf(mx, sm.peer[xb][r][tid].x);
+                    for (uint32_t r = 0; r < csize; ++r) {
+                        const float2 p = sm.peer[xb][r][tid];
+                        if (p.x > -CUDART_INF_F) z += p.y * fast_ex2(p.x - mx);
+                    }
+                }
+                sm.g[tid] = mx;
+                sm.iz[tid] = tid < n_txt && z > 0.f ? 1.f / z / (static_cast<float>(a.n_heads) * static_cast<float>(n_txt)) : 0.f;
+            }
+            if (!waited) { pdl_wait(); waited = true; }      // the accumulators were read and cleared by an earlier selection
+            soft_barrier();
+            for (int i = lane; i < npad; i += 32) {          // this warp's exponentials -> normalised, head-averaged
+                const float mk = -sm.m[warp][i];
+                my_w[i] = mk == -CUDART_INF_F ? 0.f : fast_ex2(mk - sm.g[i]) * sm.iz[i];
+            }
+            __syncwarp();
+            soft_scores(j, sm, nch, warp, lane);
+            j.slot0 += j.tr.count;
+            if (j.slot0 >= a.slots) { j.slot0 -= a.slots; j.parity0 ^= 1u; }
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == kSoftWarps + 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, kTmemColsPerSm);
+    }
+    if (csize > 1) {                          // a CTA that gave up must not leave while a peer may still send to it
+        cluster_arrive_release();
+        cluster_wait_acquire();
+    }
+    if (a.stamps && tid == 0 && blockIdx.x < kStampSlots) a.stamps[2 * blockIdx.x + 1] = global_ns();
+}
+
+int padded_text(const BatchDesc& bd)
+{
+    int n = 1;
+    for (int b = 0; b < bd.n; ++b) n = std::max(n, bd.s[b].n_txt);
+    return (n + 15) / 16 * 16;
+}
+int max_tiles(const BatchDesc& bd)
+{
+    int t = 1;
+    for (int b = 0; b < bd.n; ++b)
+        t = std::max(t, (bd.s[b].n_2d + kKeyTile - 1) / kKeyTile + (bd.s[b].n_3d + kKeyTile - 1) / kKeyTile);
+    return t;
+}
+
+cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUtensorMap* tk, StreamArgs& a, int cluster,
+                            int sms, size_t smem, cudaStream_t stream)
+{
+    auto kern = salience_stream_kernel;
+    static KernelSetup ks;
+    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kStreamThreads, smem, kTmemColsPerSm);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(sms / cluster * cluster));
+    cfg.blockDim = dim3(kStreamThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1] = pdl_attribute();
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    // Clusters that run at once: fewer than multiprocessors / cluster size (a cluster lies inside a GPC: 33 of 4, 15 of 8
+    // on a B200), and a second wave of a persistent grid would double its time.  The shared-memory footprint is the same
+    // for every launch, so the answer is looked up once per size.
+    static std::atomic<int> fits[kMaxCluster + 1];
+    int n = fits[cluster].load(std::memory_order_relaxed);
+    if (n == 0) {
+        cfg.numAttrs = 1;
+        const cudaError_t eo = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+        if (eo != cudaSuccess) return eo;
+        if (n < 1) return cudaErrorInvalidConfiguration;
+        fits[cluster].store(n, std::memory_order_relaxed);
+        cfg.numAttrs = 2;
+    }
+    cfg.gridDim = dim3(static_cast<unsigned>(std::min(a.n_jobs, n) * cluster));
+    return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, a);
+}
+
+}  // namespace
+
+cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
+                                   const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
+                                   bool free_running, int32_t* rearm, unsigned long long* stamps, cudaStream_t stream)
+{
+    const int sms = sm_count_of_current_device();
+    const int npad = padded_text(bd), tiles = max_tiles(bd);
+    StreamArgs a;
+    a.n_heads = n_heads; a.kv_group = kv_group; a.head_dim = head_dim; a.esize = esize;
+    a.width = npad;
+    a.slots = std::min(kMaxSlots, kTmemColsPerSm / npad);
+    a.n_jobs = bd.n * n_heads;
+    a.acc64 = acc64; a.status = status; a.free_running = free_running ? 1 : 0; a.rearm = rearm; a.stamps = stamps;
+    // The smallest cluster whose CTAs hold their share of a job's logits in tensor memory; a larger one while jobs are
+    // fewer than multiprocessors and the tiles can still be shared out.
+    int cluster = 1;
+    while (cluster < kMaxCluster && ((tiles + cluster - 1) / cluster > a.slots || (a.n_jobs * cluster * 2 <= sms && cluster * 2 <= tiles)))
+        cluster *= 2;
+    if ((tiles + cluster - 1) / cluster > a.slots) return cudaErrorInvalidConfiguration;
+    const size_t q_bytes = 2 * static_cast<size_t>((head_dim * esize + 127) / 128) * npad * 128;
+    a.stages = static_cast<int>(std::min<size_t>(kMaxStages, (kStreamSmem - 1024 - q_bytes) / kStageBytes));
+    if (a.stages < 4) return cudaErrorInvalidConfiguration;
+    return launch_stream(bd, tmap_q, tmap_k, a, cluster, sms, kStreamSmem, stream);
+}
+
+}  // namespace mvla

@@ -729,3 +729,50 @@ def test_step_with_two_threads_per_key_in_every_shape_of_the_scoring_kernel(n_tx
     for t in range(2):
         run_and_check_step(ctx, wl, t, states)
     ctx.close()
+
+
+@pytest.mark.parametrize("batch,H,n_txt,n_2d,n_3d,kw", [
+    (8, 16, (1, 16, 17, 64), (128, 129, 1), (255, 300, 513), {}),            # every padded text length; ragged tiles of one key up
+    (12, 16, (5, 9), (130, 40), (37, 200), {"dtype": "fp8"}),                # 8-bit keys, 16-query slots
+    (10, 16, (33, 48), (256, 100), (129, 384), {"n_kv_heads": 4}),           # grouped key heads
+    (9, 16, (40, 20), (200, 60), (70, 300), {"d": 96}),                      # a partial swizzle row
+    (6, 8, (64, 3), (1000, 700), (900, 1047), {"d": 256}),                   # two stages per tile; clusters of two
+    (1, 4, (64,), (2048,), (2048,), {"D": 512}),                             # the most tiles: clusters of eight
+    (2, 4, (17, 50), (1500, 2000), (1200, 77), {"text_first": True})])       # more than 2048 tokens, 1024-thread tail
+def test_streaming_scoring_kernel_at_the_edges_of_its_shapes(batch, H, n_txt, n_2d, n_3d, kw):
+    """Batches whose CTAs do not all run at once, and samples of more than 16 key tiles, go through the streaming
+    scoring kernel; two action steps, so that its ring state and the accumulators it leaves are exercised twice."""
+    kw = {"D": 256, "d": 64, **kw}
+    wl = W.small_workload(71, batch=batch, H=H, n_txt=n_txt, n_2d=n_2d, n_3d=n_3d, keep=(0.3, 0.5, 0.2), steps=2, **kw)
+    ctx = mvla.context_for(wl)
+    states = [oracle.State(s.n_vis) for s in wl.samples]
+    for step in range(2):
+        if "n_kv_heads" not in kw:
+            run_and_check_step(ctx, wl, step, states)
+            continue
+        t, dev = wl.steps[step], device_tensors(wl, step)        # the oracle's step takes ungrouped keys: scores only
+        out = ctx.prune_step(0, wl.samples, wl.mode, dev["q"], dev["k"], dev["v"], dev["hidden"])
+        attn, vis = out.attn.cpu().numpy(), 0
+        for s in wl.samples:
+            assert_salience_close(attn[vis:vis + s.n_vis], oracle.salience_gqa(t.q, t.k, H, kw["n_kv_heads"], kw["d"], s))
+            vis += s.n_vis
+    ctx.close()
+
+
+@pytest.mark.parametrize("gain", [30.0, 300.0])
+def test_streaming_scoring_kernel_moves_its_references_when_exponents_would_overflow(gain):
+    """Keys whose logits grow from tile to tile by far more than an fp32 exponent holds."""
+    wl = W.small_workload(72, batch=10, D=256, H=16, d=64, n_txt=(20, 33), n_2d=(300, 128), n_3d=(260, 400))
+    t = wl.steps[0]
+    for s in wl.samples:
+        for off, n in ((s.off_2d, s.n_2d), (s.off_3d, s.n_3d)):
+            k = t.k[s.seq_off + off: s.seq_off + off + n]
+            k *= (1.0 + gain * (np.arange(n) // 128)).astype(np.float32)[:, None, None]
+    t.k[:] = W.round_to_dtype(t.k, "bf16")
+    ctx, dev = mvla.context_for(wl), device_tensors(wl)
+    out = ctx.prune_step(0, wl.samples, wl.mode, dev["q"], dev["k"], dev["v"], dev["hidden"])
+    attn, vis = out.attn.cpu().numpy(), 0
+    for s in wl.samples:
+        assert_salience_close(attn[vis:vis + s.n_vis], oracle.salience_gqa(t.q, t.k, 16, 16, 64, s))
+        vis += s.n_vis
+    ctx.close()
