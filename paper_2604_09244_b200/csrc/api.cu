@@ -361,7 +361,8 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     }
     cudaError_t e;
     const bool streaming = ctx->use_umma && acc64 && !alpha.ptr && !with_cache && stream_pays(ctx, bd, tiles_per_cta, cluster);
-    const bool fast = streaming || (ctx->use_umma && fast_salience_supported(tiles_per_cta));
+    const bool f32 = c.dtype == MVLA_DTYPE_FP32 && acc64 && !alpha.ptr && f32_salience_supported(tiles_per_cta, npad, c.head_dim);
+    const bool fast = streaming || f32 || (ctx->use_umma && fast_salience_supported(tiles_per_cta));
     // The norms do not depend on the scores: with `norms_beside` (fast kernel only) they are launched AFTER
     // the scoring kernel and run beside it instead of in front of it.
     norms_beside = norms_beside && fast;
@@ -372,6 +373,10 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     if (streaming) {
         e = launch_salience_stream(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk, acc64,
                                    ctx->status_dev, free_running, rearm, stamps, st);
+        if (used_acc64) *used_acc64 = true;
+    } else if (f32) {
+        e = launch_salience_f32(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<const float*>(q), static_cast<const float*>(k),
+                                tiles_per_cta, cluster, npad, acc64, ctx->status_dev, rearm, stamps, st);
         if (used_acc64) *used_acc64 = true;
     } else if (fast) {
         e = launch_salience_fast(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk,

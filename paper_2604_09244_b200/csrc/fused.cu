@@ -58,6 +58,151 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
     return false;
 }
 
+// Shared memory of the softmax part.
+struct FastSmem {
+    float m[kMaxText];                       // local max per query (scaled, log2 domain), -inf replaced by 0
+    alignas(16) float w[kMaxText];           // final weight per query
+    float2 peer[kMaxCluster][kMaxText];      // (raw local max, local sum) of every CTA of the cluster
+    float2 loc[kMaxText];                    // this CTA's pairs, staged for the push
+    float wred[4][kMaxText];
+};
+// What the softmax part writes.
+struct FastOut {
+    float* part;
+    int64_t part_stride;
+    unsigned long long* acc64;
+    int* status;
+    int free_running, n_heads;
+    AlphaOut alpha;
+};
+
+// From the raw dot products of this thread's key(s) -- L[t * TC + i]: tile t, text query c0 + i -- to the outputs.
+// vis0[t], valid[t]: the tiles' first visual index and number of keys.
+template <int TCOL, int NTILE, int SPLIT>
+__device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT], const SampleDev& s, const int (&valid)[NTILE],
+                                               const int (&vis0)[NTILE], bool ok, int npad, int h, float cscale, uint32_t bar_x,
+                                               FastSmem& sm, const FastOut& o)
+{
+    constexpr int TC = TCOL / SPLIT, NT = kFastThreads * SPLIT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int key = tid & (kFastThreads - 1), kwarp = warp & 3, c0 = (tid / kFastThreads) * TC;
+    const uint32_t crank = cluster_ctarank(), csize = gridDim.x;
+    // The registers keep the raw dot products; the scale enters with the exponent below (one FFMA).  Keys
+    // past the end of a ragged tile are masked; a full tile needs no pass over the registers at all, and
+    // columns past the padded query count are never looked at.
+#pragma unroll
+    for (int t = 0; t < NTILE; ++t) {
+        if (ok && valid[t] == kKeyTile) continue;         // block-uniform
+        const bool live = ok && key < valid[t];
+#pragma unroll
+        for (int i = 0; i < TC; ++i) L[t * TC + i] = live ? L[t * TC + i] : -CUDART_INF_F;
+    }
+
+    // ---- local maximum per query
+#pragma unroll
+    for (int qc = 0; qc < TC / 16; ++qc) {
+        if (c0 + qc * 16 >= npad) break;
+        float m[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            m[i] = L[qc * 16 + i];
+#pragma unroll
+            for (int t = 1; t < NTILE; ++t) m[i] = fmaxf(m[i], L[t * TC + qc * 16 + i]);
+        }
+        const float red = warp_reduce16<true>(m, lane);
+        if ((lane & 1) == 0) sm.wred[kwarp][c0 + qc * 16 + col16(lane)] = red;
+    }
+    __syncthreads();
+    float m_raw = -CUDART_INF_F;
+    if (tid < npad) {
+        m_raw = fmaxf(fmaxf(sm.wred[0][tid], sm.wred[1][tid]), fmaxf(sm.wred[2][tid], sm.wred[3][tid])) * cscale;
+        sm.m[tid] = (m_raw == -CUDART_INF_F) ? 0.f : m_raw;
+    }
+    __syncthreads();
+
+    // ---- exponentials (kept in registers) and the local denominator per query
+#pragma unroll
+    for (int qc = 0; qc < TC / 16; ++qc) {
+        if (c0 + qc * 16 >= npad) break;
+        float sum[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const float mm = sm.m[c0 + qc * 16 + i];
+            sum[i] = 0.f;
+#pragma unroll
+            for (int t = 0; t < NTILE; ++t) {
+                const float e = ex2_approx(fmaf(L[t * TC + qc * 16 + i], cscale, -mm));
+                L[t * TC + qc * 16 + i] = e;
+                sum[i] += e;
+            }
+        }
+        const float red = warp_reduce16<false>(sum, lane);
+        if ((lane & 1) == 0) sm.wred[kwarp][c0 + qc * 16 + col16(lane)] = red;
+    }
+    __syncthreads();
+
+    // ---- exchange (max, sum) with the other key tiles of this (sample, head)
+    if (tid < npad)
+        sm.loc[tid] = make_float2(m_raw, (sm.wred[0][tid] + sm.wred[1][tid]) + (sm.wred[2][tid] + sm.wred[3][tid]));
+    __syncthreads();
+    cluster_wait_acquire();                   // every peer is running and has initialised its barriers
+    for (int p = tid; p < npad * static_cast<int>(csize); p += NT) {
+        const int i = p % npad;
+        const uint32_t r = static_cast<uint32_t>(p / npad);
+        st_async_peer_f32x2(smem_u32(&sm.peer[crank][i]), bar_x, r, sm.loc[i]);
+    }
+    __syncwarp();
+    if (tid < npad) {                         // the warps that combine the pairs wait for them; the others park below
+        const bool okx = mbar_wait_cluster(bar_x, 0);
+        if (!okx) *reinterpret_cast<volatile int*>(o.status) = MVLA_ERR_TIMEOUT;
+        float gmax = -CUDART_INF_F;
+        for (uint32_t r = 0; r < csize; ++r) gmax = fmaxf(gmax, sm.peer[r][tid].x);
+        float z = 0.f;
+        for (uint32_t r = 0; r < csize; ++r) {
+            const float2 pr = sm.peer[r][tid];
+            if (pr.x > -CUDART_INF_F) z += pr.y * ex2_approx(pr.x - gmax);
+        }
+        const float inv_hn = 1.f / (static_cast<float>(o.n_heads) * static_cast<float>(s.n_txt));
+        sm.w[tid] = (tid < s.n_txt && z > 0.f && okx) ? ex2_approx(sm.m[tid] - gmax) / z * inv_hn : 0.f;
+    }
+    __syncthreads();
+
+    // ---- per key: sum over queries of the normalised probabilities (this head's contribution)
+    if (!o.free_running) pdl_wait();            // the accumulators were read and cleared by an earlier selection
+#pragma unroll
+    for (int t = 0; t < NTILE; ++t) {
+        if (valid[t] <= 0) continue;
+        float acc = 0.f;
+#pragma unroll
+        for (int qc = 0; qc < TC / 16; ++qc) {
+            if (c0 + qc * 16 >= npad) break;  // columns past the padded query count were never exponentiated
+#pragma unroll
+            for (int i = 0; i < 16; ++i)      // sm.w is 0 past the text queries
+                acc = fmaf(L[t * TC + qc * 16 + i], sm.w[c0 + qc * 16 + i], acc);
+        }
+        if (key < valid[t]) {
+            if (o.acc64)                        // (with SPLIT = 2 both halves of the queries add into the key's accumulator)
+                atomicAdd(o.acc64 + s.vis_off + vis0[t] + key, __float2ull_rn(acc * kFixScale));
+            if constexpr (SPLIT == 1) {
+                if (!o.acc64 && o.part)           // neither: the caller wants the attention copy only
+                    o.part[static_cast<int64_t>(h) * o.part_stride + s.vis_off + vis0[t] + key] = acc;
+                if (o.alpha.ptr) {              // the attention itself, for the per-patch indicators: this key's row of queries
+                    float4* ap = reinterpret_cast<float4*>(o.alpha.ptr + static_cast<int64_t>(h) * o.alpha.stride_h +
+                                                           static_cast<int64_t>(s.vis_off + vis0[t] + key) * o.alpha.stride_j);
+                    const float hn = static_cast<float>(o.n_heads) * static_cast<float>(s.n_txt);   // sm.w carries 1 / (H n_t)
+#pragma unroll
+                    for (int g4 = 0; g4 < TCOL / 4; ++g4) {   // 16-byte stores: a handful of instructions (sm.w is 0 past the text queries)
+                        if (4 * g4 >= npad || 4 * g4 >= o.alpha.stride_j) break;
+                        const float4 w4 = *reinterpret_cast<const float4*>(&sm.w[4 * g4]);
+                        ap[g4] = make_float4(L[t * TCOL + 4 * g4] * w4.x * hn, L[t * TCOL + 4 * g4 + 1] * w4.y * hn,
+                                             L[t * TCOL + 4 * g4 + 2] * w4.z * hn, L[t * TCOL + 4 * g4 + 3] * w4.w * hn);
+                    }
+                }
+            }
+        }
+    }
+}
+
 // grid = (cluster size, n_heads, samples), cluster = (cluster size, 1, 1), 128 x SPLIT threads.
 // TCOL: tensor-memory columns per tile (>= padded query count); NTILE: key tiles per CTA.
 // SPLIT: threads per key.  1: a thread holds all the logits of its key.  2 (fixed-point accumulators only, no
@@ -78,17 +223,13 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
     static_assert(TC % 16 == 0, "a thread holds whole groups of 16 queries");
     extern __shared__ uint8_t dyn_smem_raw[];
     uint8_t* dyn_smem = dyn_smem_raw + ((1024u - (smem_u32(dyn_smem_raw) & 1023u)) & 1023u);   // swizzle atoms are 1 KB
-    __shared__ float s_m[kMaxText];                       // local max per query (scaled, log2 domain), -inf replaced by 0
-    __shared__ alignas(16) float s_w[kMaxText];           // final weight per query
-    __shared__ float2 s_peer[kMaxCluster][kMaxText];      // (raw local max, local sum) of every CTA of the cluster
-    __shared__ float2 s_loc[kMaxText];                    // this CTA's pairs, staged for the push
-    __shared__ float s_wred[4][kMaxText];
+    __shared__ FastSmem sm;
     __shared__ __align__(8) uint64_t s_bar[3];
     __shared__ uint32_t s_tmem;
 
     const SampleDev& s = bd.s[blockIdx.z];
     const int h = blockIdx.y;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int key = tid & (kFastThreads - 1);            // key of the tile(s) this thread works on
     const int kwarp = warp & 3;                           // its warp among the four that cover the 128 keys (= tensor-memory lane quarter)
     const int c0 = (tid / kFastThreads) * TC;             // first of its text queries
@@ -152,7 +293,7 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
                 tma_load_3d(smem_u32(Ks + (t * khalves + kh) * 16384), &tmap_k, kh * box_elems, h / kv_group, row0, bar_full);
         }
     }
-    if (tid < kMaxText) s_w[tid] = 0.f;
+    if (tid < kMaxText) sm.w[tid] = 0.f;
     __syncwarp();
     cluster_arrive_release();                 // publishes this CTA's barriers; matched by the wait before the first remote store
     uint32_t tmem_cols = 32;
@@ -248,120 +389,8 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
             }
         }
     }
-    // The registers keep the raw dot products; the scale enters with the exponent below (one FFMA).  Keys
-    // past the end of a ragged tile are masked; a full tile needs no pass over the registers at all, and
-    // columns past the padded query count are never looked at.
-#pragma unroll
-    for (int t = 0; t < NTILE; ++t) {
-        if (ok && valid[t] == kKeyTile) continue;         // block-uniform
-        const bool live = ok && key < valid[t];
-#pragma unroll
-        for (int i = 0; i < TC; ++i) L[t * TC + i] = live ? L[t * TC + i] : -CUDART_INF_F;
-    }
-
-    // ---- local maximum per query
-#pragma unroll
-    for (int qc = 0; qc < TC / 16; ++qc) {
-        if (c0 + qc * 16 >= npad) break;
-        float m[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            m[i] = L[qc * 16 + i];
-#pragma unroll
-            for (int t = 1; t < NTILE; ++t) m[i] = fmaxf(m[i], L[t * TC + qc * 16 + i]);
-        }
-        const float red = warp_reduce16<true>(m, lane);
-        if ((lane & 1) == 0) s_wred[kwarp][c0 + qc * 16 + col16(lane)] = red;
-    }
-    __syncthreads();
-    float m_raw = -CUDART_INF_F;
-    if (tid < npad) {
-        m_raw = fmaxf(fmaxf(s_wred[0][tid], s_wred[1][tid]), fmaxf(s_wred[2][tid], s_wred[3][tid])) * cscale;
-        s_m[tid] = (m_raw == -CUDART_INF_F) ? 0.f : m_raw;
-    }
-    __syncthreads();
-
-    // ---- exponentials (kept in registers) and the local denominator per query
-#pragma unroll
-    for (int qc = 0; qc < TC / 16; ++qc) {
-        if (c0 + qc * 16 >= npad) break;
-        float sum[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float mm = s_m[c0 + qc * 16 + i];
-            sum[i] = 0.f;
-#pragma unroll
-            for (int t = 0; t < NTILE; ++t) {
-                const float e = ex2_approx(fmaf(L[t * TC + qc * 16 + i], cscale, -mm));
-                L[t * TC + qc * 16 + i] = e;
-                sum[i] += e;
-            }
-        }
-        const float red = warp_reduce16<false>(sum, lane);
-        if ((lane & 1) == 0) s_wred[kwarp][c0 + qc * 16 + col16(lane)] = red;
-    }
-    __syncthreads();
-
-    // ---- exchange (max, sum) with the other key tiles of this (sample, head)
-    if (tid < npad)
-        s_loc[tid] = make_float2(m_raw, (s_wred[0][tid] + s_wred[1][tid]) + (s_wred[2][tid] + s_wred[3][tid]));
-    __syncthreads();
-    cluster_wait_acquire();                   // every peer is running and has initialised its barriers
-    for (int p = tid; p < npad * static_cast<int>(csize); p += NT) {
-        const int i = p % npad;
-        const uint32_t r = static_cast<uint32_t>(p / npad);
-        st_async_peer_f32x2(smem_u32(&s_peer[crank][i]), bar_x, r, s_loc[i]);
-    }
-    __syncwarp();
-    if (tid < npad) {                         // the warps that combine the pairs wait for them; the others park below
-        const bool okx = mbar_wait_cluster(bar_x, 0);
-        if (!okx) *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
-        float gmax = -CUDART_INF_F;
-        for (uint32_t r = 0; r < csize; ++r) gmax = fmaxf(gmax, s_peer[r][tid].x);
-        float z = 0.f;
-        for (uint32_t r = 0; r < csize; ++r) {
-            const float2 pr = s_peer[r][tid];
-            if (pr.x > -CUDART_INF_F) z += pr.y * ex2_approx(pr.x - gmax);
-        }
-        const float inv_hn = 1.f / (static_cast<float>(n_heads) * static_cast<float>(s.n_txt));
-        s_w[tid] = (tid < s.n_txt && z > 0.f && okx) ? ex2_approx(s_m[tid] - gmax) / z * inv_hn : 0.f;
-    }
-    __syncthreads();
-
-    // ---- per key: sum over queries of the normalised probabilities (this head's contribution)
-    if (!free_running) pdl_wait();            // the accumulators were read and cleared by an earlier selection
-#pragma unroll
-    for (int t = 0; t < NTILE; ++t) {
-        if (valid[t] <= 0) continue;
-        float acc = 0.f;
-#pragma unroll
-        for (int qc = 0; qc < TC / 16; ++qc) {
-            if (c0 + qc * 16 >= npad) break;  // columns past the padded query count were never exponentiated
-#pragma unroll
-            for (int i = 0; i < 16; ++i)      // s_w is 0 past the text queries
-                acc = fmaf(L[t * TC + qc * 16 + i], s_w[c0 + qc * 16 + i], acc);
-        }
-        if (key < valid[t]) {
-            if (acc64)                        // (with SPLIT = 2 both halves of the queries add into the key's accumulator)
-                atomicAdd(acc64 + s.vis_off + vis0[t] + key, __float2ull_rn(acc * kFixScale));
-            if constexpr (SPLIT == 1) {
-                if (!acc64 && part)           // neither: the caller wants the attention copy only
-                    part[static_cast<int64_t>(h) * part_stride + s.vis_off + vis0[t] + key] = acc;
-                if (alpha.ptr) {              // the attention itself, for the per-patch indicators: this key's row of queries
-                    float4* ap = reinterpret_cast<float4*>(alpha.ptr + static_cast<int64_t>(h) * alpha.stride_h +
-                                                           static_cast<int64_t>(s.vis_off + vis0[t] + key) * alpha.stride_j);
-                    const float hn = static_cast<float>(n_heads) * static_cast<float>(s.n_txt);   // s_w carries 1 / (H n_t)
-#pragma unroll
-                    for (int g4 = 0; g4 < TCOL / 4; ++g4) {   // 16-byte stores: a handful of instructions (s_w is 0 past the text queries)
-                        if (4 * g4 >= npad || 4 * g4 >= alpha.stride_j) break;
-                        const float4 w4 = *reinterpret_cast<const float4*>(&s_w[4 * g4]);
-                        ap[g4] = make_float4(L[t * TCOL + 4 * g4] * w4.x * hn, L[t * TCOL + 4 * g4 + 1] * w4.y * hn,
-                                             L[t * TCOL + 4 * g4 + 2] * w4.z * hn, L[t * TCOL + 4 * g4 + 3] * w4.w * hn);
-                    }
-                }
-            }
-        }
-    }
+    softmax_scores<TCOL, NTILE, SPLIT>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
+                                       FastOut{part, part_stride, acc64, status, free_running, n_heads, alpha});
 
     tc_fence_before();
     __syncthreads();
@@ -369,6 +398,121 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
     if (stamps && tid == 0) {
         const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
         if (cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
+    }
+}
+
+// ------------------------------------------------------------------ fp32 inputs
+// The same chain for fp32 q / k: plain FMAs instead of the tensor cores (their fp32 forms round the operands).  Rows
+// arrive as bulk copies of d floats each, on a pitch of d + 4 (an odd number of 16-byte units, so that 16-byte reads of
+// neighbouring rows do not conflict); a thread computes the dot products of its key with its half of the text queries,
+// the key's piece in registers against broadcasts of the queries.  Dot products are summed in element order.
+// Bound by latency at the sizes this path serves (2.2 MB a step at 192 tokens, 8 heads x 64): the loads of all rows of a
+// CTA go out at once, where scalar loads through registers kept a few in flight, and the step runs as two chained
+// kernels like that of the other types (24.6 -> 14.8 us a step at that size).
+template <int TCOL, int NTILE>
+__global__ void __launch_bounds__(kFastThreads * 2, 1)
+salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restrict__ q, const float* __restrict__ k, int n_heads, int kv_group,
+                    int d, int npad_max, unsigned long long* __restrict__ acc64, int* status, int32_t* __restrict__ rearm,
+                    unsigned long long* __restrict__ stamps)
+{
+    constexpr int TC = TCOL / 2, NT = kFastThreads * 2;
+    extern __shared__ __align__(16) float rows[];         // [npad_max queries, then NTILE x 128 keys][d + 4]
+    __shared__ FastSmem sm;
+    __shared__ __align__(8) uint64_t s_bar[2];
+    const SampleDev& s = bd.s[blockIdx.z];
+    const int h = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int key = tid & (kFastThreads - 1), c0 = (tid / kFastThreads) * TC;
+    const int npad = min(npad_max, (s.n_txt + 15) & ~15);
+    const int tt0 = static_cast<int>(cluster_ctarank()) * NTILE;
+    const int pitch = d + 4;
+    const float cscale = 1.4426950408889634f * rsqrtf(static_cast<float>(d));   // log2 domain
+    const uint32_t bar_full = smem_u32(&s_bar[0]), bar_x = smem_u32(&s_bar[1]);
+    int valid[NTILE], vis0[NTILE];
+    TileInfo ti[NTILE];
+#pragma unroll
+    for (int t = 0; t < NTILE; ++t) {
+        ti[t] = tile_info(s, tt0 + t);
+        valid[t] = ti[t].valid;
+        vis0[t] = ti[t].vis0;
+    }
+    if (warp == 0) {                          // the loads go out first
+        if (lane == 0) {
+            mbar_init(bar_full, 1);
+            mbar_init(bar_x, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            mbar_expect_tx(bar_x, gridDim.x * static_cast<uint32_t>(npad) * 8u);
+            pdl_wait();
+            if (stamps) {
+                const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+                if (cta < kStampSlots) stamps[2 * cta] = global_ns();
+            }
+            int live = s.n_txt;
+#pragma unroll
+            for (int t = 0; t < NTILE; ++t) live += valid[t];
+            mbar_expect_tx(bar_full, static_cast<uint32_t>(live) * static_cast<uint32_t>(d) * 4u);
+        }
+        __syncwarp();
+        const uint32_t bytes = static_cast<uint32_t>(d) * 4u;
+        const int64_t qrow = static_cast<int64_t>(n_heads) * d, krow = static_cast<int64_t>(n_heads / kv_group) * d;
+        const float* qs = q + (static_cast<int64_t>(s.seq_off) + s.off_txt) * qrow + static_cast<int64_t>(h) * d;
+        for (int i = lane; i < s.n_txt; i += 32) bulk_load(smem_u32(rows + i * pitch), qs + i * qrow, bytes, bar_full);
+#pragma unroll
+        for (int t = 0; t < NTILE; ++t) {
+            const float* ks = k + static_cast<int64_t>(ti[t].row0) * krow + static_cast<int64_t>(h / kv_group) * d;
+            for (int i = lane; i < valid[t]; i += 32)
+                bulk_load(smem_u32(rows + (npad_max + t * kKeyTile + i) * pitch), ks + i * krow, bytes, bar_full);
+        }
+    } else {                                  // query rows that do not exist read as zero
+        for (int i = tid - 32; i < (npad - s.n_txt) * d; i += NT - 32) rows[(s.n_txt + i / d) * pitch + i % d] = 0.f;
+    }
+    if (tid < kMaxText) sm.w[tid] = 0.f;
+    __syncwarp();
+    cluster_arrive_release();                 // publishes this CTA's barriers; matched by the wait before the first remote store
+    __syncthreads();
+    pdl_trigger();                            // (see salience_fast_kernel)
+    if (rearm && blockIdx.x == 0 && blockIdx.y == 0)
+        for (int i = tid; i < s.n_out; i += NT) rearm[s.out_off + i] = -1;
+    bool ok = true;
+    if (tid == 0) {
+        ok = mbar_wait(bar_full, 0);
+        if (!ok) {                            // report, then give the copies one more bounded chance to land
+            *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
+            mbar_wait(bar_full, 0);
+        }
+    }
+    ok = __syncthreads_and(ok) != 0;
+    if (ok) mbar_wait(bar_full, 0);           // complete: makes the copied rows visible to every thread
+    float L[NTILE * TC];
+#pragma unroll
+    for (int i = 0; i < NTILE * TC; ++i) L[i] = 0.f;
+    if (c0 < npad) {
+#pragma unroll
+        for (int t = 0; t < NTILE; ++t) {
+            if (valid[t] <= 0) continue;
+            const float4* kr = reinterpret_cast<const float4*>(rows + (npad_max + t * kKeyTile + key) * pitch);
+#pragma unroll 2
+            for (int c = 0; c < d / 4; ++c) {
+                const float4 k4 = kr[c];
+#pragma unroll
+                for (int i = 0; i < TC; ++i) {
+                    const float4 q4 = *reinterpret_cast<const float4*>(rows + (c0 + i) * pitch + 4 * c);
+                    float& acc = L[t * TC + i];
+                    acc = fmaf(k4.x, q4.x, acc);
+                    acc = fmaf(k4.y, q4.y, acc);
+                    acc = fmaf(k4.z, q4.z, acc);
+                    acc = fmaf(k4.w, q4.w, acc);
+                }
+            }
+        }
+    }
+    softmax_scores<TCOL, NTILE, 2>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
+                                   FastOut{nullptr, 0, acc64, status, 0, n_heads, AlphaOut{nullptr, 0, 0}});
+    if (stamps) {
+        __syncthreads();
+        if (tid == 0) {
+            const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+            if (cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
+        }
     }
 }
 
@@ -403,7 +547,51 @@ cudaError_t launch_fast_t(const BatchDesc& bd, int n_heads, int kv_group, int he
     return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, n_heads, kv_group, head_dim, esize, npad, part, part_stride, acc64, status, free_running, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols);
 }
 
+template <int TCOL, int NTILE>
+cudaError_t launch_f32_t(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, const float* q, const float* k, int cluster, int npad,
+                         unsigned long long* acc64, int* status, int32_t* rearm, unsigned long long* stamps, cudaStream_t stream)
+{
+    const size_t smem = sizeof(float) * static_cast<size_t>(npad + NTILE * kKeyTile) * (head_dim + 4);
+    auto kern = salience_f32_kernel<TCOL, NTILE>;
+    static KernelSetup ks;
+    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kFastThreads * 2, smem, 0);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster, n_heads, bd.n);
+    cfg.blockDim = dim3(kFastThreads * 2);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1] = pdl_attribute();
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, bd, q, k, n_heads, kv_group, head_dim, npad, acc64, status, rearm, stamps);
+}
+
 }  // namespace
+
+// fp32: two key tiles per CTA at most, and all rows of a CTA in shared memory beside the kernel's own 9 KB.
+bool f32_salience_supported(int tiles_per_cta, int npad, int head_dim)
+{
+    return tiles_per_cta <= 2 && sizeof(float) * static_cast<size_t>(npad + tiles_per_cta * kKeyTile) * (head_dim + 4) <= 216 * 1024;
+}
+
+cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, const float* q, const float* k, int tiles_per_cta,
+                                int cluster, int npad, unsigned long long* acc64, int* status, int32_t* rearm, unsigned long long* stamps,
+                                cudaStream_t stream)
+{
+    if (!f32_salience_supported(tiles_per_cta, npad, head_dim)) return cudaErrorInvalidConfiguration;
+#define MVLA_F32(TC, NTL)                                                                                       \
+    if (npad <= TC && tiles_per_cta == NTL)                                                                     \
+        return launch_f32_t<TC, NTL>(bd, n_heads, kv_group, head_dim, q, k, cluster, npad, acc64, status, rearm, stamps, stream);
+    MVLA_F32(32, 1) MVLA_F32(64, 1) MVLA_F32(32, 2) MVLA_F32(64, 2)
+#undef MVLA_F32
+    return cudaErrorInvalidConfiguration;
+}
 
 bool fast_salience_supported(int tiles_per_cta) { return tiles_per_cta >= 1 && tiles_per_cta <= 2; }
 

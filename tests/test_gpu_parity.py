@@ -776,3 +776,22 @@ def test_streaming_scoring_kernel_moves_its_references_when_exponents_would_over
         assert_salience_close(attn[vis:vis + s.n_vis], oracle.salience_gqa(t.q, t.k, 16, 16, 64, s))
         vis += s.n_vis
     ctx.close()
+
+
+@pytest.mark.parametrize("n_txt,n_2d,n_3d,d,hkv", [
+    ((1, 17), (128, 1), (129, 40), 64, 0),                # one query, one key in a tile
+    ((33, 64), (100, 256), (300, 0), 128, 2),             # both halves of the queries; an empty modality; grouped keys
+    ((16, 48), (700, 513), (500, 640), 96, 0),            # two key tiles per CTA
+    ((20, 5), (130, 60), (200, 90), 256, 0)])             # the longest rows
+def test_fp32_step_at_the_edges_of_its_scoring_kernel(n_txt, n_2d, n_3d, d, hkv):
+    wl = W.small_workload(73, batch=2, D=256, H=4, d=d, dtype="fp32", n_txt=n_txt, n_2d=n_2d, n_3d=n_3d, n_kv_heads=hkv)
+    ctx, dev, t = mvla.context_for(wl), device_tensors(wl), wl.steps[0]
+    if not hkv:
+        run_and_check_step(ctx, wl, 0, [oracle.State(s.n_vis) for s in wl.samples])
+    else:
+        out = ctx.prune_step(0, wl.samples, wl.mode, dev["q"], dev["k"], dev["v"], dev["hidden"])
+        attn, vis = out.attn.cpu().numpy(), 0
+        for s in wl.samples:
+            assert_salience_close(attn[vis:vis + s.n_vis], oracle.salience_gqa(t.q, t.k, 4, hkv, d, s))
+            vis += s.n_vis
+    ctx.close()
