@@ -360,7 +360,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
         if (r != MVLA_OK) return r;
     }
     cudaError_t e;
-    const bool streaming = ctx->use_umma && acc64 && !alpha.ptr && !with_cache && stream_pays(ctx, bd, tiles_per_cta, cluster);
+    const bool streaming = ctx->use_umma && (acc64 || alpha.ptr) && !with_cache && stream_pays(ctx, bd, tiles_per_cta, cluster);
     const bool f32 = c.dtype == MVLA_DTYPE_FP32 && acc64 && !alpha.ptr && f32_salience_supported(tiles_per_cta, npad, c.head_dim);
     const bool fast = streaming || f32 || (ctx->use_umma && fast_salience_supported(tiles_per_cta));
     // The norms do not depend on the scores: with `norms_beside` (fast kernel only) they are launched AFTER
@@ -372,8 +372,8 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     }
     if (streaming) {
         e = launch_salience_stream(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk, acc64,
-                                   ctx->status_dev, free_running, rearm, stamps, st);
-        if (used_acc64) *used_acc64 = true;
+                                   ctx->status_dev, free_running, alpha, rearm, rearm_rec, stamps, st);
+        if (used_acc64) *used_acc64 = acc64 != nullptr;
     } else if (f32) {
         e = launch_salience_f32(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<const float*>(q), static_cast<const float*>(k),
                                 tiles_per_cta, cluster, npad, acc64, ctx->status_dev, rearm, stamps, st);
@@ -402,13 +402,6 @@ mvla_ctx::Range range_of(const void* p, size_t bytes)
 {
     const char* c = static_cast<const char*>(p);
     return {c, c ? c + bytes : c};
-}
-
-bool chunk_is_fast(const mvla_ctx* ctx, const Plan& plan, int first, int n)
-{
-    int max_tiles = 1;
-    for (int b = first; b < first + n; ++b) max_tiles = std::max(max_tiles, tiles_of(plan.s[b]));
-    return ctx->use_umma && fast_salience_supported((max_tiles + kMaxCluster - 1) / kMaxCluster);
 }
 
 GateParams gate_params(const mvla_ctx* ctx, int32_t mode, bool has_l1)
@@ -540,16 +533,13 @@ int32_t validate_patch(const mvla_ctx* ctx, int32_t batch, const mvla_sample* sa
     return MVLA_OK;
 }
 
-// Layout of the attention copy: [head][visual token of the batch][text query, padded to whole 128-byte lines]
-int64_t alpha_row(const mvla_ctx* ctx) { return (static_cast<int64_t>(ctx->cfg.max_text) + 31) / 32 * 32; }
-size_t alpha_floats(const mvla_ctx* ctx)
-{
-    return static_cast<size_t>(ctx->cfg.n_heads) * ctx->vis_all * static_cast<size_t>(alpha_row(ctx));
-}
+// Layout of the attention copy: [head][four text queries][visual token of the batch][4]
+int64_t alpha_head(const mvla_ctx* ctx) { return (static_cast<int64_t>(ctx->cfg.max_text) + 3) / 4 * static_cast<int64_t>(ctx->vis_all) * 4; }
+size_t alpha_floats(const mvla_ctx* ctx) { return static_cast<size_t>(ctx->cfg.n_heads) * static_cast<size_t>(alpha_head(ctx)); }
 
 AlphaOut alpha_of(const mvla_ctx* ctx, unsigned set)
 {
-    return AlphaOut{ctx->alpha_ws + set * alpha_floats(ctx), static_cast<int64_t>(ctx->vis_all) * alpha_row(ctx), alpha_row(ctx)};
+    return AlphaOut{ctx->alpha_ws + set * alpha_floats(ctx), alpha_head(ctx), static_cast<int64_t>(ctx->vis_all) * 4};
 }
 
 PatchParams patch_params(const mvla_ctx* ctx)
@@ -644,8 +634,7 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
     const unsigned par = ctx->step_parity;
     bool forked = false;
     ForkPlan fp;
-    if ((flags & MVLA_FLAG_INPUTS_STABLE) && ctx->patch_sets == kSets && batch <= kMaxChunk &&
-        chunk_is_fast(ctx, plan, 0, batch)) {
+    if ((flags & MVLA_FLAG_INPUTS_STABLE) && ctx->patch_sets == kSets && batch <= kMaxChunk && ctx->use_umma) {
         forked = true;
         const size_t nvis_b = static_cast<size_t>(plan.total_vis), npat_b = nvis_b / 2, in_rows = static_cast<size_t>(in->rows);
         const size_t hb = static_cast<size_t>(ctx->cfg.d_model) * ctx->elem, kb = static_cast<size_t>(kv_bytes);
@@ -671,7 +660,7 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
     float* attn = out->attn ? out->attn : ctx->patch_attn_ws + set * ctx->vis_all;
     float* x = out->patch_x ? out->patch_x : ctx->patch_x_ws + set * (ctx->vis_all / 2 + 1) * 4;
     const BatchDesc whole = chunk_of(plan, 0, std::min(batch, kMaxChunk));
-    if (!forked && batch <= kMaxChunk && chunk_is_fast(ctx, plan, 0, batch) && patch_tail_supported(whole)) {
+    if (!forked && batch <= kMaxChunk && ctx->use_umma && patch_tail_supported(whole)) {
         // two kernels: scoring (leaves the attention copy, re-arms the hand-over words), then indicators,
         // stages 1-4 and the row copy in one
         int32_t* list = ctx->tail_list + par * ctx->rows_all;
@@ -763,9 +752,12 @@ static int32_t mvla_prune_create_impl(const mvla_config* cfg, mvla_ctx** out)
     }
     DeviceGuard guard(c.device);
     if (!guard.ok) return MVLA_ERR_CUDA;
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, c.device) != cudaSuccess) return MVLA_ERR_CUDA;
-    if (prop.major != 10) return MVLA_ERR_UNSUPPORTED;        // built for sm_100a only
+    // (two attributes: the full property record takes 2.5 ms to look up)
+    int major = 0, sm_count = 0;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c.device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess)
+        return MVLA_ERR_CUDA;
+    if (major != 10) return MVLA_ERR_UNSUPPORTED;             // built for sm_100a only
 
     mvla_ctx* ctx = new (std::nothrow) mvla_ctx();
     if (!ctx) return MVLA_ERR_OOM;
@@ -783,7 +775,7 @@ static int32_t mvla_prune_create_impl(const mvla_config* cfg, mvla_ctx** out)
     ctx->tail_list = nullptr;
     ctx->tail_ticket = nullptr;
     ctx->patch_rec = nullptr;
-    ctx->sm_count = prop.multiProcessorCount;
+    ctx->sm_count = sm_count;
     ctx->stage_event = nullptr;
     ctx->stamps = nullptr;
     ctx->lcache = nullptr;

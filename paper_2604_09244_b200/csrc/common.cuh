@@ -124,13 +124,14 @@ cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t 
 // launch_select_copy's CTAs exchange, see there).  With `rearm_rec` (the patch-by-patch tail, launch_patch_tail)
 // it is words [cap_off, cap_off + kHandWords + n_txt + n_vis) instead, and the three 8-byte words of every patch in
 // `rearm_rec` ([vis_off / 2 + p][3]) are set to all ones.
-// Optional copy of the attention itself for the patch-by-patch path, the text queries of a (head, token)
-// next to one another (what the scoring kernel's thread holds, and what the indicators of a patch read):
-// ptr[(h * stride_h) + (vis_off + j) * stride_j + i] = alpha[h, i, j]   (null: not written).
-// stride_j is a multiple of 4 and ptr 16-byte aligned; entries i in [n_txt, stride_j) may be overwritten.
+// Optional copy of the attention itself for the patch-by-patch path, four text queries of a (head, token) next to one
+// another and the tokens behind one another:
+// ptr[h * stride_h + (i / 4) * stride_q + (vis_off + j) * 4 + i % 4] = alpha[h, i, j]   (null: not written).
+// A scoring thread holds the queries of one token, a warp 32 neighbouring tokens: each of its 16-byte stores is part of
+// 512 contiguous bytes, and so is each 16-byte load of the indicators.  Queries that pad the last four are zero.
 struct AlphaOut {
     float* ptr;
-    int64_t stride_h, stride_j;
+    int64_t stride_h, stride_q;
 };
 
 bool fast_salience_supported(int tiles_per_cta);
@@ -149,10 +150,12 @@ cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, 
                                 int cluster, int npad, unsigned long long* acc64, int* status, int32_t* rearm, unsigned long long* stamps,
                                 cudaStream_t stream);
 // The same scores into the same fixed-point accumulators by the streaming kernel (stream.cu): persistent CTAs, key
-// tiles through a shared-memory ring; for batches and for samples of any size.  `free_running`, `rearm`, `stamps` as above.
+// tiles through a shared-memory ring; for batches and for samples of any size.  `free_running`, `alpha`, `rearm`, `stamps` as
+// above; with `alpha` there may be no accumulators.
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
-                                   bool free_running, int32_t* rearm, unsigned long long* stamps, cudaStream_t stream);
+                                   bool free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
+                                   unsigned long long* stamps, cudaStream_t stream);
 
 // Salience: per-head partial scores part[h][vis] (already scaled by 1/(H n_t)).
 // `use_umma`: tensor-core path (bf16 only).  tmaps: device-usable tensor maps (passed by value).
@@ -162,6 +165,8 @@ cudaError_t launch_salience(const BatchDesc& bd, int dtype, int n_heads, int kv_
                             int cluster, int npad, float* part, int64_t part_stride,
                             int* status, AlphaOut alpha, cudaStream_t stream);
 
+// attn[j] = the fixed-point accumulator j as fp32; the accumulator is zero again afterwards.
+cudaError_t launch_take_scores(unsigned long long* acc64, int total_vis, float* attn, cudaStream_t stream);
 // attn[j] = sum_h part[h][j]  (fixed head order).
 cudaError_t launch_head_reduce(const float* part, int64_t part_stride, int n_heads, int total_vis,
                                float* attn, cudaStream_t stream);

@@ -187,14 +187,13 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
                 if (!o.acc64 && o.part)           // neither: the caller wants the attention copy only
                     o.part[static_cast<int64_t>(h) * o.part_stride + s.vis_off + vis0[t] + key] = acc;
                 if (o.alpha.ptr) {              // the attention itself, for the per-patch indicators: this key's row of queries
-                    float4* ap = reinterpret_cast<float4*>(o.alpha.ptr + static_cast<int64_t>(h) * o.alpha.stride_h +
-                                                           static_cast<int64_t>(s.vis_off + vis0[t] + key) * o.alpha.stride_j);
+                    float* ap = o.alpha.ptr + static_cast<int64_t>(h) * o.alpha.stride_h + static_cast<int64_t>(s.vis_off + vis0[t] + key) * 4;
                     const float hn = static_cast<float>(o.n_heads) * static_cast<float>(s.n_txt);   // sm.w carries 1 / (H n_t)
 #pragma unroll
                     for (int g4 = 0; g4 < TCOL / 4; ++g4) {   // 16-byte stores: a handful of instructions (sm.w is 0 past the text queries)
-                        if (4 * g4 >= npad || 4 * g4 >= o.alpha.stride_j) break;
+                        if (4 * g4 >= s.n_txt) break;
                         const float4 w4 = *reinterpret_cast<const float4*>(&sm.w[4 * g4]);
-                        ap[g4] = make_float4(L[t * TCOL + 4 * g4] * w4.x * hn, L[t * TCOL + 4 * g4 + 1] * w4.y * hn,
+                        *reinterpret_cast<float4*>(ap + g4 * o.alpha.stride_q) = make_float4(L[t * TCOL + 4 * g4] * w4.x * hn, L[t * TCOL + 4 * g4 + 1] * w4.y * hn,
                                              L[t * TCOL + 4 * g4 + 2] * w4.z * hn, L[t * TCOL + 4 * g4 + 3] * w4.w * hn);
                     }
                 }

@@ -29,10 +29,10 @@ __device__ __forceinline__ unsigned long long ld_relaxed_gpu_u64(const unsigned 
     return v;
 }
 
-// Indicators of a block of PP = 2, 4 or 8 patches (8 floats = one 32-byte sector per (head, query); fewer
-// patches per CTA when the batch is too small to fill the SMs otherwise), by a CTA of kIndThreads threads.
-// Thread = (patch, group): the group walks the (head, query) pairs with stride 512 / PP, so a CTA has
-// all its loads of a pass in flight at once (a few per thread).
+// Indicators of a block of PP = 2, 4 or 8 patches (fewer patches per CTA when the batch is too small to fill the SMs
+// otherwise), by a CTA of kIndThreads threads.  Thread = (patch, group): the group walks the (head, four queries)
+// pieces of 16 bytes with stride 512 / PP, so a CTA has all its loads of a pass in flight at once (one to a few per
+// thread, where single floats were four times as many).
 // Also writes the per-token scores of the patch's two tokens: a_j = ||alpha_j||_1 / (H n_t).
 // The L1 feature norms of the CTA's 2 PP rows (Sec. 3.1.2) are taken here too, 256 / PP threads per row,
 // their loads issued before the kernel waits for the attention copy of the kernel before it.
@@ -61,8 +61,10 @@ __device__ __forceinline__ void patch_indicators_block(const SampleDev& s, int b
     const int p = p0 + pl;
     const bool live = p < P;
     const int npairs = n_heads * s.n_txt;
-    const float* base = alpha.ptr + static_cast<int64_t>(s.vis_off + p) * alpha.stride_j;   // the patch's 2D token; its 3D token is P rows on
-    const int64_t to3 = static_cast<int64_t>(P) * alpha.stride_j;
+    const int nq4 = (s.n_txt + 3) >> 2, npieces = n_heads * nq4;   // pieces of four queries (padded with zeros)
+    const float* base = alpha.ptr + static_cast<int64_t>(s.vis_off + p) * 4;   // the patch's 2D token; its 3D token is P tokens on
+    const int64_t to3 = static_cast<int64_t>(P) * 4;
+    auto piece = [&](const float* a) { return __ldcg(reinterpret_cast<const float4*>(a)); };
 
     // ---- feature norms: row r of the CTA = 2D token p0 + r (r < PP) or 3D token p0 + r - PP.  The first
     //      kNormKeep 16-byte pieces of a thread are loaded here and added up further down, once the loads of
@@ -128,25 +130,35 @@ __device__ __forceinline__ void patch_indicators_block(const SampleDev& s, int b
         __syncthreads();
     };
 
-    // pass 1: <a3, a2>, <a2, a2>, ||a2||_1, ||a3||_1.  The first kKeep pairs of a thread stay in registers for
+    // pass 1: <a3, a2>, <a2, a2>, ||a2||_1, ||a3||_1.  The first kKeep pieces of a thread stay in registers for
     // pass 2 (all of them at the shapes this path is built for): the attention copy is read once.
-    constexpr int kKeep = 16;
-    float r2[kKeep], r3[kKeep];
+    constexpr int kKeep = 6;
+    float4 r2[kKeep], r3[kKeep];
     float v[4] = {0.f, 0.f, 0.f, 0.f};
-    const int nq = min(kKeep, (npairs + kIndGroups - 1) / kIndGroups);   // block-uniform: slots in use
-    // pair idx = g + q kIndGroups is (head h, query i); stepping q moves (h, i) by a fixed amount
-    const int step_h = kIndGroups / s.n_txt, step_i = kIndGroups - step_h * s.n_txt;
-    int h = g / s.n_txt, i = g - h * s.n_txt;
+    auto add_piece = [&](const float4& a2, const float4& a3) {
+        v[0] = fmaf(a3.x, a2.x, v[0]); v[0] = fmaf(a3.y, a2.y, v[0]); v[0] = fmaf(a3.z, a2.z, v[0]); v[0] = fmaf(a3.w, a2.w, v[0]);
+        v[1] = fmaf(a2.x, a2.x, v[1]); v[1] = fmaf(a2.y, a2.y, v[1]); v[1] = fmaf(a2.z, a2.z, v[1]); v[1] = fmaf(a2.w, a2.w, v[1]);
+        v[2] += (fabsf(a2.x) + fabsf(a2.y)) + (fabsf(a2.z) + fabsf(a2.w));
+        v[3] += (fabsf(a3.x) + fabsf(a3.y)) + (fabsf(a3.z) + fabsf(a3.w));
+    };
+    auto orthogonal = [](float coef, const float4& a2, const float4& a3) {
+        return (fabsf(fmaf(-coef, a2.x, a3.x)) + fabsf(fmaf(-coef, a2.y, a3.y))) +
+               (fabsf(fmaf(-coef, a2.z, a3.z)) + fabsf(fmaf(-coef, a2.w, a3.w)));
+    };
+    const int nq = min(kKeep, (npieces + kIndGroups - 1) / kIndGroups);   // block-uniform: slots in use
+    // piece idx = g + q kIndGroups is (head h, four queries i); stepping q moves (h, i) by a fixed amount
+    const int step_h = kIndGroups / nq4, step_i = kIndGroups - step_h * nq4;
+    int h = g / nq4, i = g - h * nq4;
 #pragma unroll
     for (int q = 0; q < kKeep; ++q) {                     // all loads of the thread in flight at once
-        r2[q] = 0.f; r3[q] = 0.f;
+        r2[q] = make_float4(0.f, 0.f, 0.f, 0.f); r3[q] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (q >= nq) continue;                            // uniform
-        if (live && g + q * kIndGroups < npairs) {
-            const float* a = base + static_cast<int64_t>(h) * alpha.stride_h + i;
-            r2[q] = __ldcg(a); r3[q] = __ldcg(a + to3);
+        if (live && g + q * kIndGroups < npieces) {
+            const float* a = base + static_cast<int64_t>(h) * alpha.stride_h + static_cast<int64_t>(i) * alpha.stride_q;
+            r2[q] = piece(a); r3[q] = piece(a + to3);
         }
         h += step_h; i += step_i;
-        if (i >= s.n_txt) { i -= s.n_txt; ++h; }
+        if (i >= nq4) { i -= nq4; ++h; }
     }
     {                                                     // the feature norms, now that every load is in flight
         float acc = 0.f;
@@ -159,23 +171,16 @@ __device__ __forceinline__ void patch_indicators_block(const SampleDev& s, int b
         if (lane == 0) rown[warp] = acc;                  // read after the barriers of the first reduction
     }
 #pragma unroll
-    for (int q = 0; q < kKeep; ++q) {                     // (a pair that does not exist adds zeros)
+    for (int q = 0; q < kKeep; ++q) {                     // (a piece that does not exist adds zeros)
         if (q >= nq) break;                               // uniform
-        v[0] = fmaf(r3[q], r2[q], v[0]);
-        v[1] = fmaf(r2[q], r2[q], v[1]);
-        v[2] += fabsf(r2[q]);
-        v[3] += fabsf(r3[q]);
+        add_piece(r2[q], r3[q]);
     }
     if (live) {
-#pragma unroll 4
-        for (int idx = g + kKeep * kIndGroups; idx < npairs; idx += kIndGroups) {
-            const int hh = idx / s.n_txt, ii = idx - hh * s.n_txt;
-            const float* a = base + static_cast<int64_t>(hh) * alpha.stride_h + ii;
-            const float a2 = __ldcg(a), a3 = __ldcg(a + to3);
-            v[0] = fmaf(a3, a2, v[0]);
-            v[1] = fmaf(a2, a2, v[1]);
-            v[2] += fabsf(a2);
-            v[3] += fabsf(a3);
+#pragma unroll 2
+        for (int idx = g + kKeep * kIndGroups; idx < npieces; idx += kIndGroups) {
+            const int hh = idx / nq4, ii = idx - hh * nq4;
+            const float* a = base + static_cast<int64_t>(hh) * alpha.stride_h + static_cast<int64_t>(ii) * alpha.stride_q;
+            add_piece(piece(a), piece(a + to3));
         }
     }
     reduce(v, 4);
@@ -187,14 +192,14 @@ __device__ __forceinline__ void patch_indicators_block(const SampleDev& s, int b
 #pragma unroll
     for (int q = 0; q < kKeep; ++q) {
         if (q >= nq) break;                               // uniform
-        o[0] += fabsf(fmaf(-coef, r2[q], r3[q]));
+        o[0] += orthogonal(coef, r2[q], r3[q]);
     }
     if (live) {
-#pragma unroll 4
-        for (int idx = g + kKeep * kIndGroups; idx < npairs; idx += kIndGroups) {
-            const int hh = idx / s.n_txt, ii = idx - hh * s.n_txt;
-            const float* a = base + static_cast<int64_t>(hh) * alpha.stride_h + ii;
-            o[0] += fabsf(fmaf(-coef, __ldcg(a), __ldcg(a + to3)));
+#pragma unroll 2
+        for (int idx = g + kKeep * kIndGroups; idx < npieces; idx += kIndGroups) {
+            const int hh = idx / nq4, ii = idx - hh * nq4;
+            const float* a = base + static_cast<int64_t>(hh) * alpha.stride_h + static_cast<int64_t>(ii) * alpha.stride_q;
+            o[0] += orthogonal(coef, piece(a), piece(a + to3));
         }
     }
     reduce(o, 1);

@@ -10,6 +10,7 @@
 // later in a fixed order so that the result does not depend on scheduling.
 #include "common.cuh"
 #include "device_utils.cuh"
+#include "select_impl.cuh"
 #include "tmem_plan.h"
 
 #include <math_constants.h>
@@ -264,9 +265,10 @@ salience_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CU
                     const float e = exp2f(v[i] - s_m[cb + i]);
                     const float pr = (cb + i < s.n_txt) ? e * s_w[cb + i] : 0.f;
                     acc += pr;
-                    if (alpha.ptr && cb + i < s.n_txt && tid < ti.valid)   // the attention itself (per-patch indicators)
-                        alpha.ptr[static_cast<int64_t>(h) * alpha.stride_h + static_cast<int64_t>(s.vis_off + ti.vis0 + tid) * alpha.stride_j +
-                                  cb + i] = pr * (static_cast<float>(n_heads) * static_cast<float>(s.n_txt));
+                    if (alpha.ptr && cb + i < ((s.n_txt + 3) & ~3) && tid < ti.valid)   // the attention itself (per-patch indicators)
+                        alpha.ptr[static_cast<int64_t>(h) * alpha.stride_h + static_cast<int64_t>((cb + i) >> 2) * alpha.stride_q +
+                                  static_cast<int64_t>(s.vis_off + ti.vis0 + tid) * 4 + (i & 3)] =
+                            pr * (static_cast<float>(n_heads) * static_cast<float>(s.n_txt));
                 }
             }
         }
@@ -292,6 +294,16 @@ __global__ void head_reduce_kernel(const float* __restrict__ part, int64_t part_
     float acc = 0.f;
     for (int h = 0; h < n_heads; ++h) acc += part[static_cast<int64_t>(h) * part_stride + j];
     attn[j] = acc;
+}
+
+__global__ void take_scores_kernel(unsigned long long* __restrict__ acc64, int total_vis, float* __restrict__ attn)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();                               // launched while the scoring kernel still runs: wait for its sums
+    pdl_trigger();
+    if (j >= total_vis) return;
+    attn[j] = __ull2float_rn(__ldcg(acc64 + j)) * kFixInv;   // one rounding: the exact head sum to fp32
+    acc64[j] = 0ull;
 }
 
 // One warp per visual row; 16-byte loads; fixed reduction order.
@@ -417,6 +429,19 @@ cudaError_t launch_head_reduce(const float* part, int64_t part_stride, int n_hea
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, head_reduce_kernel, part, part_stride, n_heads, total_vis, attn);
+}
+
+cudaError_t launch_take_scores(unsigned long long* acc64, int total_vis, float* attn, cudaStream_t stream)
+{
+    if (total_vis <= 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((total_vis + 255) / 256);
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1] = {pdl_attribute()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, take_scores_kernel, acc64, total_vis, attn);
 }
 
 cudaError_t launch_l1norm(const BatchDesc& bd, int dtype, int d_model, const void* hidden, float* l1,

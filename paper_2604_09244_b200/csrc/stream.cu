@@ -43,7 +43,9 @@ struct StreamArgs {
     unsigned long long* acc64;
     int* status;
     int free_running;
+    AlphaOut alpha;               // with it there may be no accumulators
     int32_t* rearm;               // see launch_salience_fast
+    unsigned long long* rearm_rec;
     unsigned long long* stamps;
 };
 
@@ -185,7 +187,11 @@ struct JobTiles {
 // What a softmax warp needs to know about a job.
 struct SoftJob {
     JobTiles tr;
-    unsigned long long* acc;      // the sample's accumulators
+    unsigned long long* acc;      // the sample's accumulators, or null
+    float* alpha;                 // the sample's attention copy of this head, or null
+    int64_t stride_q;
+    int n_txt;
+    float hn;                     // heads x text queries: the weights carry its inverse
     int slot0, slots, width;      // slot of the job's first tile, slots in the ring, columns per slot
     uint32_t parity0;             // parity of that slot's use
     uint32_t lane_base;           // tensor-memory address of the warp's 32 lanes
@@ -322,7 +328,8 @@ __device__ __forceinline__ void soft_exps(const SoftJob& j, StreamSmem& sm, int 
 }
 
 // Per key, the sum of its exponentials weighted by sm.w[warp] (the normalised, head-averaged attention mass), added into
-// the accumulators; a tile's slot is free once the four warps of its group are done.
+// the accumulators, or (ALPHA) the normalised exponentials one by one into the attention copy; a tile's slot is free once the four warps of its group are done.
+template <bool ALPHA>
 __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, int nch, int warp, int lane)
 {
     const int key = (warp & 3) * 32 + lane;
@@ -331,12 +338,20 @@ __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, in
     for (int t = warp >> 2; t < j.tr.count; t += 2) {
         const uint32_t cols = j.cols(t);
         float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        const bool live = key < j.tr.valid(t);
+        float* const ap = ALPHA ? j.alpha + static_cast<int64_t>(j.tr.vis0(t) + key) * 4 : nullptr;
         auto add16 = [&](const float (&v)[16], int c) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float4 w4 = *reinterpret_cast<const float4*>(&my_w[c * 16 + 4 * i]);
-                acc[0] = fma2(make_float2(v[4 * i], v[4 * i + 1]), make_float2(w4.x, w4.y), acc[0]);
-                acc[1] = fma2(make_float2(v[4 * i + 2], v[4 * i + 3]), make_float2(w4.z, w4.w), acc[1]);
+                if constexpr (ALPHA) {                           // the attention itself (weights are zero past the text queries)
+                    if (live && c * 16 + 4 * i < j.n_txt)
+                        *reinterpret_cast<float4*>(ap + (c * 4 + i) * j.stride_q) =
+                            make_float4(v[4 * i] * w4.x * j.hn, v[4 * i + 1] * w4.y * j.hn, v[4 * i + 2] * w4.z * j.hn, v[4 * i + 3] * w4.w * j.hn);
+                } else {
+                    acc[0] = fma2(make_float2(v[4 * i], v[4 * i + 1]), make_float2(w4.x, w4.y), acc[0]);
+                    acc[1] = fma2(make_float2(v[4 * i + 2], v[4 * i + 3]), make_float2(w4.z, w4.w), acc[1]);
+                }
             }
         };
         int c = 0;
@@ -359,8 +374,10 @@ __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, in
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sm.tempty[j.slot(t)]));
-        const float a = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
-        if (key < j.tr.valid(t)) atomicAdd(j.acc + j.tr.vis0(t) + key, __float2ull_rn(a * kFixScale));
+        if constexpr (!ALPHA) {
+            const float a = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
+            if (live) atomicAdd(j.acc + j.tr.vis0(t) + key, __float2ull_rn(a * kFixScale));
+        }
     }
     __syncwarp();
 }
@@ -509,6 +526,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
     } else {
         // ---------------------------------------------------------------- softmax
         SoftJob j;
+        j.alpha = nullptr; j.stride_q = a.alpha.stride_q;
         j.slot0 = 0; j.slots = a.slots; j.width = W; j.parity0 = 0;
         j.lane_base = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         j.cscale = 1.4426950408889634f * rsqrtf(static_cast<float>(a.head_dim));   // log2 domain
@@ -520,8 +538,17 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             j.tr = JobTiles(s, crank, lg);
             j.acc = a.acc64 + s.vis_off;
             const int n_txt = s.n_txt, npad = (n_txt + 15) & ~15;
-            if (a.rearm && h == 0 && crank == 0)      // the tail kernel's hand-over words; their last users finished long ago
-                for (int i = tid; i < s.n_out; i += kSoftThreads) a.rearm[s.out_off + i] = -1;
+            j.n_txt = n_txt;
+            j.hn = static_cast<float>(a.n_heads) * static_cast<float>(n_txt);
+            if (a.alpha.ptr) j.alpha = a.alpha.ptr + static_cast<int64_t>(h) * a.alpha.stride_h + static_cast<int64_t>(s.vis_off) * 4;
+            if (a.rearm && h == 0 && crank == 0) {    // the tail kernel's hand-over words; their last users finished long ago
+                if (!a.rearm_rec) {
+                    for (int i = tid; i < s.n_out; i += kSoftThreads) a.rearm[s.out_off + i] = -1;
+                } else {                              // the patch-by-patch tail: its list words, and three words per patch
+                    for (int i = tid; i < kHandWords + s.n_txt + s.n_2d + s.n_3d; i += kSoftThreads) a.rearm[s.cap_off + i] = -1;
+                    for (int i = tid; i < 3 * s.n_2d; i += kSoftThreads) a.rearm_rec[static_cast<int64_t>(s.vis_off / 2) * 3 + i] = ~0ull;
+                }
+            }
             const int nch = npad >> 4;
             {
                 int c = 0;
@@ -554,7 +581,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
                     }
                 }
                 sm.g[tid] = mx;
-                sm.iz[tid] = tid < n_txt && z > 0.f ? 1.f / z / (static_cast<float>(a.n_heads) * static_cast<float>(n_txt)) : 0.f;
+                sm.iz[tid] = tid < n_txt && z > 0.f ? 1.f / z / j.hn : 0.f;
             }
             if (!waited) { pdl_wait(); waited = true; }      // the accumulators were read and cleared by an earlier selection
             soft_barrier();
@@ -563,7 +590,8 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
                 my_w[i] = mk == -CUDART_INF_F ? 0.f : fast_ex2(mk - sm.g[i]) * sm.iz[i];
             }
             __syncwarp();
-            soft_scores(j, sm, nch, warp, lane);
+            if (a.alpha.ptr) soft_scores<true>(j, sm, nch, warp, lane);
+            else soft_scores<false>(j, sm, nch, warp, lane);
             j.slot0 += j.tr.count;
             if (j.slot0 >= a.slots) { j.slot0 -= a.slots; j.parity0 ^= 1u; }
         }
@@ -637,7 +665,8 @@ cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUte
 
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
-                                   bool free_running, int32_t* rearm, unsigned long long* stamps, cudaStream_t stream)
+                                   bool free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
+                                   unsigned long long* stamps, cudaStream_t stream)
 {
     const int sms = sm_count_of_current_device();
     const int npad = padded_text(bd), tiles = max_tiles(bd);
@@ -646,7 +675,8 @@ cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_grou
     a.width = npad;
     a.slots = std::min(kMaxSlots, kTmemColsPerSm / npad);
     a.n_jobs = bd.n * n_heads;
-    a.acc64 = acc64; a.status = status; a.free_running = free_running ? 1 : 0; a.rearm = rearm; a.stamps = stamps;
+    a.acc64 = acc64; a.status = status; a.free_running = free_running ? 1 : 0; a.alpha = alpha; a.rearm = rearm;
+    a.rearm_rec = rearm_rec; a.stamps = stamps;
     // The smallest cluster whose CTAs hold their share of a job's logits in tensor memory; a larger one while jobs are
     // fewer than multiprocessors and the tiles can still be shared out.
     int cluster = 1;

@@ -324,3 +324,16 @@ def test_patch_step_in_one_tail_kernel_at_the_edges_of_its_shapes(batch, n_txt, 
         total += n
     assert checked >= 0.8 * total
     ctx.close()
+
+
+@pytest.mark.parametrize("batch,H,d,n_txt,n_patch", [
+    (12, 16, 64, (33, 16, 50, 1), (130, 60, 200)),        # every padded text length, ragged tiles
+    (3, 8, 128, (64, 18), (2048, 1100)),                  # more than 16 key tiles a sample: clusters
+])
+def test_patch_step_scored_by_the_streaming_kernel(batch, H, d, n_txt, n_patch):
+    wl = W.patch_workload(58, batch=batch, D=256, H=H, d=d, n_txt=n_txt, n_patch=n_patch, steps=2)
+    ctx = mvla.context_for(wl)
+    states = [oracle.PatchState(s.n_2d) for s in wl.samples]
+    for step in (0, 1):
+        run_patch_step(ctx, wl, step, states)
+    ctx.close()
