@@ -318,6 +318,20 @@ int32_t check_sticky(mvla_ctx* ctx)
     return (ctx->status_host && *reinterpret_cast<volatile int*>(ctx->status_host) != 0) ? MVLA_ERR_TIMEOUT : MVLA_OK;
 }
 
+// Visual tokens of a launch's samples.
+int visual_tokens(const BatchDesc& bd)
+{
+    const SampleDev& last = bd.s[bd.n - 1];
+    return last.vis_off + last.n_2d + last.n_3d - bd.s[0].vis_off;
+}
+
+// A launch of the step failed after the scoring kernel was enqueued: the fixed-point accumulators of the
+// chunk must not keep this step's sums (the kernel that clears them will not run).
+void clear_accumulators(unsigned long long* acc64, const BatchDesc& bd, cudaStream_t st)
+{
+    cudaMemsetAsync(acc64 + bd.s[0].vis_off, 0, static_cast<size_t>(visual_tokens(bd)) * sizeof(unsigned long long), st);
+}
+
 // Which of the two tensor-core scoring kernels.  The latency-shaped one of fused.cu covers up to 16 key tiles a sample
 // and is the faster one while its CTAs all run at once (three with one key tile to a multiprocessor, two with two tiles);
 // from the second wave on the streaming one is (stream.cu).  Measured at 32 heads, 256 + 512 tokens, whole step in us,
@@ -329,14 +343,14 @@ bool stream_pays(const mvla_ctx* ctx, const BatchDesc& bd, int tiles_per_cta, in
            bd.n * ctx->cfg.n_heads * cluster > ctx->sm_count * (tiles_per_cta == 1 ? 3 : 2);
 }
 
-// Salience of one chunk (+ L1 norms into `l1` when asked).  The per-head contributions land in
+// Salience of one chunk (+ L1 norms into `l1` when asked; + the scores as fp32 into `attn_out` when asked).  The per-head contributions land in
 // ctx->part, or, when `want_acc64` and the register-resident tensor-core kernel covers the shape, in the
 // fixed-point accumulators ctx->acc64 (*used_acc64 = true).
 int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, const void* k, int64_t rows,
                            const void* hidden, float* l1, unsigned long long* acc64, bool* used_acc64,
                            bool free_running, cudaStream_t st, AlphaOut alpha = AlphaOut{nullptr, 0, 0},
                            int32_t* rearm = nullptr, bool norms_beside = false, unsigned long long* stamps = nullptr,
-                           bool with_cache = false, unsigned long long* rearm_rec = nullptr)
+                           bool with_cache = false, unsigned long long* rearm_rec = nullptr, float* attn_out = nullptr)
 {
     if (used_acc64) *used_acc64 = false;
     const mvla_config& c = ctx->cfg;
@@ -367,7 +381,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     // the scoring kernel and run beside it instead of in front of it.
     norms_beside = norms_beside && fast;
     if (hidden && l1 && !norms_beside) {
-        e = launch_l1norm(bd, ctx->hidden_dtype, c.d_model, hidden, l1, false, st);
+        e = launch_l1norm(bd, ctx->hidden_dtype, c.d_model, hidden, l1, false, nullptr, nullptr, st);
         if (e != cudaSuccess) return fail_cuda(ctx, e);
     }
     if (streaming) {
@@ -391,9 +405,17 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     }
     if (e == cudaErrorInvalidConfiguration) return MVLA_ERR_UNSUPPORTED;
     if (e != cudaSuccess) return fail_cuda(ctx, e);
-    if (hidden && l1 && norms_beside) {
-        e = launch_l1norm(bd, ctx->hidden_dtype, c.d_model, hidden, l1, true, st);
-        if (e != cudaSuccess) return fail_cuda(ctx, e);
+    const bool take = attn_out && used_acc64 && *used_acc64;      // scores wanted as fp32: the norm kernel takes them, if there is one
+    e = cudaSuccess;
+    if (hidden && l1 && norms_beside)
+        e = launch_l1norm(bd, ctx->hidden_dtype, c.d_model, hidden, l1, true, take ? acc64 : nullptr, attn_out, st);
+    else if (take)
+        e = launch_take_scores(acc64 + bd.s[0].vis_off, visual_tokens(bd), attn_out + bd.s[0].vis_off, st);
+    else if (attn_out)
+        e = launch_head_reduce(ctx->part + bd.s[0].vis_off, ctx->part_stride, c.n_heads, visual_tokens(bd), attn_out + bd.s[0].vis_off, st);
+    if (e != cudaSuccess) {
+        if (take) clear_accumulators(acc64, bd, st);
+        return fail_cuda(ctx, e);
     }
     return MVLA_OK;
 }
@@ -413,16 +435,6 @@ GateParams gate_params(const mvla_ctx* ctx, int32_t mode, bool has_l1)
     gp.adaptive = mode == MVLA_MODE_ADAPTIVE;
     gp.has_l1 = has_l1;
     return gp;
-}
-
-// A launch of the step failed after the scoring kernel was enqueued: the fixed-point accumulators of the
-// chunk must not keep this step's sums (the selection that clears them will not run).
-void clear_accumulators(unsigned long long* acc64, const BatchDesc& bd, cudaStream_t st)
-{
-    const SampleDev& first = bd.s[0];
-    const SampleDev& last = bd.s[bd.n - 1];
-    const size_t n = static_cast<size_t>(last.vis_off + last.n_2d + last.n_3d - first.vis_off);
-    cudaMemsetAsync(acc64 + first.vis_off, 0, n * sizeof(unsigned long long), st);
 }
 
 // ---- overlap of neighbouring prune steps (MVLA_FLAG_INPUTS_STABLE) ----
@@ -920,13 +932,17 @@ static int32_t mvla_salience_impl(mvla_ctx* ctx, int32_t batch, const mvla_sampl
     if (rc != MVLA_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const bool want_l1 = hidden && l1_out;
+    // the kernels of the fused step, into a scratch set of this call's own
+    ctx->step_parity = (ctx->step_parity + 1u) % kSets;
+    ctx->sel_valid[ctx->step_parity] = false;        // this set is used outside the event chain
+    unsigned long long* acc64 = ctx->acc64 + ctx->step_parity * ctx->vis_all;
     for (int first = 0; first < batch; first += kMaxChunk) {
         const BatchDesc bd = chunk_of(plan, first, std::min(kMaxChunk, batch - first));
-        rc = run_salience_chunk(ctx, bd, q, k, rows, want_l1 ? hidden : nullptr, l1_out, nullptr, nullptr, false, st);
+        bool used_acc64 = false;
+        rc = run_salience_chunk(ctx, bd, q, k, rows, want_l1 ? hidden : nullptr, l1_out, acc64, &used_acc64, false, st,
+                                AlphaOut{nullptr, 0, 0}, nullptr, true, nullptr, false, nullptr, attn_out);
         if (rc != MVLA_OK) return rc;
     }
-    const cudaError_t e = launch_head_reduce(ctx->part, ctx->part_stride, ctx->cfg.n_heads, plan.total_vis, attn_out, st);
-    if (e != cudaSuccess) return fail_cuda(ctx, e);
     return MVLA_OK;
 }
 

@@ -296,26 +296,31 @@ __global__ void head_reduce_kernel(const float* __restrict__ part, int64_t part_
     attn[j] = acc;
 }
 
+// One rounding: the exact head sum to fp32; the accumulator is ready for the next call.
+__device__ __forceinline__ void take_score(unsigned long long* acc, float* attn)
+{
+    *attn = __ull2float_rn(__ldcg(acc)) * kFixInv;
+    *acc = 0ull;
+}
 __global__ void take_scores_kernel(unsigned long long* __restrict__ acc64, int total_vis, float* __restrict__ attn)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();                               // launched while the scoring kernel still runs: wait for its sums
     pdl_trigger();
-    if (j >= total_vis) return;
-    attn[j] = __ull2float_rn(__ldcg(acc64 + j)) * kFixInv;   // one rounding: the exact head sum to fp32
-    acc64[j] = 0ull;
+    if (j < total_vis) take_score(acc64 + j, attn + j);
 }
 
 // One warp per visual row; 16-byte loads; fixed reduction order.
 // Launched with programmatic serialization: the kernel after it may become resident at once, and this
 // kernel itself needs nothing from the kernel before it except that the hidden rows are final, which the
 // launch order guarantees (see the callers).  It therefore does its work first and waits for its
-// predecessor LAST, only so that "this kernel is complete" keeps implying "its predecessor is complete"
-// for whatever follows.
+// predecessor LAST, so that "this kernel is complete" keeps implying "its predecessor is complete" for whatever
+// follows -- and, with `acc64`, to take the scores that the predecessor has left in the accumulators: one kernel
+// less on the chain of the stand-alone scores.
 template <typename T>
 __global__ void __launch_bounds__(256)
 l1norm_kernel(const __grid_constant__ BatchDesc bd, int d_model, const T* __restrict__ hidden,
-              float* __restrict__ l1, int early)
+              float* __restrict__ l1, int early, unsigned long long* __restrict__ acc64, float* __restrict__ attn)
 {
     if (early) pdl_trigger();
     else pdl_wait();
@@ -350,6 +355,7 @@ l1norm_kernel(const __grid_constant__ BatchDesc bd, int d_model, const T* __rest
     for (int off = 16; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (lane == 0) l1[s.vis_off + j] = acc;
     if (early) pdl_wait();
+    if (acc64 && lane == 0) take_score(acc64 + s.vis_off + j, attn + s.vis_off + j);
 }
 
 template <typename T, bool UMMA>
@@ -445,7 +451,7 @@ cudaError_t launch_take_scores(unsigned long long* acc64, int total_vis, float* 
 }
 
 cudaError_t launch_l1norm(const BatchDesc& bd, int dtype, int d_model, const void* hidden, float* l1,
-                          bool beside_predecessor, cudaStream_t stream)
+                          bool beside_predecessor, unsigned long long* acc64, float* attn, cudaStream_t stream)
 {
     int max_nv = 0;
     for (int b = 0; b < bd.n; ++b) max_nv = max(max_nv, bd.s[b].n_2d + bd.s[b].n_3d);
@@ -459,8 +465,8 @@ cudaError_t launch_l1norm(const BatchDesc& bd, int dtype, int d_model, const voi
     cfg.numAttrs = beside_predecessor ? 1 : 0;
     const int early = beside_predecessor ? 1 : 0;
     if (dtype == MVLA_DTYPE_BF16)
-        return cudaLaunchKernelEx(&cfg, l1norm_kernel<__nv_bfloat16>, bd, d_model, static_cast<const __nv_bfloat16*>(hidden), l1, early);
-    return cudaLaunchKernelEx(&cfg, l1norm_kernel<float>, bd, d_model, static_cast<const float*>(hidden), l1, early);
+        return cudaLaunchKernelEx(&cfg, l1norm_kernel<__nv_bfloat16>, bd, d_model, static_cast<const __nv_bfloat16*>(hidden), l1, early, acc64, attn);
+    return cudaLaunchKernelEx(&cfg, l1norm_kernel<float>, bd, d_model, static_cast<const float*>(hidden), l1, early, acc64, attn);
 }
 
 }  // namespace mvla
