@@ -395,8 +395,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     } else if (fast) {
         e = launch_salience_fast(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk,
                                  tiles_per_cta, cluster, npad,
-                                 alpha.ptr && !acc64 ? nullptr : ctx->part,     // the patch path reads the attention copy only
-                                 ctx->part_stride, acc64, ctx->status_dev, free_running, alpha, rearm, rearm_rec, stamps,
+                                 acc64, ctx->status_dev, free_running, alpha, rearm, rearm_rec, stamps,
                                  with_cache ? ctx->lcache : nullptr, ctx->max_vis, ctx->cache_cols, st);
         if (used_acc64) *used_acc64 = acc64 != nullptr;
     } else {

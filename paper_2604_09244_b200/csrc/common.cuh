@@ -110,10 +110,9 @@ cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t 
 
 // ---- launchers (each enqueues on `stream` and returns the launch status) ----
 
-// bf16 tensor-core salience with logits held in registers (one or two key tiles per CTA).  With
-// `acc64` the per-head contributions are added into 64-bit fixed-point accumulators (scale 2^60, one
-// per visual token, zero on entry); without it they go to part[h][vis] as in launch_salience (nowhere when
-// `part` is null too: only the attention copy is wanted).
+// bf16 tensor-core salience with logits held in registers (one or two key tiles per CTA).  The per-head
+// contributions are added into the 64-bit fixed-point accumulators `acc64` (scale 2^60, one per visual token, zero on
+// entry); nowhere when it is null: only the attention copy is wanted.
 // `free_running`: the kernel does not wait for the kernel before it in its stream (the caller orders
 // everything it depends on with events).
 // `lcache`: logit cache [state][head][cache_vis][cache_cols] fp32 (raw dot products), or null; which tiles are
@@ -140,7 +139,7 @@ bool fast_salience_supported(int tiles_per_cta);
 // `esize`: bytes per element of q and k (2: bf16, 1: e4m3).
 cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tmap_q,
                                  const CUtensorMap* tmap_k, int tiles_per_cta, int cluster, int npad,
-                                 float* part, int64_t part_stride, unsigned long long* acc64, int* status,
+                                 unsigned long long* acc64, int* status,
                                  bool free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                                  float* lcache, int cache_vis, int cache_cols, cudaStream_t stream);
 

@@ -24,6 +24,7 @@ namespace mvla {
 namespace {
 
 constexpr int kFastThreads = 128;
+constexpr float kRescaleAt = 64.f;       // exponents (log2) above this: the warp's reference becomes its maximum
 
 __device__ __forceinline__ float ex2_approx(float x)
 {
@@ -58,19 +59,15 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
     return false;
 }
 
-// Shared memory of the softmax part.
+// Shared memory of the softmax part, per warp of the four that cover a tile's 128 keys, and per query.
 struct FastSmem {
-    float m[kMaxText];                       // local max per query (scaled, log2 domain), -inf replaced by 0
-    alignas(16) float w[kMaxText];           // final weight per query
-    float2 peer[kMaxCluster][kMaxText];      // (raw local max, local sum) of every CTA of the cluster
-    float2 loc[kMaxText];                    // this CTA's pairs, staged for the push
-    float wred[4][kMaxText];
+    alignas(16) float m[4][kMaxText];        // -reference of the exponents (log2 domain)
+    alignas(16) float w[4][kMaxText];        // sum of the exponentials, then their weight in the scores
+    float2 peer[kMaxCluster][kMaxText];      // (reference, sum) of every CTA of the cluster
 };
 // What the softmax part writes.
 struct FastOut {
-    float* part;
-    int64_t part_stride;
-    unsigned long long* acc64;
+    unsigned long long* acc64;               // null: the attention copy only
     int* status;
     int free_running, n_heads;
     AlphaOut alpha;
@@ -78,15 +75,22 @@ struct FastOut {
 
 // From the raw dot products of this thread's key(s) -- L[t * TC + i]: tile t, text query c0 + i -- to the outputs.
 // vis0[t], valid[t]: the tiles' first visual index and number of keys.
+//
+// A warp takes its exponentials against a reference of its own, the logits of its first key, not against a maximum
+// over the CTA's keys: fp32 is as precise at 2^40 as at 1, so a reference only has to keep the exponents from
+// overflowing, and the two shared-memory round trips, two block barriers and the butterfly that found the maximum leave
+// the chain (a warp whose exponents exceed kRescaleAt takes its true maxima after all).  The pairs (reference, sum) of
+// the four warps are combined per query, then those of the cluster's CTAs.
 template <int TCOL, int NTILE, int SPLIT>
 __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT], const SampleDev& s, const int (&valid)[NTILE],
                                                const int (&vis0)[NTILE], bool ok, int npad, int h, float cscale, uint32_t bar_x,
                                                FastSmem& sm, const FastOut& o)
 {
-    constexpr int TC = TCOL / SPLIT, NT = kFastThreads * SPLIT;
+    constexpr int TC = TCOL / SPLIT;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int key = tid & (kFastThreads - 1), kwarp = warp & 3, c0 = (tid / kFastThreads) * TC;
     const uint32_t crank = cluster_ctarank(), csize = gridDim.x;
+    float* const nm = sm.m[kwarp] + c0;
     // The registers keep the raw dot products; the scale enters with the exponent below (one FFMA).  Keys
     // past the end of a ragged tile are masked; a full tile needs no pass over the registers at all, and
     // columns past the padded query count are never looked at.
@@ -98,105 +102,131 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
         for (int i = 0; i < TC; ++i) L[t * TC + i] = live ? L[t * TC + i] : -CUDART_INF_F;
     }
 
-    // ---- local maximum per query
+    // ---- references: the warp's first key (zero for a warp without one: its exponentials are all zero)
+    if (lane == 0) {
 #pragma unroll
-    for (int qc = 0; qc < TC / 16; ++qc) {
-        if (c0 + qc * 16 >= npad) break;
-        float m[16];
+        for (int i = 0; i < TC; i += 4) {
+            if ((i & 15) == 0 && c0 + i >= npad) break;
+            float r[4];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            m[i] = L[qc * 16 + i];
+            for (int k = 0; k < 4; ++k) {
+                r[k] = L[i + k];
 #pragma unroll
-            for (int t = 1; t < NTILE; ++t) m[i] = fmaxf(m[i], L[t * TC + qc * 16 + i]);
+                for (int t = 1; t < NTILE; ++t) r[k] = valid[0] > kwarp * 32 ? r[k] : L[t * TC + i + k];
+                r[k] = r[k] == -CUDART_INF_F ? 0.f : -r[k] * cscale;
+            }
+            *reinterpret_cast<float4*>(nm + i) = make_float4(r[0], r[1], r[2], r[3]);
         }
-        const float red = warp_reduce16<true>(m, lane);
-        if ((lane & 1) == 0) sm.wred[kwarp][c0 + qc * 16 + col16(lane)] = red;
     }
-    __syncthreads();
-    float m_raw = -CUDART_INF_F;
-    if (tid < npad) {
-        m_raw = fmaxf(fmaxf(sm.wred[0][tid], sm.wred[1][tid]), fmaxf(sm.wred[2][tid], sm.wred[3][tid])) * cscale;
-        sm.m[tid] = (m_raw == -CUDART_INF_F) ? 0.f : m_raw;
+    __syncwarp();
+    {
+        float top = -CUDART_INF_F;
+#pragma unroll
+        for (int i = 0; i < TC; i += 4) {
+            if ((i & 15) == 0 && c0 + i >= npad) break;
+            const float4 m4 = *reinterpret_cast<const float4*>(nm + i);
+#pragma unroll
+            for (int t = 0; t < NTILE; ++t)
+                top = fmaxf(top, fmaxf(fmaxf(fmaf(L[t * TC + i], cscale, m4.x), fmaf(L[t * TC + i + 1], cscale, m4.y)),
+                                       fmaxf(fmaf(L[t * TC + i + 2], cscale, m4.z), fmaf(L[t * TC + i + 3], cscale, m4.w))));
+        }
+        if (__any_sync(0xffffffffu, top > kRescaleAt)) {  // rare
+#pragma unroll
+            for (int qc = 0; qc < TC / 16; ++qc) {
+                if (c0 + qc * 16 >= npad) break;
+                float m[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    m[i] = L[qc * 16 + i];
+#pragma unroll
+                    for (int t = 1; t < NTILE; ++t) m[i] = fmaxf(m[i], L[t * TC + qc * 16 + i]);
+                }
+                const float red = warp_reduce16<true>(m, lane);
+                __syncwarp();
+                if ((lane & 1) == 0) nm[qc * 16 + col16(lane)] = -red * cscale;
+            }
+            __syncwarp();
+        }
     }
-    __syncthreads();
 
-    // ---- exponentials (kept in registers) and the local denominator per query
+    // ---- exponentials (kept in registers) and their sum per query
 #pragma unroll
     for (int qc = 0; qc < TC / 16; ++qc) {
         if (c0 + qc * 16 >= npad) break;
         float sum[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            const float mm = sm.m[c0 + qc * 16 + i];
+            const float mm = nm[qc * 16 + i];
             sum[i] = 0.f;
 #pragma unroll
             for (int t = 0; t < NTILE; ++t) {
-                const float e = ex2_approx(fmaf(L[t * TC + qc * 16 + i], cscale, -mm));
+                const float e = ex2_approx(fmaf(L[t * TC + qc * 16 + i], cscale, mm));
                 L[t * TC + qc * 16 + i] = e;
                 sum[i] += e;
             }
         }
         const float red = warp_reduce16<false>(sum, lane);
-        if ((lane & 1) == 0) sm.wred[kwarp][c0 + qc * 16 + col16(lane)] = red;
+        if ((lane & 1) == 0) sm.w[kwarp][c0 + qc * 16 + col16(lane)] = red;
     }
     __syncthreads();
 
-    // ---- exchange (max, sum) with the other key tiles of this (sample, head)
-    if (tid < npad)
-        sm.loc[tid] = make_float2(m_raw, (sm.wred[0][tid] + sm.wred[1][tid]) + (sm.wred[2][tid] + sm.wred[3][tid]));
-    __syncthreads();
+    // ---- one thread per query: the pairs of the CTA's warps, exchanged with the other key tiles of this (sample, head)
     cluster_wait_acquire();                   // every peer is running and has initialised its barriers
-    for (int p = tid; p < npad * static_cast<int>(csize); p += NT) {
-        const int i = p % npad;
-        const uint32_t r = static_cast<uint32_t>(p / npad);
-        st_async_peer_f32x2(smem_u32(&sm.peer[crank][i]), bar_x, r, sm.loc[i]);
-    }
-    __syncwarp();
-    if (tid < npad) {                         // the warps that combine the pairs wait for them; the others park below
+    if (tid < npad) {                         // (the other warps park at the barrier below)
+        float ref[4], mx = -CUDART_INF_F, z = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {         // (a warp with a key has a sum of at least one: its reference's)
+            ref[k] = sm.w[k][tid] > 0.f ? -sm.m[k][tid] : -CUDART_INF_F;
+            mx = fmaxf(mx, ref[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (ref[k] > -CUDART_INF_F) z += sm.w[k][tid] * ex2_approx(ref[k] - mx);
+        for (uint32_t r = 0; r < csize; ++r) st_async_peer_f32x2(smem_u32(&sm.peer[crank][tid]), bar_x, r, make_float2(mx, z));
+        const float inv_hn = 1.f / (static_cast<float>(o.n_heads) * static_cast<float>(s.n_txt));
         const bool okx = mbar_wait_cluster(bar_x, 0);
         if (!okx) *reinterpret_cast<volatile int*>(o.status) = MVLA_ERR_TIMEOUT;
-        float gmax = -CUDART_INF_F;
-        for (uint32_t r = 0; r < csize; ++r) gmax = fmaxf(gmax, sm.peer[r][tid].x);
-        float z = 0.f;
+        mx = -CUDART_INF_F;
+        for (uint32_t r = 0; r < csize; ++r) mx = fmaxf(mx, sm.peer[r][tid].x);
+        z = 0.f;
         for (uint32_t r = 0; r < csize; ++r) {
             const float2 pr = sm.peer[r][tid];
-            if (pr.x > -CUDART_INF_F) z += pr.y * ex2_approx(pr.x - gmax);
+            if (pr.x > -CUDART_INF_F) z += pr.y * ex2_approx(pr.x - mx);
         }
-        const float inv_hn = 1.f / (static_cast<float>(o.n_heads) * static_cast<float>(s.n_txt));
-        sm.w[tid] = (tid < s.n_txt && z > 0.f && okx) ? ex2_approx(sm.m[tid] - gmax) / z * inv_hn : 0.f;
+        const float iz = (tid < s.n_txt && z > 0.f && okx) ? inv_hn / z : 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) sm.w[k][tid] = ref[k] > -CUDART_INF_F ? ex2_approx(ref[k] - mx) * iz : 0.f;
     }
     __syncthreads();
 
     // ---- per key: sum over queries of the normalised probabilities (this head's contribution)
-    if (!o.free_running) pdl_wait();            // the accumulators were read and cleared by an earlier selection
+    const float* const w = sm.w[kwarp] + c0;  // 0 past the text queries
+    if (!o.free_running) pdl_wait();          // the accumulators were read and cleared by an earlier selection
 #pragma unroll
     for (int t = 0; t < NTILE; ++t) {
-        if (valid[t] <= 0) continue;
-        float acc = 0.f;
+        if (key >= valid[t]) continue;
+        if (o.acc64) {                        // (with SPLIT = 2 both halves of the queries add into the key's accumulator)
+            float acc = 0.f;
 #pragma unroll
-        for (int qc = 0; qc < TC / 16; ++qc) {
-            if (c0 + qc * 16 >= npad) break;  // columns past the padded query count were never exponentiated
-#pragma unroll
-            for (int i = 0; i < 16; ++i)      // sm.w is 0 past the text queries
-                acc = fmaf(L[t * TC + qc * 16 + i], sm.w[c0 + qc * 16 + i], acc);
+            for (int i = 0; i < TC; i += 4) {
+                if ((i & 15) == 0 && c0 + i >= npad) break;   // columns past the padded query count were never exponentiated
+                const float4 w4 = *reinterpret_cast<const float4*>(w + i);
+                acc = fmaf(L[t * TC + i], w4.x, acc);
+                acc = fmaf(L[t * TC + i + 1], w4.y, acc);
+                acc = fmaf(L[t * TC + i + 2], w4.z, acc);
+                acc = fmaf(L[t * TC + i + 3], w4.w, acc);
+            }
+            atomicAdd(o.acc64 + s.vis_off + vis0[t] + key, __float2ull_rn(acc * kFixScale));
         }
-        if (key < valid[t]) {
-            if (o.acc64)                        // (with SPLIT = 2 both halves of the queries add into the key's accumulator)
-                atomicAdd(o.acc64 + s.vis_off + vis0[t] + key, __float2ull_rn(acc * kFixScale));
-            if constexpr (SPLIT == 1) {
-                if (!o.acc64 && o.part)           // neither: the caller wants the attention copy only
-                    o.part[static_cast<int64_t>(h) * o.part_stride + s.vis_off + vis0[t] + key] = acc;
-                if (o.alpha.ptr) {              // the attention itself, for the per-patch indicators: this key's row of queries
-                    float* ap = o.alpha.ptr + static_cast<int64_t>(h) * o.alpha.stride_h + static_cast<int64_t>(s.vis_off + vis0[t] + key) * 4;
-                    const float hn = static_cast<float>(o.n_heads) * static_cast<float>(s.n_txt);   // sm.w carries 1 / (H n_t)
+        if (o.alpha.ptr) {                    // the attention itself, for the per-patch indicators: this key's row of queries
+            float* ap = o.alpha.ptr + static_cast<int64_t>(h) * o.alpha.stride_h + static_cast<int64_t>(s.vis_off + vis0[t] + key) * 4;
+            const float hn = static_cast<float>(o.n_heads) * static_cast<float>(s.n_txt);   // the weights carry 1 / (H n_t)
 #pragma unroll
-                    for (int g4 = 0; g4 < TCOL / 4; ++g4) {   // 16-byte stores: a handful of instructions (sm.w is 0 past the text queries)
-                        if (4 * g4 >= s.n_txt) break;
-                        const float4 w4 = *reinterpret_cast<const float4*>(&sm.w[4 * g4]);
-                        *reinterpret_cast<float4*>(ap + g4 * o.alpha.stride_q) = make_float4(L[t * TCOL + 4 * g4] * w4.x * hn, L[t * TCOL + 4 * g4 + 1] * w4.y * hn,
-                                             L[t * TCOL + 4 * g4 + 2] * w4.z * hn, L[t * TCOL + 4 * g4 + 3] * w4.w * hn);
-                    }
-                }
+            for (int i = 0; i < TC; i += 4) { // 16-byte stores: a handful of instructions
+                if (c0 + i >= s.n_txt) break;
+                const float4 w4 = *reinterpret_cast<const float4*>(w + i);
+                *reinterpret_cast<float4*>(ap + ((c0 + i) >> 2) * o.alpha.stride_q) =
+                    make_float4(L[t * TC + i] * w4.x * hn, L[t * TC + i + 1] * w4.y * hn, L[t * TC + i + 2] * w4.z * hn, L[t * TC + i + 3] * w4.w * hn);
             }
         }
     }
@@ -204,15 +234,14 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
 
 // grid = (cluster size, n_heads, samples), cluster = (cluster size, 1, 1), 128 x SPLIT threads.
 // TCOL: tensor-memory columns per tile (>= padded query count); NTILE: key tiles per CTA.
-// SPLIT: threads per key.  1: a thread holds all the logits of its key.  2 (fixed-point accumulators only, no
-// attention copy): threads t and t + 128 hold one half of the text queries each -- the chain through max,
-// exponentials, sums and weighted sum is half as long per warp, and a scheduler has two warps to alternate
-// between; both halves add into the key's accumulator.
+// SPLIT: threads per key.  1: a thread holds all the logits of its key.  2: threads t and t + 128 hold one half of the
+// text queries each -- the chain through exponentials, sums and weighted sum is half as long per warp, and a scheduler
+// has two warps to alternate between; both halves add into the key's accumulator.
 template <int TCOL, int NTILE, int SPLIT>
 __global__ void __launch_bounds__(kFastThreads * SPLIT, 1)
 salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,
                      const __grid_constant__ CUtensorMap tmap_k, int n_heads, int kv_group, int head_dim, int esize, int npad_max,
-                     float* __restrict__ part, int64_t part_stride, unsigned long long* __restrict__ acc64,
+                     unsigned long long* __restrict__ acc64,
                      int* status, int free_running, const AlphaOut alpha, int32_t* __restrict__ rearm, unsigned long long* __restrict__ rearm_rec,
                      unsigned long long* __restrict__ stamps, float* __restrict__ lcache, int cache_vis, int cache_cols)
 {
@@ -260,7 +289,11 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
     // row of this thread's key in the cache: [state][head][visual index][column]
     const int64_t cache_row0 = caching ? ((static_cast<int64_t>(s.cache_state) * n_heads + h) * cache_vis) * cache_cols : 0;
 
-    if (tid == 0) {                           // the loads go out first; everything else overlaps with them
+    // ---- before the wait for the kernel before this one: everything that does not read its results.  In particular the
+    //      cluster arrive: a release waits for all that its thread has issued, and behind the loads it took as long as
+    //      they did (0.6 us behind six boxes, 1.4 us behind ten).
+    const bool one = warp == 0 && elect_one();
+    if (one) {
         prefetch_tensormap(&tmap_q);
         prefetch_tensormap(&tmap_k);
         mbar_init(bar_full, 1);
@@ -268,31 +301,7 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
         mbar_init(bar_x, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         mbar_expect_tx(bar_x, csize * static_cast<uint32_t>(npad) * 8u);     // every CTA of the cluster sends npad pairs
-        // Inputs may come from the kernel before this one -- unless the host has established (stable
-        // inputs, scratch ordered by events) that nothing this kernel touches depends on it.
-        if (!free_running) pdl_wait();
-        if (stamps) {                         // measurement aid: when this CTA was free to start its loads
-            const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-            if (cta < kStampSlots) stamps[2 * cta] = global_ns();
-        }
-        int live = 0;                         // key tiles to fetch: those that exist and do not come from the cache
-#pragma unroll
-        for (int t = 0; t < NTILE; ++t) live += valid[t] > 0 && from_k[t];
-        // (no tile to compute: nothing is fetched, both barriers below complete at once)
-        mbar_expect_tx(bar_full, live > 0 ? static_cast<uint32_t>(khalves) * (npad * 128 + live * 16384) : 0u);
-        for (int kh = 0; kh < khalves && live > 0; ++kh)
-            for (int c = 0; c < npad / 16; ++c)
-                tma_load_3d(smem_u32(Qs + kh * npad * 128 + c * 2048), &tmap_q, kh * box_elems, h,
-                            s.seq_off + s.off_txt + c * 16, bar_full);
-#pragma unroll
-        for (int t = 0; t < NTILE; ++t) {
-            if (valid[t] <= 0 || !from_k[t]) continue;
-            const int row0 = tile_info(s, tt0 + t).row0;
-            for (int kh = 0; kh < khalves; ++kh)
-                tma_load_3d(smem_u32(Ks + (t * khalves + kh) * 16384), &tmap_k, kh * box_elems, h / kv_group, row0, bar_full);
-        }
     }
-    if (tid < kMaxText) sm.w[tid] = 0.f;
     __syncwarp();
     cluster_arrive_release();                 // publishes this CTA's barriers; matched by the wait before the first remote store
     uint32_t tmem_cols = 32;
@@ -300,13 +309,6 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
     // blocks until the columns are free: the launcher has made sure that the CTAs resident on a multiprocessor
     // never ask for more than its 512 columns together, so no CTA waits here for one that waits for it
     if (warp == 1) tmem_alloc(smem_u32(&s_tmem), tmem_cols);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = s_tmem;
-    // Thread 0 is past its wait for the kernel before this one, so whatever that kernel wrote is
-    // complete: the next kernel may become resident now and may read such data in its prologue.
-    pdl_trigger();
     // One CTA per sample re-arms the words through which the kernel after this one hands the kept list from
     // its selecting CTA to its copying CTAs (-1: not yet known).  Their last users finished long ago.
     if (rearm && blockIdx.x == 0 && blockIdx.y == 0) {
@@ -317,36 +319,82 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
             for (int i = tid; i < 3 * s.n_2d; i += NT) rearm_rec[static_cast<int64_t>(s.vis_off / 2) * 3 + i] = ~0ull;
         }
     }
+    int row0[NTILE], live = 0;                // key tiles to fetch: those that exist and do not come from the cache
+#pragma unroll
+    for (int t = 0; t < NTILE; ++t) {
+        row0[t] = tile_info(s, tt0 + t).row0;
+        live += valid[t] > 0 && from_k[t];
+    }
+    const int hk = h / kv_group, qrow = s.seq_off + s.off_txt, nq = npad / 16;
+    const uint32_t k_smem = smem_u32(Ks), q_smem = smem_u32(Qs);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = s_tmem;
 
-    if (tid == 0) {
+    // Warp 0 loads and multiplies: it runs these loops as a whole warp, all values the same in every lane, and one
+    // elected lane issues, so that coordinates and descriptors stay in uniform registers.  (In a single-thread branch
+    // every operand is moved to a uniform register one by one: 0.1 us more for the MMAs of a tile.)
+    if (warp == 0) {
+        // Inputs may come from the kernel before this one -- unless the host has established (stable
+        // inputs, scratch ordered by events) that nothing this kernel touches depends on it.
+        if (!free_running) pdl_wait();
+        // (no tile to compute: nothing is fetched, both barriers below complete at once)
+        if (one) mbar_expect_tx(bar_full, live > 0 ? static_cast<uint32_t>(khalves) * (npad * 128 + live * 16384) : 0u);
+#pragma unroll
+        for (int t = 0; t < NTILE; ++t) {
+            if (valid[t] <= 0 || !from_k[t]) continue;
+            for (int kh = 0; kh < khalves; ++kh)
+                if (one) tma_load_3d(k_smem + static_cast<uint32_t>(t * khalves + kh) * 16384u, &tmap_k, kh * box_elems, hk, row0[t], bar_full);
+        }
+        for (int kh = 0; kh < khalves && live > 0; ++kh)
+            for (int c = 0; c < nq; ++c)
+                if (one) tma_load_3d(q_smem + static_cast<uint32_t>(kh * npad * 128 + c * 2048), &tmap_q, kh * box_elems, h, qrow + c * 16, bar_full);
+        // Whatever the kernel before this one wrote is complete: the next kernel may become resident now and may read
+        // such data in its prologue.
+        pdl_trigger();
+        if (stamps && one) {                  // measurement aid: when this CTA was free to start its loads
+            const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+            if (cta < kStampSlots) stamps[2 * cta] = global_ns();
+        }
+    }
+    // Only warp 0 polls the barriers; the other threads park at the block barrier below (a hardware
+    // wait), so while a CTA waits for its predecessor, its loads or its MMAs it leaves the issue slots and
+    // the shared-memory pipe of the multiprocessor to the CTAs that share it.
+    bool ok = true;
+    if (warp == 0) {
         bool got = mbar_wait(bar_full, 0);
         if (!got) {                           // report, then give the copies one more bounded chance to land
             *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
             got = mbar_wait(bar_full, 0);
         }
+        __syncwarp();
+        got = __all_sync(0xffffffffu, got);
+        tc_fence_after();
         if (got) {
-            tc_fence_after();
             const uint32_t idesc = idesc_by_size(esize, npad);
+            const int ksteps = (d * esize + 31) / 32;              // an instruction consumes 32 bytes of every row
+            const uint64_t k_desc = smem_desc_sw128(k_smem), q_desc = smem_desc_sw128(q_smem);   // (addresses / 16 in the low bits)
 #pragma unroll
             for (int t = 0; t < NTILE; ++t) {
                 if (valid[t] <= 0 || !from_k[t]) continue;
-                for (int kb = 0; kb < khalves * 4; ++kb) {     // columns past d are zeros: they add nothing
-                    const int kh = kb >> 2, kin = kb & 3;          // 4 K-steps of 16 inside a 64-wide half
-                    const uint64_t a = smem_desc_sw128(smem_u32(Ks + (t * khalves + kh) * 16384) + kin * 32);
-                    const uint64_t b = smem_desc_sw128(smem_u32(Qs + kh * npad * 128) + kin * 32);
-                    umma_by_size(esize, tmem_base + t * TCOL, a, b, idesc, kb > 0 ? 1u : 0u);
+                for (int kh = 0; kh < khalves; ++kh) {
+                    const uint64_t kd = k_desc + static_cast<uint64_t>(t * khalves + kh) * (16384 >> 4);
+                    const uint64_t qd = q_desc + static_cast<uint64_t>(kh * npad) * (128 >> 4);
+                    const int n = min(4, ksteps - kh * 4);
+                    if (one) {
+                        if (esize == 2)
+                            for (int kb = 0; kb < n; ++kb) umma_bf16(tmem_base + t * TCOL, kd + 2 * kb, qd + 2 * kb, idesc, kh + kb > 0 ? 1u : 0u);
+                        else
+                            for (int kb = 0; kb < n; ++kb) umma_e4m3(tmem_base + t * TCOL, kd + 2 * kb, qd + 2 * kb, idesc, kh + kb > 0 ? 1u : 0u);
+                    }
                 }
             }
         }
-        umma_commit(bar_mma);                 // arrives once every MMA issued above has finished
-    }
-    // Only thread 0 polls the barriers; the other threads park at the block barrier below (a hardware
-    // wait), so while a CTA waits for its predecessor, its loads or its MMAs it leaves the issue slots and
-    // the shared-memory pipe of the multiprocessor to the CTAs that share it.
-    bool ok = true;
-    if (tid == 0) {
+        if (one) umma_commit(bar_mma);        // arrives once every MMA issued above has finished
         ok = mbar_wait(bar_mma, 0);
         if (!ok) *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
+        __syncwarp();
     }
     ok = __syncthreads_and(ok) != 0;          // block-uniform from here on (aligned instructions follow)
     tc_fence_after();
@@ -389,7 +437,7 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
         }
     }
     softmax_scores<TCOL, NTILE, SPLIT>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
-                                       FastOut{part, part_stride, acc64, status, free_running, n_heads, alpha});
+                                       FastOut{acc64, status, free_running, n_heads, alpha});
 
     tc_fence_before();
     __syncthreads();
@@ -434,13 +482,22 @@ salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restric
         valid[t] = ti[t].valid;
         vis0[t] = ti[t].vis0;
     }
-    if (warp == 0) {                          // the loads go out first
+    // before the wait for the kernel before this one (see salience_fast_kernel)
+    if (tid == 0) {
+        mbar_init(bar_full, 1);
+        mbar_init(bar_x, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        mbar_expect_tx(bar_x, gridDim.x * static_cast<uint32_t>(npad) * 8u);
+    }
+    __syncwarp();
+    cluster_arrive_release();                 // publishes this CTA's barriers; matched by the wait before the first remote store
+    for (int i = tid; i < (npad - s.n_txt) * d; i += NT) rows[(s.n_txt + i / d) * pitch + i % d] = 0.f;   // query rows that do not exist
+    if (rearm && blockIdx.x == 0 && blockIdx.y == 0)
+        for (int i = tid; i < s.n_out; i += NT) rearm[s.out_off + i] = -1;
+    __syncthreads();
+    if (warp == 0) {
+        pdl_wait();
         if (lane == 0) {
-            mbar_init(bar_full, 1);
-            mbar_init(bar_x, 1);
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            mbar_expect_tx(bar_x, gridDim.x * static_cast<uint32_t>(npad) * 8u);
-            pdl_wait();
             if (stamps) {
                 const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
                 if (cta < kStampSlots) stamps[2 * cta] = global_ns();
@@ -461,16 +518,8 @@ salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restric
             for (int i = lane; i < valid[t]; i += 32)
                 bulk_load(smem_u32(rows + (npad_max + t * kKeyTile + i) * pitch), ks + i * krow, bytes, bar_full);
         }
-    } else {                                  // query rows that do not exist read as zero
-        for (int i = tid - 32; i < (npad - s.n_txt) * d; i += NT - 32) rows[(s.n_txt + i / d) * pitch + i % d] = 0.f;
+        pdl_trigger();
     }
-    if (tid < kMaxText) sm.w[tid] = 0.f;
-    __syncwarp();
-    cluster_arrive_release();                 // publishes this CTA's barriers; matched by the wait before the first remote store
-    __syncthreads();
-    pdl_trigger();                            // (see salience_fast_kernel)
-    if (rearm && blockIdx.x == 0 && blockIdx.y == 0)
-        for (int i = tid; i < s.n_out; i += NT) rearm[s.out_off + i] = -1;
     bool ok = true;
     if (tid == 0) {
         ok = mbar_wait(bar_full, 0);
@@ -505,7 +554,7 @@ salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restric
         }
     }
     softmax_scores<TCOL, NTILE, 2>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
-                                   FastOut{nullptr, 0, acc64, status, 0, n_heads, AlphaOut{nullptr, 0, 0}});
+                                   FastOut{acc64, status, 0, n_heads, AlphaOut{nullptr, 0, 0}});
     if (stamps) {
         __syncthreads();
         if (tid == 0) {
@@ -517,7 +566,7 @@ salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restric
 
 template <int TCOL, int NTILE, int SPLIT>
 cudaError_t launch_fast_t(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tq,
-                          const CUtensorMap* tk, int cluster, int npad, float* part, int64_t part_stride,
+                          const CUtensorMap* tk, int cluster, int npad,
                           unsigned long long* acc64, int* status, int free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                           float* lcache, int cache_vis, int cache_cols, cudaStream_t stream)
 {
@@ -543,7 +592,7 @@ cudaError_t launch_fast_t(const BatchDesc& bd, int n_heads, int kv_group, int he
     attr[1] = pdl_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, n_heads, kv_group, head_dim, esize, npad, part, part_stride, acc64, status, free_running, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols);
+    return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, n_heads, kv_group, head_dim, esize, npad, acc64, status, free_running, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols);
 }
 
 template <int TCOL, int NTILE>
@@ -596,19 +645,17 @@ bool fast_salience_supported(int tiles_per_cta) { return tiles_per_cta >= 1 && t
 
 cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tmap_q,
                                  const CUtensorMap* tmap_k, int tiles_per_cta, int cluster, int npad,
-                                 float* part, int64_t part_stride, unsigned long long* acc64, int* status,
+                                 unsigned long long* acc64, int* status,
                                  bool free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                                  float* lcache, int cache_vis, int cache_cols, cudaStream_t stream)
 {
     const int tcol = npad <= 16 ? 16 : (npad <= 32 ? 32 : 64);
-    // two threads per key where the kernel's outputs allow it (see the kernel) and a thread still holds 16 queries
-    const int split = (acc64 && !alpha.ptr && tcol >= 32) ? 2 : 1;
+    const int split = tcol >= 32 ? 2 : 1;     // two threads per key while a thread still holds 16 queries
 #define MVLA_FAST(TC, NTL, SP)                                                                                  \
     if (tcol == TC && tiles_per_cta == NTL && split == SP)                                                      \
-        return launch_fast_t<TC, NTL, SP>(bd, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, part, part_stride, \
+        return launch_fast_t<TC, NTL, SP>(bd, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, \
                                           acc64, status, free_running ? 1 : 0, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream);
-    MVLA_FAST(16, 1, 1) MVLA_FAST(32, 1, 1) MVLA_FAST(64, 1, 1) MVLA_FAST(16, 2, 1) MVLA_FAST(32, 2, 1) MVLA_FAST(64, 2, 1)
-    MVLA_FAST(32, 1, 2) MVLA_FAST(64, 1, 2) MVLA_FAST(32, 2, 2) MVLA_FAST(64, 2, 2)
+    MVLA_FAST(16, 1, 1) MVLA_FAST(16, 2, 1) MVLA_FAST(32, 1, 2) MVLA_FAST(64, 1, 2) MVLA_FAST(32, 2, 2) MVLA_FAST(64, 2, 2)
 #undef MVLA_FAST
     return cudaErrorInvalidConfiguration;
 }

@@ -87,12 +87,6 @@ __device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatil
     *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
     return false;
 }
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-    return p != 0;
-}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
