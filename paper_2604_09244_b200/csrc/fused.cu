@@ -81,7 +81,7 @@ struct FastOut {
 // overflowing, and the two shared-memory round trips, two block barriers and the butterfly that found the maximum leave
 // the chain (a warp whose exponents exceed kRescaleAt takes its true maxima after all).  The pairs (reference, sum) of
 // the four warps are combined per query, then those of the cluster's CTAs.
-template <int TCOL, int NTILE, int SPLIT>
+template <int TCOL, int NTILE, int SPLIT, bool ALPHA>
 __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT], const SampleDev& s, const int (&valid)[NTILE],
                                                const int (&vis0)[NTILE], bool ok, int npad, int h, float cscale, uint32_t bar_x,
                                                FastSmem& sm, const FastOut& o)
@@ -205,7 +205,7 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
 #pragma unroll
     for (int t = 0; t < NTILE; ++t) {
         if (key >= valid[t]) continue;
-        if (o.acc64) {                        // (with SPLIT = 2 both halves of the queries add into the key's accumulator)
+        if constexpr (!ALPHA) {               // (with SPLIT = 2 both halves of the queries add into the key's accumulator)
             float acc = 0.f;
 #pragma unroll
             for (int i = 0; i < TC; i += 4) {
@@ -218,7 +218,7 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
             }
             atomicAdd(o.acc64 + s.vis_off + vis0[t] + key, __float2ull_rn(acc * kFixScale));
         }
-        if (o.alpha.ptr) {                    // the attention itself, for the per-patch indicators: this key's row of queries
+        if constexpr (ALPHA) {                // the attention itself, for the per-patch indicators: this key's row of queries
             float* ap = o.alpha.ptr + static_cast<int64_t>(h) * o.alpha.stride_h + static_cast<int64_t>(s.vis_off + vis0[t] + key) * 4;
             const float hn = static_cast<float>(o.n_heads) * static_cast<float>(s.n_txt);   // the weights carry 1 / (H n_t)
 #pragma unroll
@@ -234,10 +234,13 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
 
 // grid = (cluster size, n_heads, samples), cluster = (cluster size, 1, 1), 128 x SPLIT threads.
 // TCOL: tensor-memory columns per tile (>= padded query count); NTILE: key tiles per CTA.
+// KIND: what else the kernel does.  Its code runs once per launch, from a cold instruction cache: code that a step does
+// not use still costs it time (0.5 us for 1.5 KB), so the variants are compiled apart.
 // SPLIT: threads per key.  1: a thread holds all the logits of its key.  2: threads t and t + 128 hold one half of the
 // text queries each -- the chain through exponentials, sums and weighted sum is half as long per warp, and a scheduler
 // has two warps to alternate between; both halves add into the key's accumulator.
-template <int TCOL, int NTILE, int SPLIT>
+enum { kPlain = 0, kWithCache = 1, kForPatches = 2 };   // scores only; with the logit cache; the attention copy instead of scores
+template <int TCOL, int NTILE, int SPLIT, int KIND>
 __global__ void __launch_bounds__(kFastThreads * SPLIT, 1)
 salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,
                      const __grid_constant__ CUtensorMap tmap_k, int n_heads, int kv_group, int head_dim, int esize, int npad_max,
@@ -277,7 +280,7 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
     int valid[NTILE], vis0[NTILE];
     bool from_k[NTILE];                       // the tile's logits come from K (TMA + MMA); false: from the logit cache
     bool any_live = false;
-    const bool caching = lcache != nullptr && s.cache_state >= 0;
+    const bool caching = KIND == kWithCache && s.cache_state >= 0;
 #pragma unroll
     for (int t = 0; t < NTILE; ++t) {
         const TileInfo ti = tile_info(s, tt0 + t);
@@ -312,7 +315,7 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
     // One CTA per sample re-arms the words through which the kernel after this one hands the kept list from
     // its selecting CTA to its copying CTAs (-1: not yet known).  Their last users finished long ago.
     if (rearm && blockIdx.x == 0 && blockIdx.y == 0) {
-        if (!rearm_rec) {
+        if constexpr (KIND != kForPatches) {
             for (int i = tid; i < s.n_out; i += NT) rearm[s.out_off + i] = -1;
         } else {                              // the patch-by-patch tail: its list words, and three words per patch
             for (int i = tid; i < kHandWords + s.n_txt + s.n_2d + s.n_3d; i += NT) rearm[s.cap_off + i] = -1;
@@ -419,7 +422,7 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
     }
     // Logit cache: a computed tile leaves its raw dot products for the next action step, a reused tile takes
     // the previous step's instead (128 bytes per key and head at 32 queries: half a key row, and no MMA).
-    if (caching && ok) {
+    if (KIND == kWithCache && caching && ok) {
 #pragma unroll
         for (int t = 0; t < NTILE; ++t) {
             if (key >= valid[t]) continue;
@@ -436,7 +439,7 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
             }
         }
     }
-    softmax_scores<TCOL, NTILE, SPLIT>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
+    softmax_scores<TCOL, NTILE, SPLIT, KIND == kForPatches>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
                                        FastOut{acc64, status, free_running, n_heads, alpha});
 
     tc_fence_before();
@@ -553,7 +556,7 @@ salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restric
             }
         }
     }
-    softmax_scores<TCOL, NTILE, 2>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
+    softmax_scores<TCOL, NTILE, 2, false>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
                                    FastOut{acc64, status, 0, n_heads, AlphaOut{nullptr, 0, 0}});
     if (stamps) {
         __syncthreads();
@@ -564,14 +567,14 @@ salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restric
     }
 }
 
-template <int TCOL, int NTILE, int SPLIT>
+template <int TCOL, int NTILE, int SPLIT, int KIND>
 cudaError_t launch_fast_t(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tq,
                           const CUtensorMap* tk, int cluster, int npad,
                           unsigned long long* acc64, int* status, int free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                           float* lcache, int cache_vis, int cache_cols, cudaStream_t stream)
 {
     size_t smem = 1024 + static_cast<size_t>((head_dim * esize + 127) / 128) * (static_cast<size_t>(NTILE) * 16384 + npad * 128);
-    auto kern = salience_fast_kernel<TCOL, NTILE, SPLIT>;
+    auto kern = salience_fast_kernel<TCOL, NTILE, SPLIT, KIND>;
     // resident CTAs x tensor-memory columns must not exceed the 512 of a multiprocessor
     const int tmem_cols = tmem_cols_for(TCOL * NTILE);
     smem = smem_for_tmem(smem, tmem_cols);
@@ -651,11 +654,15 @@ cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group,
 {
     const int tcol = npad <= 16 ? 16 : (npad <= 32 ? 32 : 64);
     const int split = tcol >= 32 ? 2 : 1;     // two threads per key while a thread still holds 16 queries
-#define MVLA_FAST(TC, NTL, SP)                                                                                  \
-    if (tcol == TC && tiles_per_cta == NTL && split == SP)                                                      \
-        return launch_fast_t<TC, NTL, SP>(bd, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, \
-                                          acc64, status, free_running ? 1 : 0, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream);
+    if ((acc64 == nullptr) == (alpha.ptr == nullptr)) return cudaErrorInvalidConfiguration;      // one or the other
+    const int kind = alpha.ptr ? kForPatches : (lcache ? kWithCache : kPlain);
+#define MVLA_FAST1(TC, NTL, SP, KD)                                                                             \
+    if (tcol == TC && tiles_per_cta == NTL && split == SP && kind == KD)                                        \
+        return launch_fast_t<TC, NTL, SP, KD>(bd, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, acc64, status, \
+                                              free_running ? 1 : 0, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream);
+#define MVLA_FAST(TC, NTL, SP) MVLA_FAST1(TC, NTL, SP, kPlain) MVLA_FAST1(TC, NTL, SP, kWithCache) MVLA_FAST1(TC, NTL, SP, kForPatches)
     MVLA_FAST(16, 1, 1) MVLA_FAST(16, 2, 1) MVLA_FAST(32, 1, 2) MVLA_FAST(64, 1, 2) MVLA_FAST(32, 2, 2) MVLA_FAST(64, 2, 2)
+#undef MVLA_FAST1
 #undef MVLA_FAST
     return cudaErrorInvalidConfiguration;
 }
