@@ -28,8 +28,9 @@ __device__ __forceinline__ void st_stream(uint4* p, const uint4& v)
 }
 
 // grid.x covers chunk_rows * segs_per_row_all warp-units.
+template <class BD>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
-compact_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CompactArgs a, const int32_t* __restrict__ kept_idx,
+compact_kernel(const __grid_constant__ BD bd, const __grid_constant__ CompactArgs a, const int32_t* __restrict__ kept_idx,
                int32_t chunk_rows, int32_t chunk_row0, const int32_t* __restrict__ out_offsets,
                int32_t chunk_first, int32_t batch_total)
 {
@@ -55,11 +56,11 @@ compact_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ Com
         if (out_offsets) {            // offsets known only on the device: scan the whole batch
             while (b + 1 < batch_total && orow >= out_offsets[b + 1]) ++b;
             b -= chunk_first;
-            if (b < 0 || b >= bd.n) continue;    // row belongs to another launch's samples
+            if (b < 0 || b >= bd.count()) continue;    // row belongs to another launch's samples
         } else {
-            while (b + 1 < bd.n && orow >= bd.s[b + 1].out_off) ++b;
+            while (b + 1 < bd.count() && orow >= bd.at(b + 1).out_off) ++b;
         }
-        const int64_t srow = static_cast<int64_t>(bd.s[b].seq_off) + kept_idx[orow];
+        const int64_t srow = static_cast<int64_t>(bd.at(b).seq_off) + kept_idx[orow];
 
         const int tsel = u >= a.seg_begin[2] ? 2 : (u >= a.seg_begin[1] ? 1 : 0);
         const int seg = u - a.seg_begin[tsel];
@@ -140,8 +141,10 @@ cudaError_t launch_compact(const BatchDesc& bd, const CompactJob& job, const int
     cudaLaunchAttribute attr[1] = {pdl_attribute()};
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, compact_kernel, bd, a, kept_idx, chunk_rows, chunk_row0, out_offsets, chunk_first,
-                              batch_total);
+    return with_desc(bd, [&](const auto& d) {
+        return cudaLaunchKernelEx(&cfg, compact_kernel<std::decay_t<decltype(d)>>, d, a, kept_idx, chunk_rows, chunk_row0, out_offsets,
+                                  chunk_first, batch_total);
+    });
 }
 
 }  // namespace mvla

@@ -240,9 +240,9 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
 // text queries each -- the chain through exponentials, sums and weighted sum is half as long per warp, and a scheduler
 // has two warps to alternate between; both halves add into the key's accumulator.
 enum { kPlain = 0, kWithCache = 1, kForPatches = 2 };   // scores only; with the logit cache; the attention copy instead of scores
-template <int TCOL, int NTILE, int SPLIT, int KIND>
+template <int TCOL, int NTILE, int SPLIT, int KIND, class BD>
 __global__ void __launch_bounds__(kFastThreads * SPLIT, 1)
-salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,
+salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUtensorMap tmap_q,
                      const __grid_constant__ CUtensorMap tmap_k, int n_heads, int kv_group, int head_dim, int esize, int npad_max,
                      unsigned long long* __restrict__ acc64,
                      int* status, int free_running, const AlphaOut alpha, int32_t* __restrict__ rearm, unsigned long long* __restrict__ rearm_rec,
@@ -258,7 +258,7 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
     __shared__ __align__(8) uint64_t s_bar[3];
     __shared__ uint32_t s_tmem;
 
-    const SampleDev& s = bd.s[blockIdx.z];
+    const SampleDev& s = bd.at(blockIdx.z);
     const int h = blockIdx.y;
     const int tid = threadIdx.x, warp = tid >> 5;
     const int key = tid & (kFastThreads - 1);            // key of the tile(s) this thread works on
@@ -459,9 +459,9 @@ salience_fast_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant
 // Bound by latency at the sizes this path serves (2.2 MB a step at 192 tokens, 8 heads x 64): the loads of all rows of a
 // CTA go out at once, where scalar loads through registers kept a few in flight, and the step runs as two chained
 // kernels like that of the other types (24.6 -> 14.8 us a step at that size).
-template <int TCOL, int NTILE>
+template <int TCOL, int NTILE, class BD>
 __global__ void __launch_bounds__(kFastThreads * 2, 1)
-salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restrict__ q, const float* __restrict__ k, int n_heads, int kv_group,
+salience_f32_kernel(const __grid_constant__ BD bd, const float* __restrict__ q, const float* __restrict__ k, int n_heads, int kv_group,
                     int d, int npad_max, unsigned long long* __restrict__ acc64, int* status, int32_t* __restrict__ rearm,
                     unsigned long long* __restrict__ stamps)
 {
@@ -469,7 +469,7 @@ salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restric
     extern __shared__ __align__(16) float rows[];         // [npad_max queries, then NTILE x 128 keys][d + 4]
     __shared__ FastSmem sm;
     __shared__ __align__(8) uint64_t s_bar[2];
-    const SampleDev& s = bd.s[blockIdx.z];
+    const SampleDev& s = bd.at(blockIdx.z);
     const int h = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int key = tid & (kFastThreads - 1), c0 = (tid / kFastThreads) * TC;
     const int npad = min(npad_max, (s.n_txt + 15) & ~15);
@@ -567,14 +567,14 @@ salience_f32_kernel(const __grid_constant__ BatchDesc bd, const float* __restric
     }
 }
 
-template <int TCOL, int NTILE, int SPLIT, int KIND>
-cudaError_t launch_fast_t(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tq,
+template <int TCOL, int NTILE, int SPLIT, int KIND, class BD>
+cudaError_t launch_fast_t(const BD& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tq,
                           const CUtensorMap* tk, int cluster, int npad,
                           unsigned long long* acc64, int* status, int free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                           float* lcache, int cache_vis, int cache_cols, cudaStream_t stream)
 {
     size_t smem = 1024 + static_cast<size_t>((head_dim * esize + 127) / 128) * (static_cast<size_t>(NTILE) * 16384 + npad * 128);
-    auto kern = salience_fast_kernel<TCOL, NTILE, SPLIT, KIND>;
+    auto kern = salience_fast_kernel<TCOL, NTILE, SPLIT, KIND, BD>;
     // resident CTAs x tensor-memory columns must not exceed the 512 of a multiprocessor
     const int tmem_cols = tmem_cols_for(TCOL * NTILE);
     smem = smem_for_tmem(smem, tmem_cols);
@@ -598,12 +598,12 @@ cudaError_t launch_fast_t(const BatchDesc& bd, int n_heads, int kv_group, int he
     return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, n_heads, kv_group, head_dim, esize, npad, acc64, status, free_running, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols);
 }
 
-template <int TCOL, int NTILE>
-cudaError_t launch_f32_t(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, const float* q, const float* k, int cluster, int npad,
+template <int TCOL, int NTILE, class BD>
+cudaError_t launch_f32_t(const BD& bd, int n_heads, int kv_group, int head_dim, const float* q, const float* k, int cluster, int npad,
                          unsigned long long* acc64, int* status, int32_t* rearm, unsigned long long* stamps, cudaStream_t stream)
 {
     const size_t smem = sizeof(float) * static_cast<size_t>(npad + NTILE * kKeyTile) * (head_dim + 4);
-    auto kern = salience_f32_kernel<TCOL, NTILE>;
+    auto kern = salience_f32_kernel<TCOL, NTILE, BD>;
     static KernelSetup ks;
     const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kFastThreads * 2, smem, 0);
     if (e != cudaSuccess) return e;
@@ -638,7 +638,8 @@ cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, 
     if (!f32_salience_supported(tiles_per_cta, npad, head_dim)) return cudaErrorInvalidConfiguration;
 #define MVLA_F32(TC, NTL)                                                                                       \
     if (npad <= TC && tiles_per_cta == NTL)                                                                     \
-        return launch_f32_t<TC, NTL>(bd, n_heads, kv_group, head_dim, q, k, cluster, npad, acc64, status, rearm, stamps, stream);
+        return with_desc(bd, [&](const auto& d) {                                                               \
+            return launch_f32_t<TC, NTL>(d, n_heads, kv_group, head_dim, q, k, cluster, npad, acc64, status, rearm, stamps, stream); });
     MVLA_F32(32, 1) MVLA_F32(64, 1) MVLA_F32(32, 2) MVLA_F32(64, 2)
 #undef MVLA_F32
     return cudaErrorInvalidConfiguration;
@@ -658,8 +659,9 @@ cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group,
     const int kind = alpha.ptr ? kForPatches : (lcache ? kWithCache : kPlain);
 #define MVLA_FAST1(TC, NTL, SP, KD)                                                                             \
     if (tcol == TC && tiles_per_cta == NTL && split == SP && kind == KD)                                        \
-        return launch_fast_t<TC, NTL, SP, KD>(bd, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, acc64, status, \
-                                              free_running ? 1 : 0, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream);
+        return with_desc(bd, [&](const auto& d) {                                                               \
+            return launch_fast_t<TC, NTL, SP, KD>(d, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, acc64, status, \
+                                                  free_running ? 1 : 0, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream); });
 #define MVLA_FAST(TC, NTL, SP) MVLA_FAST1(TC, NTL, SP, kPlain) MVLA_FAST1(TC, NTL, SP, kWithCache) MVLA_FAST1(TC, NTL, SP, kForPatches)
     MVLA_FAST(16, 1, 1) MVLA_FAST(16, 2, 1) MVLA_FAST(32, 1, 2) MVLA_FAST(64, 1, 2) MVLA_FAST(32, 2, 2) MVLA_FAST(64, 2, 2)
 #undef MVLA_FAST1

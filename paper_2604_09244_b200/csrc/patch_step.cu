@@ -23,34 +23,34 @@ struct PatchTailPlan {
     int16_t cta0[kMaxChunk + 1];      // first copying CTA of every sample (counted from 0); cta0[n] = their number
 };
 
-template <typename T, int PP>
+template <typename T, int PP, class BD>
 __global__ void __launch_bounds__(kTailThreads, 1)
-patch_tail_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ PatchTailPlan tp, int n_heads,
+patch_tail_kernel(const __grid_constant__ BD bd, const __grid_constant__ PatchTailPlan tp, int n_heads,
                   const AlphaOut alpha, const T* __restrict__ hidden, int d_model, float* __restrict__ x_out,
                   float* __restrict__ attn_out, unsigned long long* rec, const PatchParams pp, const PatchIO io,
                   const __grid_constant__ CompactArgs ca, int32_t* list, unsigned int* ticket_counter)
 {
-    const int n_ind = tp.ind0[bd.n];
+    const int n_ind = tp.ind0[bd.count()];
     int c = cta_ticket(ticket_counter);
     if (c < n_ind) {
         int b = 0;
-        while (b + 1 < bd.n && c >= tp.ind0[b + 1]) ++b;
-        patch_indicators_block<T, PP>(bd.s[b], c - tp.ind0[b], n_heads, alpha, hidden, d_model, x_out, attn_out, rec, true);
+        while (b + 1 < bd.count() && c >= tp.ind0[b + 1]) ++b;
+        patch_indicators_block<T, PP>(bd.at(b), c - tp.ind0[b], n_heads, alpha, hidden, d_model, x_out, attn_out, rec, true);
         return;
     }
     c -= n_ind;
-    if (c < bd.n) {
+    if (c < bd.count()) {
         __shared__ PatchSmemT<kTailThreads> sm;
-        const SampleDev& s = bd.s[c];
-        const bool copying = tp.cta0[bd.n] > 0;
-        patch_select_block<kTailThreads>(s, c, bd.n, pp, io, sm, rec, copying ? list + s.cap_off : nullptr);
+        const SampleDev& s = bd.at(c);
+        const bool copying = tp.cta0[bd.count()] > 0;
+        patch_select_block<kTailThreads>(s, c, bd.count(), pp, io, sm, rec, copying ? list + s.cap_off : nullptr);
         return;
     }
     // ---- row copy
-    c -= bd.n;
+    c -= bd.count();
     int b = 0;
-    while (b + 1 < bd.n && c >= tp.cta0[b + 1]) ++b;
-    const SampleDev& s = bd.s[b];
+    while (b + 1 < bd.count() && c >= tp.cta0[b + 1]) ++b;
+    const SampleDev& s = bd.at(b);
     const int tid = threadIdx.x, lane = tid & 31;
     const int part = c - tp.cta0[b], nparts = tp.cta0[b + 1] - tp.cta0[b];
     const int w = part * (kTailThreads / 32) + (tid >> 5), nw = nparts * (kTailThreads / 32);
@@ -151,8 +151,9 @@ cudaError_t launch_patch_tail(const BatchDesc& bd, int n_heads, AlphaOut alpha, 
     cfg.numAttrs = 1;
 #define MVLA_TAIL(T, PPV)                                                                                     \
     if (per == PPV)                                                                                           \
-        return cudaLaunchKernelEx(&cfg, patch_tail_kernel<T, PPV>, bd, tp, n_heads, alpha,                    \
-                                  static_cast<const T*>(hidden), d_model, x_out, attn_out, rec, pp, io, ca, list, ticket_counter);
+        return with_desc(bd, [&](const auto& d) {                                                             \
+            return cudaLaunchKernelEx(&cfg, patch_tail_kernel<T, PPV, std::decay_t<decltype(d)>>, d, tp, n_heads, alpha, \
+                                      static_cast<const T*>(hidden), d_model, x_out, attn_out, rec, pp, io, ca, list, ticket_counter); });
     if (dtype == MVLA_DTYPE_BF16) { MVLA_TAIL(__nv_bfloat16, 8) MVLA_TAIL(__nv_bfloat16, 4) MVLA_TAIL(__nv_bfloat16, 2) }
     else { MVLA_TAIL(float, 8) MVLA_TAIL(float, 4) MVLA_TAIL(float, 2) }
 #undef MVLA_TAIL

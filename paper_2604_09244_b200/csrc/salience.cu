@@ -317,14 +317,14 @@ __global__ void take_scores_kernel(unsigned long long* __restrict__ acc64, int t
 // predecessor LAST, so that "this kernel is complete" keeps implying "its predecessor is complete" for whatever
 // follows -- and, with `acc64`, to take the scores that the predecessor has left in the accumulators: one kernel
 // less on the chain of the stand-alone scores.
-template <typename T>
+template <typename T, class BD>
 __global__ void __launch_bounds__(256)
-l1norm_kernel(const __grid_constant__ BatchDesc bd, int d_model, const T* __restrict__ hidden,
+l1norm_kernel(const __grid_constant__ BD bd, int d_model, const T* __restrict__ hidden,
               float* __restrict__ l1, int early, unsigned long long* __restrict__ acc64, float* __restrict__ attn)
 {
     if (early) pdl_trigger();
     else pdl_wait();
-    const SampleDev& s = bd.s[blockIdx.y];
+    const SampleDev& s = bd.at(blockIdx.y);
     const int nv = s.n_2d + s.n_3d;
     const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (j >= nv) {
@@ -465,8 +465,14 @@ cudaError_t launch_l1norm(const BatchDesc& bd, int dtype, int d_model, const voi
     cfg.numAttrs = beside_predecessor ? 1 : 0;
     const int early = beside_predecessor ? 1 : 0;
     if (dtype == MVLA_DTYPE_BF16)
-        return cudaLaunchKernelEx(&cfg, l1norm_kernel<__nv_bfloat16>, bd, d_model, static_cast<const __nv_bfloat16*>(hidden), l1, early, acc64, attn);
-    return cudaLaunchKernelEx(&cfg, l1norm_kernel<float>, bd, d_model, static_cast<const float*>(hidden), l1, early, acc64, attn);
+        return with_desc(bd, [&](const auto& d) {
+            return cudaLaunchKernelEx(&cfg, l1norm_kernel<__nv_bfloat16, std::decay_t<decltype(d)>>, d, d_model,
+                                      static_cast<const __nv_bfloat16*>(hidden), l1, early, acc64, attn);
+        });
+    return with_desc(bd, [&](const auto& d) {
+        return cudaLaunchKernelEx(&cfg, l1norm_kernel<float, std::decay_t<decltype(d)>>, d, d_model, static_cast<const float*>(hidden), l1,
+                                  early, acc64, attn);
+    });
 }
 
 }  // namespace mvla

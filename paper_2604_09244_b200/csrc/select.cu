@@ -10,12 +10,12 @@
 namespace mvla {
 namespace {
 
-template <int NT, int CAP>
+template <int NT, int CAP, class BD>
 __global__ void __launch_bounds__(NT, 1)
-select_kernel(const __grid_constant__ BatchDesc bd, const GateParams gp, const SelectIO io)
+select_kernel(const __grid_constant__ BD bd, const GateParams gp, const SelectIO io)
 {
     __shared__ SelectSmem<NT, CAP> sm;
-    select_sample<NT, CAP>(bd.s[blockIdx.x], blockIdx.x, gp, io, sm);
+    select_sample<NT, CAP>(bd.at(blockIdx.x), blockIdx.x, gp, io, sm);
 }
 
 }  // namespace
@@ -33,9 +33,12 @@ cudaError_t launch_select(const BatchDesc& bd, const GateParams& gp, const Selec
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     // few elements per thread keep the chain short: the capacity is the smallest that holds the largest sample
-    if (wide) return cudaLaunchKernelEx(&cfg, select_kernel<1024, kMaxVis>, bd, gp, io);
-    if (max_vis > 1024) return cudaLaunchKernelEx(&cfg, select_kernel<512, 2048>, bd, gp, io);
-    return cudaLaunchKernelEx(&cfg, select_kernel<512, 1024>, bd, gp, io);
+    return with_desc(bd, [&](const auto& d) {
+        using BD = std::decay_t<decltype(d)>;
+        if (wide) return cudaLaunchKernelEx(&cfg, select_kernel<1024, kMaxVis, BD>, d, gp, io);
+        if (max_vis > 1024) return cudaLaunchKernelEx(&cfg, select_kernel<512, 2048, BD>, d, gp, io);
+        return cudaLaunchKernelEx(&cfg, select_kernel<512, 1024, BD>, d, gp, io);
+    });
 }
 
 }  // namespace mvla

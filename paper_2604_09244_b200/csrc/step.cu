@@ -43,34 +43,34 @@ __global__ void wait_probe_kernel(const int* never_set, uint64_t limit_ns, int* 
 // dispatched in: a copying CTA never keeps its selecting CTA from running.  (Taking the roles in the order
 // in which the CTAs start, by a ticket from an atomic counter as the patch-by-patch tail does, cost 0.4 us per
 // step here: 296 atomics on one word.)  All waits are bounded all the same.
-template <int NT, int CAP>
-__global__ void __launch_bounds__(NT)
-select_copy_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ TailPlan tp, const GateParams gp,
+template <int NT, int CAP, class BD>
+__global__ void __launch_bounds__(NT, 1024 / NT)      // as many CTAs to a multiprocessor as the launcher counts on
+select_copy_kernel(const __grid_constant__ BD bd, const __grid_constant__ TailPlan tp, const GateParams gp,
                    const SelectIO io, const __grid_constant__ CompactArgs ca, int32_t* __restrict__ list, int* status,
                    unsigned long long* __restrict__ stamps)
 {
     const int tid = threadIdx.x, lane = tid & 31;
     const int cta = blockIdx.x;
-    if (cta < bd.n) {
+    if (cta < bd.count()) {
         // ---- selection of one sample, by one CTA
         __shared__ SelectSmem<NT, CAP> sm;
         const int b = cta;
         SelectRole role;
         role.late_pdl = true;
         role.l1_late = true;                                // the norms may come from a kernel that ran beside the scoring
-        if (tp.cta0[bd.n] > 0) role.kept_sm = list + bd.s[b].out_off;   // every word is its own "ready" signal
-        select_sample<NT, CAP>(bd.s[b], b, gp, io, sm, role, [&]() {}, [&]() {
+        if (tp.cta0[bd.count()] > 0) role.kept_sm = list + bd.at(b).out_off;   // every word is its own "ready" signal
+        select_sample<NT, CAP>(bd.at(b), b, gp, io, sm, role, [&]() {}, [&]() {
             if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
         });
         if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta] = stamps[2 * cta + 1];   // placeholder start, see the copiers
         return;
     }
     // ---- row copy
-    const int c = cta - bd.n;
+    const int c = cta - bd.count();
     int b = 0;
-    while (b + 1 < bd.n && c >= tp.cta0[b + 1]) ++b;
+    while (b + 1 < bd.count() && c >= tp.cta0[b + 1]) ++b;
     const int part = c - tp.cta0[b], nparts = tp.cta0[b + 1] - tp.cta0[b];
-    const SampleDev& s = bd.s[b];
+    const SampleDev& s = bd.at(b);
     const int w = part * (NT / 32) + (tid >> 5), nw = nparts * (NT / 32);
 
     // Output position of the text rows: known on the host when the split is (FIXED budgets, cold start),
@@ -112,8 +112,8 @@ select_copy_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__
     }
 }
 
-template <int NT, int CAP>
-cudaError_t launch_t(const BatchDesc& bd, const TailPlan& tp, const GateParams& gp, const SelectIO& io, const CompactArgs& ca,
+template <int NT, int CAP, class BD>
+cudaError_t launch_t(const BD& bd, const TailPlan& tp, const GateParams& gp, const SelectIO& io, const CompactArgs& ca,
                      int32_t* list, int* status, unsigned long long* stamps, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
@@ -123,7 +123,7 @@ cudaError_t launch_t(const BatchDesc& bd, const TailPlan& tp, const GateParams& 
     cudaLaunchAttribute attr[1] = {pdl_attribute()};
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, select_copy_kernel<NT, CAP>, bd, tp, gp, io, ca, list, status, stamps);
+    return cudaLaunchKernelEx(&cfg, select_copy_kernel<NT, CAP, BD>, bd, tp, gp, io, ca, list, status, stamps);
 }
 
 int max_vis_of(const BatchDesc& bd)
@@ -178,9 +178,12 @@ cudaError_t launch_select_copy(const BatchDesc& bd, const GateParams& gp, const 
         for (int b = 0; b < bd.n; ++b) tp.cta0[b] = 0;       // nothing to copy: selection only
     }
     for (int b = bd.n; b <= kMaxChunk; ++b) tp.cta0[b] = static_cast<int16_t>(next);
-    if (max_vis_of(bd) <= 1024) return launch_t<512, 1024>(bd, tp, gp, io, ca, list, status, stamps, stream);
-    if (max_vis_of(bd) > 2048) return launch_t<1024, kMaxVis>(bd, tp, gp, io, ca, list, status, stamps, stream);
-    return launch_t<512, 2048>(bd, tp, gp, io, ca, list, status, stamps, stream);
+    const int nv = max_vis_of(bd);
+    return with_desc(bd, [&](const auto& d) {
+        if (nv <= 1024) return launch_t<512, 1024>(d, tp, gp, io, ca, list, status, stamps, stream);
+        if (nv <= 2048) return launch_t<512, 2048>(d, tp, gp, io, ca, list, status, stamps, stream);
+        return launch_t<1024, kMaxVis>(d, tp, gp, io, ca, list, status, stamps, stream);
+    });
 }
 
 }  // namespace mvla
