@@ -277,7 +277,7 @@ int tiles_of(const SampleDev& s)
     return (s.n_2d + kKeyTile - 1) / kKeyTile + (s.n_3d + kKeyTile - 1) / kKeyTile;
 }
 
-// 3-D view (head_dim, heads, rows) of a token-major [rows, H, d] bf16 or e4m3 tensor; boxes of 128 bytes x 1 x
+// 3-D view (head_dim, heads, rows) of a token-major [rows, H, d] tensor; boxes of 128 bytes x 1 x
 // `box_rows` land in shared memory as `box_rows` rows of 128 bytes with the 128-byte swizzle.
 int32_t tensor_map(mvla_ctx* ctx, int which, const void* ptr, int64_t rows, int box_rows, const CUtensorMap** out)
 {
@@ -300,7 +300,7 @@ int32_t tensor_map(mvla_ctx* ctx, int which, const void* ptr, int64_t rows, int 
     cuuint64_t strides[2] = {static_cast<cuuint64_t>(c.head_dim) * es, static_cast<cuuint64_t>(c.head_dim) * heads * es};
     cuuint32_t box[3] = {static_cast<cuuint32_t>(128 / es), 1, static_cast<cuuint32_t>(box_rows)};
     cuuint32_t estr[3] = {1, 1, 1};
-    const CUtensorMapDataType dt = es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    const CUtensorMapDataType dt = es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     slot->ptr = nullptr;
     const CUresult r = ctx->encode(&slot->map, dt, 3, const_cast<void*>(ptr), dims,
                                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -366,7 +366,8 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     const int cluster = (max_tiles + tiles_per_cta - 1) / tiles_per_cta;
     const int npad = (max_txt + 15) / 16 * 16;
     const CUtensorMap *tq = nullptr, *tk = nullptr;
-    if (ctx->use_umma) {
+    const bool f32 = c.dtype == MVLA_DTYPE_FP32 && acc64 && !alpha.ptr && f32_salience_supported(tiles_per_cta, npad, c.head_dim);
+    if (ctx->use_umma || f32) {
         int32_t r = tensor_map(ctx, 0, q, rows, 16, &tq);
         if (r != MVLA_OK) return r;
         tk = tq;                              // (the slot not to be reused)
@@ -375,7 +376,6 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     }
     cudaError_t e;
     const bool streaming = ctx->use_umma && (acc64 || alpha.ptr) && !with_cache && stream_pays(ctx, bd, tiles_per_cta, cluster);
-    const bool f32 = c.dtype == MVLA_DTYPE_FP32 && acc64 && !alpha.ptr && f32_salience_supported(tiles_per_cta, npad, c.head_dim);
     const bool fast = streaming || f32 || (ctx->use_umma && fast_salience_supported(tiles_per_cta));
     // The norms do not depend on the scores: with `norms_beside` (fast kernel only) they are launched AFTER
     // the scoring kernel and run beside it instead of in front of it.
@@ -389,8 +389,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
                                    ctx->status_dev, free_running, alpha, rearm, rearm_rec, stamps, st);
         if (used_acc64) *used_acc64 = acc64 != nullptr;
     } else if (f32) {
-        e = launch_salience_f32(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<const float*>(q), static_cast<const float*>(k),
-                                tiles_per_cta, cluster, npad, acc64, ctx->status_dev, rearm, stamps, st);
+        e = launch_salience_f32(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, tq, tk, tiles_per_cta, cluster, npad, acc64, ctx->status_dev, rearm, stamps, st);
         if (used_acc64) *used_acc64 = true;
     } else if (fast) {
         e = launch_salience_fast(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk,
@@ -865,7 +864,7 @@ static int32_t mvla_prune_create_impl(const mvla_config* cfg, mvla_ctx** out)
         *ctx->status_host = 0;
         e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->status_dev), ctx->status_host, 0);
     }
-    if (e == cudaSuccess && ctx->use_umma) {
+    if (e == cudaSuccess) {
         void* fn = nullptr;
         cudaDriverEntryPointQueryResult qres;
         e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &qres);

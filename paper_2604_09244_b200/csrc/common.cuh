@@ -164,7 +164,8 @@ cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group,
 
 // The same scores into the same fixed-point accumulators from fp32 q / k (plain FMAs), where the shape fits.
 bool f32_salience_supported(int tiles_per_cta, int npad, int head_dim);
-cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, const float* q, const float* k, int tiles_per_cta,
+cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, const CUtensorMap* tmap_q,
+                                const CUtensorMap* tmap_k, int tiles_per_cta,
                                 int cluster, int npad, unsigned long long* acc64, int* status, int32_t* rearm, unsigned long long* stamps,
                                 cudaStream_t stream);
 // The same scores into the same fixed-point accumulators by the streaming kernel (stream.cu): persistent CTAs, key

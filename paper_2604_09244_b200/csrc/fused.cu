@@ -453,28 +453,33 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
 
 // ------------------------------------------------------------------ fp32 inputs
 // The same chain for fp32 q / k: plain FMAs instead of the tensor cores (their fp32 forms round the operands).  Rows
-// arrive as bulk copies of d floats each, on a pitch of d + 4 (an odd number of 16-byte units, so that 16-byte reads of
-// neighbouring rows do not conflict); a thread computes the dot products of its key with its half of the text queries,
+// arrive as TMA boxes of 32 floats x 128 keys (or 16 queries) with the 128-byte swizzle, in which 16-byte reads of
+// neighbouring rows do not conflict; a thread computes the dot products of its key with its half of the text queries,
 // the key's piece in registers against broadcasts of the queries.  Dot products are summed in element order.
-// Bound by latency at the sizes this path serves (2.2 MB a step at 192 tokens, 8 heads x 64): the loads of all rows of a
-// CTA go out at once, where scalar loads through registers kept a few in flight, and the step runs as two chained
-// kernels like that of the other types (24.6 -> 14.8 us a step at that size).
+// Bound by latency at the sizes this path serves (2.2 MB a step at 192 tokens, 8 heads x 64): the loads of a CTA go out at
+// once, where scalar loads through registers kept a few in flight, and the step runs as chained kernels like that of the
+// other types (24.6 -> 14.4 us a step at that size with a bulk copy per row, 10.3 with boxes: 144 small copies took
+// their time to issue).
 template <int TCOL, int NTILE, class BD>
 __global__ void __launch_bounds__(kFastThreads * 2, 1)
-salience_f32_kernel(const __grid_constant__ BD bd, const float* __restrict__ q, const float* __restrict__ k, int n_heads, int kv_group,
-                    int d, int npad_max, unsigned long long* __restrict__ acc64, int* status, int32_t* __restrict__ rearm,
+salience_f32_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
+                    int n_heads, int kv_group, int d, int npad_max, unsigned long long* __restrict__ acc64, int* status, int32_t* __restrict__ rearm,
                     unsigned long long* __restrict__ stamps)
 {
     constexpr int TC = TCOL / 2, NT = kFastThreads * 2;
-    extern __shared__ __align__(16) float rows[];         // [npad_max queries, then NTILE x 128 keys][d + 4]
+    extern __shared__ uint8_t dyn_smem_raw[];
+    const int boxes = d / 32;                             // head dims are multiples of 32
+    // The queries come first: a thread reads a whole half of TCOL queries, rows past the padded ones (up to 2 KB past the
+    // last box) included, and what it reads there must exist.
+    uint8_t* Qs = dyn_smem_raw + ((1024u - (smem_u32(dyn_smem_raw) & 1023u)) & 1023u);   // [box][npad rows x 128 B]
+    uint8_t* Ks = Qs + boxes * npad_max * 128;            // [tile][box][128 rows x 128 B]
     __shared__ FastSmem sm;
     __shared__ __align__(8) uint64_t s_bar[2];
     const SampleDev& s = bd.at(blockIdx.z);
-    const int h = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5;
     const int key = tid & (kFastThreads - 1), c0 = (tid / kFastThreads) * TC;
     const int npad = min(npad_max, (s.n_txt + 15) & ~15);
     const int tt0 = static_cast<int>(cluster_ctarank()) * NTILE;
-    const int pitch = d + 4;
     const float cscale = 1.4426950408889634f * rsqrtf(static_cast<float>(d));   // log2 domain
     const uint32_t bar_full = smem_u32(&s_bar[0]), bar_x = smem_u32(&s_bar[1]);
     int valid[NTILE], vis0[NTILE];
@@ -486,7 +491,10 @@ salience_f32_kernel(const __grid_constant__ BD bd, const float* __restrict__ q, 
         vis0[t] = ti[t].vis0;
     }
     // before the wait for the kernel before this one (see salience_fast_kernel)
-    if (tid == 0) {
+    const bool one = warp == 0 && elect_one();
+    if (one) {
+        prefetch_tensormap(&tmap_q);
+        prefetch_tensormap(&tmap_k);
         mbar_init(bar_full, 1);
         mbar_init(bar_x, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -494,34 +502,30 @@ salience_f32_kernel(const __grid_constant__ BD bd, const float* __restrict__ q, 
     }
     __syncwarp();
     cluster_arrive_release();                 // publishes this CTA's barriers; matched by the wait before the first remote store
-    for (int i = tid; i < (npad - s.n_txt) * d; i += NT) rows[(s.n_txt + i / d) * pitch + i % d] = 0.f;   // query rows that do not exist
     if (rearm && blockIdx.x == 0 && blockIdx.y == 0)
         for (int i = tid; i < s.n_out; i += NT) rearm[s.out_off + i] = -1;
+    const int hk = h / kv_group, qrow = s.seq_off + s.off_txt, nq = npad / 16;
+    int live = 0;
+#pragma unroll
+    for (int t = 0; t < NTILE; ++t) live += valid[t] > 0;
     __syncthreads();
     if (warp == 0) {
         pdl_wait();
-        if (lane == 0) {
-            if (stamps) {
-                const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-                if (cta < kStampSlots) stamps[2 * cta] = global_ns();
-            }
-            int live = s.n_txt;
-#pragma unroll
-            for (int t = 0; t < NTILE; ++t) live += valid[t];
-            mbar_expect_tx(bar_full, static_cast<uint32_t>(live) * static_cast<uint32_t>(d) * 4u);
-        }
-        __syncwarp();
-        const uint32_t bytes = static_cast<uint32_t>(d) * 4u;
-        const int64_t qrow = static_cast<int64_t>(n_heads) * d, krow = static_cast<int64_t>(n_heads / kv_group) * d;
-        const float* qs = q + (static_cast<int64_t>(s.seq_off) + s.off_txt) * qrow + static_cast<int64_t>(h) * d;
-        for (int i = lane; i < s.n_txt; i += 32) bulk_load(smem_u32(rows + i * pitch), qs + i * qrow, bytes, bar_full);
+        if (one) mbar_expect_tx(bar_full, static_cast<uint32_t>(boxes) * (npad * 128 + live * 16384));
 #pragma unroll
         for (int t = 0; t < NTILE; ++t) {
-            const float* ks = k + static_cast<int64_t>(ti[t].row0) * krow + static_cast<int64_t>(h / kv_group) * d;
-            for (int i = lane; i < valid[t]; i += 32)
-                bulk_load(smem_u32(rows + (npad_max + t * kKeyTile + i) * pitch), ks + i * krow, bytes, bar_full);
+            if (valid[t] <= 0) continue;
+            for (int x = 0; x < boxes; ++x)
+                if (one) tma_load_3d(smem_u32(Ks) + static_cast<uint32_t>(t * boxes + x) * 16384u, &tmap_k, x * 32, hk, ti[t].row0, bar_full);
         }
+        for (int x = 0; x < boxes; ++x)
+            for (int c = 0; c < nq; ++c)
+                if (one) tma_load_3d(smem_u32(Qs) + static_cast<uint32_t>(x * npad * 128 + c * 2048), &tmap_q, x * 32, h, qrow + c * 16, bar_full);
         pdl_trigger();
+        if (stamps && one) {
+            const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+            if (cta < kStampSlots) stamps[2 * cta] = global_ns();
+        }
     }
     bool ok = true;
     if (tid == 0) {
@@ -540,18 +544,21 @@ salience_f32_kernel(const __grid_constant__ BD bd, const float* __restrict__ q, 
 #pragma unroll
         for (int t = 0; t < NTILE; ++t) {
             if (valid[t] <= 0) continue;
-            const float4* kr = reinterpret_cast<const float4*>(rows + (npad_max + t * kKeyTile + key) * pitch);
+            for (int x = 0; x < boxes; ++x) {
+                const uint8_t* kr = Ks + (t * boxes + x) * 16384 + key * 128;
+                const uint8_t* qr = Qs + (x * npad + c0) * 128;
 #pragma unroll 2
-            for (int c = 0; c < d / 4; ++c) {
-                const float4 k4 = kr[c];
+                for (int c = 0; c < 8; ++c) {             // 16-byte piece c of row r lies at c ^ (r mod 8)
+                    const float4 k4 = *reinterpret_cast<const float4*>(kr + ((c ^ (key & 7)) << 4));
 #pragma unroll
-                for (int i = 0; i < TC; ++i) {
-                    const float4 q4 = *reinterpret_cast<const float4*>(rows + (c0 + i) * pitch + 4 * c);
-                    float& acc = L[t * TC + i];
-                    acc = fmaf(k4.x, q4.x, acc);
-                    acc = fmaf(k4.y, q4.y, acc);
-                    acc = fmaf(k4.z, q4.z, acc);
-                    acc = fmaf(k4.w, q4.w, acc);
+                    for (int i = 0; i < TC; ++i) {        // (c0 is a multiple of 16)
+                        const float4 q4 = *reinterpret_cast<const float4*>(qr + i * 128 + ((c ^ (i & 7)) << 4));
+                        float& acc = L[t * TC + i];
+                        acc = fmaf(k4.x, q4.x, acc);
+                        acc = fmaf(k4.y, q4.y, acc);
+                        acc = fmaf(k4.z, q4.z, acc);
+                        acc = fmaf(k4.w, q4.w, acc);
+                    }
                 }
             }
         }
@@ -599,10 +606,10 @@ cudaError_t launch_fast_t(const BD& bd, int n_heads, int kv_group, int head_dim,
 }
 
 template <int TCOL, int NTILE, class BD>
-cudaError_t launch_f32_t(const BD& bd, int n_heads, int kv_group, int head_dim, const float* q, const float* k, int cluster, int npad,
+cudaError_t launch_f32_t(const BD& bd, int n_heads, int kv_group, int head_dim, const CUtensorMap* tq, const CUtensorMap* tk, int cluster, int npad,
                          unsigned long long* acc64, int* status, int32_t* rearm, unsigned long long* stamps, cudaStream_t stream)
 {
-    const size_t smem = sizeof(float) * static_cast<size_t>(npad + NTILE * kKeyTile) * (head_dim + 4);
+    const size_t smem = 1024 + static_cast<size_t>(head_dim / 32) * (NTILE * 16384 + npad * 128);
     auto kern = salience_f32_kernel<TCOL, NTILE, BD>;
     static KernelSetup ks;
     const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kFastThreads * 2, smem, 0);
@@ -620,18 +627,19 @@ cudaError_t launch_f32_t(const BD& bd, int n_heads, int kv_group, int head_dim, 
     attr[1] = pdl_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, bd, q, k, n_heads, kv_group, head_dim, npad, acc64, status, rearm, stamps);
+    return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, n_heads, kv_group, head_dim, npad, acc64, status, rearm, stamps);
 }
 
 }  // namespace
 
-// fp32: two key tiles per CTA at most, and all rows of a CTA in shared memory beside the kernel's own 9 KB.
+// fp32: two key tiles per CTA at most, and all rows of a CTA in shared memory beside the kernel's own 7 KB.
 bool f32_salience_supported(int tiles_per_cta, int npad, int head_dim)
 {
-    return tiles_per_cta <= 2 && sizeof(float) * static_cast<size_t>(npad + tiles_per_cta * kKeyTile) * (head_dim + 4) <= 216 * 1024;
+    return tiles_per_cta <= 2 && 1024 + head_dim / 32 * (tiles_per_cta * 16384 + npad * 128) <= 218 * 1024;
 }
 
-cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, const float* q, const float* k, int tiles_per_cta,
+cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, const CUtensorMap* tmap_q,
+                                const CUtensorMap* tmap_k, int tiles_per_cta,
                                 int cluster, int npad, unsigned long long* acc64, int* status, int32_t* rearm, unsigned long long* stamps,
                                 cudaStream_t stream)
 {
@@ -639,7 +647,7 @@ cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, 
 #define MVLA_F32(TC, NTL)                                                                                       \
     if (npad <= TC && tiles_per_cta == NTL)                                                                     \
         return with_desc(bd, [&](const auto& d) {                                                               \
-            return launch_f32_t<TC, NTL>(d, n_heads, kv_group, head_dim, q, k, cluster, npad, acc64, status, rearm, stamps, stream); });
+            return launch_f32_t<TC, NTL>(d, n_heads, kv_group, head_dim, tmap_q, tmap_k, cluster, npad, acc64, status, rearm, stamps, stream); });
     MVLA_F32(32, 1) MVLA_F32(64, 1) MVLA_F32(32, 2) MVLA_F32(64, 2)
 #undef MVLA_F32
     return cudaErrorInvalidConfiguration;
