@@ -9,7 +9,7 @@
 //      smallest and largest key of each modality in shared memory                        [barrier A]
 //   2. modality sums -> the four indicators, smoothed too; dual threshold (Sec. 4.1), target-object
 //      rule (Sec. 4.2), fusion (Sec. 4.4), budget split: one thread, while the others already count
-//      their keys into a histogram of 1024 bins per modality laid over the RANGE of the keys
+//      their keys into a histogram of 1024 or 4096 bins per modality laid over the RANGE of the keys
 //      (bin = (key - smallest) >> shift), so one pass separates a few hundred scores     [barrier B]
 //   3. one warp per modality finds the bin that holds the k-th largest key (two 32-way scans)
 //                                                                                         [barrier C]
@@ -30,8 +30,11 @@ namespace mvla {
 constexpr float kFixScale = 1152921504606846976.f;          // 2^60
 constexpr float kFixInv = 1.f / 1152921504606846976.f;      // 2^-60, exact
 
-constexpr int kSelBins = 1024;      // histogram bins per modality
-constexpr int kSelBinBits = 10;
+// Histogram bins per modality.  A few strong tokens stretch the range that the bins share and the bulk of the scores
+// falls into a few dozen of 1024 bins: with more than 1024 tokens the threshold bin then holds some hundred keys and has to
+// be split again (1.5 us); four times the bins keep it below kCandMax for 0.1 us more in the search.  (Up to 1024 tokens
+// it held 6 to 20 keys.)
+constexpr int sel_bin_bits(int cap) { return cap <= 1024 ? 10 : 12; }
 constexpr int kCandMax = 32;        // keys of the threshold bin ranked from a list; above that the bin is split again
 
 // what happens to the keys of the threshold bin of a modality
@@ -49,9 +52,10 @@ enum : int {
 // of such instructions a warp issues between two barriers, and 16-byte accesses are used wherever possible.
 template <int NT, int CAP = kMaxVis>
 struct SelectSmem {
-    // bin r (0 = largest keys) of lane r / 32 lives at hist_pos(r): the 32 bins of a lane are eight int4, and
-    // for each of the eight the 32 lanes read consecutive int4 (no bank conflict)
-    alignas(16) int hist[2][kSelBins];
+    // bin r (0 = largest keys) lives at hist_pos(r): the bins of a lane of the search are BINS / 128 int4, and for each
+    // of them the 32 lanes read consecutive int4 (no bank conflict)
+    static constexpr int kBits = sel_bin_bits(CAP), kBins = 1 << kBits;
+    alignas(16) int hist[2][kBins];
     alignas(16) float red[NT / 32][8];       // per-warp partial sums: scores 2D, 3D; norms 2D, 3D; smoothed scores 2D, 3D
     alignas(16) uint32_t ext[NT / 32][4];    // per-warp smallest / largest key: min 2D, max 2D, min 3D, max 3D
     alignas(16) uint32_t cand_key[2][kCandMax];
@@ -63,9 +67,11 @@ struct SelectSmem {
     int krem[2];                             // still to be taken from the keys under examination
     float zf[2];                             // factors of the optional normalised scores
 };
+template <int BITS>
 __device__ __forceinline__ int hist_pos(int r)
 {
-    return (((r & 31) >> 2) << 7) + ((r >> 5) << 2) + (r & 3);
+    constexpr int kLane = BITS - 5;                        // bins of a lane: 2^kLane
+    return (((r & ((1 << kLane) - 1)) >> 2) << 7) + ((r >> kLane) << 2) + (r & 3);
 }
 
 // fp32 -> uint32 whose unsigned order is the float order; NaN sorts below everything.
@@ -155,12 +161,14 @@ struct NoHook {
 };
 
 // One warp: the bin that holds the k-th largest of the keys counted in `h` (1 <= k <= number counted).
+template <int BITS>
 __device__ __forceinline__ void find_threshold_bin(const int* h, int k, int lane, int& tbin, int& need, int& cnt)
 {
     const int4* h4 = reinterpret_cast<const int4*>(h);
+    constexpr int kVec = 1 << (BITS - 7);                              // int4 per lane
     int mine = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {                                      // bins 32 lane .. 32 lane + 31
+    for (int i = 0; i < kVec; ++i) {                                   // bins 4 kVec lane ..
         const int4 v = h4[(i << 5) + lane];
         mine += (v.x + v.y) + (v.z + v.w);
     }
@@ -168,14 +176,29 @@ __device__ __forceinline__ void find_threshold_bin(const int* h, int k, int lane
     const unsigned hit = __ballot_sync(0xffffffffu, inc - mine < k && k <= inc);
     const int L = max(__ffs(hit) - 1, 0);
     const int above_l = __shfl_sync(0xffffffffu, inc - mine, L);
-    const int c = h[hist_pos(32 * L + lane)];                          // the 32 bins of that lane, one per lane
-    const int inc2 = warp_incl_scan(c, lane);
-    const int above = above_l + inc2 - c;
-    const unsigned hit2 = __ballot_sync(0xffffffffu, above < k && k <= above + c);
-    const int i = max(__ffs(hit2) - 1, 0);
-    tbin = 32 * L + i;
-    need = k - __shfl_sync(0xffffffffu, above, i);
-    cnt = __shfl_sync(0xffffffffu, c, i);
+    if constexpr (kVec == 8) {                                         // the 32 bins of that lane, one per lane
+        const int c = h[hist_pos<BITS>(32 * L + lane)];
+        const int inc2 = warp_incl_scan(c, lane);
+        const int above = above_l + inc2 - c;
+        const unsigned hit2 = __ballot_sync(0xffffffffu, above < k && k <= above + c);
+        const int i = max(__ffs(hit2) - 1, 0);
+        tbin = 32 * L + i;
+        need = k - __shfl_sync(0xffffffffu, above, i);
+        cnt = __shfl_sync(0xffffffffu, c, i);
+    } else {                                                           // 128 bins, four per lane
+        static_assert(kVec == 32 || kVec == 8, "one int4 per lane");
+        const int4 c = h4[(lane << 5) + L];
+        const int tot = (c.x + c.y) + (c.z + c.w);
+        const int above = above_l + warp_incl_scan(tot, lane) - tot;
+        const unsigned hit2 = __ballot_sync(0xffffffffu, above < k && k <= above + tot);
+        const int i = max(__ffs(hit2) - 1, 0);
+        const int a1 = above + c.x, a2 = a1 + c.y, a3 = a2 + c.z;      // which of the lane's four
+        const int w = k <= a1 ? 0 : k <= a2 ? 1 : k <= a3 ? 2 : 3;
+        const int nd = k - (w == 0 ? above : w == 1 ? a1 : w == 2 ? a2 : a3), cw = w == 0 ? c.x : w == 1 ? c.y : w == 2 ? c.z : c.w;
+        tbin = 128 * L + 4 * i + __shfl_sync(0xffffffffu, w, i);
+        need = __shfl_sync(0xffffffffu, nd, i);
+        cnt = __shfl_sync(0xffffffffu, cw, i);
+    }
 }
 
 // `before_wait` runs ahead of the wait for the previous kernel (late_pdl only); `after_list` runs as soon as
@@ -188,6 +211,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
 {
     constexpr int EPT = CAP / NT;                         // elements per thread, strided by NT
     constexpr int NW = NT / 32;
+    constexpr int kSelBinBits = SelectSmem<NT, CAP>::kBits, kSelBins = SelectSmem<NT, CAP>::kBins;
     static_assert(EPT >= 1 && EPT * NT == CAP, "thread count must divide the capacity");
     static_assert(EPT * NW <= 128, "the emission prefix is taken by one warp, four entries per lane");
     static_assert((2 * kCandMax * 8) % NT == 0 || NT % (2 * kCandMax * 8) == 0, "whole warps rank the listed keys");
@@ -303,7 +327,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
         const uint32_t hi2 = __reduce_max_sync(0xffffffffu, x4.y);
         lo3 = __reduce_min_sync(0xffffffffu, x4.z);
         const uint32_t hi3 = __reduce_max_sync(0xffffffffu, x4.w);
-        sh2 = hi2 > lo2 ? max(0, (32 - __clz(hi2 - lo2)) - kSelBinBits) : -1;       // (key - lo) >> shift < 1024
+        sh2 = hi2 > lo2 ? max(0, (32 - __clz(hi2 - lo2)) - kSelBinBits) : -1;       // (key - lo) >> shift < bins
         sh3 = hi3 > lo3 ? max(0, (32 - __clz(hi3 - lo3)) - kSelBinBits) : -1;
     }
 
@@ -390,7 +414,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
             const int sh = is3 ? sh3 : sh2;
             if (st[e] == 2 && (is3 ? act3 : act2) && sh >= 0) {
                 const int r = kSelBins - 1 - static_cast<int>((key[e] - (is3 ? lo3 : lo2)) >> sh);
-                atomicAdd(&sm.hist[is3 ? 1 : 0][hist_pos(r)], 1);
+                atomicAdd(&sm.hist[is3 ? 1 : 0][hist_pos<kSelBinBits>(r)], 1);
             }
         }
         __syncthreads();                                                                   // ---- barrier B
@@ -403,7 +427,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
             else if (sh < 0) { mode = SEL_TIES; need = k; }                // equal keys only: index order decides
             else {
                 int cnt;
-                find_threshold_bin(sm.hist[m], k, lane, tbin, need, cnt);
+                find_threshold_bin<kSelBinBits>(sm.hist[m], k, lane, tbin, need, cnt);
                 mode = need == cnt ? SEL_BIN_ALL : (cnt <= kCandMax ? SEL_LIST : (sh == 0 ? SEL_TIES : SEL_REFINE));
             }
             if (lane == 0) { sm.ctl[m] = mode; sm.ctl[2 + m] = tbin; sm.ctl[4 + m] = need; sm.krem[m] = need; }
