@@ -71,7 +71,7 @@ struct mvla_ctx {
     int32_t* tail_list;          // [kSets][rows_all] kept list as the copying CTAs read it (-1 between launches)
     unsigned int* tail_ticket;   // [kSets] ticket counters of the patch-by-patch tail (zero between launches)
     unsigned long long* patch_rec;   // [kSets][vis_all / 2][3] hand-over words of the patch-by-patch tail (all ones between launches)
-    size_t rows_all;             // max_batch * (kHandWords + max_text + max_vis)
+    size_t rows_all;             // max_batch * (kHandWords + kListStride (max_text + max_vis))
     int sm_count;                // multiprocessors of the device
     // reuse of the previous step's logits (cfg.logit_cache)
     float* lcache;               // [n_prune_points * n_slots][H][max_vis][cache_cols] raw dot products
@@ -205,7 +205,7 @@ int32_t make_plan(mvla_ctx* ctx, int32_t prune_point, int32_t batch, const mvla_
         const int nv = in.n_2d + in.n_3d;
         d.vis_off = vis_off;
         d.cap_off = cap_off;
-        cap_off += kHandWords + in.n_txt + nv;
+        cap_off += kHandWords + kListStride * (in.n_txt + nv);
         vis_off += nv;
         d.k_2d_fixed = -1;
         d.cache_state = -1;
@@ -828,7 +828,7 @@ static int32_t mvla_prune_create_impl(const mvla_config* cfg, mvla_ctx** out)
     alloc(&ctx->mhat_state, 2 * n_state * 4);
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->acc64), kSets * vis_all * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(ctx->acc64, 0, kSets * vis_all * sizeof(unsigned long long));
-    ctx->rows_all = static_cast<size_t>(c.max_batch) * (kHandWords + c.max_text + ctx->max_vis);
+    ctx->rows_all = static_cast<size_t>(c.max_batch) * (kHandWords + kListStride * (c.max_text + ctx->max_vis));
     // (+ 1: a word that no launch ever writes, for mvla_selftest_wait_timeout)
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->tail_list), (kSets * ctx->rows_all + 1) * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(ctx->tail_list, 0xFF, (kSets * ctx->rows_all + 1) * sizeof(int32_t));

@@ -18,6 +18,10 @@ namespace mvla {
 // to be written", word 1 the sample's first output row), then one word per row of the sample.
 constexpr int kHandLines = 8;
 constexpr int kHandWords = kHandLines * 32;
+// Distance in words between the hand-over words of neighbouring rows in the fused tails.  A row's word is polled by as
+// many warps as move its segments (a dozen); side by side, 32 words shared a line of the L2 and its pollers were served
+// one after another: eight words a line shorten a step by 2 to 3 % (four a line: no more).
+constexpr int kListStride = 4;
 constexpr int kMaxChunk = 32;        // samples carried by one launch (descriptors travel as kernel parameters)
 constexpr int kKeyTile = 128;        // visual keys per tile = rows of one MMA
 constexpr int kMaxCluster = 8;       // portable cluster size
@@ -30,7 +34,7 @@ constexpr unsigned kStampSlots = 4096;      // CTAs per kernel that leave time s
 struct SampleDev {
     int32_t seq_off, off_txt, n_txt, off_2d, n_2d, off_3d, n_3d;
     int32_t vis_off;        // offset of the sample in packed [sum n_vis] arrays
-    int32_t cap_off;        // sum of (kHandWords + n_txt + n_vis) over the samples before this one: its hand-over words in the patch-by-patch tail
+    int32_t cap_off;        // sum of (kHandWords + kListStride (n_txt + n_vis)) over the samples before this one: its hand-over words in the patch-by-patch tail
     int32_t out_off;        // first output row
     int32_t n_out;          // kept rows = n_txt + budget
     int32_t budget;         // kept visual tokens (host known)
@@ -138,9 +142,9 @@ cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t 
 // computed and stored and which are read back is in the descriptors (cache_state, tile_compute).
 // `stamps`: when not null, CTA c (linear index, below kStampSlots) writes the global timer when it was free to
 // start its loads to stamps[2 c] and when it ended to stamps[2 c + 1].
-// `rearm`: when not null, words [out_off, out_off + n_out) of every sample are set to -1 (the kept list that
+// `rearm`: when not null, words kListStride x [out_off, out_off + n_out) of every sample are set to -1 (the kept list that
 // launch_select_copy's CTAs exchange, see there).  With `rearm_rec` (the patch-by-patch tail, launch_patch_tail)
-// it is words [cap_off, cap_off + kHandWords + n_txt + n_vis) instead, and the three 8-byte words of every patch in
+// it is the hand-over words of every sample from cap_off on instead, and the three 8-byte words of every patch in
 // `rearm_rec` ([vis_off / 2 + p][3]) are set to all ones.
 // Optional copy of the attention itself for the patch-by-patch path, four text queries of a (head, token) next to one
 // another and the tokens behind one another:
@@ -284,7 +288,7 @@ cudaError_t launch_patch_indicators(const BatchDesc& bd, int n_heads, AlphaOut a
 cudaError_t launch_patch_select(const BatchDesc& bd, const PatchParams& pp, const PatchIO& io, cudaStream_t stream);
 // Indicators, stages 1-4 and the row copy of the patch-by-patch step in one kernel behind the scoring kernel
 // (which must have re-armed `list` and `rec`, see launch_salience_fast).  `rec`: [sum P][3] 8-byte words;
-// `list`: 4-byte words, kHandWords + n_txt + n_vis per sample from cap_off on.  io.x / io.attn are not read.
+// `list`: 4-byte words, kHandWords + kListStride (n_txt + n_vis) per sample from cap_off on.  io.x / io.attn are not read.
 // `ticket_counter`: one word, zero before the first launch, used by one launch at a time (it returns to zero with
 // every launch): the CTAs take their roles in the order in which they start (copy_impl.cuh: cta_ticket).
 bool patch_tail_supported(const BatchDesc& bd);

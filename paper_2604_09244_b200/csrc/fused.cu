@@ -316,9 +316,10 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
     // its selecting CTA to its copying CTAs (-1: not yet known).  Their last users finished long ago.
     if (rearm && blockIdx.x == 0 && blockIdx.y == 0) {
         if constexpr (KIND != kForPatches) {
-            for (int i = tid; i < s.n_out; i += NT) rearm[s.out_off + i] = -1;
+            for (int i = tid; i < s.n_out; i += NT) rearm[(s.out_off + i) * kListStride] = -1;
         } else {                              // the patch-by-patch tail: its list words, and three words per patch
-            for (int i = tid; i < kHandWords + s.n_txt + s.n_2d + s.n_3d; i += NT) rearm[s.cap_off + i] = -1;
+            for (int i = tid; i < kHandWords; i += NT) rearm[s.cap_off + i] = -1;
+            for (int i = tid; i < s.n_txt + s.n_2d + s.n_3d; i += NT) rearm[s.cap_off + kHandWords + i * kListStride] = -1;
             for (int i = tid; i < 3 * s.n_2d; i += NT) rearm_rec[static_cast<int64_t>(s.vis_off / 2) * 3 + i] = ~0ull;
         }
     }
@@ -334,6 +335,26 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = s_tmem;
+
+    // Logit cache: a reused tile takes the previous action step's dot products instead of K (128 bytes per key and head
+    // at 32 queries: half a key row, and no MMA).  They were written two kernels ago, so they are fetched before the wait,
+    // too, instead of behind the MMAs, where they are needed.
+    float L[NTILE * TC];                      // L[t * TC + i]: tile t, text query c0 + i
+#pragma unroll
+    for (int i = 0; i < NTILE * TC; ++i) L[i] = 0.f;
+    if constexpr (KIND == kWithCache) {
+#pragma unroll
+        for (int t = 0; t < NTILE; ++t) {
+            if (!caching || from_k[t] || key >= valid[t]) continue;
+            const float4* row = reinterpret_cast<const float4*>(lcache + cache_row0 + static_cast<int64_t>(vis0[t] + key) * cache_cols + c0);
+#pragma unroll
+            for (int i = 0; i < TC; i += 4) {
+                if (c0 + i >= npad) break;
+                const float4 v = __ldcg(row + i / 4);
+                L[t * TC + i] = v.x; L[t * TC + i + 1] = v.y; L[t * TC + i + 2] = v.z; L[t * TC + i + 3] = v.w;
+            }
+        }
+    }
 
     // Warp 0 loads and multiplies: it runs these loops as a whole warp, all values the same in every lane, and one
     // elected lane issues, so that coordinates and descriptors stay in uniform registers.  (In a single-thread branch
@@ -402,40 +423,29 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
     ok = __syncthreads_and(ok) != 0;          // block-uniform from here on (aligned instructions follow)
     tc_fence_after();
 
-    // ---- all logits of this thread's key(s) into registers, scaled to the log2 domain, masked
-    float L[NTILE * TC];                      // L[t * TC + i]: tile t, text query c0 + i
-    if (any_live && ok) {
-        if constexpr (SPLIT == 1) {
-            tmem_ld_cols<CC>(tmem_base + (static_cast<uint32_t>(kwarp * 32) << 16), L);
-        } else {
-#pragma unroll
-            for (int t = 0; t < NTILE; ++t) {
-                float part_l[TC];
-                tmem_ld_cols<TC>(tmem_base + static_cast<uint32_t>(t * TCOL + c0) + (static_cast<uint32_t>(kwarp * 32) << 16), part_l);
-#pragma unroll
-                for (int i = 0; i < TC; ++i) L[t * TC + i] = part_l[i];
-            }
-        }
+    // ---- all logits of this thread's key(s) into registers
+    if constexpr (SPLIT == 1 && KIND != kWithCache) {
+        if (any_live && ok) tmem_ld_cols<CC>(tmem_base + (static_cast<uint32_t>(kwarp * 32) << 16), L);
     } else {
 #pragma unroll
-        for (int i = 0; i < NTILE * TC; ++i) L[i] = 0.f;
+        for (int t = 0; t < NTILE; ++t) {
+            if (!any_live || !ok || !from_k[t]) continue;                    // block-uniform
+            float part_l[TC];
+            tmem_ld_cols<TC>(tmem_base + static_cast<uint32_t>(t * TCOL + c0) + (static_cast<uint32_t>(kwarp * 32) << 16), part_l);
+#pragma unroll
+            for (int i = 0; i < TC; ++i) L[t * TC + i] = part_l[i];
+        }
     }
-    // Logit cache: a computed tile leaves its raw dot products for the next action step, a reused tile takes
-    // the previous step's instead (128 bytes per key and head at 32 queries: half a key row, and no MMA).
-    if (KIND == kWithCache && caching && ok) {
+    // Logit cache: a computed tile leaves its raw dot products for the next action step.
+    if constexpr (KIND == kWithCache) {
 #pragma unroll
         for (int t = 0; t < NTILE; ++t) {
-            if (key >= valid[t]) continue;
+            if (!caching || !ok || !from_k[t] || key >= valid[t]) continue;
             float4* row = reinterpret_cast<float4*>(lcache + cache_row0 + static_cast<int64_t>(vis0[t] + key) * cache_cols + c0);
 #pragma unroll
-            for (int i = 0; i < TC / 4; ++i) {
-                if (c0 + 4 * i >= npad) break;
-                if (from_k[t]) {
-                    row[i] = make_float4(L[t * TC + 4 * i], L[t * TC + 4 * i + 1], L[t * TC + 4 * i + 2], L[t * TC + 4 * i + 3]);
-                } else {
-                    const float4 v = __ldcg(row + i);
-                    L[t * TC + 4 * i] = v.x; L[t * TC + 4 * i + 1] = v.y; L[t * TC + 4 * i + 2] = v.z; L[t * TC + 4 * i + 3] = v.w;
-                }
+            for (int i = 0; i < TC; i += 4) {
+                if (c0 + i >= npad) break;
+                row[i / 4] = make_float4(L[t * TC + i], L[t * TC + i + 1], L[t * TC + i + 2], L[t * TC + i + 3]);
             }
         }
     }
@@ -503,7 +513,7 @@ salience_f32_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUten
     __syncwarp();
     cluster_arrive_release();                 // publishes this CTA's barriers; matched by the wait before the first remote store
     if (rearm && blockIdx.x == 0 && blockIdx.y == 0)
-        for (int i = tid; i < s.n_out; i += NT) rearm[s.out_off + i] = -1;
+        for (int i = tid; i < s.n_out; i += NT) rearm[(s.out_off + i) * kListStride] = -1;
     const int hk = h / kv_group, qrow = s.seq_off + s.off_txt, nq = npad / 16;
     int live = 0;
 #pragma unroll

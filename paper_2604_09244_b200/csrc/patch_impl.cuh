@@ -270,12 +270,12 @@ __device__ __forceinline__ int ld_volatile_i32(const int* p)
 // `rec`: null: indicators and scores come from io.x / io.attn, written by the kernel before this one; else
 //        they are taken, patch by patch, from the 8-byte words that patch_indicators_block writes in the
 //        same kernel (bounded wait for each).
-// `list`: when not null, kHandWords + `cap` 4-byte words (all -1 before the launch) for CTAs of the same
+// `list`: when not null, kHandWords + kListStride `cap` 4-byte words (all -1 before the launch) for CTAs of the same
 //        kernel that copy the rows: in each of the first kHandLines lines of 32 words, word 0 = 1 once the
 //        masks are decided (the list follows shortly: time to start polling it), word 1 = first output
 //        row of the sample, word 2 = number of rows it keeps (written before word 1 by the same thread;
 //        a reader takes word 2 only after it has seen word 1 and re-reads it until it is there); word
-//        kHandWords + r = index inside the sample of the token that goes to the sample's output row r.
+//        kHandWords + kListStride r = index inside the sample of the token that goes to the sample's output row r.
 template <int NT>
 __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_local, int n_in_launch, const PatchParams& pp,
                                                    const PatchIO& io, PatchSmemT<NT>& sm, const unsigned long long* rec,
@@ -553,7 +553,7 @@ __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_loc
     const int baset = (s.off_2d < s.off_txt ? k2 : 0) + (s.off_3d < s.off_txt ? k3 : 0);
     for (int i = tid; i < s.n_txt; i += NT) {
         io.kept_idx[out_off + baset + i] = s.off_txt + i;
-        if (list) list[kHandWords + baset + i] = s.off_txt + i;
+        if (list) list[kHandWords + (baset + i) * kListStride] = s.off_txt + i;
     }
     int run = 0;
     for (int j0 = 0; j0 < nv; j0 += NT) {              // block-uniform
@@ -566,7 +566,7 @@ __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_loc
             const int pos = j < P ? base2 + r : base3 + (r - k2);
             const int val = j < P ? s.off_2d + j : s.off_3d + (j - P);
             io.kept_idx[out_off + pos] = val;
-            if (list) list[kHandWords + pos] = val;
+            if (list) list[kHandWords + pos * kListStride] = val;
         }
     }
     if (tid == 0) bookkeeping(out_off);                           // nobody in this kernel waits for these

@@ -84,7 +84,7 @@ patch_tail_kernel(const __grid_constant__ BD bd, const __grid_constant__ PatchTa
     }
     words += kHandWords;
     copy_rows(ca, n_rows, w, nw, lane, [&](int i, int64_t& srow, int64_t& drow) {
-        const int v = poll_word(words + i, t0, kLimitNs);     // the whole warp reads one word: one request
+        const int v = poll_word(words + i * kListStride, t0, kLimitNs);     // the whole warp reads one word: one request
         if (v < 0) {                                                   // gave up: report, leave the row alone
             *reinterpret_cast<volatile int*>(io.status) = MVLA_ERR_TIMEOUT;
             return false;

@@ -510,7 +510,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
     int32_t* const kept_sm = role.kept_sm;
     for (int i = tid; i < s.n_txt; i += NT) {
         if (leader) io.kept_idx[s.out_off + baset + i] = s.off_txt + i;
-        if (kept_sm) kept_sm[baset + i] = s.off_txt + i;
+        if (kept_sm) kept_sm[(baset + i) * kListStride] = s.off_txt + i;
     }
     // Exclusive prefix of the per-(slice, warp) counts in sm.wtot, for this warp's entry of every slice:
     // one scan per warp (each warp for itself: no further barrier), then one shuffle per slice.
@@ -576,7 +576,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
         const int pos = j < n2 ? base2 + r : base3 + (r - k2);
         const int val = j < n2 ? s.off_2d + j : s.off_3d + (j - n2);
         if (leader) io.kept_idx[s.out_off + pos] = val;
-        if (kept_sm) kept_sm[pos] = val;
+        if (kept_sm) kept_sm[pos * kListStride] = val;
     }
     after_list();
     if (role.late_pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -58,7 +58,7 @@ select_copy_kernel(const __grid_constant__ BD bd, const __grid_constant__ TailPl
         SelectRole role;
         role.late_pdl = true;
         role.l1_late = true;                                // the norms may come from a kernel that ran beside the scoring
-        if (tp.cta0[bd.count()] > 0) role.kept_sm = list + bd.at(b).out_off;   // every word is its own "ready" signal
+        if (tp.cta0[bd.count()] > 0) role.kept_sm = list + bd.at(b).out_off * kListStride;   // every word is its own "ready" signal
         select_sample<NT, CAP>(bd.at(b), b, gp, io, sm, role, [&]() {}, [&]() {
             if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
         });
@@ -92,11 +92,11 @@ select_copy_kernel(const __grid_constant__ BD bd, const __grid_constant__ TailPl
 
     {
         const int n_rows = s.n_out - (text_early ? s.n_txt : 0);
-        const int32_t* kept = list + s.out_off;
+        const int32_t* kept = list + s.out_off * kListStride;
         const uint64_t t0 = global_ns();
         copy_rows(ca, n_rows, w, nw, lane, [&](int i, int64_t& srow, int64_t& drow) {
             const int r = (text_early && i >= baset) ? i + s.n_txt : i;       // skip the text rows copied before
-            const int v = poll_word(kept + r, t0, 1000000000ull);   // the whole warp reads one word: one request
+            const int v = poll_word(kept + r * kListStride, t0, 1000000000ull);   // the whole warp reads one word: one request
             if (v < 0) {                                    // gave up: report, leave the row alone
                 *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
                 return false;

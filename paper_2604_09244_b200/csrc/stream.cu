@@ -537,9 +537,11 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             if (a.alpha.ptr) j.alpha = a.alpha.ptr + static_cast<int64_t>(h) * a.alpha.stride_h + static_cast<int64_t>(s.vis_off) * 4;
             if (a.rearm && h == 0 && crank == 0) {    // the tail kernel's hand-over words; their last users finished long ago
                 if (!a.rearm_rec) {
-                    for (int i = tid; i < s.n_out; i += kSoftThreads) a.rearm[s.out_off + i] = -1;
+                    for (int i = tid; i < s.n_out; i += kSoftThreads) a.rearm[(s.out_off + i) * kListStride] = -1;
                 } else {                              // the patch-by-patch tail: its list words, and three words per patch
-                    for (int i = tid; i < kHandWords + s.n_txt + s.n_2d + s.n_3d; i += kSoftThreads) a.rearm[s.cap_off + i] = -1;
+                    for (int i = tid; i < kHandWords; i += kSoftThreads) a.rearm[s.cap_off + i] = -1;
+                    for (int i = tid; i < s.n_txt + s.n_2d + s.n_3d; i += kSoftThreads)
+                        a.rearm[s.cap_off + kHandWords + i * kListStride] = -1;
                     for (int i = tid; i < 3 * s.n_2d; i += kSoftThreads) a.rearm_rec[static_cast<int64_t>(s.vis_off / 2) * 3 + i] = ~0ull;
                 }
             }
