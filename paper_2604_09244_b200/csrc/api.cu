@@ -348,7 +348,7 @@ bool stream_pays(const mvla_ctx* ctx, const BatchDesc& bd, int tiles_per_cta, in
 // fixed-point accumulators ctx->acc64 (*used_acc64 = true).
 int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, const void* k, int64_t rows,
                            const void* hidden, float* l1, unsigned long long* acc64, bool* used_acc64,
-                           bool free_running, cudaStream_t st, AlphaOut alpha = AlphaOut{nullptr, 0, 0},
+                           cudaStream_t st, AlphaOut alpha = AlphaOut{nullptr, 0, 0},
                            int32_t* rearm = nullptr, bool norms_beside = false, unsigned long long* stamps = nullptr,
                            bool with_cache = false, unsigned long long* rearm_rec = nullptr, float* attn_out = nullptr)
 {
@@ -386,7 +386,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     }
     if (streaming) {
         e = launch_salience_stream(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk, acc64,
-                                   ctx->status_dev, free_running, alpha, rearm, rearm_rec, stamps, st);
+                                   ctx->status_dev, alpha, rearm, rearm_rec, stamps, st);
         if (used_acc64) *used_acc64 = acc64 != nullptr;
     } else if (f32) {
         e = launch_salience_f32(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, tq, tk, tiles_per_cta, cluster, npad, acc64, ctx->status_dev, rearm, stamps, st);
@@ -394,7 +394,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     } else if (fast) {
         e = launch_salience_fast(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk,
                                  tiles_per_cta, cluster, npad,
-                                 acc64, ctx->status_dev, free_running, alpha, rearm, rearm_rec, stamps,
+                                 acc64, ctx->status_dev, alpha, rearm, rearm_rec, stamps,
                                  with_cache ? ctx->lcache : nullptr, ctx->max_vis, ctx->cache_cols, st);
         if (used_acc64) *used_acc64 = acc64 != nullptr;
     } else {
@@ -572,7 +572,7 @@ int32_t run_patch_indicators(mvla_ctx* ctx, unsigned set, const Plan& plan, int3
     const AlphaOut alpha = alpha_of(ctx, set);
     for (int first = 0; first < batch; first += kMaxChunk) {
         const BatchDesc bd = chunk_of(plan, first, std::min(kMaxChunk, batch - first));
-        const int32_t rc = run_salience_chunk(ctx, bd, q, k, rows, nullptr, nullptr, nullptr, nullptr, false, st, alpha);
+        const int32_t rc = run_salience_chunk(ctx, bd, q, k, rows, nullptr, nullptr, nullptr, nullptr, st, alpha);
         if (rc != MVLA_OK) return rc;
     }
     for (int first = 0; first < batch; first += kMaxChunk) {
@@ -677,7 +677,7 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
         unsigned long long* rec = ctx->patch_rec + par * (ctx->vis_all / 2 + 1) * 3;
         const AlphaOut alpha = alpha_of(ctx, set);
         ph.mark("mvla: scoring (+ attention copy)");
-        rc = run_salience_chunk(ctx, whole, in->q, in->k, in->rows, nullptr, nullptr, nullptr, nullptr, false, st, alpha,
+        rc = run_salience_chunk(ctx, whole, in->q, in->k, in->rows, nullptr, nullptr, nullptr, nullptr, st, alpha,
                                 list, false, nullptr, false, rec);
         if (rc != MVLA_OK) return rc;
         const PatchParams pp = patch_params(ctx);
@@ -937,7 +937,7 @@ static int32_t mvla_salience_impl(mvla_ctx* ctx, int32_t batch, const mvla_sampl
     for (int first = 0; first < batch; first += kMaxChunk) {
         const BatchDesc bd = chunk_of(plan, first, std::min(kMaxChunk, batch - first));
         bool used_acc64 = false;
-        rc = run_salience_chunk(ctx, bd, q, k, rows, want_l1 ? hidden : nullptr, l1_out, acc64, &used_acc64, false, st,
+        rc = run_salience_chunk(ctx, bd, q, k, rows, want_l1 ? hidden : nullptr, l1_out, acc64, &used_acc64, st,
                                 AlphaOut{nullptr, 0, 0}, nullptr, true, nullptr, false, nullptr, attn_out);
         if (rc != MVLA_OK) return rc;
     }
@@ -1208,7 +1208,7 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         const bool tail = !forked;
         ph.mark("mvla: scoring");
         rc = run_salience_chunk(ctx, bd, in->q, in->k, in->rows, adaptive ? in->hidden : nullptr, l1_ws, acc64,
-                                &used_acc64, false, forked ? ctx->aux[par] : st, AlphaOut{nullptr, 0, 0},
+                                &used_acc64, forked ? ctx->aux[par] : st, AlphaOut{nullptr, 0, 0},
                                 tail ? ctx->tail_list + par * ctx->rows_all : nullptr, tail, tail ? ctx->stamps : nullptr,
                                 cache_on);
         if (rc != MVLA_OK) return rc;
@@ -1238,9 +1238,9 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         io.chunk_first = first; io.total_out = plan.total_out; io.write_total = first + n == batch;
         io.n_in_launch = n;
         if (!forked && used_acc64) {
-            // one kernel for selection and row copy: every CTA repeats its sample's selection, then copies
+            // one kernel: a CTA per sample selects, the others copy rows as the kept list becomes known
             ctx->sel_valid[par] = false;             // this set was used outside the event chain
-                ph.mark("mvla: selection + row copy");
+            ph.mark("mvla: selection + row copy");
             const cudaError_t e2 = launch_select_copy(bd, gp, io, job, ctx->tail_list + par * ctx->rows_all,
                                                       ctx->status_dev,
                                                       ctx->stamps ? ctx->stamps + 2 * kStampSlots : nullptr, st);

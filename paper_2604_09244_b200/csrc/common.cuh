@@ -136,8 +136,6 @@ cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t 
 // bf16 tensor-core salience with logits held in registers (one or two key tiles per CTA).  The per-head
 // contributions are added into the 64-bit fixed-point accumulators `acc64` (scale 2^60, one per visual token, zero on
 // entry); nowhere when it is null: only the attention copy is wanted.
-// `free_running`: the kernel does not wait for the kernel before it in its stream (the caller orders
-// everything it depends on with events).
 // `lcache`: logit cache [state][head][cache_vis][cache_cols] fp32 (raw dot products), or null; which tiles are
 // computed and stored and which are read back is in the descriptors (cache_state, tile_compute).
 // `stamps`: when not null, CTA c (linear index, below kStampSlots) writes the global timer when it was free to
@@ -163,7 +161,7 @@ bool fast_salience_supported(int tiles_per_cta);
 cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tmap_q,
                                  const CUtensorMap* tmap_k, int tiles_per_cta, int cluster, int npad,
                                  unsigned long long* acc64, int* status,
-                                 bool free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
+                                 AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                                  float* lcache, int cache_vis, int cache_cols, cudaStream_t stream);
 
 // The same scores into the same fixed-point accumulators from fp32 q / k (plain FMAs), where the shape fits.
@@ -173,11 +171,10 @@ cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, 
                                 int cluster, int npad, unsigned long long* acc64, int* status, int32_t* rearm, unsigned long long* stamps,
                                 cudaStream_t stream);
 // The same scores into the same fixed-point accumulators by the streaming kernel (stream.cu): persistent CTAs, key
-// tiles through a shared-memory ring; for batches and for samples of any size.  `free_running`, `alpha`, `rearm`, `stamps` as
-// above; with `alpha` there may be no accumulators.
+// tiles through a shared-memory ring; for batches and for samples of any size.  `alpha`, `rearm`, `stamps` as above; with `alpha` there may be no accumulators.
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
-                                   bool free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
+                                   AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
                                    unsigned long long* stamps, cudaStream_t stream);
 
 // Salience: per-head partial scores part[h][vis] (already scaled by 1/(H n_t)).

@@ -1,9 +1,17 @@
-// Fast salience kernel for bf16 (Sec. 3.2.1 of the paper).
+// Latency-shaped scoring kernels (Sec. 3.2.1 of the paper): bf16 and e4m3 on the tensor cores, fp32 by FMAs; for
+// launches whose CTAs all run at once (batches and larger samples: stream.cu).
 //
 // Same decomposition as the generic salience kernel (one cluster per (sample, head), one CTA per one or
 // two tiles of 128 keys; TMA -> shared memory -> tcgen05.mma -> tensor memory), but built as one short
-// dependency chain, because at ~40 KB of input per CTA the kernel is latency bound:
-//   * the loads are issued before anything else; tensor-memory allocation overlaps with them;
+// dependency chain, because at ~40 KB of input per CTA the kernel is latency bound.  Of the 5 us that one sample of
+// 768 tokens and 32 heads of 128 takes (2.6 us would be its share of the key stream at full bandwidth), 1.5 are the
+// tiles' flight, 0.6 the MMAs, 1.7 the softmax with the exchange, the rest launch and drain.  So:
+//   * everything that reads nothing of the kernel before comes before the wait for it (barriers, cluster arrive,
+//     tensor-memory allocation, hand-over words, load operands): a release issued behind the loads waits as long as
+//     they do.  A step of one frame 12.8 -> 12.0 us, eight action steps 161.8 -> 153.4;
+//   * a variant per use (scores, with the logit cache, with the attention copy): the code runs once per launch from
+//     a cold instruction cache, and what a step does not use cost eight action steps 4 us;
+//   * exponents are taken against the logits of each warp's first key, not a maximum: two block barriers less;
 //   * each thread reads ALL its logits from tensor memory once (one wide tcgen05.ld) and keeps them in
 //     registers through max -> exp2 -> sum -> weighted sum;
 //   * the per-query (max, sum) pairs travel between the CTAs of a cluster as asynchronous remote
@@ -69,7 +77,7 @@ struct FastSmem {
 struct FastOut {
     unsigned long long* acc64;               // null: the attention copy only
     int* status;
-    int free_running, n_heads;
+    int n_heads;
     AlphaOut alpha;
 };
 
@@ -201,7 +209,7 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
 
     // ---- per key: sum over queries of the normalised probabilities (this head's contribution)
     const float* const w = sm.w[kwarp] + c0;  // 0 past the text queries
-    if (!o.free_running) pdl_wait();          // the accumulators were read and cleared by an earlier selection
+    pdl_wait();                               // the accumulators were read and cleared by an earlier selection
 #pragma unroll
     for (int t = 0; t < NTILE; ++t) {
         if (key >= valid[t]) continue;
@@ -245,7 +253,7 @@ __global__ void __launch_bounds__(kFastThreads * SPLIT, 1)
 salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUtensorMap tmap_q,
                      const __grid_constant__ CUtensorMap tmap_k, int n_heads, int kv_group, int head_dim, int esize, int npad_max,
                      unsigned long long* __restrict__ acc64,
-                     int* status, int free_running, const AlphaOut alpha, int32_t* __restrict__ rearm, unsigned long long* __restrict__ rearm_rec,
+                     int* status, const AlphaOut alpha, int32_t* __restrict__ rearm, unsigned long long* __restrict__ rearm_rec,
                      unsigned long long* __restrict__ stamps, float* __restrict__ lcache, int cache_vis, int cache_cols)
 {
     constexpr int CC = TCOL * NTILE;                      // tensor-memory columns of the CTA
@@ -360,9 +368,8 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
     // elected lane issues, so that coordinates and descriptors stay in uniform registers.  (In a single-thread branch
     // every operand is moved to a uniform register one by one: 0.1 us more for the MMAs of a tile.)
     if (warp == 0) {
-        // Inputs may come from the kernel before this one -- unless the host has established (stable
-        // inputs, scratch ordered by events) that nothing this kernel touches depends on it.
-        if (!free_running) pdl_wait();
+        // Inputs may come from the kernel before this one.
+        pdl_wait();
         // (no tile to compute: nothing is fetched, both barriers below complete at once)
         if (one) mbar_expect_tx(bar_full, live > 0 ? static_cast<uint32_t>(khalves) * (npad * 128 + live * 16384) : 0u);
 #pragma unroll
@@ -450,7 +457,7 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
         }
     }
     softmax_scores<TCOL, NTILE, SPLIT, KIND == kForPatches>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
-                                       FastOut{acc64, status, free_running, n_heads, alpha});
+                                       FastOut{acc64, status, n_heads, alpha});
 
     tc_fence_before();
     __syncthreads();
@@ -574,7 +581,7 @@ salience_f32_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUten
         }
     }
     softmax_scores<TCOL, NTILE, 2, false>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
-                                   FastOut{acc64, status, 0, n_heads, AlphaOut{nullptr, 0, 0}});
+                                   FastOut{acc64, status, n_heads, AlphaOut{nullptr, 0, 0}});
     if (stamps) {
         __syncthreads();
         if (tid == 0) {
@@ -587,7 +594,7 @@ salience_f32_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUten
 template <int TCOL, int NTILE, int SPLIT, int KIND, class BD>
 cudaError_t launch_fast_t(const BD& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tq,
                           const CUtensorMap* tk, int cluster, int npad,
-                          unsigned long long* acc64, int* status, int free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
+                          unsigned long long* acc64, int* status, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                           float* lcache, int cache_vis, int cache_cols, cudaStream_t stream)
 {
     size_t smem = 1024 + static_cast<size_t>((head_dim * esize + 127) / 128) * (static_cast<size_t>(NTILE) * 16384 + npad * 128);
@@ -612,7 +619,7 @@ cudaError_t launch_fast_t(const BD& bd, int n_heads, int kv_group, int head_dim,
     attr[1] = pdl_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, n_heads, kv_group, head_dim, esize, npad, acc64, status, free_running, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols);
+    return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, n_heads, kv_group, head_dim, esize, npad, acc64, status, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols);
 }
 
 template <int TCOL, int NTILE, class BD>
@@ -668,7 +675,7 @@ bool fast_salience_supported(int tiles_per_cta) { return tiles_per_cta >= 1 && t
 cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tmap_q,
                                  const CUtensorMap* tmap_k, int tiles_per_cta, int cluster, int npad,
                                  unsigned long long* acc64, int* status,
-                                 bool free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
+                                 AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                                  float* lcache, int cache_vis, int cache_cols, cudaStream_t stream)
 {
     const int tcol = npad <= 16 ? 16 : (npad <= 32 ? 32 : 64);
@@ -679,7 +686,7 @@ cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group,
     if (tcol == TC && tiles_per_cta == NTL && split == SP && kind == KD)                                        \
         return with_desc(bd, [&](const auto& d) {                                                               \
             return launch_fast_t<TC, NTL, SP, KD>(d, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, acc64, status, \
-                                                  free_running ? 1 : 0, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream); });
+                                                  alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream); });
 #define MVLA_FAST(TC, NTL, SP) MVLA_FAST1(TC, NTL, SP, kPlain) MVLA_FAST1(TC, NTL, SP, kWithCache) MVLA_FAST1(TC, NTL, SP, kForPatches)
     MVLA_FAST(16, 1, 1) MVLA_FAST(16, 2, 1) MVLA_FAST(32, 1, 2) MVLA_FAST(64, 1, 2) MVLA_FAST(32, 2, 2) MVLA_FAST(64, 2, 2)
 #undef MVLA_FAST1

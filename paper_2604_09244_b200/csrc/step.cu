@@ -12,6 +12,9 @@
 //   * what nobody waits for (smoothed state, indicators and diagnostics when the budgets came from the
 //     host, optional score outputs) is written after the list.
 // The scoring kernel that runs before this one re-arms the words, so nothing is left to do at the end.
+// A word is polled by the dozen warps that move its row's segments, and polls of one line of the L2 are served one
+// after another: neighbouring rows' words lie kListStride words apart (8 words a line instead of 32: eight action steps
+// 143.5 -> 141.2 us, three views 20.8 -> 20.4; 4 words a line were no better).
 #include "common.cuh"
 #include "device_utils.cuh"
 #include "copy_impl.cuh"

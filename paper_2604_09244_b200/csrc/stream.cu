@@ -10,10 +10,14 @@
 //     two buffers of their own): 128-160 KB in flight per multiprocessor whatever the softmax is doing;
 //   * one thread issues the MMAs of a tile into the next free tensor-memory slot (slots are a ring too);
 //   * eight warps take the softmax: a warp reads its own 32 tensor-memory lanes of every other tile, against references of
-//     its own, so that a job has two block barriers in all.  Exponentials go back to tensor memory; per-key contributions are added into the 64-bit fixed-point
-//     accumulators (scale 2^60: the sum over heads is exact and independent of scheduling).
+//     its own, so that a job has two block barriers in all.  Exponentials go back to tensor memory; per-key contributions
+//     are added into the 64-bit fixed-point accumulators (scale 2^60: the sum over heads is exact and independent of
+//     scheduling).
 // What bounds it: HBM (the keys are read once); softmax arithmetic comes second (16 exponentials per clock and
 // multiprocessor: half of the time of the key stream at 48 queries, nine tenths at 64).
+// Whole steps against one short-lived CTA per two tiles (and, above 2048 tokens, the generic kernel): 16 requests of 768
+// tokens 121 -> 97 us, 8 of 3584 tokens 695 -> 184, 16 patch-by-patch steps of 512 tokens 139 -> 97.
+// More softmax warps (12, 16), two tiles per warp at once and prefetching the next tile's columns were all slower.
 #include "common.cuh"
 #include "device_utils.cuh"
 #include "select_impl.cuh"
@@ -42,7 +46,6 @@ struct StreamArgs {
     int n_jobs;                   // samples x heads
     unsigned long long* acc64;
     int* status;
-    int free_running;
     AlphaOut alpha;               // with it there may be no accumulators
     int32_t* rearm;               // see launch_salience_fast
     unsigned long long* rearm_rec;
@@ -434,7 +437,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             prefetch_tensormap(&tmap_q);
             prefetch_tensormap(&tmap_k);
         }
-        if (!a.free_running) pdl_wait();
+        pdl_wait();
         if (a.stamps && one && blockIdx.x < kStampSlots) a.stamps[2 * blockIdx.x] = global_ns();
         pdl_trigger();                        // whatever the kernel before this one wrote is complete
         const int box_elems = 128 / a.esize;
@@ -525,7 +528,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
         j.lane_base = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         j.cscale = 1.4426950408889634f * rsqrtf(static_cast<float>(a.head_dim));   // log2 domain
         float* const my_w = sm.w[warp];
-        bool waited = a.free_running != 0;
+        bool waited = false;
         int jn = 0;
         for (int job = first_job, b = b_first, h = h_first; job < a.n_jobs; job += job_step, ++jn, advance(b, h)) {
             const SampleDev& s = bd.s[b];
@@ -659,9 +662,13 @@ cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUte
 
 }  // namespace
 
+// no CTA with 32 columns of tensor memory (at least 1/17 of the shared memory, smem_for_tmem) fits beside one
+static_assert(kSmemPerSm - static_cast<int>(kStreamSmem + sizeof(StreamSmem)) - kSmemReservedPerCta < kSmemPerSm / 17,
+              "the streaming kernel must be alone with the tensor memory of its multiprocessor");
+
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
-                                   bool free_running, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
+                                   AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
                                    unsigned long long* stamps, cudaStream_t stream)
 {
     const int sms = sm_count_of_current_device();
@@ -671,7 +678,7 @@ cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_grou
     a.width = npad;
     a.slots = std::min(kMaxSlots, kTmemColsPerSm / npad);
     a.n_jobs = bd.n * n_heads;
-    a.acc64 = acc64; a.status = status; a.free_running = free_running ? 1 : 0; a.alpha = alpha; a.rearm = rearm;
+    a.acc64 = acc64; a.status = status; a.alpha = alpha; a.rearm = rearm;
     a.rearm_rec = rearm_rec; a.stamps = stamps;
     // The smallest cluster whose CTAs hold their share of a job's logits in tensor memory; a larger one while jobs are
     // fewer than multiprocessors and the tiles can still be shared out.

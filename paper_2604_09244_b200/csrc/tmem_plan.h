@@ -47,10 +47,10 @@ inline size_t smem_for_tmem(size_t dyn_smem, int tmem_cols)
     return padded <= static_cast<size_t>(kSmemMaxPerCta) ? padded : 0;
 }
 
-// Dynamic shared memory of the streaming scoring kernel, which takes all 512 columns: it leaves 28 KB of a
-// multiprocessor less the kernel's static part (21 KB) and the reserved part, and no kernel that uses tensor memory
-// gets by with less than 13 KB (smem_for_tmem for 32 columns), so whoever runs beside it has none.  Kernels without
-// shared memory (the feature norms) still fit.
-constexpr size_t kStreamSmem = 200 * 1024;
+// Dynamic shared memory of the streaming scoring kernel, which takes all 512 columns: with the kernel's static
+// part (13.25 KB) and the reserved part it leaves 5.75 KB of a multiprocessor, and no kernel that uses tensor memory gets
+// by with less than 13 KB (smem_for_tmem for 32 columns), so whoever runs beside it has none.  Kernels without shared
+// memory (the feature norms) still fit.
+constexpr size_t kStreamSmem = 208 * 1024;
 
 }  // namespace mvla
