@@ -386,7 +386,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     }
     if (streaming) {
         e = launch_salience_stream(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk, acc64,
-                                   ctx->status_dev, alpha, rearm, rearm_rec, stamps, st);
+                                   ctx->status_dev, alpha, rearm, rearm_rec, stamps, hidden && l1 && norms_beside, st);
         if (used_acc64) *used_acc64 = acc64 != nullptr;
     } else if (f32) {
         e = launch_salience_f32(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, tq, tk, tiles_per_cta, cluster, npad, acc64, ctx->status_dev, rearm, stamps, st);

@@ -171,11 +171,12 @@ cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, 
                                 int cluster, int npad, unsigned long long* acc64, int* status, int32_t* rearm, unsigned long long* stamps,
                                 cudaStream_t stream);
 // The same scores into the same fixed-point accumulators by the streaming kernel (stream.cu): persistent CTAs, key
-// tiles through a shared-memory ring; for batches and for samples of any size.  `alpha`, `rearm`, `stamps` as above; with `alpha` there may be no accumulators.
+// tiles through a shared-memory ring; for batches and for samples of any size.  `alpha`, `rearm`, `stamps` as above; with
+// `alpha` there may be no accumulators.  `norms_beside`: launch_l1norm follows and is to run beside it.
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
                                    AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
-                                   unsigned long long* stamps, cudaStream_t stream);
+                                   unsigned long long* stamps, bool norms_beside, cudaStream_t stream);
 
 // Salience: per-head partial scores part[h][vis] (already scaled by 1/(H n_t)).
 // `use_umma`: tensor-core path (bf16 only).  tmaps: device-usable tensor maps (passed by value).

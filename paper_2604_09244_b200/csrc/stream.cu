@@ -380,7 +380,13 @@ __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, in
 }
 
 // grid = clusters x cluster size (1-D), kStreamThreads threads, one CTA per multiprocessor.
-__global__ void __launch_bounds__(kStreamThreads, 1)
+// ROOM: the feature norms are to run beside this kernel.  Its ten warps put three on two of a multiprocessor's four
+// register files (16384 registers each): at the 168 registers a thread that the compiler takes these are full, no CTA of
+// the norms fits, and they start when the scores are done.  144 leave room for two warps of 32 registers in each (adaptive
+// steps, 10 requests of 190 tokens 31.2 -> 24.1 us, 4 of 768 33.6 -> 27.1); 128 spill in the softmax (16 requests of 768
+// tokens 97 -> 106).  Without norms the registers are worth more (16 patch-by-patch steps 96.3 us, 99.1 with 144).
+template <bool ROOM>
+__global__ void __maxnreg__(ROOM ? 144 : 168)
 salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,
                        const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ StreamArgs a)
 {
@@ -537,7 +543,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             const int n_txt = s.n_txt, npad = (n_txt + 15) & ~15;
             j.n_txt = n_txt;
             j.hn = static_cast<float>(a.n_heads) * static_cast<float>(n_txt);
-            if (a.alpha.ptr) j.alpha = a.alpha.ptr + static_cast<int64_t>(h) * a.alpha.stride_h + static_cast<int64_t>(s.vis_off) * 4;
+            if (!ROOM && a.alpha.ptr) j.alpha = a.alpha.ptr + static_cast<int64_t>(h) * a.alpha.stride_h + static_cast<int64_t>(s.vis_off) * 4;
             if (a.rearm && h == 0 && crank == 0) {    // the tail kernel's hand-over words; their last users finished long ago
                 if (!a.rearm_rec) {
                     for (int i = tid; i < s.n_out; i += kSoftThreads) a.rearm[(s.out_off + i) * kListStride] = -1;
@@ -589,7 +595,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
                 my_w[i] = mk == -CUDART_INF_F ? 0.f : fast_ex2(mk - sm.g[i]) * sm.iz[i];
             }
             __syncwarp();
-            if (a.alpha.ptr) soft_scores<true>(j, sm, nch, warp, lane);
+            if (!ROOM && a.alpha.ptr) soft_scores<true>(j, sm, nch, warp, lane);
             else soft_scores<false>(j, sm, nch, warp, lane);
             j.slot0 += j.tr.count;
             if (j.slot0 >= a.slots) { j.slot0 -= a.slots; j.parity0 ^= 1u; }
@@ -623,10 +629,11 @@ int max_tiles(const BatchDesc& bd)
     return t;
 }
 
+template <bool ROOM>
 cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUtensorMap* tk, StreamArgs& a, int cluster,
                             int sms, size_t smem, cudaStream_t stream)
 {
-    auto kern = salience_stream_kernel;
+    auto kern = salience_stream_kernel<ROOM>;
     static KernelSetup ks;
     const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kStreamThreads, smem, kTmemColsPerSm);
     if (e != cudaSuccess) return e;
@@ -669,7 +676,7 @@ static_assert(kSmemPerSm - static_cast<int>(kStreamSmem + sizeof(StreamSmem)) - 
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
                                    AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
-                                   unsigned long long* stamps, cudaStream_t stream)
+                                   unsigned long long* stamps, bool norms_beside, cudaStream_t stream)
 {
     const int sms = sm_count_of_current_device();
     const int npad = padded_text(bd), tiles = max_tiles(bd);
@@ -689,7 +696,8 @@ cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_grou
     const size_t q_bytes = 2 * static_cast<size_t>((head_dim * esize + 127) / 128) * npad * 128;
     a.stages = static_cast<int>(std::min<size_t>(kMaxStages, (kStreamSmem - 1024 - q_bytes) / kStageBytes));
     if (a.stages < 4) return cudaErrorInvalidConfiguration;
-    return launch_stream(bd, tmap_q, tmap_k, a, cluster, sms, kStreamSmem, stream);
+    if (norms_beside && !alpha.ptr) return launch_stream<true>(bd, tmap_q, tmap_k, a, cluster, sms, kStreamSmem, stream);
+    return launch_stream<false>(bd, tmap_q, tmap_k, a, cluster, sms, kStreamSmem, stream);
 }
 
 }  // namespace mvla
