@@ -759,6 +759,19 @@ def test_streaming_scoring_kernel_at_the_edges_of_its_shapes(batch, H, n_txt, n_
     ctx.close()
 
 
+@pytest.mark.parametrize("batch,H,n_txt,n_2d,n_3d", [
+    (8, 16, (64, 1, 33), (129, 40), (255, 300)),
+    (2, 4, (17, 50), (1500, 2000), (1200, 77))])
+def test_streaming_scoring_kernel_without_norms_beside_it(batch, H, n_txt, n_2d, n_3d):
+    """Fixed budgets need no feature norms: the kernel's other register split."""
+    wl = W.small_workload(73, batch=batch, H=H, D=256, n_txt=n_txt, n_2d=n_2d, n_3d=n_3d, mode=W.MODE_FIXED, steps=2)
+    ctx = mvla.context_for(wl)
+    states = [oracle.State(s.n_vis) for s in wl.samples]
+    for step in range(2):
+        run_and_check_step(ctx, wl, step, states)
+    ctx.close()
+
+
 @pytest.mark.parametrize("gain", [30.0, 300.0])
 def test_streaming_scoring_kernel_moves_its_references_when_exponents_would_overflow(gain):
     """Keys whose logits grow from tile to tile by far more than an fp32 exponent holds."""
