@@ -16,7 +16,7 @@
 // What bounds it: HBM (the keys are read once); softmax arithmetic comes second (16 exponentials per clock and
 // multiprocessor: half of the time of the key stream at 48 queries, nine tenths at 64).
 // Whole steps against one short-lived CTA per two tiles (and, above 2048 tokens, the generic kernel): 16 requests of 768
-// tokens 121 -> 97 us, 8 of 3584 tokens 695 -> 184, 16 patch-by-patch steps of 512 tokens 139 -> 97.
+// tokens 121 -> 97 us, 8 of 3584 tokens 695 -> 162, 16 patch-by-patch steps of 512 tokens 139 -> 97.
 // More softmax warps (12, 16), two tiles per warp at once and prefetching the next tile's columns were all slower.
 #include "common.cuh"
 #include "device_utils.cuh"
