@@ -122,7 +122,8 @@ typedef struct mvla_config {
                                   which says which rows changed (mvla_tensors.changed_rows) recomputes only those
                                   (Sec. 4.3 / 5.2: consecutive frames share most of their content).
                                   n_prune_points x slots x n_heads x (max_2d + max_3d) x round16(max_text) floats.
-                                  bf16 / e4m3 tensor-core path, samples of up to 2048 visual tokens, budgeted modes */
+                                  bf16 / e4m3 tensor-core path, budgeted modes, calls of up to 32 samples of up to 16
+                                  key tiles (of 128, per modality) each; other calls run without */
     int32_t reserved0;
 } mvla_config;
 

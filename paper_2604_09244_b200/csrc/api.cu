@@ -276,6 +276,8 @@ int tiles_of(const SampleDev& s)
 {
     return (s.n_2d + kKeyTile - 1) / kKeyTile + (s.n_3d + kKeyTile - 1) / kKeyTile;
 }
+// Key tiles of a CTA where one cluster covers a (sample, head) of `tiles` tiles.
+int tiles_per_cta_of(int tiles) { return (tiles + kMaxCluster - 1) / kMaxCluster; }
 
 // 3-D view (head_dim, heads, rows) of a token-major [rows, H, d] tensor; boxes of 128 bytes x 1 x
 // `box_rows` land in shared memory as `box_rows` rows of 128 bytes with the 128-byte swizzle.
@@ -362,7 +364,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
         cached |= bd.s[b].cache_state >= 0;
     }
     with_cache = with_cache && cached;
-    const int tiles_per_cta = (max_tiles + kMaxCluster - 1) / kMaxCluster;
+    const int tiles_per_cta = tiles_per_cta_of(max_tiles);
     const int cluster = (max_tiles + tiles_per_cta - 1) / tiles_per_cta;
     const int npad = (max_txt + 15) / 16 * 16;
     const CUtensorMap *tq = nullptr, *tk = nullptr;
@@ -1133,8 +1135,11 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
     job.row_bytes[0] = static_cast<int32_t>(ctx->cfg.d_model * ctx->elem);
 
     // Reuse of the previous step's logits: which key tiles of which sample must be computed (host decision
-    // from the caller's changed_rows), for steps that are not overlapped with their neighbours.
-    const bool cache_on = ctx->lcache != nullptr && !(flags & MVLA_FLAG_INPUTS_STABLE);
+    // from the caller's changed_rows), for steps that are not overlapped with their neighbours.  Only the latency-shaped
+    // kernel reads and writes the cache, and one launch is scored by one kernel: a sample that it does not take (by
+    // tiles, not by tokens: 1100 + 900 tokens are 17 tiles) leaves the whole call without.
+    bool cache_on = ctx->lcache != nullptr && !(flags & MVLA_FLAG_INPUTS_STABLE) && batch <= kMaxChunk;
+    for (int b = 0; b < batch && cache_on; ++b) cache_on = fast_salience_supported(tiles_per_cta_of(tiles_of(plan.s[b])));
     for (int b = 0; b < batch; ++b) {
         SampleDev& d = plan.s[b];
         d.cache_state = -1;
@@ -1144,8 +1149,7 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         const int sidx = prune_point * ctx->n_slots + sm.state_slot;
         mvla_ctx::CacheSig& sig = ctx->cache_sig[sidx];
         const int tiles = tiles_of(d);
-        const bool fits = sm.n_2d + sm.n_3d <= 2048 && batch <= kMaxChunk;
-        if (!cache_on || !fits || (flags & MVLA_FLAG_NO_STATE_UPDATE)) {
+        if (!cache_on || (flags & MVLA_FLAG_NO_STATE_UPDATE)) {
             // the step runs without the cache; a dry run leaves it as it is, anything else makes it stale
             if (!(flags & MVLA_FLAG_NO_STATE_UPDATE)) sig.valid = false;
             continue;

@@ -717,6 +717,38 @@ def test_a_mask_that_hides_a_change_reuses_the_stale_logits():
     ctx.close()
 
 
+def test_logit_cache_is_left_out_of_samples_that_its_kernel_does_not_take():
+    # 9 + 8 key tiles in 2000 tokens: one tile more than the kernel that keeps logits covers.  Nothing is reused or counted,
+    # whatever the mask says, and every step is judged against the full oracle on its own inputs
+    wl = W.config5_action_iteration(T=3, D=256, H=4, d=64, n_txt=20, n_2d=1100, n_3d=900, drift="visual_local")
+    ctx = mvla.context_for(wl, logit_cache=1)
+    states = _fresh_states(wl)
+    for t in range(3):
+        run_and_check_step(ctx, wl, t, states, flags=mvla.FLAG_RESET_STATE if t == 0 else 0,
+                           changed_rows=wl.extra["changed_rows"][t] if t > 0 else None)
+        assert ctx.logit_cache_stats() == (0, 0)
+    ctx.close()
+
+
+def test_a_step_beside_a_sample_without_logit_cache_leaves_no_logits_to_reuse():
+    # the small sample (2 + 3 tiles) is stepped beside one of 17 tiles, then alone with a mask, then alone once more
+    wl = W.small_workload(83, batch=2, D=256, H=4, d=64, n_txt=(20, 30), n_2d=(150, 1100), n_3d=(300, 900))
+    ctx, small, t = mvla.context_for(wl, logit_cache=1), wl.samples[0], wl.steps[0]
+    dev = device_tensors(wl)
+    ctx.prune_step(0, wl.samples, wl.mode, dev["q"], dev["k"], dev["v"], dev["hidden"], flags=mvla.FLAG_RESET_STATE)
+    assert ctx.logit_cache_stats() == (0, 0)
+    for computed, reused in ((5, 0), (6, 4)):
+        mask = np.zeros(wl.total_rows, dtype=np.uint8)
+        mask[small.seq_off + small.off_2d:][:40] = 1
+        t.k[mask != 0] *= np.float32(-2.0)                            # (exact in bf16)
+        k = mvla.to_device(t.k, wl.dtype, "cuda")
+        out = ctx.prune_step(0, [small], wl.mode, dev["q"], k, dev["v"], dev["hidden"], changed_rows=mask)
+        torch.cuda.synchronize()
+        assert_salience_close(out.attn.cpu().numpy(), oracle.salience(t.q, t.k, wl.n_heads, wl.head_dim, small))
+        assert ctx.logit_cache_stats() == (computed, reused)
+    ctx.close()
+
+
 @pytest.mark.parametrize("n_txt,n_2d,n_3d", [(40, 700, 900), (64, 512, 640), (17, 1500, 500), (48, 100, 60)])
 def test_step_with_two_threads_per_key_in_every_shape_of_the_scoring_kernel(n_txt, n_2d, n_3d):
     # more than 16 text queries: the scoring kernel of the fused step runs with two threads per key, half of the
