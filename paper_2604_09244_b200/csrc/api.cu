@@ -257,10 +257,24 @@ int32_t make_plan(mvla_ctx* ctx, int32_t prune_point, int32_t batch, const mvla_
     return MVLA_OK;
 }
 
+int tiles_of(const SampleDev& s)
+{
+    return (s.n_2d + kKeyTile - 1) / kKeyTile + (s.n_3d + kKeyTile - 1) / kKeyTile;
+}
+
+// The step is enqueued: its samples' states move on.  So does what the logit cache holds of them: this step's logits
+// where the step ran with the cache, else (the stage calls, steps without it) nothing that a later mask could refer to.
 void commit_steps(mvla_ctx* ctx, int32_t prune_point, const Plan& plan, const mvla_sample* samples)
 {
-    for (int b = 0; b < plan.n; ++b)
-        if (plan.s[b].update_state) ctx->t_host[prune_point * ctx->n_slots + samples[b].state_slot] = plan.s[b].t;
+    for (int b = 0; b < plan.n; ++b) {
+        const SampleDev& d = plan.s[b];
+        if (!d.update_state) continue;
+        const int sidx = prune_point * ctx->n_slots + samples[b].state_slot;
+        ctx->t_host[sidx] = d.t;
+        if (!ctx->lcache) continue;
+        ctx->cache_sig[sidx] = mvla_ctx::CacheSig{d.cache_state >= 0, d.n_txt, d.n_2d, d.n_3d};
+        for (int t = 0; t < tiles_of(d) && d.cache_state >= 0; ++t) ((d.tile_compute >> t) & 1u ? ctx->tiles_computed : ctx->tiles_reused) += 1;
+    }
 }
 
 // (descriptors past the n-th are left as they are: no kernel looks at them)
@@ -272,10 +286,6 @@ BatchDesc chunk_of(const Plan& plan, int first, int n)
     return bd;
 }
 
-int tiles_of(const SampleDev& s)
-{
-    return (s.n_2d + kKeyTile - 1) / kKeyTile + (s.n_3d + kKeyTile - 1) / kKeyTile;
-}
 // Key tiles of a CTA where one cluster covers a (sample, head) of `tiles` tiles.
 int tiles_per_cta_of(int tiles) { return (tiles + kMaxCluster - 1) / kMaxCluster; }
 
@@ -1142,18 +1152,11 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
     for (int b = 0; b < batch && cache_on; ++b) cache_on = fast_salience_supported(tiles_per_cta_of(tiles_of(plan.s[b])));
     for (int b = 0; b < batch; ++b) {
         SampleDev& d = plan.s[b];
-        d.cache_state = -1;
-        d.tile_compute = 0xFFFFFFFFu;
-        if (!ctx->lcache) continue;
+        if (!cache_on || !d.update_state) continue;      // (a dry run leaves the cache as it is)
         const mvla_sample& sm = samples[b];
         const int sidx = prune_point * ctx->n_slots + sm.state_slot;
         mvla_ctx::CacheSig& sig = ctx->cache_sig[sidx];
         const int tiles = tiles_of(d);
-        if (!cache_on || (flags & MVLA_FLAG_NO_STATE_UPDATE)) {
-            // the step runs without the cache; a dry run leaves it as it is, anything else makes it stale
-            if (!(flags & MVLA_FLAG_NO_STATE_UPDATE)) sig.valid = false;
-            continue;
-        }
         d.cache_state = sidx;
         bool all = !sig.valid || (flags & MVLA_FLAG_RESET_STATE) || !in->changed_rows || sig.n_txt != sm.n_txt ||
                    sig.n_2d != sm.n_2d || sig.n_3d != sm.n_3d;
@@ -1171,8 +1174,7 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
             }
             d.tile_compute = mask;
         }
-        for (int t = 0; t < tiles; ++t) ((d.tile_compute >> t) & 1u ? ctx->tiles_computed : ctx->tiles_reused) += 1;
-        sig = mvla_ctx::CacheSig{true, sm.n_txt, sm.n_2d, sm.n_3d};
+        sig.valid = false;                               // until the step is enqueued as a whole (commit_steps)
     }
 
     // scratch set of this step

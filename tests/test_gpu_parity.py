@@ -749,6 +749,23 @@ def test_a_step_beside_a_sample_without_logit_cache_leaves_no_logits_to_reuse():
     ctx.close()
 
 
+def test_a_step_through_the_stage_calls_makes_the_cached_logits_stale():
+    # step 2 runs as salience + select: a mask for step 3 says what changed since step 2, and the cache holds step 1
+    wl = W.config5_action_iteration(T=1, D=256, H=4, d=64, n_txt=20, n_2d=150, n_3d=300)
+    ctx, s, t, dev = mvla.context_for(wl, logit_cache=1), wl.samples[0], wl.steps[0], device_tensors(wl)
+    ctx.prune_step(0, wl.samples, wl.mode, dev["q"], dev["k"], dev["v"], dev["hidden"], flags=mvla.FLAG_RESET_STATE)
+    t.k[s.off_2d:s.off_2d + 40] *= np.float32(-2.0)                   # (exact in bf16)
+    k = mvla.to_device(t.k, wl.dtype, "cuda")
+    attn, l1 = ctx.salience(wl.samples, dev["q"], k, dev["hidden"])
+    ctx.select(0, wl.samples, wl.mode, attn, l1)
+    nothing = np.zeros(s.seq_len, dtype=np.uint8)
+    out = ctx.prune_step(0, wl.samples, wl.mode, dev["q"], k, dev["v"], dev["hidden"], changed_rows=nothing)
+    torch.cuda.synchronize()
+    assert_salience_close(out.attn.cpu().numpy(), oracle.salience(t.q, t.k, wl.n_heads, wl.head_dim, s))
+    assert ctx.logit_cache_stats() == (10, 0)
+    ctx.close()
+
+
 @pytest.mark.parametrize("n_txt,n_2d,n_3d", [(40, 700, 900), (64, 512, 640), (17, 1500, 500), (48, 100, 60)])
 def test_step_with_two_threads_per_key_in_every_shape_of_the_scoring_kernel(n_txt, n_2d, n_3d):
     # more than 16 text queries: the scoring kernel of the fused step runs with two threads per key, half of the
