@@ -123,6 +123,29 @@ cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t 
     return cudaSuccess;
 }
 
+cudaError_t clusters_at_once(KernelSetup& ks, const void* kern, int threads, size_t smem, int cluster, int* count)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    *count = ks.clusters.find(dev, cluster, smem);
+    if (*count > 0) return cudaSuccess;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(cluster));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(count, kern, &cfg);
+    if (e == cudaSuccess) ks.clusters.keep(dev, cluster, smem, *count);
+    return e;
+}
+
 cudaError_t launch_compact(const BatchDesc& bd, const CompactJob& job, const int32_t* kept_idx,
                            int32_t chunk_rows, int32_t chunk_row0, const int32_t* out_offsets,
                            int32_t chunk_first, int32_t batch_total, cudaStream_t stream)

@@ -631,14 +631,19 @@ int max_tiles(const BatchDesc& bd)
 
 template <bool ROOM>
 cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUtensorMap* tk, StreamArgs& a, int cluster,
-                            int sms, size_t smem, cudaStream_t stream)
+                            size_t smem, cudaStream_t stream)
 {
     auto kern = salience_stream_kernel<ROOM>;
     static KernelSetup ks;
-    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kStreamThreads, smem, kTmemColsPerSm);
+    cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kStreamThreads, smem, kTmemColsPerSm);
     if (e != cudaSuccess) return e;
+    // a second wave of a persistent grid would double its time
+    int n = 0;
+    e = clusters_at_once(ks, reinterpret_cast<const void*>(kern), kStreamThreads, smem, cluster, &n);
+    if (e != cudaSuccess) return e;
+    if (n < 1) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(sms / cluster * cluster));
+    cfg.gridDim = dim3(static_cast<unsigned>(std::min(a.n_jobs, n) * cluster));
     cfg.blockDim = dim3(kStreamThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -650,20 +655,6 @@ cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUte
     attr[1] = pdl_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    // Clusters that run at once: fewer than multiprocessors / cluster size (a cluster lies inside a GPC: 33 of 4, 15 of 8
-    // on a B200), and a second wave of a persistent grid would double its time.  The shared-memory footprint is the same
-    // for every launch, so the answer is looked up once per size.
-    static std::atomic<int> fits[kMaxCluster + 1];
-    int n = fits[cluster].load(std::memory_order_relaxed);
-    if (n == 0) {
-        cfg.numAttrs = 1;
-        const cudaError_t eo = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-        if (eo != cudaSuccess) return eo;
-        if (n < 1) return cudaErrorInvalidConfiguration;
-        fits[cluster].store(n, std::memory_order_relaxed);
-        cfg.numAttrs = 2;
-    }
-    cfg.gridDim = dim3(static_cast<unsigned>(std::min(a.n_jobs, n) * cluster));
     return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, a);
 }
 
@@ -696,8 +687,8 @@ cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_grou
     const size_t q_bytes = 2 * static_cast<size_t>((head_dim * esize + 127) / 128) * npad * 128;
     a.stages = static_cast<int>(std::min<size_t>(kMaxStages, (kStreamSmem - 1024 - q_bytes) / kStageBytes));
     if (a.stages < 4) return cudaErrorInvalidConfiguration;
-    if (norms_beside && !alpha.ptr) return launch_stream<true>(bd, tmap_q, tmap_k, a, cluster, sms, kStreamSmem, stream);
-    return launch_stream<false>(bd, tmap_q, tmap_k, a, cluster, sms, kStreamSmem, stream);
+    if (norms_beside && !alpha.ptr) return launch_stream<true>(bd, tmap_q, tmap_k, a, cluster, kStreamSmem, stream);
+    return launch_stream<false>(bd, tmap_q, tmap_k, a, cluster, kStreamSmem, stream);
 }
 
 }  // namespace mvla
