@@ -126,12 +126,11 @@ int sm_count_of_current_device();
 // small step would see.  One object per kernel instantiation; host threads may share it.
 struct KernelSetup {
     std::atomic<int> smem_set[64];       // dynamic shared memory the kernel may use (the largest asked for so far)
-    std::atomic<int> smem_checked[64];   // dynamic shared memory whose occupancy was last checked, + 1
     ResidentClusters clusters;
 };
-// Lets `kern` use `smem` bytes of dynamic shared memory and, with `tmem_cols` > 0, makes sure that the CTAs of
-// `threads` threads that fit on a multiprocessor cannot ask for more tensor memory than it has.
-cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t smem, int tmem_cols);
+// Lets `kern` use `smem` bytes of dynamic shared memory and refuses a size with which the CTAs that fit on a
+// multiprocessor could ask for more than its tensor memory at `tmem_cols` columns each (tmem_plan.h).
+cudaError_t setup_kernel(KernelSetup& ks, const void* kern, size_t smem, int tmem_cols);
 // Clusters of `cluster` CTAs that run at once on the current device (setup_kernel comes first).  Fewer than
 // multiprocessors x CTAs / cluster size: a cluster lies inside a GPC (with one CTA per multiprocessor 33 of 4, 15 of 8 on a
 // B200).

@@ -99,8 +99,9 @@ int sm_count_of_current_device()
     return cached[dev];
 }
 
-cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t smem, int tmem_cols)
+cudaError_t setup_kernel(KernelSetup& ks, const void* kern, size_t smem, int tmem_cols)
 {
+    if (!tmem_columns_fit(smem, tmem_cols)) return cudaErrorInvalidConfiguration;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -112,13 +113,6 @@ cudaError_t setup_kernel(KernelSetup& ks, const void* kern, int threads, size_t 
         if (!known || ks.smem_set[dev].load(std::memory_order_relaxed) < bytes) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess) return e;
         if (known && ks.smem_set[dev].load(std::memory_order_relaxed) < bytes) ks.smem_set[dev].store(bytes, std::memory_order_release);
-    }
-    if (tmem_cols > 0 && !(known && ks.smem_checked[dev].load(std::memory_order_relaxed) == bytes + 1)) {
-        int resident = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, threads, smem);
-        if (e != cudaSuccess) return e;
-        if (resident * tmem_cols > kTmemColsPerSm) return cudaErrorInvalidConfiguration;
-        if (known) ks.smem_checked[dev].store(bytes + 1, std::memory_order_relaxed);
     }
     return cudaSuccess;
 }

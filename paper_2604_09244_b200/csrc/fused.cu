@@ -604,7 +604,7 @@ cudaError_t launch_fast_t(const BD& bd, int n_heads, int kv_group, int head_dim,
     smem = smem_for_tmem(smem, tmem_cols);
     if (smem == 0) return cudaErrorInvalidConfiguration;
     static KernelSetup ks;
-    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kFastThreads * SPLIT, smem, tmem_cols);
+    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), smem, tmem_cols);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster, n_heads, bd.n);
@@ -629,7 +629,7 @@ cudaError_t launch_f32_t(const BD& bd, int n_heads, int kv_group, int head_dim, 
     const size_t smem = 1024 + static_cast<size_t>(head_dim / 32) * (NTILE * 16384 + npad * 128);
     auto kern = salience_f32_kernel<TCOL, NTILE, BD>;
     static KernelSetup ks;
-    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kFastThreads * 2, smem, 0);
+    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), smem, 0);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster, n_heads, bd.n);

@@ -383,7 +383,7 @@ cudaError_t launch_salience_t(const BatchDesc& bd, int n_heads, int kv_group, in
         if (smem == 0) return cudaErrorInvalidConfiguration;
     }
     static KernelSetup ks;
-    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kThreads, smem, tmem_cols);
+    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), smem, tmem_cols);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster, n_heads, bd.n);

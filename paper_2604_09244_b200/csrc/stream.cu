@@ -635,7 +635,7 @@ cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUte
 {
     auto kern = salience_stream_kernel<ROOM>;
     static KernelSetup ks;
-    cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), kStreamThreads, smem, kTmemColsPerSm);
+    cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), smem, kTmemColsPerSm);
     if (e != cudaSuccess) return e;
     // a second wave of a persistent grid would double its time
     int n = 0;

@@ -7,8 +7,9 @@
 // blocked in the allocation behind CTA B, which waits for its peer B', blocked in the allocation on SM X
 // behind A.  No bounded mbarrier wait can break it.  So the launchers make sure that
 //     resident CTAs per multiprocessor x columns per CTA <= 512
-// by asking for enough dynamic shared memory that no more CTAs than that fit, and check the result with the
-// occupancy calculator before every launch configuration is used.
+// by asking for enough dynamic shared memory that no more CTAs than that fit.  (The runtime's occupancy calculator is no
+// check of this: it answers one CTA per multiprocessor for every kernel that allocates tensor memory, where three of the
+// scoring kernel's do run side by side.)
 #pragma once
 
 #include <stddef.h>
@@ -45,6 +46,12 @@ inline size_t smem_for_tmem(size_t dyn_smem, int tmem_cols)
     const size_t footprint = kSmemPerSm / (max_ctas + 1) + 1;      // (max_ctas + 1) of these do not fit
     const size_t padded = footprint - kSmemReservedPerCta;
     return padded <= static_cast<size_t>(kSmemMaxPerCta) ? padded : 0;
+}
+
+// Whether the CTAs that fit cannot ask for more columns than there are (`tmem_cols` each; 0: no tensor memory).
+inline bool tmem_columns_fit(size_t dyn_smem, int tmem_cols)
+{
+    return tmem_cols <= kTmemColsPerSm && (tmem_cols <= 0 || ctas_by_smem(dyn_smem) <= kTmemColsPerSm / tmem_cols);
 }
 
 // Dynamic shared memory of the streaming scoring kernel, which takes all 512 columns: with the kernel's static

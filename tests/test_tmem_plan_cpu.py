@@ -26,6 +26,8 @@ int main()
                     const size_t got = smem_for_tmem(dyn, cols);
                     if (got == 0 || got < dyn || got > static_cast<size_t>(kSmemMaxPerCta)) { std::printf("bad size %zu\n", got); return 1; }
                     if (ctas_by_smem(got) * cols > kTmemColsPerSm) { std::printf("over-subscribed\n"); return 1; }
+                    // what every launcher is checked by accepts this size, and the unpadded one only where it needed none
+                    if (!tmem_columns_fit(got, cols) || tmem_columns_fit(dyn, cols) != (got == dyn)) { std::printf("not told apart\n"); return 1; }
                     // the padding is the smallest that works: one CTA fewer would still have fitted the columns
                     if (got > dyn && (ctas_by_smem(got) + 1) * cols <= kTmemColsPerSm) { std::printf("padded too far\n"); return 1; }
                     padded += got > dyn;
@@ -34,7 +36,8 @@ int main()
     // the shape the advisory named: 128-byte key rows, 3 tiles, more than 32 queries -> 256 columns, 65 KB
     if (ctas_by_smem(smem_for_tmem(1024 + 1 * (3 * 16384 + 64 * 128), tmem_cols_for(3 * 64))) * 256 > 512) return 1;
     if (tmem_cols_for(1) != 32 || tmem_cols_for(33) != 64 || tmem_cols_for(512) != 512) return 1;
-    if (smem_for_tmem(40000, 1024) != 0) return 1;
+    if (smem_for_tmem(40000, 1024) != 0 || tmem_columns_fit(40000, 1024)) return 1;
+    if (!tmem_columns_fit(0, 0) || !tmem_columns_fit(kStreamSmem, 512) || tmem_columns_fit(kSmemPerSm / 2 - kSmemReservedPerCta, 512)) return 1;
     std::printf("%d %d\n", checked, padded);
     return 0;
 }
