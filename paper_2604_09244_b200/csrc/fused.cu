@@ -89,10 +89,12 @@ struct FastOut {
 // overflowing, and the two shared-memory round trips, two block barriers and the butterfly that found the maximum leave
 // the chain (a warp whose exponents exceed kRescaleAt takes its true maxima after all).  The pairs (reference, sum) of
 // the four warps are combined per query, then those of the cluster's CTAs.
-template <int TCOL, int NTILE, int SPLIT, bool ALPHA>
+//
+// `before_exchange` runs when every warp has its logits in registers and before anything waits for another CTA.
+template <int TCOL, int NTILE, int SPLIT, bool ALPHA, class Hook>
 __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT], const SampleDev& s, const int (&valid)[NTILE],
                                                const int (&vis0)[NTILE], bool ok, int npad, int h, float cscale, uint32_t bar_x,
-                                               FastSmem& sm, const FastOut& o)
+                                               FastSmem& sm, const FastOut& o, Hook before_exchange)
 {
     constexpr int TC = TCOL / SPLIT;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -177,6 +179,7 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
         if ((lane & 1) == 0) sm.w[kwarp][c0 + qc * 16 + col16(lane)] = red;
     }
     __syncthreads();
+    before_exchange();
 
     // ---- one thread per query: the pairs of the CTA's warps, exchanged with the other key tiles of this (sample, head)
     cluster_wait_acquire();                   // every peer is running and has initialised its barriers
@@ -317,9 +320,11 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
     cluster_arrive_release();                 // publishes this CTA's barriers; matched by the wait before the first remote store
     uint32_t tmem_cols = 32;
     while (tmem_cols < static_cast<uint32_t>(CC)) tmem_cols <<= 1;
-    // blocks until the columns are free: the launcher has made sure that the CTAs resident on a multiprocessor
-    // never ask for more than its 512 columns together, so no CTA waits here for one that waits for it
-    if (warp == 1) tmem_alloc(smem_u32(&s_tmem), tmem_cols);
+    // Blocks until the columns are free.  Whoever holds some on this multiprocessor gives them back without waiting for
+    // another CTA: this kernel before its exchange (below), the streaming kernel is never beside it, and the CTAs of the
+    // generic kernel that fit beside one another never ask for more than there is (tmem_plan.h).  (Warp 3: it has no part
+    // in the exchange.)
+    if (warp == 3) tmem_alloc(smem_u32(&s_tmem), tmem_cols);
     // One CTA per sample re-arms the words through which the kernel after this one hands the kept list from
     // its selecting CTA to its copying CTAs (-1: not yet known).  Their last users finished long ago.
     if (rearm && blockIdx.x == 0 && blockIdx.y == 0) {
@@ -456,15 +461,20 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
             }
         }
     }
-    softmax_scores<TCOL, NTILE, SPLIT, KIND == kForPatches>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
-                                       FastOut{acc64, status, n_heads, alpha});
-
     tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, tmem_cols);    // the warp that allocated
-    if (stamps && tid == 0) {
-        const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-        if (cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
+    softmax_scores<TCOL, NTILE, SPLIT, KIND == kForPatches>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
+                                       FastOut{acc64, status, n_heads, alpha}, [&]() {
+        if (warp == 3) {
+            tc_fence_after();
+            tmem_dealloc(tmem_base, tmem_cols);
+        }
+    });
+    if (stamps) {
+        __syncthreads();
+        if (tid == 0) {
+            const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+            if (cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
+        }
     }
 }
 
@@ -581,7 +591,7 @@ salience_f32_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUten
         }
     }
     softmax_scores<TCOL, NTILE, 2, false>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
-                                   FastOut{acc64, status, n_heads, AlphaOut{nullptr, 0, 0}});
+                                   FastOut{acc64, status, n_heads, AlphaOut{nullptr, 0, 0}}, []() {});
     if (stamps) {
         __syncthreads();
         if (tid == 0) {

@@ -1,7 +1,7 @@
 // Host arithmetic that keeps tensor memory from deadlocking the scoring kernels.
 //
 // A multiprocessor has 512 columns of tensor memory.  tcgen05.alloc blocks until its columns are free, and
-// the scoring kernels hold their columns while they wait for the other CTAs of their cluster.  If the CTAs
+// the generic scoring kernel holds its columns while it waits for the other CTAs of its cluster.  If the CTAs
 // that fit on a multiprocessor by registers, threads and shared memory could together ask for more than
 // 512 columns, this cycle is possible: CTA A holds columns on SM X and waits for its peer A' on SM Y; A' is
 // blocked in the allocation behind CTA B, which waits for its peer B', blocked in the allocation on SM X
@@ -10,6 +10,9 @@
 // by asking for enough dynamic shared memory that no more CTAs than that fit.  (The runtime's occupancy calculator is no
 // check of this: it answers one CTA per multiprocessor for every kernel that allocates tensor memory, where three of the
 // scoring kernel's do run side by side.)
+// That bounds the CTAs of one launch.  Launches of other shapes, streams or contexts may share the multiprocessor, with
+// other columns per byte of shared memory: so the latency-shaped kernel gives its columns back before it waits for its
+// cluster, and the streaming kernel (below) leaves no room for any other holder.
 #pragma once
 
 #include <stddef.h>
