@@ -345,14 +345,29 @@ void clear_accumulators(unsigned long long* acc64, const BatchDesc& bd, cudaStre
 }
 
 // Which of the two tensor-core scoring kernels.  The latency-shaped one of fused.cu covers up to 16 key tiles a sample
-// and is the faster one while its CTAs all run at once (three with one key tile to a multiprocessor, two with two tiles);
-// from the second wave on the streaming one is (stream.cu).  Measured at 32 heads, 256 + 512 tokens, whole step in us,
-// latency-shaped / streaming: 2 samples 16.1 / 17.1, 3 samples (576 CTAs) 22.0 / 20.8, 4 samples 27.5 / 23.9, 16
-// samples 120 / 97; 768 + 1023 tokens: 1 sample (224 CTAs) 18.5 / 20.9, 2 samples 33.9 / 30.8.
-bool stream_pays(const mvla_ctx* ctx, const BatchDesc& bd, int tiles_per_cta, int cluster)
+// and is the faster one while its CTAs all run at once; from the second wave on the streaming one is (stream.cu).  What runs
+// at once goes by shared memory, and is counted as no more than three CTAs to a multiprocessor with one key tile and two with
+// two (with short rows more fit, and share its time).  Measured on whole steps in us, latency-shaped / streaming:
+//   heads of 128, 256 + 512 tokens: 2 samples of 32 heads 16.1 / 17.1, 3 samples (576 CTAs) 22.0 / 20.8, 4 samples
+//     27.5 / 23.9, 16 samples 120 / 97; 768 + 1023 tokens: 1 sample (224 CTAs of two tiles) 18.5 / 20.9, 2 samples 33.9 / 30.8;
+//   16 heads of 256, of which two CTAs of one tile fit, or one of two tiles; fixed budgets: 320 CTAs 30.8 / 26.5, 336
+//     25.4 / 23.0, 384 26.7 / 26.4; 768 + 768 tokens (16 clusters of 6, 22 at once) 17.5 / 22.7, 768 + 1023 (16 of 7, 15 at
+//     once) 26.0 / 24.0, 2 samples of 640 + 512 (32 of 5, 26 at once) 29.1 / 26.3, 3 samples 25.7 / 25.2.
+// With the feature norms beside the scores two tiles a CTA behave the same (28.2 / 25.5 for 768 + 1023, 43.1 / 32.9 for two
+// samples; 32.8 / 34.2 for three of 640 + 512), one tile does not: batches of small samples leave the norms behind the streaming
+// kernel instead of beside it (384 CTAs: 4 samples 30.0 / 28.7, 12 samples 29.5 / 33.3).  There the line stays at three CTAs.
+cudaError_t stream_pays(const mvla_ctx* ctx, const BatchDesc& bd, int tiles_per_cta, int cluster, int npad, bool for_patches,
+                        bool norms_beside, bool* pays)
 {
-    return !fast_salience_supported(tiles_per_cta) ||
-           bd.n * ctx->cfg.n_heads * cluster > ctx->sm_count * (tiles_per_cta == 1 ? 3 : 2);
+    const int clusters = bd.n * ctx->cfg.n_heads, ctas = clusters * cluster, cap = tiles_per_cta == 1 ? 3 : 2;
+    *pays = !fast_salience_supported(tiles_per_cta) || ctas > ctx->sm_count * cap;
+    // (two CTAs of one tile always fit: 106 KB each with 64 queries of the longest rows)
+    if (*pays || (tiles_per_cta == 1 && (norms_beside || ctas <= ctx->sm_count * 2))) return cudaSuccess;
+    int per_sm = 0, at_once = 0;
+    const cudaError_t e = fast_salience_residency(bd, ctx->cfg.head_dim, static_cast<int>(ctx->qk_elem), tiles_per_cta, cluster, npad,
+                                                  for_patches, &per_sm, &at_once);
+    *pays = per_sm > 1 ? ctas > ctx->sm_count * std::min(per_sm, cap) : clusters > at_once;
+    return e;
 }
 
 // Salience of one chunk (+ L1 norms into `l1` when asked; + the scores as fp32 into `attn_out` when asked).  The per-head contributions land in
@@ -387,7 +402,11 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
         if (r != MVLA_OK) return r;
     }
     cudaError_t e;
-    const bool streaming = ctx->use_umma && (acc64 || alpha.ptr) && !with_cache && stream_pays(ctx, bd, tiles_per_cta, cluster);
+    bool streaming = false;
+    if (ctx->use_umma && (acc64 || alpha.ptr) && !with_cache) {
+        e = stream_pays(ctx, bd, tiles_per_cta, cluster, npad, alpha.ptr != nullptr, norms_beside && hidden && l1, &streaming);
+        if (e != cudaSuccess) return e == cudaErrorInvalidConfiguration ? MVLA_ERR_UNSUPPORTED : fail_cuda(ctx, e);
+    }
     const bool fast = streaming || f32 || (ctx->use_umma && fast_salience_supported(tiles_per_cta));
     // The norms do not depend on the scores: with `norms_beside` (fast kernel only) they are launched AFTER
     // the scoring kernel and run beside it instead of in front of it.

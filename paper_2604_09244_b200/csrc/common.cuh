@@ -131,9 +131,9 @@ struct KernelSetup {
 // Lets `kern` use `smem` bytes of dynamic shared memory and refuses a size with which the CTAs that fit on a
 // multiprocessor could ask for more than its tensor memory at `tmem_cols` columns each (tmem_plan.h).
 cudaError_t setup_kernel(KernelSetup& ks, const void* kern, size_t smem, int tmem_cols);
-// Clusters of `cluster` CTAs that run at once on the current device (setup_kernel comes first).  Fewer than
-// multiprocessors x CTAs / cluster size: a cluster lies inside a GPC (with one CTA per multiprocessor 33 of 4, 15 of 8 on a
-// B200).
+// Clusters of `cluster` CTAs that run at once on the current device (setup_kernel comes first), for a kernel with tensor
+// memory of which one CTA fits on a multiprocessor.  Fewer than multiprocessors / cluster size: a cluster lies inside a GPC (33
+// of 4, 15 of 8 on a B200).  (Where two CTAs fit the runtime's answer is the same, and too small: 32 of 8 do run at once.)
 cudaError_t clusters_at_once(KernelSetup& ks, const void* kern, int threads, size_t smem, int cluster, int* count);
 
 // ---- launchers (each enqueues on `stream` and returns the launch status) ----
@@ -168,6 +168,11 @@ cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group,
                                  unsigned long long* acc64, int* status,
                                  AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                                  float* lcache, int cache_vis, int cache_cols, cudaStream_t stream);
+
+// Of such a launch without the logit cache: CTAs that fit on a multiprocessor, and, where that is one, clusters (one per
+// sample and head) that run at once on the device.
+cudaError_t fast_salience_residency(const BatchDesc& bd, int head_dim, int esize, int tiles_per_cta, int cluster, int npad,
+                                    bool for_patches, int* per_sm, int* clusters);
 
 // The same scores into the same fixed-point accumulators from fp32 q / k (plain FMAs), where the shape fits.
 bool f32_salience_supported(int tiles_per_cta, int npad, int head_dim);

@@ -73,6 +73,7 @@ struct FastSmem {
     alignas(16) float w[4][kMaxText];        // sum of the exponentials, then their weight in the scores
     float2 peer[kMaxCluster][kMaxText];      // (reference, sum) of every CTA of the cluster
 };
+constexpr size_t kFastStaticSmem = sizeof(FastSmem) + 32;   // of salience_fast_kernel: + its barriers and a tensor-memory address
 // What the softmax part writes.
 struct FastOut {
     unsigned long long* acc64;               // null: the attention copy only
@@ -601,24 +602,39 @@ salience_f32_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUten
     }
 }
 
+// One variant of the kernel with the set-up that goes with it.
 template <int TCOL, int NTILE, int SPLIT, int KIND, class BD>
+struct FastVariant {
+    static constexpr int kThreads = kFastThreads * SPLIT;
+    static constexpr auto kern = salience_fast_kernel<TCOL, NTILE, SPLIT, KIND, BD>;
+    static const void* address() { return reinterpret_cast<const void*>(kern); }
+    static KernelSetup& setup()
+    {
+        static KernelSetup ks;
+        return ks;
+    }
+    // dynamic shared memory of a launch, with the kernel ready for it
+    static cudaError_t prepare(int head_dim, int esize, int npad, size_t* smem)
+    {
+        // resident CTAs x tensor-memory columns must not exceed the 512 of a multiprocessor
+        const int tmem_cols = tmem_cols_for(TCOL * NTILE);
+        *smem = smem_for_tmem(1024 + static_cast<size_t>((head_dim * esize + 127) / 128) * (static_cast<size_t>(NTILE) * 16384 + npad * 128), tmem_cols);
+        return *smem == 0 ? cudaErrorInvalidConfiguration : setup_kernel(setup(), address(), *smem, tmem_cols);
+    }
+};
+
+template <class V, class BD>
 cudaError_t launch_fast_t(const BD& bd, int n_heads, int kv_group, int head_dim, int esize, const CUtensorMap* tq,
                           const CUtensorMap* tk, int cluster, int npad,
                           unsigned long long* acc64, int* status, AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                           float* lcache, int cache_vis, int cache_cols, cudaStream_t stream)
 {
-    size_t smem = 1024 + static_cast<size_t>((head_dim * esize + 127) / 128) * (static_cast<size_t>(NTILE) * 16384 + npad * 128);
-    auto kern = salience_fast_kernel<TCOL, NTILE, SPLIT, KIND, BD>;
-    // resident CTAs x tensor-memory columns must not exceed the 512 of a multiprocessor
-    const int tmem_cols = tmem_cols_for(TCOL * NTILE);
-    smem = smem_for_tmem(smem, tmem_cols);
-    if (smem == 0) return cudaErrorInvalidConfiguration;
-    static KernelSetup ks;
-    const cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), smem, tmem_cols);
+    size_t smem = 0;
+    const cudaError_t e = V::prepare(head_dim, esize, npad, &smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster, n_heads, bd.n);
-    cfg.blockDim = dim3(kFastThreads * SPLIT);
+    cfg.blockDim = dim3(V::kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -629,7 +645,23 @@ cudaError_t launch_fast_t(const BD& bd, int n_heads, int kv_group, int head_dim,
     attr[1] = pdl_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, n_heads, kv_group, head_dim, esize, npad, acc64, status, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols);
+    return cudaLaunchKernelEx(&cfg, V::kern, bd, *tq, *tk, n_heads, kv_group, head_dim, esize, npad, acc64, status, alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols);
+}
+
+// use(variant, descriptors) with the variant that scores a launch
+template <class F>
+cudaError_t with_fast_variant(const BatchDesc& bd, int npad, int tiles_per_cta, int kind, F use)
+{
+    const int tcol = npad <= 16 ? 16 : (npad <= 32 ? 32 : 64);
+    const int split = tcol >= 32 ? 2 : 1;     // two threads per key while a thread still holds 16 queries
+#define MVLA_FAST1(TC, NTL, SP, KD)                                                                             \
+    if (tcol == TC && tiles_per_cta == NTL && split == SP && kind == KD)                                        \
+        return with_desc(bd, [&](const auto& d) { return use(FastVariant<TC, NTL, SP, KD, std::decay_t<decltype(d)>>{}, d); });
+#define MVLA_FAST(TC, NTL, SP) MVLA_FAST1(TC, NTL, SP, kPlain) MVLA_FAST1(TC, NTL, SP, kWithCache) MVLA_FAST1(TC, NTL, SP, kForPatches)
+    MVLA_FAST(16, 1, 1) MVLA_FAST(16, 2, 1) MVLA_FAST(32, 1, 2) MVLA_FAST(64, 1, 2) MVLA_FAST(32, 2, 2) MVLA_FAST(64, 2, 2)
+#undef MVLA_FAST1
+#undef MVLA_FAST
+    return cudaErrorInvalidConfiguration;
 }
 
 template <int TCOL, int NTILE, class BD>
@@ -688,20 +720,24 @@ cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group,
                                  AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
                                  float* lcache, int cache_vis, int cache_cols, cudaStream_t stream)
 {
-    const int tcol = npad <= 16 ? 16 : (npad <= 32 ? 32 : 64);
-    const int split = tcol >= 32 ? 2 : 1;     // two threads per key while a thread still holds 16 queries
     if ((acc64 == nullptr) == (alpha.ptr == nullptr)) return cudaErrorInvalidConfiguration;      // one or the other
-    const int kind = alpha.ptr ? kForPatches : (lcache ? kWithCache : kPlain);
-#define MVLA_FAST1(TC, NTL, SP, KD)                                                                             \
-    if (tcol == TC && tiles_per_cta == NTL && split == SP && kind == KD)                                        \
-        return with_desc(bd, [&](const auto& d) {                                                               \
-            return launch_fast_t<TC, NTL, SP, KD>(d, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, acc64, status, \
-                                                  alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream); });
-#define MVLA_FAST(TC, NTL, SP) MVLA_FAST1(TC, NTL, SP, kPlain) MVLA_FAST1(TC, NTL, SP, kWithCache) MVLA_FAST1(TC, NTL, SP, kForPatches)
-    MVLA_FAST(16, 1, 1) MVLA_FAST(16, 2, 1) MVLA_FAST(32, 1, 2) MVLA_FAST(64, 1, 2) MVLA_FAST(32, 2, 2) MVLA_FAST(64, 2, 2)
-#undef MVLA_FAST1
-#undef MVLA_FAST
-    return cudaErrorInvalidConfiguration;
+    return with_fast_variant(bd, npad, tiles_per_cta, alpha.ptr ? kForPatches : (lcache ? kWithCache : kPlain), [&](auto v, const auto& d) {
+        return launch_fast_t<decltype(v)>(d, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, acc64, status,
+                                          alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream);
+    });
+}
+
+cudaError_t fast_salience_residency(const BatchDesc& bd, int head_dim, int esize, int tiles_per_cta, int cluster, int npad,
+                                    bool for_patches, int* per_sm, int* clusters)
+{
+    return with_fast_variant(bd, npad, tiles_per_cta, for_patches ? kForPatches : kPlain, [&](auto v, const auto&) {
+        using V = decltype(v);
+        size_t smem = 0;
+        const cudaError_t e = V::prepare(head_dim, esize, npad, &smem);
+        if (e != cudaSuccess) return e;
+        *per_sm = ctas_by_smem(smem + kFastStaticSmem);      // (registers allow two CTAs of two tiles and three of one)
+        return *per_sm > 1 ? cudaSuccess : clusters_at_once(V::setup(), V::address(), V::kThreads, smem, cluster, clusters);
+    });
 }
 
 }  // namespace mvla

@@ -821,6 +821,31 @@ def test_streaming_scoring_kernel_without_norms_beside_it(batch, H, n_txt, n_2d,
     ctx.close()
 
 
+@pytest.mark.parametrize("batch,d,n_txt,n_2d,n_3d,mode,at_once", [
+    (1, 256, 20, 768, 768, W.MODE_ADAPTIVE, True),        # 16 clusters of 6 CTAs with two tiles, one CTA to a multiprocessor
+    (1, 256, 20, 768, 1023, W.MODE_ADAPTIVE, False),      # 16 of 7: one more than lie inside the device's GPCs
+    (1, 128, 64, 768, 1023, W.MODE_ADAPTIVE, True),       # rows half as long: two CTAs fit
+    (1, 160, 64, 1023, 1000, W.MODE_ADAPTIVE, False),     # 16 of 8, rows of one and a quarter boxes
+    (2, 256, 7, 640, 512, W.MODE_FIXED, False),           # 32 of 5
+    (4, 256, 33, 256, 512, W.MODE_FIXED, False),          # 384 CTAs of one tile, two fit: 296 at once
+    (4, 256, 33, 256, 512, W.MODE_ADAPTIVE, True),        # ... with norms beside the scores the line is three to a multiprocessor
+    (4, 128, 33, 256, 512, W.MODE_FIXED, True),           # ... and three fit
+])
+def test_scoring_kernel_goes_by_what_fits_on_the_device(batch, d, n_txt, n_2d, n_3d, mode, at_once):
+    """16 heads on both sides of the line between the two scoring kernels, told apart by how many CTAs leave time stamps:
+    the latency-shaped kernel has one per one or two key tiles."""
+    wl = W.small_workload(74, batch=batch, D=128, H=16, d=d, n_txt=(n_txt,), n_2d=(n_2d,), n_3d=(n_3d,), keep=(0.3,), mode=mode, steps=2)
+    ctx, states = mvla.context_for(wl), [oracle.State(s.n_vis) for s in wl.samples]
+    tiles = -(-n_2d // 128) + -(-n_3d // 128)
+    ctas = batch * 16 * -(-tiles // -(-tiles // 8))
+    for step in range(2):
+        stamps = torch.zeros(2, ctx.STAMP_SLOTS, 2, dtype=torch.int64, device="cuda")
+        ctx.set_kernel_stamps(stamps)
+        run_and_check_step(ctx, wl, step, states)
+        assert (int((stamps[0, :, 1] != 0).sum()) == ctas) == at_once
+    ctx.close()
+
+
 @pytest.mark.parametrize("gain", [30.0, 300.0])
 def test_streaming_scoring_kernel_moves_its_references_when_exponents_would_overflow(gain):
     """Keys whose logits grow from tile to tile by far more than an fp32 exponent holds."""
