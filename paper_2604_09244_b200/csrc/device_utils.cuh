@@ -70,22 +70,59 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// Bounded wait: gives up after about one second and reports false.  (No suspend-time hint on the try: with
-// one it was measured to notice the completed phase about a microsecond late.)
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
-    const uint64_t t0 = global_ns();
-    for (uint32_t it = 0; it < kSpinLimit; ++it) {
-        uint32_t ok;
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// Whether the phase of this parity is complete.  CLUSTER: with acquire at cluster scope (arrivals and data come from other
+// CTAs).  (No suspend-time hint: with one it was measured to notice the completed phase about a microsecond late.)
+template <bool CLUSTER>
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    if constexpr (CLUSTER)
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    else
         asm volatile("{\n\t.reg .pred p;\n\t"
                      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (ok) return true;
+    return ok != 0;
+}
+// Bounded wait: gives up after about one second and reports false.
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
+{
+    const uint64_t t0 = global_ns();
+    for (uint32_t it = 0; it < kSpinLimit; ++it) {
+        if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
         if ((it & 63u) == 63u && global_ns() - t0 > 1000000000ull) break;
     }
     return false;
 }
+// Asynchronous 8-byte store into the shared memory of CTA `rank` (same offset as `local_addr`); on
+// landing it credits 8 bytes to that CTA's mbarrier at the offset of `local_bar`: the data and its
+// "ready" signal travel together, one way.
+__device__ __forceinline__ void st_async_pair(uint32_t local_addr, uint32_t local_bar, uint32_t rank, float2 v)
+{
+    uint32_t raddr, rbar;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(raddr) : "r"(local_addr), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbar) : "r"(local_bar), "r"(rank));
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
+                 ::"r"(raddr), "f"(v.x), "f"(v.y), "r"(rbar) : "memory");
+}
+// 2^x in one instruction.
+__device__ __forceinline__ float ex2_approx(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// Exponents are taken against a reference that need not be the maximum; one (log2) above this moves the warp's reference.
+constexpr float kRescaleAt = 64.f;
 // One box of a 3-D tiled tensor map -> this CTA's shared memory; completion counted on `bar`.
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z,
                                             uint32_t bar)

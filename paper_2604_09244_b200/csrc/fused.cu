@@ -32,40 +32,6 @@ namespace mvla {
 namespace {
 
 constexpr int kFastThreads = 128;
-constexpr float kRescaleAt = 64.f;       // exponents (log2) above this: the warp's reference becomes its maximum
-
-__device__ __forceinline__ float ex2_approx(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-// Asynchronous 8-byte store into the shared memory of CTA `rank` (same offset as `local_addr`); on
-// landing it credits 8 bytes to that CTA's mbarrier at the offset of `local_bar`: the data and its
-// "ready" signal travel together, one way.
-__device__ __forceinline__ void st_async_peer_f32x2(uint32_t local_addr, uint32_t local_bar, uint32_t rank, float2 v)
-{
-    uint32_t raddr, rbar;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(raddr) : "r"(local_addr), "r"(rank));
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbar) : "r"(local_bar), "r"(rank));
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
-                 ::"r"(raddr), "f"(v.x), "f"(v.y), "r"(rbar) : "memory");
-}
-// Bounded wait with acquire at cluster scope (the arrivals come from other CTAs).
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
-{
-    const uint64_t t0 = global_ns();
-    for (uint32_t it = 0; it < kSpinLimit; ++it) {
-        uint32_t ok;
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (ok) return true;
-        if ((it & 63u) == 63u && global_ns() - t0 > 1000000000ull) break;
-    }
-    return false;
-}
 
 // Shared memory of the softmax part, per warp of the four that cover a tile's 128 keys, and per query.
 struct FastSmem {
@@ -194,9 +160,9 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (ref[k] > -CUDART_INF_F) z += sm.w[k][tid] * ex2_approx(ref[k] - mx);
-        for (uint32_t r = 0; r < csize; ++r) st_async_peer_f32x2(smem_u32(&sm.peer[crank][tid]), bar_x, r, make_float2(mx, z));
+        for (uint32_t r = 0; r < csize; ++r) st_async_pair(smem_u32(&sm.peer[crank][tid]), bar_x, r, make_float2(mx, z));
         const float inv_hn = 1.f / (static_cast<float>(o.n_heads) * static_cast<float>(s.n_txt));
-        const bool okx = mbar_wait_cluster(bar_x, 0);
+        const bool okx = mbar_wait<true>(bar_x, 0);
         if (!okx) *reinterpret_cast<volatile int*>(o.status) = MVLA_ERR_TIMEOUT;
         mx = -CUDART_INF_F;
         for (uint32_t r = 0; r < csize; ++r) mx = fmaxf(mx, sm.peer[r][tid].x);

@@ -33,7 +33,6 @@ constexpr int kSoftThreads = kSoftWarps * 32;
 constexpr int kStreamThreads = kSoftThreads + 64;     // + the loading warp and the MMA warp
 constexpr int kMaxStages = 12;
 constexpr uint32_t kStageBytes = 16384;               // 128 keys x 128 bytes: one swizzled box of a key tile
-constexpr float kRescaleAt = 64.f;                    // exponents (log2) above this move a warp's reference
 constexpr int kMaxSlots = 32;
 // Pairs of job n go to buffer n mod 2: a CTA sends those of job n + 2 only after it has the pairs of job n + 1 of every
 // peer, which that peer sent when it was done with job n's.
@@ -71,14 +70,7 @@ __device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatil
 {
     uint64_t t0 = 0;
     for (uint32_t it = 0; it < kSpinLimit; ++it) {
-        uint32_t ok;
-        if constexpr (CLUSTER)
-            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-                         "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        else
-            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                         "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (ok) return true;
+        if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
         if ((it & 63u) == 63u) {
             if (*aborted) return false;
             const uint64_t now = global_ns();
@@ -90,18 +82,8 @@ __device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatil
     *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
     return false;
 }
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 // Barrier of the softmax warps.
 __device__ __forceinline__ void soft_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kSoftThreads) : "memory"); }
-__device__ __forceinline__ float fast_ex2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
@@ -112,14 +94,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
                    "r"(__float_as_uint(v[15])) : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void st_async_pair(uint32_t local_addr, uint32_t local_bar, uint32_t rank, float2 v)
-{
-    uint32_t raddr, rbar;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(raddr) : "r"(local_addr), "r"(rank));
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbar) : "r"(local_bar), "r"(rank));
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
-                 ::"r"(raddr), "f"(v.x), "f"(v.y), "r"(rbar) : "memory");
-}
 
 // Two fp32 operations per instruction.
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
@@ -217,7 +191,7 @@ __device__ __noinline__ void raise_references(uint32_t cols_t, uint32_t lane_bas
         const int col = c * 16 + col16(lane);
         const float old = -nm[col], now = fmaxf(old, red);
         __syncwarp();
-        if ((lane & 1) == 0) { nm[col] = -now; w[col] = fast_ex2(old - now); }
+        if ((lane & 1) == 0) { nm[col] = -now; w[col] = ex2_approx(old - now); }
         __syncwarp();
         for (int u = group; u < t; u += 2) {
             const int slot = first_slot + u;
@@ -305,8 +279,8 @@ __device__ __forceinline__ void soft_exps(const SoftJob& j, StreamSmem& sm, int 
         for (int c = 0; c < N; ++c) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                v[c][2 * i] = fast_ex2(v[c][2 * i]);
-                v[c][2 * i + 1] = fast_ex2(v[c][2 * i + 1]);
+                v[c][2 * i] = ex2_approx(v[c][2 * i]);
+                v[c][2 * i + 1] = ex2_approx(v[c][2 * i + 1]);
                 sum[c * 8 + i] = add2(sum[c * 8 + i], make_float2(v[c][2 * i], v[c][2 * i + 1]));
             }
             tmem_st16(cols + c * 16, v[c]);
@@ -569,7 +543,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
                 for (int k = 0; k < kSoftWarps; ++k) { mk[k] = -sm.m[k][tid]; mx = fmaxf(mx, mk[k]); }
 #pragma unroll
                 for (int k = 0; k < kSoftWarps; ++k)
-                    if (mk[k] > -CUDART_INF_F) z += sm.w[k][tid] * fast_ex2(mk[k] - mx);
+                    if (mk[k] > -CUDART_INF_F) z += sm.w[k][tid] * ex2_approx(mk[k] - mx);
                 if (csize > 1) {
                     const int xb = jn & (kPairBufs - 1);
                     const uint32_t xbar = smem_u32(&sm.xbar[xb]);
@@ -582,7 +556,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
                     for (uint32_t r = 0; r < csize; ++r) mx = fmaxf(mx, sm.peer[xb][r][tid].x);
                     for (uint32_t r = 0; r < csize; ++r) {
                         const float2 p = sm.peer[xb][r][tid];
-                        if (p.x > -CUDART_INF_F) z += p.y * fast_ex2(p.x - mx);
+                        if (p.x > -CUDART_INF_F) z += p.y * ex2_approx(p.x - mx);
                     }
                 }
                 sm.g[tid] = mx;
@@ -592,7 +566,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             soft_barrier();
             for (int i = lane; i < npad; i += 32) {          // this warp's exponentials -> normalised, head-averaged
                 const float mk = -sm.m[warp][i];
-                my_w[i] = mk == -CUDART_INF_F ? 0.f : fast_ex2(mk - sm.g[i]) * sm.iz[i];
+                my_w[i] = mk == -CUDART_INF_F ? 0.f : ex2_approx(mk - sm.g[i]) * sm.iz[i];
             }
             __syncwarp();
             if (!ROOM && a.alpha.ptr) soft_scores<true>(j, sm, nch, warp, lane);
