@@ -34,7 +34,7 @@ def _compile_cuda(tmp: str, verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     flags = ["-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a", "-Xcompiler", "-fPIC",
              "-I", os.path.join(ROOT, "include"), "-I", CSRC] + (["-Xptxas=-v"] if verbose else [])
-    flags += os.environ.get("MVLA_NVCC_FLAGS", "").split()     # extra compiler flags, e.g. -D tuning macros
+    flags += os.environ.get("MVLA_NVCC_FLAGS", "").split()     # extra compiler flags
 
     def one(f):
         obj = os.path.join(tmp, f + ".o")

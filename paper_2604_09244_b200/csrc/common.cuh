@@ -28,8 +28,8 @@ constexpr int kKeyTile = 128;        // visual keys per tile = rows of one MMA
 constexpr int kMaxCluster = 8;       // portable cluster size
 constexpr int kMaxText = 64;
 constexpr int kMaxVis = 4096;
-constexpr uint32_t kSpinLimit = 1u << 22;
-constexpr unsigned kStampSlots = 4096;      // CTAs per kernel that leave time stamps when asked to (mvla_set_kernel_stamps)   // bounded device-side waits (each try sleeps, see wait loops)
+constexpr uint32_t kSpinLimit = 1u << 22;   // tries of a bounded device-side wait (the clock ends it earlier, see the wait loops)
+constexpr unsigned kStampSlots = 4096;      // CTAs per kernel that leave time stamps when asked to (mvla_set_kernel_stamps)
 
 // Device-side view of one sample; everything the host can compute is computed there.
 struct SampleDev {

@@ -13,7 +13,7 @@
 //     a cold instruction cache, and what a step does not use cost eight action steps 4 us;
 //   * exponents are taken against the logits of each warp's first key, not a maximum: two block barriers less;
 //   * each thread reads ALL its logits from tensor memory once (one wide tcgen05.ld) and keeps them in
-//     registers through max -> exp2 -> sum -> weighted sum;
+//     registers through exp2 -> sum -> weighted sum;
 //   * the per-query (max, sum) pairs travel between the CTAs of a cluster as asynchronous remote
 //     shared-memory stores that credit the receiver's mbarrier when they land (st.async with
 //     complete_tx): one one-way trip, no cluster-wide hardware barrier and no fence on the critical path;

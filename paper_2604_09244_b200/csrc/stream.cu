@@ -357,8 +357,8 @@ __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, in
 // ROOM: the feature norms are to run beside this kernel.  Its ten warps put three on two of a multiprocessor's four
 // register files (16384 registers each): at the 168 registers a thread that the compiler takes these are full, no CTA of
 // the norms fits, and they start when the scores are done.  144 leave room for two warps of 32 registers in each (adaptive
-// steps, 10 requests of 190 tokens 31.2 -> 24.1 us, 4 of 768 33.6 -> 27.1); 128 spill in the softmax (16 requests of 768
-// tokens 97 -> 106).  Without norms the registers are worth more (16 patch-by-patch steps 96.3 us, 99.1 with 144).
+// steps, 10 requests of 190 tokens 31.2 -> 24.1 us, 4 of 768 33.6 -> 27.1) at the price of 8 bytes a thread stored and 24
+// loaded; with 128 these are 68 and 144 (16 requests of 768 tokens 97 -> 106).  Without norms the registers are worth more (16 patch-by-patch steps 96.3 us, 99.1 with 144).
 template <bool ROOM>
 __global__ void __maxnreg__(ROOM ? 144 : 168)
 salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,

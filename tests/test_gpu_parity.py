@@ -107,7 +107,8 @@ def test_salience_small_ragged(dtype, path, text_first):
 
 
 def test_salience_many_tiles_and_max_text():
-    # 2500 keys -> 21 tiles -> 3 tiles per CTA in a cluster of 7; 64 text queries (the maximum)
+    # 2500 keys -> 20 tiles; 64 text queries (the maximum): the streaming kernel in clusters, and the generic one by FMAs with
+    # 3 tiles per CTA in a cluster of 7
     wl = W.small_workload(32, batch=1, D=128, H=2, d=128, dtype="bf16", n_txt=(64,), n_2d=(1100,), n_3d=(1400,))
     for path in (mvla.SALIENCE_AUTO, mvla.SALIENCE_FMA):
         ctx = mvla.context_for(wl, salience_path=path)
@@ -785,7 +786,7 @@ def test_step_with_two_threads_per_key_in_every_shape_of_the_scoring_kernel(n_tx
     (12, 16, (5, 9), (130, 40), (37, 200), {"dtype": "fp8"}),                # 8-bit keys, 16-query slots
     (10, 16, (33, 48), (256, 100), (129, 384), {"n_kv_heads": 4}),           # grouped key heads
     (9, 16, (40, 20), (200, 60), (70, 300), {"d": 96}),                      # a partial swizzle row
-    (6, 8, (64, 3), (1000, 700), (900, 1047), {"d": 256}),                   # two stages per tile; clusters of two
+    (6, 8, (64, 3), (1000, 700), (900, 1047), {"d": 256}),                   # four stages per tile; clusters of two
     (1, 4, (64,), (2048,), (2048,), {"D": 512}),                             # the most tiles: clusters of eight
     (2, 4, (17, 50), (1500, 2000), (1200, 77), {"text_first": True})])       # more than 2048 tokens, 1024-thread tail
 def test_streaming_scoring_kernel_at_the_edges_of_its_shapes(batch, H, n_txt, n_2d, n_3d, kw):
