@@ -372,9 +372,9 @@ cudaError_t stream_pays(const mvla_ctx* ctx, const BatchDesc& bd, int tiles_per_
     return e;
 }
 
-// Salience of one chunk (+ L1 norms into `l1` when asked; + the scores as fp32 into `attn_out` when asked).  The per-head contributions land in
-// ctx->part, or, when `want_acc64` and the register-resident tensor-core kernel covers the shape, in the
-// fixed-point accumulators ctx->acc64 (*used_acc64 = true).
+// Salience of one chunk (+ L1 norms into `l1` when asked; + the scores as fp32 into `attn_out` when asked).  The per-head
+// contributions are added into the fixed-point accumulators `acc64` (*used_acc64 = true) where a kernel that does so covers the
+// shape, else they land in ctx->part.
 int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, const void* k, int64_t rows,
                            const void* hidden, float* l1, unsigned long long* acc64, bool* used_acc64,
                            cudaStream_t st, AlphaOut alpha = AlphaOut{nullptr, 0, 0},
