@@ -14,8 +14,8 @@ template <int NT, int CAP, class BD>
 __global__ void __launch_bounds__(NT, 1)
 select_kernel(const __grid_constant__ BD bd, const GateParams gp, const SelectIO io)
 {
-    __shared__ SelectSmem<NT, CAP> sm;
-    select_sample<NT, CAP>(bd.at(blockIdx.x), blockIdx.x, gp, io, sm);
+    __shared__ SelectSmem<NT, CAP / NT> sm;
+    select_sample<NT, CAP / NT>(bd.at(blockIdx.x), blockIdx.x, gp, io, sm);
 }
 
 }  // namespace

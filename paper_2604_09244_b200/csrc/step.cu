@@ -56,13 +56,12 @@ select_copy_kernel(const __grid_constant__ BD bd, const __grid_constant__ TailPl
     const int cta = blockIdx.x;
     if (cta < bd.count()) {
         // ---- selection of one sample, by one CTA
-        __shared__ SelectSmem<NT, CAP> sm;
+        __shared__ SelectSmem<NT, CAP / NT> sm;
         const int b = cta;
         SelectRole role;
         role.late_pdl = true;
-        role.l1_late = true;                                // the norms may come from a kernel that ran beside the scoring
-        if (tp.cta0[bd.count()] > 0) role.kept_sm = list + bd.at(b).out_off * kListStride;   // every word is its own "ready" signal
-        select_sample<NT, CAP>(bd.at(b), b, gp, io, sm, role, [&]() {}, [&]() {
+        if (tp.cta0[bd.count()] > 0) role.list = list + bd.at(b).out_off * kListStride;   // every word is its own "ready" signal
+        select_sample<NT, CAP / NT>(bd.at(b), b, gp, io, sm, role, [&]() {
             if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
         });
         if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta] = stamps[2 * cta + 1];   // placeholder start, see the copiers

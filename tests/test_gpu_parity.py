@@ -83,6 +83,49 @@ def test_select_text_first_and_negative_scores():
     ctx.close()
 
 
+def _scores_of_shape(shape, n, rng):
+    """Scores that put the threshold into every part of the selection's histogram: a window around the mean, open ends."""
+    if shape == "softmax":                       # what the scoring kernels leave: a bulk below the mean, a few strong ones
+        x = np.exp(0.05 * rng.standard_normal(n)) * np.where(rng.random(n) < 0.05, 20.0, 1.0)
+        return x / x.sum()
+    if shape == "one_token_has_it_all":          # the threshold far below the window
+        x = 1e-9 * (1.0 + rng.random(n))
+        x[rng.integers(n)] = 1.0
+        return x
+    if shape == "above_the_window":              # not normalised: everything in the last bin
+        return 1e3 + rng.random(n)
+    if shape == "narrow":                        # thousands of keys within a few units in the last place, many equal
+        return (1.0 + 2.0 ** -23 * rng.integers(0, 40, size=n)) / n
+    if shape == "two_scales":                    # one end of the window and the other
+        return np.where(rng.random(n) < 0.5, 1e-12, 64.0) * (1.0 + 2.0 ** -20 * rng.integers(0, 1 << 12, size=n))
+    x = rng.standard_normal(n) * 10.0 ** rng.integers(-30, 30, size=n).astype(np.float64)       # any float, infinities and zeros
+    x[rng.random(n) < 0.1] = 0.0
+    x[rng.random(n) < 0.02] = np.inf
+    x[rng.random(n) < 0.02] = -np.inf
+    return x
+
+
+@pytest.mark.parametrize("shape", ["softmax", "one_token_has_it_all", "above_the_window", "narrow", "two_scales", "any_float"])
+def test_select_finds_the_threshold_wherever_it_lies(shape):
+    # sizes around the capacities of the kernel's variants (1024, 2048, 4096 tokens); exact: the k largest, lower index first
+    rng = np.random.default_rng(11)
+    for n2, n3 in ((1, 1), (0, 2), (31, 33), (512, 512), (513, 512), (1024, 1024), (5, 2044), (1024, 1025), (2048, 2048)):
+        ctx = mvla.PruneContext(dtype=torch.float32, n_heads=2, head_dim=64, d_model=64, max_batch=1, max_text=8,
+                                max_2d=max(n2, 1), max_3d=max(n3, 1), cold_start_full_keep=0)
+        for keep in (0.02, 0.4, 0.97):
+            s = W.layout_2d_3d_txt(0, 3, n2, n3, keep_2d=keep, keep_3d=keep)
+            attn = _scores_of_shape(shape, n2 + n3, rng).astype(np.float32)
+            out = ctx.select(0, [s], mvla.MODE_FIXED, torch.from_numpy(attn).cuda(), flags=mvla.FLAG_RESET_STATE)
+            torch.cuda.synchronize()
+            k2, k3 = (int(k) for k in out.budgets.cpu().numpy()[0])
+            kept = out.kept_idx.cpu().numpy()[:out.out_offsets.cpu().numpy()[1]]
+            best2 = np.argsort(-attn[:n2], kind="stable")[:k2]
+            best3 = n2 + np.argsort(-attn[n2:], kind="stable")[:k3]
+            want = np.concatenate([np.sort(best2), np.sort(best3), n2 + n3 + np.arange(3)])
+            assert np.array_equal(kept, want), (shape, n2, n3, keep)
+        ctx.close()
+
+
 # ------------------------------------------------------------------ salience
 @pytest.mark.parametrize("dtype,path", [("fp32", mvla.SALIENCE_AUTO), ("bf16", mvla.SALIENCE_FMA),
                                         ("bf16", mvla.SALIENCE_AUTO)])
