@@ -169,6 +169,30 @@ __device__ __forceinline__ void umma_by_size(int esize, uint32_t d_tmem, uint64_
     if (esize == 2) umma_bf16(d_tmem, a_desc, b_desc, idesc, accumulate);
     else umma_e4m3(d_tmem, a_desc, b_desc, idesc, accumulate);
 }
+// A descriptor whose start address lies 16 x `units` bytes further on (below 256 KB: the low word does not carry).
+__device__ __forceinline__ uint64_t desc_plus(uint64_t desc, uint32_t units)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(static_cast<uint32_t>(desc) + units), "r"(static_cast<uint32_t>(desc >> 32)));
+    return d;
+}
+// The MMAs over one box (128-byte swizzle rows) of both operands: `n` of them, 32 bytes of every row each, the first of them
+// accumulating when asked and the others always.  Four in a row without a loop, in 32-bit descriptor arithmetic: issued
+// one by one in a loop over run-time sizes the eight MMAs of a key tile of 128 bf16 elements took 750 cycles, like this 370 to 400,
+// which is what they take to execute (N = 16 to 64).
+__device__ __forceinline__ void umma_box(int esize, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, int n, bool accumulate)
+{
+    const uint32_t first = accumulate ? 1u : 0u;
+    if (n == 4 && esize == 2) {
+#pragma unroll
+        for (uint32_t kb = 0; kb < 4; ++kb) umma_bf16(d_tmem, desc_plus(a_desc, 2 * kb), desc_plus(b_desc, 2 * kb), idesc, kb ? 1u : first);
+    } else if (n == 4) {
+#pragma unroll
+        for (uint32_t kb = 0; kb < 4; ++kb) umma_e4m3(d_tmem, desc_plus(a_desc, 2 * kb), desc_plus(b_desc, 2 * kb), idesc, kb ? 1u : first);
+    } else {                                  // the last box of a head dim that is no multiple of 128 bytes
+        for (int kb = 0; kb < n; ++kb) umma_by_size(esize, d_tmem, a_desc + 2 * kb, b_desc + 2 * kb, idesc, kb ? 1u : first);
+    }
+}
 __device__ __forceinline__ void umma_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");

@@ -382,15 +382,9 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
             for (int t = 0; t < NTILE; ++t) {
                 if (valid[t] <= 0 || !from_k[t]) continue;
                 for (int kh = 0; kh < khalves; ++kh) {
-                    const uint64_t kd = k_desc + static_cast<uint64_t>(t * khalves + kh) * (16384 >> 4);
-                    const uint64_t qd = q_desc + static_cast<uint64_t>(kh * npad) * (128 >> 4);
-                    const int n = min(4, ksteps - kh * 4);
-                    if (one) {
-                        if (esize == 2)
-                            for (int kb = 0; kb < n; ++kb) umma_bf16(tmem_base + t * TCOL, kd + 2 * kb, qd + 2 * kb, idesc, kh + kb > 0 ? 1u : 0u);
-                        else
-                            for (int kb = 0; kb < n; ++kb) umma_e4m3(tmem_base + t * TCOL, kd + 2 * kb, qd + 2 * kb, idesc, kh + kb > 0 ? 1u : 0u);
-                    }
+                    if (one)
+                        umma_box(esize, tmem_base + t * TCOL, desc_plus(k_desc, static_cast<uint32_t>(t * khalves + kh) * (16384 >> 4)),
+                                 desc_plus(q_desc, static_cast<uint32_t>(kh * npad) * (128 >> 4)), idesc, min(4, ksteps - kh * 4), kh > 0);
                 }
             }
         }

@@ -482,14 +482,10 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
                     ok = ring_wait<false>(smem_u32(&sm.kfull[stage]), phase, aborted, a.status);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t kd = k_desc0 + static_cast<uint64_t>(stage) * (kStageBytes >> 4);
-                    const uint64_t qd = q_desc0 + ((static_cast<uint64_t>(qb) * q_bytes + static_cast<uint64_t>(kh * npad) * 128) >> 4);
+                    const uint64_t kd = desc_plus(k_desc0, static_cast<uint32_t>(stage) * (kStageBytes >> 4));
+                    const uint64_t qd = desc_plus(q_desc0, (static_cast<uint32_t>(qb) * q_bytes + static_cast<uint32_t>(kh * npad) * 128u) >> 4);
                     if (one) {
-                        const int n = min(4, ksteps - kh * 4);
-                        if (a.esize == 2)
-                            for (int kb = 0; kb < n; ++kb) umma_bf16(tmem_base + slot * W, kd + 2 * kb, qd + 2 * kb, idesc, kh + kb > 0 ? 1u : 0u);
-                        else
-                            for (int kb = 0; kb < n; ++kb) umma_e4m3(tmem_base + slot * W, kd + 2 * kb, qd + 2 * kb, idesc, kh + kb > 0 ? 1u : 0u);
+                        umma_box(a.esize, tmem_base + slot * W, kd, qd, idesc, min(4, ksteps - kh * 4), kh > 0);
                         umma_commit(smem_u32(&sm.kempty[stage]));
                     }
                     if (++stage == a.stages) { stage = 0; phase ^= 1; }
