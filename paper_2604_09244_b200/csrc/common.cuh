@@ -14,9 +14,10 @@
 
 namespace mvla {
 
-// Hand-over words of the patch-by-patch tail, per sample from word cap_off on: kHandLines lines of 32 words
-// (identical copies, so that the copying CTAs do not all poll one line of the L2: word 0 "the list is about
-// to be written", word 1 the sample's first output row), then one word per row of the sample.
+// Hand-over words of the patch-by-patch tail, from word cap_off of the launch's first sample on: kHandLines lines of 32
+// words (identical copies, so that the copying CTAs do not all poll one line of the L2: word 0 "a list is about
+// to be written", word 1 the rows that the batch keeps), then one word per output row.  (Every sample reserves and
+// re-arms words for lines of its own and its rows; the launch uses them as one run.)
 constexpr int kHandLines = 8;
 constexpr int kHandWords = kHandLines * 32;
 // Distance in words between the hand-over words of neighbouring rows in the fused tails.  A row's word is polled by as
@@ -296,7 +297,7 @@ cudaError_t launch_patch_indicators(const BatchDesc& bd, int n_heads, AlphaOut a
 cudaError_t launch_patch_select(const BatchDesc& bd, const PatchParams& pp, const PatchIO& io, cudaStream_t stream);
 // Indicators, stages 1-4 and the row copy of the patch-by-patch step in one kernel behind the scoring kernel
 // (which must have re-armed `list` and `rec`, see launch_salience_fast).  `rec`: [sum P][3] 8-byte words;
-// `list`: 4-byte words, kHandWords + kListStride (n_txt + n_vis) per sample from cap_off on.  io.x / io.attn are not read.
+// `list`: 4-byte words, kHandWords + kListStride (n_txt + n_vis) for every sample from its cap_off on.  io.x / io.attn are not read.
 // `ticket_counter`: one word, zero before the first launch, used by one launch at a time (it returns to zero with
 // every launch): the CTAs take their roles in the order in which they start (copy_impl.cuh: cta_ticket).
 bool patch_tail_supported(const BatchDesc& bd);

@@ -34,12 +34,16 @@ __device__ __forceinline__ void st_row(uint4* p, const uint4& v)
 // Copies `n_rows` rows.  The work is cut into 2 KB segments of one row of one tensor; warp `w` of `nw`
 // takes segments w, w + nw, ... and keeps two of them (8 x 16 bytes per lane) in flight.
 // rows(i, src_row, dst_row): absolute source and destination row of the i-th row of the list; false: skip it.
-template <class RowFn>
-__device__ __forceinline__ void copy_rows(const CompactArgs& a, int n_rows, int w, int nw, int lane, RowFn rows)
+// ended(): the list turned out to be shorter (asked after rows(), once per two segments).
+struct NotEnded {
+    __device__ bool operator()() const { return false; }
+};
+template <class RowFn, class Ended = NotEnded>
+__device__ __forceinline__ void copy_rows(const CompactArgs& a, int n_rows, int w, int nw, int lane, RowFn rows, Ended ended = Ended())
 {
     const int per_row = a.seg_begin[3];
     const int n_units = n_rows * per_row;
-    for (int u0 = w; u0 < n_units; u0 += 2 * nw) {
+    for (int u0 = w; u0 < n_units && !ended(); u0 += 2 * nw) {
         uint4 v[2][4];
         const uint4* sp[2];
         uint4* dp[2];

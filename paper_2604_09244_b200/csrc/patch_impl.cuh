@@ -270,12 +270,11 @@ __device__ __forceinline__ int ld_volatile_i32(const int* p)
 // `rec`: null: indicators and scores come from io.x / io.attn, written by the kernel before this one; else
 //        they are taken, patch by patch, from the 8-byte words that patch_indicators_block writes in the
 //        same kernel (bounded wait for each).
-// `list`: when not null, kHandWords + kListStride `cap` 4-byte words (all -1 before the launch) for CTAs of the same
-//        kernel that copy the rows: in each of the first kHandLines lines of 32 words, word 0 = 1 once the
-//        masks are decided (the list follows shortly: time to start polling it), word 1 = first output
-//        row of the sample, word 2 = number of rows it keeps (written before word 1 by the same thread;
-//        a reader takes word 2 only after it has seen word 1 and re-reads it until it is there); word
-//        kHandWords + kListStride r = index inside the sample of the token that goes to the sample's output row r.
+// `list`: when not null, kHandWords + kListStride x (rows that the launch's samples may keep) 4-byte words (all -1 before
+//        the launch) for CTAs of the same kernel that copy the rows: in each of the first kHandLines lines of 32 words,
+//        word 0 = 1 once the masks of some sample are decided (its list follows shortly: time to start polling),
+//        word 1 = number of rows that the batch keeps, once it is known; word kHandWords + kListStride r = source row of
+//        output row r.
 template <int NT>
 __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_local, int n_in_launch, const PatchParams& pp,
                                                    const PatchIO& io, PatchSmemT<NT>& sm, const unsigned long long* rec,
@@ -487,9 +486,10 @@ __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_loc
     //      (A sample that is alone in its launch and first in its batch starts at row 0: nothing to wait for.)
     const bool alone = n_in_launch == 1;                          // nobody in this launch to wait for or to tell
     const bool first_row_known = alone && b_glob == 0;
+    const bool last = b_glob == io.batch_total - 1;
     auto bookkeeping = [&](int off) {                             // lane 0 of warp 0
         io.out_offsets[b_glob] = off;
-        if (b_glob == io.batch_total - 1) io.out_offsets[io.batch_total] = off + n_out;
+        if (last) io.out_offsets[io.batch_total] = off + n_out;
         if (io.counts) { io.counts[b_glob * 2] = k2; io.counts[b_glob * 2 + 1] = k3; }
         if (io.diag) {
             mvla_patch_diag dg;
@@ -502,7 +502,7 @@ __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_loc
         }
     };
     if (first_row_known) {
-        if (list && tid < kHandLines) { list[32 * tid + 2] = n_out; list[32 * tid + 1] = 0; }
+        if (list && last && tid < kHandLines) list[32 * tid + 1] = n_out;
         if (tid == 0) { sm.out_off = 0; io.nout_ws[b_glob] = n_out; }   // later launches of this call read the count in stream order
     } else {
         if (warp == 0) {
@@ -530,7 +530,7 @@ __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_loc
 #pragma unroll
             for (int o = 16; o >= 1; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
             if (!__all_sync(0xffffffffu, ok) && lane == 0) *reinterpret_cast<volatile int*>(io.status) = MVLA_ERR_TIMEOUT;
-            if (list && lane < kHandLines) { list[32 * lane + 2] = n_out; list[32 * lane + 1] = off; }
+            if (list && last && lane < kHandLines) list[32 * lane + 1] = off + n_out;
             if (lane == 0) {
                 sm.out_off = off;
                 // every wait of this CTA is over: the CTA that gets here last clears the flags of the launch
@@ -553,7 +553,7 @@ __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_loc
     const int baset = (s.off_2d < s.off_txt ? k2 : 0) + (s.off_3d < s.off_txt ? k3 : 0);
     for (int i = tid; i < s.n_txt; i += NT) {
         io.kept_idx[out_off + baset + i] = s.off_txt + i;
-        if (list) list[kHandWords + (baset + i) * kListStride] = s.off_txt + i;
+        if (list) list[kHandWords + (out_off + baset + i) * kListStride] = s.seq_off + s.off_txt + i;
     }
     int run = 0;
     for (int j0 = 0; j0 < nv; j0 += NT) {              // block-uniform
@@ -566,7 +566,7 @@ __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_loc
             const int pos = j < P ? base2 + r : base3 + (r - k2);
             const int val = j < P ? s.off_2d + j : s.off_3d + (j - P);
             io.kept_idx[out_off + pos] = val;
-            if (list) list[kHandWords + pos * kListStride] = val;
+            if (list) list[kHandWords + (out_off + pos) * kListStride] = s.seq_off + val;
         }
     }
     if (tid == 0) bookkeeping(out_off);                           // nobody in this kernel waits for these

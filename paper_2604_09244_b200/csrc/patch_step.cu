@@ -4,7 +4,9 @@
 //     words, to the CTA that runs the stages after it;
 //   * one CTA per sample: temporal predictor, dual threshold, K-Means, semantic rules, fusion, masks
 //     (stages 1-4), reading each patch's words as they appear; it writes the kept list as 4-byte words;
-//   * the remaining CTAs copy the surviving rows, each warp polling the word of the row it is to move.
+//   * the remaining CTAs copy the surviving rows, each warp polling the word of the row it is to move.  Output rows are
+//     dealt out over all of them, whatever sample they belong to: which samples keep many rows shows only here, and with CTAs of
+//     its own per sample the one with the most rows was copied 17 us longer than the median one (16 samples of 512 tokens).
 // No kernel boundary, fence or flag lies between the three roles: every word is its own signal, re-armed
 // (all ones) by the scoring kernel of the same step.  The roles go by ticket (cta_ticket: the order in which the
 // CTAs started), so a consumer only ever waits for CTAs that are already running; every wait is bounded all the same.
@@ -20,7 +22,8 @@ constexpr int kTailThreads = kIndThreads;
 
 struct PatchTailPlan {
     int16_t ind0[kMaxChunk + 1];      // first indicator CTA of every sample; ind0[n] = their number
-    int16_t cta0[kMaxChunk + 1];      // first copying CTA of every sample (counted from 0); cta0[n] = their number
+    int16_t copiers;                  // copying CTAs
+    int32_t rows;                     // rows that the samples may keep
 };
 
 template <typename T, int PP, class BD>
@@ -42,57 +45,76 @@ patch_tail_kernel(const __grid_constant__ BD bd, const __grid_constant__ PatchTa
     if (c < bd.count()) {
         __shared__ PatchSmemT<kTailThreads> sm;
         const SampleDev& s = bd.at(c);
-        const bool copying = tp.cta0[bd.count()] > 0;
-        patch_select_block<kTailThreads>(s, c, bd.count(), pp, io, sm, rec, copying ? list + s.cap_off : nullptr);
+        patch_select_block<kTailThreads>(s, c, bd.count(), pp, io, sm, rec, tp.copiers > 0 ? list + bd.at(0).cap_off : nullptr);
         return;
     }
     // ---- row copy
     c -= bd.count();
-    int b = 0;
-    while (b + 1 < bd.count() && c >= tp.cta0[b + 1]) ++b;
-    const SampleDev& s = bd.at(b);
     const int tid = threadIdx.x, lane = tid & 31;
-    const int part = c - tp.cta0[b], nparts = tp.cta0[b + 1] - tp.cta0[b];
-    const int w = part * (kTailThreads / 32) + (tid >> 5), nw = nparts * (kTailThreads / 32);
+    const int w = c * (kTailThreads / 32) + (tid >> 5), nw = tp.copiers * (kTailThreads / 32);
     asm volatile("griddepcontrol.wait;" ::: "memory");      // the words were re-armed by the kernel before this one
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // One warp of the CTA waits, at a low rate, for the hint that the list is about to be written and for the
-    // sample's first output row (its own copy of both); only then do all warps poll the words of their rows.
-    // Thousands of warps polling while the selecting CTA works would slow that CTA's own memory traffic.
-    __shared__ int s_first, s_rows;
-    const int32_t* words = list + s.cap_off;
+    // One warp of the CTA waits, at a low rate, for the hint that a list is about to be written (its own copy of it); only
+    // then do all warps poll the words of their rows.  Thousands of warps polling while the selecting CTAs work would slow
+    // those CTAs' own memory traffic.
+    const int32_t* words = list + bd.at(0).cap_off;
+    const int32_t* mine = words + 32 * (c % kHandLines);
     const uint64_t t0 = global_ns();
     constexpr uint64_t kLimitNs = 1000000000ull;
+    __shared__ int s_hint, s_rows;
     if (tid < 32) {
-        const int32_t* mine = words + 32 * (part % kHandLines);
-        int hint = -1, first = -1, n_rows = -1;
+        int hint = -1, rows = -1;
         for (uint32_t it = 0; it < kSpinLimit; ++it) {
             if (hint < 0) hint = ld_relaxed_gpu(mine);
-            if (hint >= 0 && first < 0) first = ld_relaxed_gpu(mine + 1);
-            if (first >= 0) n_rows = ld_relaxed_gpu(mine + 2);
-            if (n_rows >= 0) break;
+            if (hint >= 0) rows = ld_relaxed_gpu(mine + 1);
+            if (rows >= 0 || (hint >= 0 && bd.count() > 1)) break;      // (a sample alone: its count comes with the hint)
             if ((it & 63u) == 63u && global_ns() - t0 > kLimitNs) break;
             __nanosleep(hint < 0 ? 200 : 40);
         }
-        if (lane == 0) { s_first = first; s_rows = n_rows; }
+        if (lane == 0) { s_hint = hint; s_rows = rows; }
     }
     __syncthreads();
-    const int out_off = s_first, n_rows = s_rows;           // first output row of the sample, rows it keeps
-    if (out_off < 0 || n_rows < 0) {
+    int n_rows = s_rows;                                    // rows that the batch keeps, once this warp knows
+    if (s_hint < 0 || (n_rows < 0 && bd.count() == 1)) {
         if (tid == 0) *reinterpret_cast<volatile int*>(io.status) = MVLA_ERR_TIMEOUT;
         return;
     }
     words += kHandWords;
-    copy_rows(ca, n_rows, w, nw, lane, [&](int i, int64_t& srow, int64_t& drow) {
-        const int v = poll_word(words + i * kListStride, t0, kLimitNs);     // the whole warp reads one word: one request
-        if (v < 0) {                                                   // gave up: report, leave the row alone
-            *reinterpret_cast<volatile int*>(io.status) = MVLA_ERR_TIMEOUT;
-            return false;
+    if (bd.count() == 1) {                                  // (known when the kernel is compiled)
+        copy_rows(ca, n_rows, w, nw, lane, [&](int i, int64_t& srow, int64_t& drow) {
+            const int v = poll_word(words + i * kListStride, t0, kLimitNs);     // the whole warp reads one word: one request
+            if (v < 0) {                                                   // gave up: report, leave the row alone
+                *reinterpret_cast<volatile int*>(io.status) = MVLA_ERR_TIMEOUT;
+                return false;
+            }
+            srow = v;
+            drow = i;
+            return true;
+        });
+        return;
+    }
+    bool ended = false;
+    copy_rows(ca, n_rows >= 0 ? n_rows : tp.rows, w, nw, lane, [&](int i, int64_t& srow, int64_t& drow) {
+        int v = ended ? -1 : ld_relaxed_gpu(words + i * kListStride);
+        for (uint32_t it = 0; v < 0 && !ended; ++it) {
+            if (n_rows < 0) n_rows = ld_relaxed_gpu(mine + 1);
+            if (n_rows >= 0 && i >= n_rows) {               // no such row, nor any after it
+                ended = true;
+                break;
+            }
+            if (it >= kSpinLimit || ((it & 63u) == 63u && global_ns() - t0 > kLimitNs)) {
+                *reinterpret_cast<volatile int*>(io.status) = MVLA_ERR_TIMEOUT;       // gave up: report, leave the rows alone
+                ended = true;
+                break;
+            }
+            __nanosleep(20);
+            v = ld_relaxed_gpu(words + i * kListStride);
         }
-        srow = static_cast<int64_t>(s.seq_off) + v;
-        drow = static_cast<int64_t>(out_off) + i;
+        if (v < 0) return false;
+        srow = v;
+        drow = i;
         return true;
-    });
+    }, [&]() { return ended; });
 }
 
 }  // namespace
@@ -125,22 +147,11 @@ cudaError_t launch_patch_tail(const BatchDesc& bd, int n_heads, AlphaOut alpha, 
     }
     for (int b = bd.n; b <= kMaxChunk; ++b) tp.ind0[b] = static_cast<int16_t>(next);
     const CompactArgs ca = compact_args(job);
-    int copiers = 0;
-    if (ca.seg_begin[3] > 0) {
-        // copying CTAs per sample in proportion to the rows it may keep, at least one each; together with the
-        // selecting CTAs they fill the multiprocessors once the indicator CTAs have retired
-        const int want = std::max(sm_count - bd.n, bd.n);
-        int64_t rows = 0;
-        for (int b = 0; b < bd.n; ++b) rows += bd.s[b].n_txt + bd.s[b].n_2d + bd.s[b].n_3d;
-        for (int b = 0; b < bd.n; ++b) {
-            tp.cta0[b] = static_cast<int16_t>(copiers);
-            const int64_t mine = bd.s[b].n_txt + bd.s[b].n_2d + bd.s[b].n_3d;
-            copiers += static_cast<int>(std::max<int64_t>(1, (static_cast<int64_t>(want) * mine + rows / 2) / std::max<int64_t>(rows, 1)));
-        }
-    } else {
-        for (int b = 0; b < bd.n; ++b) tp.cta0[b] = 0;
-    }
-    for (int b = bd.n; b <= kMaxChunk; ++b) tp.cta0[b] = static_cast<int16_t>(copiers);
+    // together with the selecting CTAs they fill the multiprocessors once the indicator CTAs have retired
+    const int copiers = ca.seg_begin[3] > 0 ? std::max(sm_count - bd.n, 1) : 0;
+    tp.copiers = static_cast<int16_t>(copiers);
+    tp.rows = 0;
+    for (int b = 0; b < bd.n; ++b) tp.rows += bd.s[b].n_txt + bd.s[b].n_2d + bd.s[b].n_3d;
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(next + bd.n + copiers));
