@@ -253,6 +253,86 @@ __device__ __forceinline__ double warp_sum_d(double v)
     for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     return v;
 }
+// The smallest (largest) of 64-bit patterns that order like unsigned numbers, over a warp: the high words, then the low
+// words of those that share it (two rounds of redux, 43 cycles each; a butterfly of 64-bit shuffles takes 350).
+__device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
+{
+    const unsigned hi = static_cast<unsigned>(v >> 32), m = __reduce_min_sync(0xffffffffu, hi);
+    const unsigned lo = __reduce_min_sync(0xffffffffu, hi == m ? static_cast<unsigned>(v) : 0xFFFFFFFFu);
+    return static_cast<unsigned long long>(m) << 32 | lo;
+}
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) { return ~warp_min_u64(~v); }
+
+// 1-D K-Means, K = 3 (Sec. 4.2), of the P masses by one warp, started from the smallest mass, the mean and the
+// largest: labels and centres to `sm`.  A round: assign to the nearest centre (ties to the lower one); unless nothing
+// changed, move the centres to the class means.  Nobody else has work meanwhile, so it is a chain; another warp takes the
+// baselines beside it.  Its loops over the patches are not unrolled: most samples have a number of patches that leaves an unrolled
+// loop in its remainder (157 patches 15.2 -> 14.7 us a step against eight at a time, 256 no slower; masses and labels in registers
+// instead of shared memory: 256 patches +0.2 us, 512 +3).
+template <class Smem>
+__device__ __forceinline__ void kmeans(Smem& sm, int P, int max_iter, int lane)
+{
+    double sum = 0.0;
+    unsigned long long mx = 0ull, mn = ~0ull;
+#pragma unroll 1
+    for (int p = lane; p < P; p += 32) {
+        const double m = sm.mass[p];
+        const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(m));
+        sum += m;
+        mx = max(mx, bits);
+        mn = min(mn, bits);
+        sm.massf[p] = static_cast<float>(m);
+        sm.label[p] = 255;
+    }
+    mx = warp_max_u64(mx);
+    mn = warp_min_u64(mn);
+    double c0 = __longlong_as_double(static_cast<long long>(mn)), c1 = warp_sum_d(sum) / P, c2 = __longlong_as_double(static_cast<long long>(mx));
+    int iters = 0;
+    while (iters < max_iter) {                      // warp-uniform
+        ++iters;
+        int changed = 0;
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+        int n0 = 0, n1 = 0, n2 = 0;
+        // Nearest centre.  fp32 decides wherever it can be sure: with m and the centres rounded to fp32
+        // a distance is off by at most 2^-23 (m + c), so a comparison of two distances whose fp32 values
+        // differ by more than `tol` comes out as in double; anything closer (ties included) is redone
+        // in double.  Class sums stay in double.
+        const float f0 = static_cast<float>(c0), f1 = static_cast<float>(c1), f2 = static_cast<float>(c2);
+#pragma unroll 1
+        for (int p = lane; p < P; p += 32) {
+            const double m = sm.mass[p];
+            const float mf = sm.massf[p];
+            const float tol = 4e-7f * (fabsf(mf) + fmaxf(fabsf(f0), fmaxf(fabsf(f1), fabsf(f2))));
+            const float e0 = fabsf(mf - f0), e1 = fabsf(mf - f1), e2 = fabsf(mf - f2);
+            int best = e1 < e0 ? 1 : 0;
+            const float eb = fminf(e0, e1);
+            bool sure = fabsf(e1 - e0) > tol && fabsf(e2 - eb) > tol;
+            if (e2 < eb) best = 2;
+            if (!sure) {
+                best = 0;
+                double bdist = fabs(m - c0);
+                const double d1 = fabs(m - c1), d2 = fabs(m - c2);
+                if (d1 < bdist) { bdist = d1; best = 1; }
+                if (d2 < bdist) { bdist = d2; best = 2; }
+            }
+            if (sm.label[p] != best) { sm.label[p] = static_cast<uint8_t>(best); changed = 1; }
+            s0 += best == 0 ? m : 0.0; n0 += best == 0;
+            s1 += best == 1 ? m : 0.0; n1 += best == 1;
+            s2 += best == 2 ? m : 0.0; n2 += best == 2;
+        }
+        if (!__any_sync(0xffffffffu, changed)) break;
+        s0 = warp_sum_d(s0); s1 = warp_sum_d(s1); s2 = warp_sum_d(s2);
+        n0 = __reduce_add_sync(0xffffffffu, n0); n1 = __reduce_add_sync(0xffffffffu, n1); n2 = __reduce_add_sync(0xffffffffu, n2);
+        // the three class means with one division sequence (lane k: class k)
+        const int nk = lane == 0 ? n0 : (lane == 1 ? n1 : n2);
+        const double ck = (lane == 0 ? s0 : (lane == 1 ? s1 : s2)) / max(nk, 1);
+        if (n0 > 0) c0 = __shfl_sync(0xffffffffu, ck, 0);
+        if (n1 > 0) c1 = __shfl_sync(0xffffffffu, ck, 1);
+        if (n2 > 0) c2 = __shfl_sync(0xffffffffu, ck, 2);
+    }
+    if (lane == 0) { sm.centre[0] = c0; sm.centre[1] = c1; sm.centre[2] = c2; sm.iters = iters; }
+}
+
 __device__ __forceinline__ int ld_volatile_i32(const int* p)
 {
     int v;
@@ -355,39 +435,23 @@ __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_loc
             // the patch's attention response: the mass of its two tokens
             const double m = static_cast<double>(a2[e]) + static_cast<double>(a3[e]);
             sm.mass[p] = m;
-            sm.massf[p] = static_cast<float>(m);
-            sm.label[p] = 255;
             sm.share[p] = make_float2(v.z, v.w);
         }
     }
     __syncthreads();
 
-    // ---- stage 3 preparation by one warp, without block barriers: the baselines (means of the smoothed
-    //      shares), then the 1-D K-Means, K = 3 (Sec. 4.2), started from the smallest mass, the mean and the
-    //      largest.  A round: assign to the nearest centre (ties to the lower one); unless nothing changed,
-    //      move the centres to the class means.
-    if (warp == 0) {
-        double sum_m = 0.0, sum_z = 0.0, sum_w = 0.0;
-        long long mx = 0, mn = 0x7FF0000000000000ll;             // masses are >= 0: their bit patterns order like the values
-#pragma unroll 8
-        for (int p = lane; p < P; p += 32) {                      // (unrolled: the shared-memory loads of eight patches overlap)
-            const double m = sm.mass[p];
+    // ---- stage 3 preparation: the baselines (means of the smoothed shares) by one warp, the K-Means of the masses by another
+    if (warp == 1) {
+        double sum_z = 0.0, sum_w = 0.0;
+#pragma unroll 1
+        for (int p = lane; p < P; p += 32) {
             const float2 zw = sm.share[p];
-            sum_m += m;
             sum_z += static_cast<double>(zw.x);
             sum_w += static_cast<double>(zw.y);
-            mx = max(mx, __double_as_longlong(m));
-            mn = min(mn, __double_as_longlong(m));
         }
-        sum_m = warp_sum_d(sum_m); sum_z = warp_sum_d(sum_z); sum_w = warp_sum_d(sum_w);
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-            mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, off));
-        }
-        // the three means with one division sequence: lane 0 the masses, lane 1 and 2 the shares
-        const double mean = (lane == 0 ? sum_m : (lane == 1 ? sum_z : sum_w)) / P;
-        const double mu_2d = __shfl_sync(0xffffffffu, mean, 1), mu_3d = __shfl_sync(0xffffffffu, mean, 2);
+        sum_z = warp_sum_d(sum_z); sum_w = warp_sum_d(sum_w);
+        const double mean = (lane == 0 ? sum_z : sum_w) / P;      // both with one division sequence
+        const double mu_2d = __shfl_sync(0xffffffffu, mean, 0), mu_3d = __shfl_sync(0xffffffffu, mean, 1);
         if (lane == 0) {
             sm.mu[0] = mu_2d; sm.mu[1] = mu_3d;
             // x < t for an fp32 x and a double t holds exactly when x < (t rounded up to fp32); x > t when
@@ -400,51 +464,9 @@ __device__ __forceinline__ void patch_select_block(const SampleDev& s, int b_loc
             sm.thr[5] = __double2float_rd(pp.obj_2d_min);    // M_2D  >  object rule's 2D floor
             sm.thr[6] = __double2float_ru(pp.eps_3d);        // M_3D  <  eps_3D
         }
-        double c0 = __longlong_as_double(mn), c1 = __shfl_sync(0xffffffffu, mean, 0), c2 = __longlong_as_double(mx);
-        int iters = 0;
-        while (iters < pp.kmeans_max_iter) {                      // warp-uniform
-            ++iters;
-            int changed = 0;
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-            int n0 = 0, n1 = 0, n2 = 0;
-            // Nearest centre.  fp32 decides wherever it can be sure: with m and the centres rounded to fp32
-            // a distance is off by at most 2^-23 (m + c), so a comparison of two distances whose fp32 values
-            // differ by more than `tol` comes out as in double; anything closer (ties included) is redone
-            // in double.  Class sums stay in double.
-            const float f0 = static_cast<float>(c0), f1 = static_cast<float>(c1), f2 = static_cast<float>(c2);
-#pragma unroll 8
-            for (int p = lane; p < P; p += 32) {
-                const double m = sm.mass[p];
-                const float mf = sm.massf[p];
-                const float tol = 4e-7f * (fabsf(mf) + fmaxf(fabsf(f0), fmaxf(fabsf(f1), fabsf(f2))));
-                const float e0 = fabsf(mf - f0), e1 = fabsf(mf - f1), e2 = fabsf(mf - f2);
-                int best = e1 < e0 ? 1 : 0;
-                const float eb = fminf(e0, e1);
-                bool sure = fabsf(e1 - e0) > tol && fabsf(e2 - eb) > tol;
-                if (e2 < eb) best = 2;
-                if (!sure) {
-                    best = 0;
-                    double bdist = fabs(m - c0);
-                    const double d1 = fabs(m - c1), d2 = fabs(m - c2);
-                    if (d1 < bdist) { bdist = d1; best = 1; }
-                    if (d2 < bdist) { bdist = d2; best = 2; }
-                }
-                if (sm.label[p] != best) { sm.label[p] = static_cast<uint8_t>(best); changed = 1; }
-                s0 += best == 0 ? m : 0.0; n0 += best == 0;
-                s1 += best == 1 ? m : 0.0; n1 += best == 1;
-                s2 += best == 2 ? m : 0.0; n2 += best == 2;
-            }
-            if (!__any_sync(0xffffffffu, changed)) break;
-            s0 = warp_sum_d(s0); s1 = warp_sum_d(s1); s2 = warp_sum_d(s2);
-            n0 = __reduce_add_sync(0xffffffffu, n0); n1 = __reduce_add_sync(0xffffffffu, n1); n2 = __reduce_add_sync(0xffffffffu, n2);
-            // the three class means with one division sequence (lane k: class k)
-            const int nk = lane == 0 ? n0 : (lane == 1 ? n1 : n2);
-            const double ck = (lane == 0 ? s0 : (lane == 1 ? s1 : s2)) / max(nk, 1);
-            if (n0 > 0) c0 = __shfl_sync(0xffffffffu, ck, 0);
-            if (n1 > 0) c1 = __shfl_sync(0xffffffffu, ck, 1);
-            if (n2 > 0) c2 = __shfl_sync(0xffffffffu, ck, 2);
-        }
-        if (lane == 0) { sm.centre[0] = c0; sm.centre[1] = c1; sm.centre[2] = c2; sm.iters = iters; }
+    }
+    if (warp == 0) {
+        kmeans(sm, P, pp.kmeans_max_iter, lane);
     }
     __syncthreads();
 
