@@ -379,7 +379,8 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
                            const void* hidden, float* l1, unsigned long long* acc64, bool* used_acc64,
                            cudaStream_t st, AlphaOut alpha = AlphaOut{nullptr, 0, 0},
                            int32_t* rearm = nullptr, bool norms_beside = false, unsigned long long* stamps = nullptr,
-                           bool with_cache = false, unsigned long long* rearm_rec = nullptr, float* attn_out = nullptr)
+                           bool with_cache = false, unsigned long long* rearm_rec = nullptr, float* attn_out = nullptr,
+                           bool* norms_inside = nullptr)
 {
     if (used_acc64) *used_acc64 = false;
     const mvla_config& c = ctx->cfg;
@@ -409,17 +410,24 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
         e = stream_pays(ctx, bd, tiles_per_cta, cluster, npad, alpha.ptr != nullptr, norms_beside && hidden && l1, &streaming);
         if (e != cudaSuccess) return e == cudaErrorInvalidConfiguration ? MVLA_ERR_UNSUPPORTED : fail_cuda(ctx, e);
     }
+    // With `norms_inside`: norms only if the scoring kernel takes them itself, and whether it did.
+    const bool inside = norms_inside && streaming && hidden && l1;
+    if (norms_inside) {
+        *norms_inside = inside;
+        if (!inside) hidden = nullptr;
+    }
     const bool fast = streaming || f32 || (ctx->use_umma && fast_salience_supported(tiles_per_cta));
     // The norms do not depend on the scores: with `norms_beside` (fast kernel only) they are launched AFTER
     // the scoring kernel and run beside it instead of in front of it.
-    norms_beside = norms_beside && fast;
-    if (hidden && l1 && !norms_beside) {
+    norms_beside = norms_beside && fast && !inside;
+    if (hidden && l1 && !norms_beside && !inside) {
         e = launch_l1norm(bd, ctx->hidden_dtype, c.d_model, hidden, l1, false, nullptr, nullptr, st);
         if (e != cudaSuccess) return fail_cuda(ctx, e);
     }
     if (streaming) {
         e = launch_salience_stream(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk, acc64,
-                                   ctx->status_dev, alpha, rearm, rearm_rec, stamps, hidden && l1 && norms_beside, st);
+                                   ctx->status_dev, alpha, rearm, rearm_rec, stamps, hidden && l1 && norms_beside, inside ? hidden : nullptr,
+                                   static_cast<int>(c.d_model * ctx->elem), l1, st);
         if (used_acc64) *used_acc64 = acc64 != nullptr;
     } else if (f32) {
         e = launch_salience_f32(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, tq, tk, tiles_per_cta, cluster, npad, acc64, ctx->status_dev, rearm, stamps, st);
@@ -710,8 +718,11 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
         unsigned long long* rec = ctx->patch_rec + par * (ctx->vis_all / 2 + 1) * 3;
         const AlphaOut alpha = alpha_of(ctx, set);
         ph.mark("mvla: scoring (+ attention copy)");
-        rc = run_salience_chunk(ctx, whole, in->q, in->k, in->rows, nullptr, nullptr, nullptr, nullptr, st, alpha,
-                                list, false, nullptr, false, rec);
+        // (a batch's feature norms are taken beside its scores: those are bound by the softmax, the indicators would be by the rows)
+        float* l1 = ctx->l1_ws + par * ctx->vis_all;
+        bool l1_taken = false;
+        rc = run_salience_chunk(ctx, whole, in->q, in->k, in->rows, in->hidden, l1, nullptr, nullptr, st, alpha,
+                                list, false, nullptr, false, rec, nullptr, &l1_taken);
         if (rc != MVLA_OK) return rc;
         const PatchParams pp = patch_params(ctx);
         PatchIO io;
@@ -725,7 +736,7 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
         io.chunk_first = 0;
         ph.mark("mvla: indicators + stages 1-4 + row copy");
         const cudaError_t e = launch_patch_tail(whole, ctx->cfg.n_heads, alpha, ctx->hidden_dtype, ctx->cfg.d_model, in->hidden,
-                                                x, attn, rec, pp, io, job, list, ctx->sm_count, ctx->tail_ticket + par, st);
+                                                l1_taken ? l1 : nullptr, x, attn, rec, pp, io, job, list, ctx->sm_count, ctx->tail_ticket + par, st);
         if (e != cudaSuccess) return fail_cuda(ctx, e);
         commit_steps(ctx, prune_point, plan, samples);
         if (total_kept_out) *total_kept_out = static_cast<int32_t>(cap);

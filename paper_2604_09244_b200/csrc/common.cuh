@@ -183,11 +183,12 @@ cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, 
                                 cudaStream_t stream);
 // The same scores into the same fixed-point accumulators by the streaming kernel (stream.cu): persistent CTAs, key
 // tiles through a shared-memory ring; for batches and for samples of any size.  `alpha`, `rearm`, `stamps` as above; with
-// `alpha` there may be no accumulators.  `norms_beside`: launch_l1norm follows and is to run beside it.
+// `alpha` there may be no accumulators.  `norms_beside`: launch_l1norm follows and is to run beside it.  With
+// `hidden` (bf16 rows of `row_bytes` bytes; not with `norms_beside`) the kernel takes the norms itself, into `l1`.
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
                                    AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
-                                   unsigned long long* stamps, bool norms_beside, cudaStream_t stream);
+                                   unsigned long long* stamps, bool norms_beside, const void* hidden, int row_bytes, float* l1, cudaStream_t stream);
 
 // Salience: per-head partial scores part[h][vis] (already scaled by 1/(H n_t)).
 // `use_umma`: tensor-core path (bf16 only).  tmaps: device-usable tensor maps (passed by value).
@@ -300,8 +301,9 @@ cudaError_t launch_patch_select(const BatchDesc& bd, const PatchParams& pp, cons
 // `list`: 4-byte words, kHandWords + kListStride (n_txt + n_vis) for every sample from its cap_off on.  io.x / io.attn are not read.
 // `ticket_counter`: one word, zero before the first launch, used by one launch at a time (it returns to zero with
 // every launch): the CTAs take their roles in the order in which they start (copy_impl.cuh: cta_ticket).
+// `l1`: feature norms that the scoring kernel has taken; null: taken here.
 bool patch_tail_supported(const BatchDesc& bd);
-cudaError_t launch_patch_tail(const BatchDesc& bd, int n_heads, AlphaOut alpha, int dtype, int d_model, const void* hidden,
+cudaError_t launch_patch_tail(const BatchDesc& bd, int n_heads, AlphaOut alpha, int dtype, int d_model, const void* hidden, const float* l1,
                               float* x_out, float* attn_out, unsigned long long* rec, const PatchParams& pp, const PatchIO& io,
                               const CompactJob& job, int32_t* list, int sm_count, unsigned int* ticket_counter, cudaStream_t stream);
 

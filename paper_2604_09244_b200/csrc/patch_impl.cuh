@@ -35,15 +35,16 @@ __device__ __forceinline__ unsigned long long ld_relaxed_gpu_u64(const unsigned 
 // thread, where single floats were four times as many).
 // Also writes the per-token scores of the patch's two tokens: a_j = ||alpha_j||_1 / (H n_t).
 // The L1 feature norms of the CTA's 2 PP rows (Sec. 3.1.2) are taken here too, 256 / PP threads per row,
-// their loads issued before the kernel waits for the attention copy of the kernel before it.
+// their loads issued before the kernel waits for the attention copy of the kernel before it; without NORMS that kernel has
+// taken them already (`l1`).
 //
 // `blk`: which block of PP patches of sample `s`.  `rec`: when not null, the patch's indicators and scores
 // also go, as three 8-byte words per patch ({x0, x1}, {x2, x3}, {a_2D, a_3D}; all ones before the launch),
 // to the CTA of the same kernel that runs the stages after this one: an aligned 8-byte store is
 // indivisible and no result of arithmetic has all 64 bits set, so each word is its own "ready" signal.
-template <typename T, int PP>
+template <typename T, int PP, bool NORMS>
 __device__ __forceinline__ void patch_indicators_block(const SampleDev& s, int blk, int n_heads, const AlphaOut& alpha,
-                                                       const T* __restrict__ hidden, int d_model, float* __restrict__ x_out,
+                                                       const T* __restrict__ hidden, const float* __restrict__ l1, int d_model, float* __restrict__ x_out,
                                                        float* __restrict__ attn_out, unsigned long long* __restrict__ rec, bool norms_early)
 {
     constexpr int kIndPatches = PP;
@@ -77,7 +78,7 @@ __device__ __forceinline__ void patch_indicators_block(const SampleDev& s, int b
     const int pr = p0 + (nr & (kIndPatches - 1));
     const int nvec = d_model / kVec;
     const uint4* nsrc = nullptr;
-    if (pr < P)
+    if (NORMS && pr < P)
         nsrc = reinterpret_cast<const uint4*>(hidden + static_cast<int64_t>(s.seq_off + (nr < kIndPatches ? s.off_2d : s.off_3d) + pr) * d_model);
     uint4 hv[kNormKeep];
     auto norm_loads = [&]() {
@@ -102,9 +103,14 @@ __device__ __forceinline__ void patch_indicators_block(const SampleDev& s, int b
                    fabsf(__uint_as_float(u.z)) + fabsf(__uint_as_float(u.w));
         }
     };
-    if (norms_early) norm_loads();
+    if (NORMS && norms_early) norm_loads();
     asm volatile("griddepcontrol.wait;" ::: "memory");    // the attention copy comes from the kernel before this one
-    if (!norms_early) norm_loads();
+    if (NORMS && !norms_early) norm_loads();
+    float f2 = 0.f, f3 = 0.f;                             // the norms of the patch's 2D token and its 3D token
+    if (!NORMS && g == 0 && live) {
+        f2 = __ldcg(l1 + s.vis_off + p);
+        f3 = __ldcg(l1 + s.vis_off + P + p);
+    }
 
     // Sum over the lanes of a warp that hold the same patch (the lane bits above log2 PP), then over the
     // warps in a fixed order: tot[patch][c].
@@ -160,7 +166,7 @@ __device__ __forceinline__ void patch_indicators_block(const SampleDev& s, int b
         h += step_h; i += step_i;
         if (i >= nq4) { i -= nq4; ++h; }
     }
-    {                                                     // the feature norms, now that every load is in flight
+    if constexpr (NORMS) {                                // the feature norms, now that every load is in flight
         float acc = 0.f;
 #pragma unroll
         for (int k = 0; k < kNormKeep; ++k) acc += abs_sum(hv[k]);
@@ -205,11 +211,12 @@ __device__ __forceinline__ void patch_indicators_block(const SampleDev& s, int b
     reduce(o, 1);
     if (g == 0 && live) {
         constexpr int kRowWarps = kRowThreads / 32;
-        float f2 = 0.f, f3 = 0.f;                         // the patch's 2D token, its 3D token
+        if constexpr (NORMS) {
 #pragma unroll
-        for (int w = 0; w < kRowWarps; ++w) {
-            f2 += rown[pl * kRowWarps + w];
-            f3 += rown[(kIndPatches + pl) * kRowWarps + w];
+            for (int w = 0; w < kRowWarps; ++w) {
+                f2 += rown[pl * kRowWarps + w];
+                f3 += rown[(kIndPatches + pl) * kRowWarps + w];
+            }
         }
         float4 x;
         x.x = f2 / (f2 + f3);                             // Eq. 3-1, the term of this patch

@@ -26,10 +26,10 @@ struct PatchTailPlan {
     int32_t rows;                     // rows that the samples may keep
 };
 
-template <typename T, int PP, class BD>
+template <typename T, int PP, bool NORMS, class BD>
 __global__ void __launch_bounds__(kTailThreads, 1)
 patch_tail_kernel(const __grid_constant__ BD bd, const __grid_constant__ PatchTailPlan tp, int n_heads,
-                  const AlphaOut alpha, const T* __restrict__ hidden, int d_model, float* __restrict__ x_out,
+                  const AlphaOut alpha, const T* __restrict__ hidden, const float* __restrict__ l1, int d_model, float* __restrict__ x_out,
                   float* __restrict__ attn_out, unsigned long long* rec, const PatchParams pp, const PatchIO io,
                   const __grid_constant__ CompactArgs ca, int32_t* list, unsigned int* ticket_counter)
 {
@@ -38,7 +38,7 @@ patch_tail_kernel(const __grid_constant__ BD bd, const __grid_constant__ PatchTa
     if (c < n_ind) {
         int b = 0;
         while (b + 1 < bd.count() && c >= tp.ind0[b + 1]) ++b;
-        patch_indicators_block<T, PP>(bd.at(b), c - tp.ind0[b], n_heads, alpha, hidden, d_model, x_out, attn_out, rec, true);
+        patch_indicators_block<T, PP, NORMS>(bd.at(b), c - tp.ind0[b], n_heads, alpha, hidden, l1, d_model, x_out, attn_out, rec, true);
         return;
     }
     c -= n_ind;
@@ -126,7 +126,7 @@ bool patch_tail_supported(const BatchDesc& bd)
     return bd.n >= 1 && blocks + bd.n < 30000;
 }
 
-cudaError_t launch_patch_tail(const BatchDesc& bd, int n_heads, AlphaOut alpha, int dtype, int d_model, const void* hidden,
+cudaError_t launch_patch_tail(const BatchDesc& bd, int n_heads, AlphaOut alpha, int dtype, int d_model, const void* hidden, const float* l1,
                               float* x_out, float* attn_out, unsigned long long* rec, const PatchParams& pp, const PatchIO& io,
                               const CompactJob& job, int32_t* list, int sm_count, unsigned int* ticket_counter, cudaStream_t stream)
 {
@@ -160,13 +160,17 @@ cudaError_t launch_patch_tail(const BatchDesc& bd, int n_heads, AlphaOut alpha, 
     cudaLaunchAttribute attr[1] = {pdl_attribute()};
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-#define MVLA_TAIL(T, PPV)                                                                                     \
-    if (per == PPV)                                                                                           \
+#define MVLA_TAIL1(T, PPV, NORMS)                                                                             \
+    if (per == PPV && (l1 == nullptr) == NORMS)                                                               \
         return with_desc(bd, [&](const auto& d) {                                                             \
-            return cudaLaunchKernelEx(&cfg, patch_tail_kernel<T, PPV, std::decay_t<decltype(d)>>, d, tp, n_heads, alpha, \
-                                      static_cast<const T*>(hidden), d_model, x_out, attn_out, rec, pp, io, ca, list, ticket_counter); });
-    if (dtype == MVLA_DTYPE_BF16) { MVLA_TAIL(__nv_bfloat16, 8) MVLA_TAIL(__nv_bfloat16, 4) MVLA_TAIL(__nv_bfloat16, 2) }
-    else { MVLA_TAIL(float, 8) MVLA_TAIL(float, 4) MVLA_TAIL(float, 2) }
+            return cudaLaunchKernelEx(&cfg, patch_tail_kernel<T, PPV, NORMS, std::decay_t<decltype(d)>>, d, tp, n_heads, alpha, \
+                                      static_cast<const T*>(hidden), l1, d_model, x_out, attn_out, rec, pp, io, ca, list, ticket_counter); });
+#define MVLA_TAIL(T, PPV) MVLA_TAIL1(T, PPV, true)
+    if (dtype == MVLA_DTYPE_BF16) {
+        MVLA_TAIL(__nv_bfloat16, 8) MVLA_TAIL(__nv_bfloat16, 4) MVLA_TAIL(__nv_bfloat16, 2)
+        MVLA_TAIL1(__nv_bfloat16, 8, false) MVLA_TAIL1(__nv_bfloat16, 4, false) MVLA_TAIL1(__nv_bfloat16, 2, false)
+    } else { MVLA_TAIL(float, 8) MVLA_TAIL(float, 4) MVLA_TAIL(float, 2) }
+#undef MVLA_TAIL1
 #undef MVLA_TAIL
     return cudaErrorInvalidConfiguration;
 }

@@ -31,6 +31,9 @@ namespace {
 constexpr int kSoftWarps = 8;
 constexpr int kSoftThreads = kSoftWarps * 32;
 constexpr int kStreamThreads = kSoftThreads + 64;     // + the loading warp and the MMA warp
+constexpr int kNormWarps = 2;                         // + these, in launches with the attention copy
+constexpr int kNormStages = 3;                        // pieces of rows in flight per norm warp
+constexpr uint32_t kNormPiece = 8192;
 constexpr int kMaxStages = 12;
 constexpr uint32_t kStageBytes = 16384;               // 128 keys x 128 bytes: one swizzled box of a key tile
 constexpr int kMaxSlots = 32;
@@ -49,12 +52,19 @@ struct StreamArgs {
     int32_t* rearm;               // see launch_salience_fast
     unsigned long long* rearm_rec;
     unsigned long long* stamps;
+    // feature norms (null: none): bf16 rows of `row_bytes` bytes, their L1 norms, where the pieces in flight lie in dynamic shared memory
+    const uint8_t* hidden;
+    float* l1;
+    int row_bytes;
+    uint32_t norm_off;
+    int n_samples;
 };
 
 struct StreamSmem {
     alignas(8) uint64_t kfull[kMaxStages], kempty[kMaxStages];
     uint64_t qfull[2], qempty[2];
     uint64_t tfull[kMaxSlots], tempty[kMaxSlots];
+    uint64_t nfull[kNormWarps][kNormStages];
     uint64_t xbar[kPairBufs];                      // pairs of the cluster's CTAs have landed
     alignas(16) float m[kSoftWarps][kMaxText];     // per warp and query: -reference (log2 domain; +inf: no key)
     alignas(16) float w[kSoftWarps][kMaxText];     // ... its sum of exponentials, then its weight
@@ -353,7 +363,80 @@ __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, in
     __syncwarp();
 }
 
-// grid = clusters x cluster size (1-D), kStreamThreads threads, one CTA per multiprocessor.
+// One norm warp: L1 norms of its share of the visual rows of all samples, every n_w-th of them.  Rows come by bulk
+// copies, kNormStages pieces in flight per warp, so that they take their part of the memory bandwidth without registers
+// or a CTA of their own.
+__device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs& a, StreamSmem& sm, uint32_t buf, int nw, int lane)
+{
+    const bool one = elect_one();
+    int rows = 0;                                        // of all samples
+    for (int b = 0; b < a.n_samples; ++b) rows += bd.s[b].n_2d + bd.s[b].n_3d;
+    const int w = static_cast<int>(blockIdx.x) * kNormWarps + nw, n_w = static_cast<int>(gridDim.x) * kNormWarps;
+    const int pieces = (a.row_bytes + static_cast<int>(kNormPiece) - 1) / static_cast<int>(kNormPiece), n = w < rows ? ((rows - 1 - w) / n_w + 1) * pieces : 0;
+    // The row next to be fetched: sample fb, visual index fv; and the one next to be summed goes to *out.
+    int fb = 0, fv = w;
+    float* out = a.l1 + bd.s[0].vis_off + w;             // (visual arrays are packed over the samples of the launch)
+    int fp = 0;
+    auto settle = [&]() {
+        while (fb < a.n_samples - 1 && fv >= bd.s[fb].n_2d + bd.s[fb].n_3d) { fv -= bd.s[fb].n_2d + bd.s[fb].n_3d; ++fb; }
+    };
+    settle();
+    auto fetch = [&](int st) {
+        const SampleDev& s = bd.s[fb];
+        const int row = s.seq_off + (fv < s.n_2d ? s.off_2d + fv : s.off_3d + (fv - s.n_2d));
+        const uint32_t at = static_cast<uint32_t>(fp) * kNormPiece, bytes = min(kNormPiece, static_cast<uint32_t>(a.row_bytes) - at);
+        if (one) {
+            const uint32_t bar = smem_u32(&sm.nfull[nw][st]);
+            mbar_expect_tx(bar, bytes);
+            bulk_load(buf + static_cast<uint32_t>(st) * kNormPiece, a.hidden + static_cast<int64_t>(row) * a.row_bytes + at, bytes, bar);
+        }
+        if (++fp == pieces) {
+            fp = 0;
+            fv += n_w;
+            settle();
+        }
+    };
+    pdl_wait();                                          // the rows may come from the kernel before this one
+    for (int i = 0; i < min(kNormStages, n); ++i) fetch(i);
+    int st = 0, piece = 0;
+    uint32_t phase = 0;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int i = 0; i < n; ++i) {
+        const bool ok = ring_wait<false>(smem_u32(&sm.nfull[nw][st]), phase, &sm.aborted, a.status);
+        if (!__all_sync(0xffffffffu, ok)) {              // gave up: let the copies in flight land before the CTA may end
+            const uint64_t t0 = global_ns();
+            while (global_ns() - t0 < 1000000ull) { }
+            break;
+        }
+        const uint32_t bytes = min(kNormPiece, static_cast<uint32_t>(a.row_bytes) - static_cast<uint32_t>(piece) * kNormPiece);
+        const uint32_t src = buf + static_cast<uint32_t>(st) * kNormPiece;
+#pragma unroll 4
+        for (uint32_t at = lane * 16; at < bytes; at += 512) {
+            uint32_t u[4];
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]) : "r"(src + at));
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                acc[e] += fabsf(__uint_as_float(u[e] << 16));           // low bf16
+                acc[e] += fabsf(__uint_as_float(u[e] & 0xFFFF0000u));   // high bf16
+            }
+        }
+        __syncwarp();                                    // everyone has read the piece
+        if (i + kNormStages < n) fetch(st);
+        if (++st == kNormStages) { st = 0; phase ^= 1; }
+        if (++piece == pieces) {
+            piece = 0;
+            float r = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+            for (int off = 16; off >= 1; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+            if (lane == 0) *out = r;
+            out += n_w;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[e] = 0.f;
+        }
+    }
+}
+
+// grid = clusters x cluster size (1-D), one CTA per multiprocessor.
 // ROOM: the feature norms are to run beside this kernel.  Its ten warps put three on two of a multiprocessor's four
 // register files (16384 registers each): at the 168 registers a thread that the compiler takes these are full, no CTA of
 // the norms fits, and they start when the scores are done.  144 leave room for two warps of 32 registers in each (adaptive
@@ -391,6 +474,8 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             mbar_init(smem_u32(&sm.qfull[i]), 1); mbar_init(smem_u32(&sm.qempty[i]), 1);
         }
         for (int i = 0; i < kPairBufs; ++i) mbar_init(smem_u32(&sm.xbar[i]), 1);
+        if (!ROOM)
+            for (int i = 0; i < kNormWarps * kNormStages; ++i) mbar_init(smem_u32(&sm.nfull[0][0] + i), 1);
         for (int i = 0; i < a.slots; ++i) { mbar_init(smem_u32(&sm.tfull[i]), 1); mbar_init(smem_u32(&sm.tempty[i]), 4); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sm.aborted = 0;
@@ -496,6 +581,10 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             }
             if (ok && one) umma_commit(smem_u32(&sm.qempty[qb]));
         }
+    } else if (!ROOM && warp > kSoftWarps + 1) {
+        // ---------------------------------------------------------------- feature norms
+        const int nw = warp - kSoftWarps - 2;
+        if (a.hidden) norm_warp(bd, a, sm, smem_u32(dyn) + a.norm_off + static_cast<uint32_t>(nw * kNormStages) * kNormPiece, nw, lane);
     } else {
         // ---------------------------------------------------------------- softmax
         SoftJob j;
@@ -609,12 +698,13 @@ cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUte
     if (e != cudaSuccess) return e;
     // a second wave of a persistent grid would double its time
     int n = 0;
-    e = clusters_at_once(ks, reinterpret_cast<const void*>(kern), kStreamThreads, smem, cluster, &n);
+    const int threads = kStreamThreads + (a.hidden ? 32 * kNormWarps : 0);
+    e = clusters_at_once(ks, reinterpret_cast<const void*>(kern), threads, smem, cluster, &n);
     if (e != cudaSuccess) return e;
     if (n < 1) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(std::min(a.n_jobs, n) * cluster));
-    cfg.blockDim = dim3(kStreamThreads);
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -637,7 +727,7 @@ static_assert(kSmemPerSm - static_cast<int>(kStreamSmem + sizeof(StreamSmem)) - 
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
                                    AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
-                                   unsigned long long* stamps, bool norms_beside, cudaStream_t stream)
+                                   unsigned long long* stamps, bool norms_beside, const void* hidden, int row_bytes, float* l1, cudaStream_t stream)
 {
     const int sms = sm_count_of_current_device();
     const int npad = padded_text(bd), tiles = max_tiles(bd);
@@ -655,8 +745,13 @@ cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_grou
         cluster *= 2;
     if ((tiles + cluster - 1) / cluster > a.slots) return cudaErrorInvalidConfiguration;
     const size_t q_bytes = 2 * static_cast<size_t>((head_dim * esize + 127) / 128) * npad * 128;
-    a.stages = static_cast<int>(std::min<size_t>(kMaxStages, (kStreamSmem - 1024 - q_bytes) / kStageBytes));
-    if (a.stages < 4) return cudaErrorInvalidConfiguration;
+    // shared memory: the ring of key boxes, two buffers of queries, the norm warps' pieces of rows
+    const size_t norm_bytes = hidden ? static_cast<size_t>(kNormWarps * kNormStages) * kNormPiece : 0;
+    a.stages = static_cast<int>(std::min<size_t>(kMaxStages, (kStreamSmem - 1024 - q_bytes - norm_bytes) / kStageBytes));
+    if (a.stages < 4 || (hidden && norms_beside)) return cudaErrorInvalidConfiguration;
+    a.hidden = static_cast<const uint8_t*>(hidden);
+    a.l1 = l1; a.row_bytes = row_bytes; a.n_samples = bd.n;
+    a.norm_off = static_cast<uint32_t>(a.stages * kStageBytes + q_bytes);
     if (norms_beside && !alpha.ptr) return launch_stream<true>(bd, tmap_q, tmap_k, a, cluster, kStreamSmem, stream);
     return launch_stream<false>(bd, tmap_q, tmap_k, a, cluster, kStreamSmem, stream);
 }

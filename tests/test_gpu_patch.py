@@ -337,3 +337,27 @@ def test_patch_step_scored_by_the_streaming_kernel(batch, H, d, n_txt, n_patch):
     for step in (0, 1):
         run_patch_step(ctx, wl, step, states)
     ctx.close()
+
+
+@pytest.mark.parametrize("D", [8, 2056, 4096, 4104])          # pieces of 8 KB a row: one of 16 bytes; a part; one; one and 16 bytes
+@pytest.mark.parametrize("n_patch", [(129, 64, 200, 1, 90, 130, 256, 77), (100,) * 8])
+def test_patch_step_with_feature_norms_taken_beside_the_scores(D, n_patch):
+    """Batches scored by the streaming kernel have their feature norms taken by two of its warps; rows of every sample, in
+    pieces that end anywhere; two action steps (the tail's hand-over words and the norms are written again)."""
+    wl = W.patch_workload(61, batch=8, D=D, H=32, d=64, n_txt=(5, 33, 17, 64, 16, 20, 48, 9), n_patch=n_patch, steps=2)
+    ctx = mvla.context_for(wl)
+    states = [oracle.PatchState(s.n_2d) for s in wl.samples]
+    for step in (0, 1):
+        run_patch_step(ctx, wl, step, states)
+    ctx.close()
+
+
+def test_patch_step_rows_of_very_unequal_samples():
+    """The tail deals output rows out over all copying CTAs, whatever sample they belong to: samples of a few rows beside one of
+    hundreds, the last one the smallest (nobody knows the total before it is decided)."""
+    wl = W.patch_workload(62, batch=5, D=256, H=4, d=64, n_txt=(1, 64, 3, 20, 1), n_patch=(1, 600, 2, 130, 1), steps=2, text_first=True)
+    ctx = mvla.context_for(wl)
+    states = [oracle.PatchState(s.n_2d) for s in wl.samples]
+    for step in (0, 1):
+        run_patch_step(ctx, wl, step, states)
+    ctx.close()
