@@ -22,6 +22,7 @@ constexpr int kTailThreads = kIndThreads;
 
 struct PatchTailPlan {
     int16_t ind0[kMaxChunk + 1];      // first indicator CTA of every sample; ind0[n] = their number
+    int16_t lag;                      // see the kernel
     int16_t copiers;                  // copying CTAs
     int32_t rows;                     // rows that the samples may keep
 };
@@ -33,23 +34,32 @@ patch_tail_kernel(const __grid_constant__ BD bd, const __grid_constant__ PatchTa
                   float* __restrict__ attn_out, unsigned long long* rec, const PatchParams pp, const PatchIO io,
                   const __grid_constant__ CompactArgs ca, int32_t* list, unsigned int* ticket_counter)
 {
-    const int n_ind = tp.ind0[bd.count()];
+    // Roles by ticket: the indicator CTAs of sample after sample, behind those of sample b the selecting CTA of sample b - lag
+    // (whose indicators are then about done: a selecting CTA that waits keeps a multiprocessor from the others), the selecting CTAs of
+    // the last samples, the copying CTAs.  With all selecting CTAs behind all indicator CTAs the first list of 16 samples of 512
+    // tokens came when the last indicators were done: 78.7 -> 74.2 us (74.0 with a lag of 3 samples instead of 6, 76.4 with 9).
+    const int n = bd.count(), n_ind = tp.ind0[n];
     int c = cta_ticket(ticket_counter);
-    if (c < n_ind) {
+    int sel = -1;
+    if (c < n_ind + max(0, n - tp.lag)) {
         int b = 0;
-        while (b + 1 < bd.count() && c >= tp.ind0[b + 1]) ++b;
-        patch_indicators_block<T, PP, NORMS>(bd.at(b), c - tp.ind0[b], n_heads, alpha, hidden, l1, d_model, x_out, attn_out, rec, true);
-        return;
+        while (b + 1 < n && c >= tp.ind0[b + 1] + max(0, b + 1 - tp.lag)) ++b;
+        const int at = c - tp.ind0[b] - max(0, b - tp.lag);
+        if (at < tp.ind0[b + 1] - tp.ind0[b]) {
+            patch_indicators_block<T, PP, NORMS>(bd.at(b), at, n_heads, alpha, hidden, l1, d_model, x_out, attn_out, rec, true);
+            return;
+        }
+        sel = b - tp.lag;
+    } else if (c < n_ind + n) {
+        sel = c - n_ind;
     }
-    c -= n_ind;
-    if (c < bd.count()) {
+    if (sel >= 0) {
         __shared__ PatchSmemT<kTailThreads> sm;
-        const SampleDev& s = bd.at(c);
-        patch_select_block<kTailThreads>(s, c, bd.count(), pp, io, sm, rec, tp.copiers > 0 ? list + bd.at(0).cap_off : nullptr);
+        patch_select_block<kTailThreads>(bd.at(sel), sel, n, pp, io, sm, rec, tp.copiers > 0 ? list + bd.at(0).cap_off : nullptr);
         return;
     }
+    c -= n_ind + n;
     // ---- row copy
-    c -= bd.count();
     const int tid = threadIdx.x, lane = tid & 31;
     const int w = c * (kTailThreads / 32) + (tid >> 5), nw = tp.copiers * (kTailThreads / 32);
     asm volatile("griddepcontrol.wait;" ::: "memory");      // the words were re-armed by the kernel before this one
@@ -146,6 +156,8 @@ cudaError_t launch_patch_tail(const BatchDesc& bd, int n_heads, AlphaOut alpha, 
         next += (bd.s[b].n_2d + per - 1) / per;
     }
     for (int b = bd.n; b <= kMaxChunk; ++b) tp.ind0[b] = static_cast<int16_t>(next);
+    // samples whose indicators fill the multiprocessors, and one more
+    tp.lag = static_cast<int16_t>(1 + (sm_count * bd.n + next - 1) / std::max(next, 1));
     const CompactArgs ca = compact_args(job);
     // together with the selecting CTAs they fill the multiprocessors once the indicator CTAs have retired
     const int copiers = ca.seg_begin[3] > 0 ? std::max(sm_count - bd.n, 1) : 0;
