@@ -75,7 +75,9 @@ extern "C" {
                                          writes, the library orders this call after everything enqueued so far.)
                                          Scoring and selection then run on one of a small ring of streams owned by the
                                          context, beside the selection and row copy of the steps before; the row copy
-                                         stays on `stream` and waits for the step's selection.  Every result of the
+                                         stays on `stream` and waits for the step's selection.  (Small steps of one
+                                         sample outside a stream capture stay on `stream` as a whole; their scores are
+                                         taken beside the selection and row copy of the step before.)  Every result of the
                                          call is complete in the order of `stream`, as without the flag, and the
                                          smoothed state is updated in call order.  Without the flag every kernel waits
                                          for all earlier work of `stream`. */

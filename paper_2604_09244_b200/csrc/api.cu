@@ -19,6 +19,14 @@ namespace {
 constexpr int kMaxBatch = 64;       // samples per call (mvla_prune_create refuses more)
 constexpr int kMapSlots = 16;       // tensor maps a context remembers
 constexpr int kSets = 6;            // scratch sets = prune steps that may be in flight at once
+// Steps of one sample with stable inputs, one key tile per scoring CTA, that move no more than this (keys, feature rows, text
+// queries, surviving rows in and out) are chained on the caller's stream, with the scores of a step taken beside the selection and
+// row copy of the one before: two or three launches, where the fork to a side stream is three or four launches and four event
+// calls, 10 to 14 us of host time on different hosts.  Per request of eight in a row, fork / chain in us, 32 heads: 630 tokens, heads of 64
+// (9 MB), adaptive 18.7 / 10.2, fixed 11.2 / 7.7; 750 of 128 (20 MB) 13.5 / 10.3, 11.4 to 14.4 / 10.9; 1010 of 96 (20 MB) 14.0 / 11.8, 11.5 / 11.1.
+// Above, the GPU is the limit, and a fork overlaps more: 1010 of 128 (27 MB), fixed, 11.3 / 15.1; two tiles per CTA: 1280 of
+// 64 (17 MB) 11.3 / 12.1, of 96 (26 MB) 11.4 / 14.3, adaptive 14.0 / 18.5.  (In a CUDA graph launches cost nothing: always the fork.)
+constexpr size_t kChainBytes = 20u << 20;
 
 // Tracing and logging, both on the host and off the device's path: every public call is an NVTX range (a profiler
 // shows the call and, inside mvla_prune_step, its phases around the kernels they enqueue; without a profiler
@@ -106,6 +114,7 @@ struct mvla_ctx {
     Range hist[kSets][16];
     int n_hist[kSets];
     bool hist_unknown;                         // the stream ran other work of this context since: order after it
+    cudaStream_t last_stream;                  // of the last prune step
     // Smoothed states (prune point x slot) that the step last run on each scratch set reads and writes:
     // a later selection touching one of them waits for that selection, others need not.
     int32_t state_of[kSets][kMaxChunk];
@@ -380,7 +389,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
                            cudaStream_t st, AlphaOut alpha = AlphaOut{nullptr, 0, 0},
                            int32_t* rearm = nullptr, bool norms_beside = false, unsigned long long* stamps = nullptr,
                            bool with_cache = false, unsigned long long* rearm_rec = nullptr, float* attn_out = nullptr,
-                           bool* norms_inside = nullptr)
+                           bool* norms_inside = nullptr, bool early = false)
 {
     if (used_acc64) *used_acc64 = false;
     const mvla_config& c = ctx->cfg;
@@ -436,7 +445,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
         e = launch_salience_fast(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk,
                                  tiles_per_cta, cluster, npad,
                                  acc64, ctx->status_dev, alpha, rearm, rearm_rec, stamps,
-                                 with_cache ? ctx->lcache : nullptr, ctx->max_vis, ctx->cache_cols, st);
+                                 with_cache ? ctx->lcache : nullptr, ctx->max_vis, ctx->cache_cols, early, st);
         if (used_acc64) *used_acc64 = acc64 != nullptr;
     } else {
         e = launch_salience(bd, c.dtype, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, q, k, tq, tk, ctx->use_umma, tiles_per_cta,
@@ -494,6 +503,35 @@ struct ForkPlan {
     unsigned long long cap_id = 0;       // stream capture the events of this step belong to (0: none)
 };
 
+// A buffer that a step in flight beside the others (those remembered) writes, among `r`.
+bool clashes(const mvla_ctx* ctx, unsigned par, const mvla_ctx::Range* r, int n)
+{
+    for (unsigned s = 0; s < kSets; ++s) {
+        if (s == par) continue;
+        for (int i = 0; i < n; ++i)
+            for (int j = 0; j < ctx->n_hist[s]; ++j)
+                if (r[i].lo && r[i].lo < ctx->hist[s][j].hi && ctx->hist[s][j].lo < r[i].hi) return true;
+    }
+    return false;
+}
+
+// Remembers what the step on scratch set `par` writes and which smoothed states it touches.
+void remember(mvla_ctx* ctx, unsigned par, int32_t prune_point, int32_t batch, const mvla_sample* samples, const mvla_ctx::Range* side,
+              int n_side_written, const mvla_ctx::Range* copied, int n_copied)
+{
+    if (ctx->hist_unknown) {
+        for (int& n : ctx->n_hist) n = 0;
+        for (int& n : ctx->n_state_of) n = 0;
+    }
+    int m = 0;
+    for (int i = 0; i < n_side_written; ++i) if (side[i].lo) ctx->hist[par][m++] = side[i];
+    for (int i = 0; i < n_copied; ++i) if (copied[i].lo) ctx->hist[par][m++] = copied[i];
+    ctx->n_hist[par] = m;
+    ctx->hist_unknown = false;
+    for (int b = 0; b < batch; ++b) ctx->state_of[par][b] = prune_point * ctx->n_slots + samples[b].state_slot;
+    ctx->n_state_of[par] = batch;
+}
+
 // `side`: buffers the side-stream work reads or writes, the first `n_side_written` of them written by it;
 // `copied`: buffers the row copy writes.  Enqueues the wait that opens the side stream and records what the
 // step writes and which states it touches.
@@ -504,13 +542,7 @@ int32_t plan_fork(mvla_ctx* ctx, cudaStream_t st, unsigned par, int32_t prune_po
     cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
     if (cudaStreamGetCaptureInfo(st, &cst, &fp->cap_id) != cudaSuccess) return fail_cuda(ctx, cudaGetLastError());
     if (cst != cudaStreamCaptureStatusActive) fp->cap_id = 0;
-    bool clash = ctx->hist_unknown;
-    for (unsigned s = 0; !clash && s < kSets; ++s) {
-        if (s == par) continue;
-        for (int i = 0; !clash && i < n_side; ++i)
-            for (int j = 0; !clash && j < ctx->n_hist[s]; ++j)
-                clash = side[i].lo && side[i].lo < ctx->hist[s][j].hi && ctx->hist[s][j].lo < side[i].hi;
-    }
+    const bool clash = ctx->hist_unknown || clashes(ctx, par, side, n_side);
     // earlier selections still possibly in flight that touch a smoothed state this step touches: the
     // state is updated in call order, so this step's selection waits for the most recent one per
     // state (dep_mask; that one has in turn waited for those before it).  Steps older than
@@ -536,22 +568,11 @@ int32_t plan_fork(mvla_ctx* ctx, cudaStream_t st, unsigned par, int32_t prune_po
     if (fp->ordered_after_all) {
         e = cudaEventRecord(ctx->ev_fork, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->aux[par], ctx->ev_fork, 0);
-        if (ctx->hist_unknown) {
-            for (int& n : ctx->n_hist) n = 0;
-            for (int& n : ctx->n_state_of) n = 0;
-        }
     } else {
         e = cudaStreamWaitEvent(ctx->aux[par], ctx->ev_copy[par], 0);
     }
     if (e != cudaSuccess) return fail_cuda(ctx, e);
-    // remember what this step writes
-    int m = 0;
-    for (int i = 0; i < n_side_written; ++i) if (side[i].lo) ctx->hist[par][m++] = side[i];
-    for (int i = 0; i < n_copied; ++i) if (copied[i].lo) ctx->hist[par][m++] = copied[i];
-    ctx->n_hist[par] = m;
-    ctx->hist_unknown = false;
-    for (int b = 0; b < batch; ++b) ctx->state_of[par][b] = prune_point * ctx->n_slots + samples[b].state_slot;
-    ctx->n_state_of[par] = batch;
+    remember(ctx, par, prune_point, batch, samples, side, n_side_written, copied, n_copied);
     return MVLA_OK;
 }
 
@@ -1215,7 +1236,7 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
     float* l1_ws = ctx->l1_ws + ctx->step_parity * ctx->vis_all;
     // With stable inputs (and the fast scoring kernel, whose scratch rotates over kSets sets) scoring and
     // selection go to the side stream of this step's scratch set (see plan_fork).
-    bool forked = false;
+    bool forked = false, chained = false, early = false;
     ForkPlan fp;
     const unsigned par = ctx->step_parity;
     const size_t nvis_b = static_cast<size_t>(plan.total_vis), nout_b = static_cast<size_t>(plan.total_out);
@@ -1233,11 +1254,25 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
             range_of(adaptive ? in->hidden : nullptr, in_rows * hb)};
         const mvla_ctx::Range copied[3] = {range_of(out->out_hidden, nout_b * hb), range_of(out->out_k, nout_b * kb),
                                            range_of(out->out_v, nout_b * kb)};
-        rc = plan_fork(ctx, st, par, prune_point, batch, samples, side, 10, 7, copied, 3, &fp);
-        if (rc != MVLA_OK) return rc;
+        cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cst) != cudaSuccess) return fail_cuda(ctx, cudaGetLastError());
+        const SampleDev& one = plan.s[0];
+        const size_t moved = nvis_b * (kb + (adaptive ? hb : 0)) + static_cast<size_t>(one.n_txt) * qb + 2 * nout_b * (hb + 2 * kb);
+        if (batch == 1 && moved <= kChainBytes && cst == cudaStreamCaptureStatusNone && tiles_per_cta_of(tiles_of(one)) == 1) {
+            forked = false;
+            chained = true;
+            // (the first step of a chain, and its selection and row copy in any case, wait for all earlier work of the stream)
+            early = !ctx->hist_unknown && ctx->last_stream == st && !clashes(ctx, par, side + 7, 3);
+            remember(ctx, par, prune_point, batch, samples, side, 7, copied, 3);
+            ctx->sel_valid[par] = false;               // this set is used outside the event chain
+        } else {
+            rc = plan_fork(ctx, st, par, prune_point, batch, samples, side, 10, 7, copied, 3, &fp);
+            if (rc != MVLA_OK) return rc;
+        }
     } else {
         ctx->hist_unknown = true;
     }
+    ctx->last_stream = st;
     for (int first = 0; first < batch; first += kMaxChunk) {
         const int n = std::min(kMaxChunk, batch - first);
         const BatchDesc bd = chunk_of(plan, first, n);
@@ -1247,10 +1282,10 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         ph.mark("mvla: scoring");
         rc = run_salience_chunk(ctx, bd, in->q, in->k, in->rows, adaptive ? in->hidden : nullptr, l1_ws, acc64,
                                 &used_acc64, forked ? ctx->aux[par] : st, AlphaOut{nullptr, 0, 0},
-                                tail ? ctx->tail_list + par * ctx->rows_all : nullptr, tail, tail ? ctx->stamps : nullptr,
-                                cache_on);
+                                tail ? ctx->tail_list + par * ctx->rows_all : nullptr, tail, tail && !chained ? ctx->stamps : nullptr,
+                                cache_on, nullptr, nullptr, nullptr, early);
         if (rc != MVLA_OK) return rc;
-        if (ctx->stage_event && !forked) {
+        if (ctx->stage_event && !forked && !chained) {
             // under stream capture the record must become an event-record node of the graph (an "external"
             // record): only then can the event be timed after a replay
             cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
@@ -1280,8 +1315,8 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
             ctx->sel_valid[par] = false;             // this set was used outside the event chain
             ph.mark("mvla: selection + row copy");
             const cudaError_t e2 = launch_select_copy(bd, gp, io, job, ctx->tail_list + par * ctx->rows_all,
-                                                      ctx->status_dev,
-                                                      ctx->stamps ? ctx->stamps + 2 * kStampSlots : nullptr, st);
+                                                      ctx->status_dev, chained,
+                                                      ctx->stamps && !chained ? ctx->stamps + 2 * kStampSlots : nullptr, st);
             if (e2 != cudaSuccess) {
                 clear_accumulators(acc64, bd, st);
                 return fail_cuda(ctx, e2);

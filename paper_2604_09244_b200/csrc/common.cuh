@@ -161,6 +161,7 @@ struct AlphaOut {
 };
 
 bool fast_salience_supported(int tiles_per_cta);
+// `early`: q and k are stable, and nothing still in flight but the kernel right before this one: the scores are taken beside it.
 // `kv_group`: query heads per key head (1 unless the keys are grouped); the key tensor map then has
 // n_heads / kv_group heads.
 // `esize`: bytes per element of q and k (2: bf16, 1: e4m3).
@@ -168,7 +169,7 @@ cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group,
                                  const CUtensorMap* tmap_k, int tiles_per_cta, int cluster, int npad,
                                  unsigned long long* acc64, int* status,
                                  AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
-                                 float* lcache, int cache_vis, int cache_cols, cudaStream_t stream);
+                                 float* lcache, int cache_vis, int cache_cols, bool early, cudaStream_t stream);
 
 // Of such a launch without the logit cache: CTAs that fit on a multiprocessor, and, where that is one, clusters (one per
 // sample and head) that run at once on the device.
@@ -258,10 +259,12 @@ cudaError_t launch_compact(const BatchDesc& bd, const CompactJob& job, const int
 // (bounded waits, MVLA_ERR_TIMEOUT into `status` when one runs out): no kernel boundary, fence or flag lies
 // between selection and copy.  `list`: one int per output row of the batch, all -1 when the kernel starts
 // (the scoring kernel before it re-arms them, see launch_salience_fast).
+// `stable`: the scoring kernel of a later step may run beside this one, and this one may start before the step before it is
+// complete (launch_salience_fast, `early`).  One sample of up to 1024 visual tokens.
 // The CTAs are no more than fit on the device at once, see the kernel.  `stamps`: as in launch_salience_fast
 // (start: past the wait for the kernel before; the selecting CTA's end is when the list is written).
 cudaError_t launch_select_copy(const BatchDesc& bd, const GateParams& gp, const SelectIO& io, const CompactJob& job,
-                               int32_t* list, int* status, unsigned long long* stamps, cudaStream_t stream);
+                               int32_t* list, int* status, bool stable, unsigned long long* stamps, cudaStream_t stream);
 
 // One warp runs the copying CTAs' bounded wait on `never_set` (a word that holds -1 and stays so) with the
 // given limit and reports MVLA_ERR_TIMEOUT into `status` when it runs out.

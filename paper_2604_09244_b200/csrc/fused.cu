@@ -46,6 +46,7 @@ struct FastOut {
     int* status;
     int n_heads;
     AlphaOut alpha;
+    bool early;                              // the accumulators need no wait
 };
 
 // From the raw dot products of this thread's key(s) -- L[t * TC + i]: tile t, text query c0 + i -- to the outputs.
@@ -179,7 +180,7 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
 
     // ---- per key: sum over queries of the normalised probabilities (this head's contribution)
     const float* const w = sm.w[kwarp] + c0;  // 0 past the text queries
-    pdl_wait();                               // the accumulators were read and cleared by an earlier selection
+    if (!o.early) pdl_wait();                 // the accumulators were read and cleared by an earlier selection
 #pragma unroll
     for (int t = 0; t < NTILE; ++t) {
         if (key >= valid[t]) continue;
@@ -217,7 +218,8 @@ __device__ __forceinline__ void softmax_scores(float (&L)[NTILE * TCOL / SPLIT],
 // SPLIT: threads per key.  1: a thread holds all the logits of its key.  2: threads t and t + 128 hold one half of the
 // text queries each -- the chain through exponentials, sums and weighted sum is half as long per warp, and a scheduler
 // has two warps to alternate between; both halves add into the key's accumulator.
-enum { kPlain = 0, kWithCache = 1, kForPatches = 2 };   // scores only; with the logit cache; the attention copy instead of scores
+// scores only; with the logit cache; the attention copy instead of scores; scores of a step with stable inputs, beside the kernel before
+enum { kPlain = 0, kWithCache = 1, kForPatches = 2, kEarly = 3 };
 template <int TCOL, int NTILE, int SPLIT, int KIND, class BD>
 __global__ void __launch_bounds__(kFastThreads * SPLIT, 1)
 salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUtensorMap tmap_q,
@@ -226,6 +228,7 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
                      int* status, const AlphaOut alpha, int32_t* __restrict__ rearm, unsigned long long* __restrict__ rearm_rec,
                      unsigned long long* __restrict__ stamps, float* __restrict__ lcache, int cache_vis, int cache_cols)
 {
+    constexpr bool early = KIND == kEarly;
     constexpr int CC = TCOL * NTILE;                      // tensor-memory columns of the CTA
     constexpr int TC = TCOL / SPLIT;                      // columns (text queries) of a tile that one thread holds
     constexpr int NT = kFastThreads * SPLIT;
@@ -340,8 +343,8 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
     // elected lane issues, so that coordinates and descriptors stay in uniform registers.  (In a single-thread branch
     // every operand is moved to a uniform register one by one: 0.1 us more for the MMAs of a tile.)
     if (warp == 0) {
-        // Inputs may come from the kernel before this one.
-        pdl_wait();
+        // Inputs may come from the kernel before this one (not in a step whose inputs are promised stable: `early`).
+        if (!early) pdl_wait();
         // (no tile to compute: nothing is fetched, both barriers below complete at once)
         if (one) mbar_expect_tx(bar_full, live > 0 ? static_cast<uint32_t>(khalves) * (npad * 128 + live * 16384) : 0u);
 #pragma unroll
@@ -424,12 +427,14 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
     }
     tc_fence_before();
     softmax_scores<TCOL, NTILE, SPLIT, KIND == kForPatches>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
-                                       FastOut{acc64, status, n_heads, alpha}, [&]() {
+                                       FastOut{acc64, status, n_heads, alpha, early}, [&]() {
         if (warp == 3) {
             tc_fence_after();
             tmem_dealloc(tmem_base, tmem_cols);
         }
     });
+    // "This kernel is complete" implies that the one before it is, for whoever comes after: one CTA sees to that last.
+    if (early && tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) pdl_wait();
     if (stamps) {
         __syncthreads();
         if (tid == 0) {
@@ -552,7 +557,7 @@ salience_f32_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUten
         }
     }
     softmax_scores<TCOL, NTILE, 2, false>(L, s, valid, vis0, ok, npad, h, cscale, bar_x, sm,
-                                   FastOut{acc64, status, n_heads, AlphaOut{nullptr, 0, 0}}, []() {});
+                                   FastOut{acc64, status, n_heads, AlphaOut{nullptr, 0, 0}, false}, []() {});
     if (stamps) {
         __syncthreads();
         if (tid == 0) {
@@ -617,7 +622,7 @@ cudaError_t with_fast_variant(const BatchDesc& bd, int npad, int tiles_per_cta, 
 #define MVLA_FAST1(TC, NTL, SP, KD)                                                                             \
     if (tcol == TC && tiles_per_cta == NTL && split == SP && kind == KD)                                        \
         return with_desc(bd, [&](const auto& d) { return use(FastVariant<TC, NTL, SP, KD, std::decay_t<decltype(d)>>{}, d); });
-#define MVLA_FAST(TC, NTL, SP) MVLA_FAST1(TC, NTL, SP, kPlain) MVLA_FAST1(TC, NTL, SP, kWithCache) MVLA_FAST1(TC, NTL, SP, kForPatches)
+#define MVLA_FAST(TC, NTL, SP) MVLA_FAST1(TC, NTL, SP, kPlain) MVLA_FAST1(TC, NTL, SP, kWithCache) MVLA_FAST1(TC, NTL, SP, kForPatches) MVLA_FAST1(TC, NTL, SP, kEarly)
     MVLA_FAST(16, 1, 1) MVLA_FAST(16, 2, 1) MVLA_FAST(32, 1, 2) MVLA_FAST(64, 1, 2) MVLA_FAST(32, 2, 2) MVLA_FAST(64, 2, 2)
 #undef MVLA_FAST1
 #undef MVLA_FAST
@@ -678,10 +683,10 @@ cudaError_t launch_salience_fast(const BatchDesc& bd, int n_heads, int kv_group,
                                  const CUtensorMap* tmap_k, int tiles_per_cta, int cluster, int npad,
                                  unsigned long long* acc64, int* status,
                                  AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec, unsigned long long* stamps,
-                                 float* lcache, int cache_vis, int cache_cols, cudaStream_t stream)
+                                 float* lcache, int cache_vis, int cache_cols, bool early, cudaStream_t stream)
 {
     if ((acc64 == nullptr) == (alpha.ptr == nullptr)) return cudaErrorInvalidConfiguration;      // one or the other
-    return with_fast_variant(bd, npad, tiles_per_cta, alpha.ptr ? kForPatches : (lcache ? kWithCache : kPlain), [&](auto v, const auto& d) {
+    return with_fast_variant(bd, npad, tiles_per_cta, alpha.ptr ? kForPatches : (lcache ? kWithCache : (early ? kEarly : kPlain)), [&](auto v, const auto& d) {
         return launch_fast_t<decltype(v)>(d, n_heads, kv_group, head_dim, esize, tmap_q, tmap_k, cluster, npad, acc64, status,
                                           alpha, rearm, rearm_rec, stamps, lcache, cache_vis, cache_cols, stream);
     });

@@ -128,9 +128,12 @@ __device__ __forceinline__ int block_exscan(int x, int* warp_tot, int* total)
 //              previous state and of the norms follow griddepcontrol.wait; true: the state is loaded before it
 //              (the caller guarantees that it was written before this kernel could start), and the next kernel
 //              is released only after the list.
+//   stable   : the next kernel may become resident as soon as the kernel before this one is complete, and the previous state is
+//              loaded after the wait.
 struct SelectRole {
     int32_t* list = nullptr;
     bool late_pdl = false;
+    bool stable = false;
 };
 struct NoHook {
     __device__ void operator()() const {}
@@ -156,7 +159,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
     const bool k_fixed = s.k_2d_fixed >= 0;
 
     // prologue that needs nothing from the previous kernel
-    if (!role.late_pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!role.late_pdl && !role.stable) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     auto clear_hist = [&]() {
         for (int i = tid; i < kSelBins / 4; i += NT) reinterpret_cast<uint4*>(sm.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     };
@@ -188,6 +191,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
                  "r"(gp.has_l1), "f"(gp.tau_2d), "f"(gp.tau_3d), "f"(gp.eps_3d), "l"(io.z_out));
     __syncthreads();                                       // the histogram is clear
     asm volatile("griddepcontrol.wait;" ::: "memory");      // scores come from the kernel before this one
+    if (role.stable) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // ---- 1. all loads first
     // (Loops over a thread's tokens have no early exits: the chains of its tokens then run beside one another.)

@@ -46,7 +46,7 @@ __global__ void wait_probe_kernel(const int* never_set, uint64_t limit_ns, int* 
 // dispatched in: a copying CTA never keeps its selecting CTA from running.  (Taking the roles in the order
 // in which the CTAs start, by a ticket from an atomic counter as the patch-by-patch tail does, cost 0.4 us per
 // step here: 296 atomics on one word.)  All waits are bounded all the same.
-template <int NT, int CAP, class BD>
+template <int NT, int CAP, bool STABLE, class BD>
 __global__ void __launch_bounds__(NT, 1024 / NT)      // as many CTAs to a multiprocessor as the launcher counts on
 select_copy_kernel(const __grid_constant__ BD bd, const __grid_constant__ TailPlan tp, const GateParams gp,
                    const SelectIO io, const __grid_constant__ CompactArgs ca, int32_t* __restrict__ list, int* status,
@@ -59,7 +59,8 @@ select_copy_kernel(const __grid_constant__ BD bd, const __grid_constant__ TailPl
         __shared__ SelectSmem<NT, CAP / NT> sm;
         const int b = cta;
         SelectRole role;
-        role.late_pdl = true;
+        role.late_pdl = !STABLE;
+        role.stable = STABLE;
         if (tp.cta0[bd.count()] > 0) role.list = list + bd.at(b).out_off * kListStride;   // every word is its own "ready" signal
         select_sample<NT, CAP / NT>(bd.at(b), b, gp, io, sm, role, [&]() {
             if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
@@ -82,15 +83,18 @@ select_copy_kernel(const __grid_constant__ BD bd, const __grid_constant__ TailPl
     if (s.k_2d_fixed >= 0) baset = (b2 ? s.k_2d_fixed : 0) + (b3 ? s.budget - s.k_2d_fixed : 0);
     else if (b2 == b3) baset = b2 ? s.budget : 0;
     const bool text_early = baset >= 0;
-    if (text_early)                                         // while the scores are still being computed
+    auto copy_text = [&]() {
         copy_rows(ca, s.n_txt, w, nw, lane, [&](int i, int64_t& srow, int64_t& drow) {
             srow = static_cast<int64_t>(s.seq_off) + s.off_txt + i;
             drow = static_cast<int64_t>(s.out_off) + baset + i;
             return true;
         });
+    };
+    if (!STABLE && text_early) copy_text();                 // while the scores are still being computed
     asm volatile("griddepcontrol.wait;" ::: "memory");      // keeps the chain of dependencies whole: the kernel after
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // this one may rely on the one before it being complete
     if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta] = global_ns();
+    if (STABLE && text_early) copy_text();
 
     {
         const int n_rows = s.n_out - (text_early ? s.n_txt : 0);
@@ -114,7 +118,7 @@ select_copy_kernel(const __grid_constant__ BD bd, const __grid_constant__ TailPl
     }
 }
 
-template <int NT, int CAP, class BD>
+template <int NT, int CAP, bool STABLE, class BD>
 cudaError_t launch_t(const BD& bd, const TailPlan& tp, const GateParams& gp, const SelectIO& io, const CompactArgs& ca,
                      int32_t* list, int* status, unsigned long long* stamps, cudaStream_t stream)
 {
@@ -125,7 +129,7 @@ cudaError_t launch_t(const BD& bd, const TailPlan& tp, const GateParams& gp, con
     cudaLaunchAttribute attr[1] = {pdl_attribute()};
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, select_copy_kernel<NT, CAP, BD>, bd, tp, gp, io, ca, list, status, stamps);
+    return cudaLaunchKernelEx(&cfg, select_copy_kernel<NT, CAP, STABLE, BD>, bd, tp, gp, io, ca, list, status, stamps);
 }
 
 int max_vis_of(const BatchDesc& bd)
@@ -144,12 +148,13 @@ cudaError_t launch_wait_probe(const int32_t* never_set, uint64_t limit_ns, int* 
 }
 
 cudaError_t launch_select_copy(const BatchDesc& bd, const GateParams& gp, const SelectIO& io, const CompactJob& job,
-                               int32_t* list, int* status, unsigned long long* stamps, cudaStream_t stream)
+                               int32_t* list, int* status, bool stable, unsigned long long* stamps, cudaStream_t stream)
 {
     if (bd.n < 1) return cudaErrorInvalidConfiguration;
     const CompactArgs ca = compact_args(job);
-    // CTAs on the device at once: two of 512 threads to a multiprocessor, or one of 1024 (more than 2048 visual tokens)
-    int ctas = sm_count_of_current_device() * (max_vis_of(bd) > 2048 ? 1 : 2) - bd.n;
+    // CTAs on the device at once: two of 512 threads to a multiprocessor, or one of 1024 (more than 2048 visual tokens); one of
+    // 512 where the scoring CTAs of the next step are to run beside them (two: eight requests of 671 tokens 73 -> 79 us)
+    int ctas = sm_count_of_current_device() * (max_vis_of(bd) > 2048 || stable ? 1 : 2) - bd.n;
     TailPlan tp;
     int next = 0;
     if (ca.seg_begin[3] > 0) {
@@ -182,9 +187,13 @@ cudaError_t launch_select_copy(const BatchDesc& bd, const GateParams& gp, const 
     for (int b = bd.n; b <= kMaxChunk; ++b) tp.cta0[b] = static_cast<int16_t>(next);
     const int nv = max_vis_of(bd);
     return with_desc(bd, [&](const auto& d) {
-        if (nv <= 1024) return launch_t<512, 1024>(d, tp, gp, io, ca, list, status, stamps, stream);
-        if (nv <= 2048) return launch_t<512, 2048>(d, tp, gp, io, ca, list, status, stamps, stream);
-        return launch_t<1024, kMaxVis>(d, tp, gp, io, ca, list, status, stamps, stream);
+        if constexpr (std::is_same_v<std::decay_t<decltype(d)>, OneDesc>) {
+            if (stable && nv <= 1024) return launch_t<512, 1024, true>(d, tp, gp, io, ca, list, status, stamps, stream);
+        }
+        if (stable) return cudaErrorInvalidConfiguration;
+        if (nv <= 1024) return launch_t<512, 1024, false>(d, tp, gp, io, ca, list, status, stamps, stream);
+        if (nv <= 2048) return launch_t<512, 2048, false>(d, tp, gp, io, ca, list, status, stamps, stream);
+        return launch_t<1024, kMaxVis, false>(d, tp, gp, io, ca, list, status, stamps, stream);
     });
 }
 

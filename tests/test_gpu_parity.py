@@ -456,6 +456,50 @@ def test_pipelined_steps_of_interleaved_episodes_keep_their_states_apart():
         assert all(torch.equal(x, y) for x, y in zip(got[t], ref[t])), t
 
 
+@pytest.mark.parametrize("text_first", [False, True])
+def test_chained_requests_match_serial_steps(text_first):
+    # Requests of one sample with stable inputs are chained: the scores of a step are taken beside the selection and row copy of
+    # the step before.  A sequence that mixes independent episodes, carried-over state, fixed and adaptive budgets, steps without
+    # row copy, steps whose inputs are an earlier step's output rows, and a step without the promise: the same bits as one at a time.
+    wl = W.small_workload(59, batch=1, D=512, H=4, d=128, dtype="bf16", n_txt=(21,), n_2d=(200,), n_3d=(333,), keep=(0.4,), steps=16,
+                          text_first=text_first)
+    devs = [device_tensors(wl, t) for t in range(16)]
+    s = wl.samples[0]
+    import dataclasses
+
+    def run(flag, sync):
+        ctx = mvla.context_for(wl, n_state_slots=3)
+        outs, kept = [], []
+        for t in range(16):
+            d, sample = devs[t], dataclasses.replace(s, state_slot=t % 3)
+            mode = mvla.MODE_FIXED if t % 4 == 1 else mvla.MODE_ADAPTIVE
+            rows = t % 5 != 3
+            if t in (6, 7, 12):                                # the rows that an earlier step kept, pruned again
+                prev, n = outs[t - 1 - t % 2], kept[t - 1 - t % 2]
+                q, k, v, h = d["q"][:n], prev.out_k[:n], prev.out_v[:n], prev.out_hidden[:n]
+                n3 = (n - s.n_txt) // 2
+                sample = W.layout_2d_3d_txt(0, s.n_txt, n - s.n_txt - n3, n3, keep_2d=0.5, keep_3d=0.3, keep_total=0.4, state_slot=t % 3)
+            else:
+                q, k, v, h = (d[x] for x in ("q", "k", "v", "hidden"))
+            o = ctx.alloc_outputs([sample], hidden=rows, kv=rows, extras=True)
+            ctx.prune_step(0, [sample], mode, q, k, v if rows else None, h,
+                           flags=(0 if t == 9 else flag) | (mvla.FLAG_RESET_STATE if t < 3 or t in (6, 7, 12) else 0), out=o)
+            outs.append(o)
+            kept.append(o.total_kept)
+            if sync:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        ctx.close()
+        return [(o.ahat, o.kept_idx[:n], o.budgets, o.out_offsets) + ((o.out_hidden[:n], o.out_k[:n], o.out_v[:n]) if o.out_hidden is not None else ())
+                for o, n in zip(outs, kept)]
+
+    ref = run(0, True)
+    for _ in range(3):
+        got = run(mvla.FLAG_INPUTS_STABLE, False)
+        for t in range(16):
+            assert len(got[t]) == len(ref[t]) and all(torch.equal(x, y) for x, y in zip(got[t], ref[t])), t
+
+
 def test_step_segments_in_order_3d_text_2d():
     # the three segments may come in any order; here [3D | text | 2D], two samples, adaptive budgets
     base = W.small_workload(47, batch=2, D=256, H=4, d=128, dtype="bf16", n_txt=(9, 30), n_2d=(140, 77),
