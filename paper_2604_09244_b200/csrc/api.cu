@@ -23,7 +23,7 @@ constexpr int kSets = 6;            // scratch sets = prune steps that may be in
 // queries, surviving rows in and out) are chained on the caller's stream, with the scores of a step taken beside the selection and
 // row copy of the one before: two or three launches, where the fork to a side stream is three or four launches and four event
 // calls, 10 to 14 us of host time on different hosts.  Per request of eight in a row, fork / chain in us, 32 heads: 630 tokens, heads of 64
-// (9 MB), adaptive 18.7 / 10.2, fixed 11.2 / 7.7; 750 of 128 (20 MB) 13.5 / 10.3, 11.4 to 14.4 / 10.9; 1010 of 96 (20 MB) 14.0 / 11.8, 11.5 / 11.1.
+// (9 MB), adaptive 18.7 / 10.2, fixed 11.2 / 7.6; 750 of 128 (20 MB) 13.5 / 10.3, 9.5 to 14.4 / 10.0; 1010 of 96 (20 MB) 14.0 / 11.8, 11.5 / 11.1.
 // Above, the GPU is the limit, and a fork overlaps more: 1010 of 128 (27 MB), fixed, 11.3 / 15.1; two tiles per CTA: 1280 of
 // 64 (17 MB) 11.3 / 12.1, of 96 (26 MB) 11.4 / 14.3, adaptive 14.0 / 18.5.  (In a CUDA graph launches cost nothing: always the fork.)
 constexpr size_t kChainBytes = 20u << 20;
