@@ -31,7 +31,7 @@ namespace {
 constexpr int kSoftWarps = 8;
 constexpr int kSoftThreads = kSoftWarps * 32;
 constexpr int kStreamThreads = kSoftThreads + 64;     // + the loading warp and the MMA warp
-constexpr int kNormWarps = 2;                         // + these, in launches with the attention copy
+constexpr int kNormWarps = 2;                         // + these, in launches that take the feature norms
 constexpr int kNormStages = 3;                        // pieces of rows in flight per norm warp
 constexpr uint32_t kNormPiece = 8192;
 constexpr int kMaxStages = 12;
@@ -363,27 +363,35 @@ __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, in
     __syncwarp();
 }
 
-// One norm warp: L1 norms of its share of the visual rows of all samples, every n_w-th of them.  Rows come by bulk
+// One norm warp: L1 norms of its share of the visual rows of all samples, a run of them.  Rows come by bulk
 // copies, kNormStages pieces in flight per warp, so that they take their part of the memory bandwidth without registers
-// or a CTA of their own.
+// or a CTA of their own.  What bounds it is a piece's fixed cost and the adds of its sums, not the bytes in flight (adaptive steps of
+// 16 requests of 768 tokens: two pieces in flight 99.9 us, three 98.4; pieces of 4 KB 110.8; a run of rows instead of every n_w-th, whose
+// sample has to be looked up each time, 97.8 instead of 98.4; four sums beside one another instead of one chain 94.8; eight loads at once 93.7).
 __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs& a, StreamSmem& sm, uint32_t buf, int nw, int lane)
 {
     const bool one = elect_one();
     int rows = 0;                                        // of all samples
     for (int b = 0; b < a.n_samples; ++b) rows += bd.s[b].n_2d + bd.s[b].n_3d;
     const int w = static_cast<int>(blockIdx.x) * kNormWarps + nw, n_w = static_cast<int>(gridDim.x) * kNormWarps;
-    const int pieces = (a.row_bytes + static_cast<int>(kNormPiece) - 1) / static_cast<int>(kNormPiece), n = w < rows ? ((rows - 1 - w) / n_w + 1) * pieces : 0;
-    // The row next to be fetched: sample fb, visual index fv; and the one next to be summed goes to *out.
-    int fb = 0, fv = w;
-    float* out = a.l1 + bd.s[0].vis_off + w;             // (visual arrays are packed over the samples of the launch)
-    int fp = 0;
-    auto settle = [&]() {
-        while (fb < a.n_samples - 1 && fv >= bd.s[fb].n_2d + bd.s[fb].n_3d) { fv -= bd.s[fb].n_2d + bd.s[fb].n_3d; ++fb; }
-    };
-    settle();
-    auto fetch = [&](int st) {
+    const int first = static_cast<int>(static_cast<int64_t>(rows) * w / n_w), last = static_cast<int>(static_cast<int64_t>(rows) * (w + 1) / n_w);
+    const int pieces = (a.row_bytes + static_cast<int>(kNormPiece) - 1) / static_cast<int>(kNormPiece), n = (last - first) * pieces;
+    // The row next to be fetched: visual index fv of sample fb, whose geometry stays in registers (a run-time index into the
+    // kernel's parameters costs some hundred cycles); and the one next to be summed goes to *out.
+    int fb = 0, fv = first, n_2d = 0, n_vis = 0, row_2d = 0, row_3d = 0;
+    auto sample = [&]() {
         const SampleDev& s = bd.s[fb];
-        const int row = s.seq_off + (fv < s.n_2d ? s.off_2d + fv : s.off_3d + (fv - s.n_2d));
+        n_2d = s.n_2d;
+        n_vis = s.n_2d + s.n_3d;
+        row_2d = s.seq_off + s.off_2d;
+        row_3d = s.seq_off + s.off_3d - s.n_2d;
+    };
+    sample();
+    while (fv >= n_vis && fb < a.n_samples - 1) { fv -= n_vis; ++fb; sample(); }
+    float* out = a.l1 + bd.s[0].vis_off + first;         // (visual arrays are packed over the samples of the launch)
+    int fp = 0;
+    auto fetch = [&](int st) {
+        const int row = (fv < n_2d ? row_2d : row_3d) + fv;
         const uint32_t at = static_cast<uint32_t>(fp) * kNormPiece, bytes = min(kNormPiece, static_cast<uint32_t>(a.row_bytes) - at);
         if (one) {
             const uint32_t bar = smem_u32(&sm.nfull[nw][st]);
@@ -392,8 +400,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
         }
         if (++fp == pieces) {
             fp = 0;
-            fv += n_w;
-            settle();
+            if (++fv == n_vis && fb < a.n_samples - 1) { fv = 0; ++fb; sample(); }
         }
     };
     pdl_wait();                                          // the rows may come from the kernel before this one
@@ -410,7 +417,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
         }
         const uint32_t bytes = min(kNormPiece, static_cast<uint32_t>(a.row_bytes) - static_cast<uint32_t>(piece) * kNormPiece);
         const uint32_t src = buf + static_cast<uint32_t>(st) * kNormPiece;
-#pragma unroll 4
+#pragma unroll 8
         for (uint32_t at = lane * 16; at < bytes; at += 512) {
             uint32_t u[4];
             asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]) : "r"(src + at));
@@ -429,7 +436,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
 #pragma unroll
             for (int off = 16; off >= 1; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
             if (lane == 0) *out = r;
-            out += n_w;
+            ++out;
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[e] = 0.f;
         }
@@ -703,7 +710,7 @@ cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUte
     if (e != cudaSuccess) return e;
     if (n < 1) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(std::min(a.n_jobs, n) * cluster));
+    cfg.gridDim = dim3(static_cast<unsigned>((a.hidden ? n : std::min(a.n_jobs, n)) * cluster));      // (norms are shared out over all CTAs)
     cfg.blockDim = dim3(static_cast<unsigned>(threads));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;

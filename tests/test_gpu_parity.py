@@ -896,6 +896,20 @@ def test_streaming_scoring_kernel_at_the_edges_of_its_shapes(batch, H, n_txt, n_
     ctx.close()
 
 
+@pytest.mark.parametrize("D", [8, 2056, 4096, 4104])          # pieces of 8 KB a row: one of 16 bytes; a part; one; one and 16 bytes
+@pytest.mark.parametrize("batch,H,n_txt,n_2d,n_3d,kw", [
+    (8, 32, (5, 33, 64), (0, 200, 129, 1), (130, 64, 300, 90), {}),          # a modality without tokens; samples of a few rows
+    (3, 64, (16, 48), (200, 256), (64, 77), {"dtype": "fp8", "text_first": True})])
+def test_streaming_scoring_kernel_with_norms_inside(batch, H, n_txt, n_2d, n_3d, kw, D):
+    """Adaptive batches have their feature norms taken by two warps of the scoring kernel: rows of every sample, in pieces that
+    end anywhere; two action steps."""
+    wl = W.small_workload(75, batch=batch, H=H, D=D, d=64, n_txt=n_txt, n_2d=n_2d, n_3d=n_3d, keep=(0.3, 0.5), steps=2, **{"dtype": "bf16", **kw})
+    ctx, states = mvla.context_for(wl), [oracle.State(s.n_vis) for s in wl.samples]
+    for step in range(2):
+        run_and_check_step(ctx, wl, step, states)
+    ctx.close()
+
+
 @pytest.mark.parametrize("batch,H,n_txt,n_2d,n_3d", [
     (8, 16, (64, 1, 33), (129, 40), (255, 300)),
     (2, 4, (17, 50), (1500, 2000), (1200, 77))])
