@@ -363,10 +363,10 @@ void clear_accumulators(unsigned long long* acc64, const BatchDesc& bd, cudaStre
 //     25.4 / 23.0, 384 26.7 / 26.4; 768 + 768 tokens (16 clusters of 6, 22 at once) 17.5 / 22.7, 768 + 1023 (16 of 7, 15 at
 //     once) 26.0 / 24.0, 2 samples of 640 + 512 (32 of 5, 26 at once) 29.1 / 26.3, 3 samples 25.7 / 25.2.
 // With the feature norms beside the scores two tiles a CTA behave the same (28.2 / 25.5 for 768 + 1023, 43.1 / 32.9 for two
-// samples; 32.8 / 34.2 for three of 640 + 512), one tile does not: batches of small samples leave the norms behind the streaming
-// kernel instead of beside it (384 CTAs: 4 samples 30.0 / 28.7, 12 samples 29.5 / 33.3).  There the line stays at three CTAs.  (Not
-// the best line either: 32 heads of 128, samples of 228 tokens, 8 of them 22.1 / 27.2, 10 26.1 / 24.4, 16 34.8 / 39.3, 32 67.9 /
-// 61.3.)
+// samples; 32.8 / 34.2 for three of 640 + 512), one tile does not: batches of small samples left the norms behind the streaming
+// kernel instead of beside it (384 CTAs: 4 samples 30.0 / 28.7, 12 samples 29.5 / 33.3), so there the line is at three CTAs.  With the
+// norms inside the streaming kernel (norms_inside_pays) 32 heads of 128, samples of 228 tokens: 8 of them 22.1 / 20.6, 10 26.1 / 24.0,
+// 16 34.8 / 35.6.
 cudaError_t stream_pays(const mvla_ctx* ctx, const BatchDesc& bd, int tiles_per_cta, int cluster, int npad, bool for_patches,
                         bool norms_beside, bool* pays)
 {

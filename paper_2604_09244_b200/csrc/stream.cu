@@ -16,7 +16,8 @@
 // What bounds it: HBM (the keys are read once); softmax arithmetic comes second (16 exponentials per clock and
 // multiprocessor: half of the time of the key stream at 48 queries, nine tenths at 64).
 // Whole steps against one short-lived CTA per two tiles (and, above 2048 tokens, the generic kernel): 16 requests of 768
-// tokens 121 -> 97 us, 8 of 3584 tokens 695 -> 162, 16 patch-by-patch steps of 512 tokens 139 -> 97.
+// tokens 121 -> 97 us, 8 of 3584 tokens 695 -> 162, 16 patch-by-patch steps of 512 tokens 139 -> 97.  Taking the feature norms too:
+// 16 requests 94.9 -> 93.7, 16 of 228 tokens 39.9 -> 35.6, 16 patch-by-patch steps 82.9 -> 78.7.
 // More softmax warps (12, 16), two tiles per warp at once and prefetching the next tile's columns were all slower.
 #include "common.cuh"
 #include "device_utils.cuh"
@@ -444,7 +445,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
 }
 
 // grid = clusters x cluster size (1-D), one CTA per multiprocessor.
-// ROOM: the feature norms are to run beside this kernel.  Its ten warps put three on two of a multiprocessor's four
+// ROOM: the feature norms are to run beside this kernel (they do not fit its own two norm warps; figures from before there were these).  Its ten warps put three on two of a multiprocessor's four
 // register files (16384 registers each): at the 168 registers a thread that the compiler takes these are full, no CTA of
 // the norms fits, and they start when the scores are done.  144 leave room for two warps of 32 registers in each (adaptive
 // steps, 10 requests of 190 tokens 31.2 -> 24.1 us, 4 of 768 33.6 -> 27.1) at the price of 8 bytes a thread stored and 24
