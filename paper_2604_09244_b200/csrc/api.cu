@@ -530,13 +530,16 @@ bool clashes(const mvla_ctx* ctx, unsigned par, const mvla_ctx::Range* r, int n)
     return false;
 }
 
-// Remembers what the step on scratch set `par` writes and which smoothed states it touches.
+// Remembers what the step on scratch set `par` writes and which smoothed states it touches.  The first step after work that is not
+// remembered (a call without the promise, a stage call) drops the events of all sets: they are older than that work, so every set is
+// ordered after the caller's stream once more before its events count again.
 void remember(mvla_ctx* ctx, unsigned par, int32_t prune_point, int32_t batch, const mvla_sample* samples, const mvla_ctx::Range* side,
               int n_side_written, const mvla_ctx::Range* copied, int n_copied)
 {
     if (ctx->hist_unknown) {
         for (int& n : ctx->n_hist) n = 0;
         for (int& n : ctx->n_state_of) n = 0;
+        for (bool& v : ctx->sel_valid) v = false;
     }
     int m = 0;
     for (int i = 0; i < n_side_written; ++i) if (side[i].lo) ctx->hist[par][m++] = side[i];

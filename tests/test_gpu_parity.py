@@ -500,6 +500,51 @@ def test_chained_requests_match_serial_steps(text_first):
             assert len(got[t]) == len(ref[t]) and all(torch.equal(x, y) for x, y in zip(got[t], ref[t])), t
 
 
+@pytest.mark.parametrize("reads", ["state", "rows"])
+def test_stable_steps_are_ordered_after_a_call_without_the_promise(reads):
+    # Six stable batches, so that every scratch set has events of its own; a call without the promise, kept from running for 10 ms; a
+    # stable step that has nothing to do with it; then a stable batch that reads what that call writes: the smoothed
+    # states of its slots, or the rows that it kept.  Each of six more batches runs on another scratch set.
+    import dataclasses
+    wl = W.small_workload(61, batch=2, D=256, H=4, d=128, dtype="bf16", n_txt=(9, 30), n_2d=(100, 180), n_3d=(140, 333),
+                          keep=(0.5, 0.3), steps=14, cold_start=0)
+    devs = [device_tensors(wl, t) for t in range(14)]
+
+    def slots(first):
+        return [dataclasses.replace(s, state_slot=first + i) for i, s in enumerate(wl.samples)]
+
+    def run(flag):
+        ctx = mvla.context_for(wl, n_state_slots=6)
+        outs, kept, late = [], [], None
+        for t in range(14):
+            q, k, v, h = (devs[t][x] for x in ("q", "k", "v", "hidden"))
+            samples = slots(4 if t < 6 else 0)
+            if t == 7:
+                samples = slots(2)[:1]                        # one sample: chained on the caller's stream
+            if reads == "rows" and t > 7:                     # the rows that call 6 kept, pruned again
+                k, v, h = late.out_k, late.out_v, late.out_hidden
+            o = ctx.alloc_outputs(samples, extras=True)
+            if t == 6:
+                late = o
+                for x in (o.out_k, o.out_v, o.out_hidden):
+                    x.zero_()
+                torch.cuda.synchronize()
+                if flag:
+                    torch.cuda._sleep(20_000_000)
+            ctx.prune_step(0, samples, wl.mode, q, k, v, h, flags=(0 if t == 6 else flag) | (mvla.FLAG_RESET_STATE if t in (0, 7) else 0), out=o)
+            outs.append(o)
+            kept.append(o.total_kept)
+            if not flag:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        ctx.close()
+        return [(o.ahat, o.kept_idx[:n], o.budgets, o.out_hidden[:n], o.out_v[:n]) for o, n in zip(outs, kept)]
+
+    ref, got = run(0), run(mvla.FLAG_INPUTS_STABLE)
+    for t in range(14):
+        assert all(torch.equal(x, y) for x, y in zip(got[t], ref[t])), t
+
+
 def test_step_segments_in_order_3d_text_2d():
     # the three segments may come in any order; here [3D | text | 2D], two samples, adaptive budgets
     base = W.small_workload(47, batch=2, D=256, H=4, d=128, dtype="bf16", n_txt=(9, 30), n_2d=(140, 77),
