@@ -269,6 +269,16 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
     return static_cast<unsigned long long>(m) << 32 | lo;
 }
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) { return ~warp_min_u64(~v); }
+// A double as a pattern that orders like it (scores handed in by a caller may be negative), and back.
+__device__ __forceinline__ unsigned long long order_bits(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return static_cast<unsigned long long>(b ^ (b >> 63 | static_cast<long long>(1ull << 63)));
+}
+__device__ __forceinline__ double from_order_bits(unsigned long long k)
+{
+    return __longlong_as_double(static_cast<long long>(k >> 63 ? k ^ 1ull << 63 : ~k));
+}
 
 // 1-D K-Means, K = 3 (Sec. 4.2), of the P masses by one warp, started from the smallest mass, the mean and the
 // largest: labels and centres to `sm`.  A round: assign to the nearest centre (ties to the lower one); unless nothing
@@ -284,7 +294,7 @@ __device__ __forceinline__ void kmeans(Smem& sm, int P, int max_iter, int lane)
 #pragma unroll 1
     for (int p = lane; p < P; p += 32) {
         const double m = sm.mass[p];
-        const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(m));
+        const unsigned long long bits = order_bits(m);
         sum += m;
         mx = max(mx, bits);
         mn = min(mn, bits);
@@ -293,7 +303,7 @@ __device__ __forceinline__ void kmeans(Smem& sm, int P, int max_iter, int lane)
     }
     mx = warp_max_u64(mx);
     mn = warp_min_u64(mn);
-    double c0 = __longlong_as_double(static_cast<long long>(mn)), c1 = warp_sum_d(sum) / P, c2 = __longlong_as_double(static_cast<long long>(mx));
+    double c0 = from_order_bits(mn), c1 = warp_sum_d(sum) / P, c2 = from_order_bits(mx);
     int iters = 0;
     while (iters < max_iter) {                      // warp-uniform
         ++iters;

@@ -192,6 +192,28 @@ def test_patch_select_on_given_inputs_is_exact():
     ctx.close()
 
 
+def test_patch_select_kmeans_starts_from_the_extremes_of_signed_masses():
+    # mvla_patch_select takes any scores: with negative ones the K-Means still starts from the smallest, the mean and the largest mass
+    rng = np.random.default_rng(8)
+    p = oracle.c_patch_params(tau_2d=0.35, tau_3d=0.65, cold_start_full_keep=0)
+    ctx = mvla.PruneContext(dtype=torch.bfloat16, n_heads=4, head_dim=64, d_model=256, max_batch=1, max_text=8,
+                            max_2d=700, max_3d=700, tau_2d=0.35, tau_3d=0.65, cold_start_full_keep=0, patch_path=1)
+    for P in (1, 2, 31, 33, 300, 700):
+        s = W.layout_2d_3d_txt(0, 3, P, P)
+        x, u = rng.random((P, 4)).astype(np.float32), rng.random(P).astype(np.float32)
+        one_negative = (rng.random(2 * P) ** 6).astype(np.float32)
+        one_negative[rng.integers(P)] = -3.0
+        for attn in (one_negative, rng.standard_normal(2 * P).astype(np.float32), -(rng.random(2 * P) ** 6).astype(np.float32) - 0.5):
+            out = ctx.patch_select(0, [s], torch.from_numpy(attn).cuda(), torch.from_numpy(x).cuda(), torch.from_numpy(u).cuda(),
+                                   flags=mvla.FLAG_RESET_STATE)
+            torch.cuda.synchronize()
+            r = oracle.patch_select(attn, x, u, s, p, oracle.PatchState(P))
+            labels, _ = unpack_info(out.patch_info.cpu().numpy())
+            assert np.array_equal(labels, r.labels), P
+            assert np.array_equal(out.kept_idx.cpu().numpy()[:out.out_offsets.cpu().numpy()[1]], r.kept_idx)
+    ctx.close()
+
+
 @pytest.mark.parametrize("seed", [5, 6])
 def test_patch_step_host_model_shape(seed):
     wl = W.patch_mla(seed)                       # 32 text + 256 image + 256 point tokens, D = 4096, 32 x 128, bf16
