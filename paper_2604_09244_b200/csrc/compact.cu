@@ -122,7 +122,7 @@ cudaError_t clusters_at_once(KernelSetup& ks, const void* kern, int threads, siz
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    *count = ks.clusters.find(dev, cluster, smem);
+    *count = ks.clusters.find(dev, cluster, smem, threads);
     if (*count > 0) return cudaSuccess;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -136,7 +136,7 @@ cudaError_t clusters_at_once(KernelSetup& ks, const void* kern, int threads, siz
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     e = cudaOccupancyMaxActiveClusters(count, kern, &cfg);
-    if (e == cudaSuccess) ks.clusters.keep(dev, cluster, smem, *count);
+    if (e == cudaSuccess) ks.clusters.keep(dev, cluster, smem, *count, threads);
     return e;
 }
 

@@ -35,6 +35,7 @@ constexpr int kStreamThreads = kSoftThreads + 64;     // + the loading warp and 
 constexpr int kNormWarps = 2;                         // + these, in launches that take the feature norms
 constexpr int kNormStages = 3;                        // pieces of rows in flight per norm warp
 constexpr uint32_t kNormPiece = 8192;
+constexpr int kStreamRegs = 168;                      // registers a thread, see the kernel
 constexpr int kMaxStages = 12;
 constexpr uint32_t kStageBytes = 16384;               // 128 keys x 128 bytes: one swizzled box of a key tile
 constexpr int kMaxSlots = 32;
@@ -451,7 +452,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
 // steps, 10 requests of 190 tokens 31.2 -> 24.1 us, 4 of 768 33.6 -> 27.1) at the price of 8 bytes a thread stored and 24
 // loaded; with 128 these are 68 and 144 (16 requests of 768 tokens 97 -> 106).  Without norms the registers are worth more (16 patch-by-patch steps 96.3 us, 99.1 with 144).
 template <bool ROOM>
-__global__ void __maxnreg__(ROOM ? 144 : 168)
+__global__ void __maxnreg__(ROOM ? 144 : kStreamRegs)
 salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,
                        const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ StreamArgs a)
 {
@@ -731,6 +732,7 @@ cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUte
 // no CTA with 32 columns of tensor memory (at least 1/17 of the shared memory, smem_for_tmem) fits beside one
 static_assert(kSmemPerSm - static_cast<int>(kStreamSmem + sizeof(StreamSmem)) - kSmemReservedPerCta < kSmemPerSm / 17,
               "the streaming kernel must be alone with the tensor memory of its multiprocessor");
+static_assert((kStreamThreads + 32 * kNormWarps) * kStreamRegs <= 65536, "the norm warps must fit the register file beside the others");
 
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
