@@ -1,6 +1,7 @@
 // C-ABI layer: argument validation, host-side budget arithmetic, workspace and smoothed state,
 // tensor-map construction, launch sequencing.  No stream synchronisation anywhere.
 #include "common.cuh"
+#include "rules.h"
 
 #include <cudaTypedefs.h>
 
@@ -381,21 +382,6 @@ cudaError_t stream_pays(const mvla_ctx* ctx, const BatchDesc& bd, int tiles_per_
     return e;
 }
 
-// Whether the streaming kernel takes the feature norms of a step itself, by two more warps, or a kernel beside it does.  Whole adaptive
-// steps in us, beside / inside, 32 heads of 128 unless said otherwise:
-//   4 x 768 tokens 26.1 / 24.8, 8 x 812 55.7 / 51.1, 13 x 547 with 8 key heads 51.0 / 43.1, 16 x 228 39.9 / 35.5, 16 x 768 94.9 / 93.7; e4m3
-//   26 x 217 42.9 / 35.1, 13 x 535 54.9 / 47.8; 32 x 750 172 / 184 (e4m3 132 / 136, 8 key heads 115 / 114): two warps no longer keep up
-//   with the keys;
-//   samples of more than 16 key tiles either way: 2 x 3426 77.4 / 73.3, 5 x 2224 97.4 / 98.5, 7 x 2584 115.4 / 119, 8 x 3584 160 / 168;
-//   rows of eight times the keys' bytes, where the scores of few jobs end early: e4m3, 16 heads of 256, 4 key heads, 12 x 435 (192 jobs)
-//   26.5 / 27.3, 20 x 350 (320 jobs) 37.8 / 34.8.
-bool norms_inside_pays(const mvla_ctx* ctx, const BatchDesc& bd, int max_tiles)
-{
-    const int64_t row = static_cast<int64_t>(ctx->cfg.d_model) * ctx->elem, key = static_cast<int64_t>(ctx->kv_heads) * ctx->cfg.head_dim * ctx->qk_elem;
-    const bool short_scores = row >= 8 * key && bd.n * ctx->cfg.n_heads < 2 * ctx->sm_count;
-    return max_tiles <= 16 && visual_tokens(bd) <= 88 * ctx->sm_count && !short_scores;
-}
-
 // Salience of one chunk (+ L1 norms into `l1` when asked; + the scores as fp32 into `attn_out` when asked).  The per-head
 // contributions are added into the fixed-point accumulators `acc64` (*used_acc64 = true) where a kernel that does so covers the
 // shape, else they land in ctx->part.
@@ -435,7 +421,9 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
         if (e != cudaSuccess) return e == cudaErrorInvalidConfiguration ? MVLA_ERR_UNSUPPORTED : fail_cuda(ctx, e);
     }
     // With `norms_inside`: norms only if the scoring kernel takes them itself, and whether it did.
-    const bool inside = streaming && hidden && l1 && (norms_inside || (norms_beside && norms_inside_pays(ctx, bd, max_tiles)));
+    const NormsInsideSizes sizes = {visual_tokens(bd), npad, max_tiles, bd.n * c.n_heads, c.n_heads, static_cast<int64_t>(c.d_model * ctx->elem),
+                                   static_cast<int64_t>(ctx->kv_heads * c.head_dim * ctx->qk_elem), ctx->sm_count};
+    const bool inside = streaming && hidden && l1 && (norms_inside ? patch_norms_inside_pays(c.n_heads, npad) : norms_beside && norms_inside_pays(sizes));
     if (norms_inside) {
         *norms_inside = inside;
         if (!inside) hidden = nullptr;

@@ -1,0 +1,51 @@
+// Rules of the host that choose between two ways of doing the same work, by sizes alone, and what they were measured with.
+#pragma once
+
+#include <stddef.h>
+#include <stdint.h>
+
+namespace mvla {
+
+// Whether the streaming scoring kernel takes the feature norms of an adaptive batch itself, by two more warps, or a kernel
+// beside it does.  A piece of a row (kNormPiece) takes a norm warp the same time whatever its bytes: it waits for the piece, and three
+// are in flight.  The scores hide that as far as they go, one unit per (head, text query); the kernel beside them costs bandwidth, by the bytes of a
+// row; and inside saves its launch and boundary, a fixed gain.  In units: 2048 a piece, 15 / 64 a byte, 300 000 for the launch; these put
+// the line where 800 pairs of measurements have it with the fewest calls on the wrong side.  Whole steps in us, beside / inside, 768 tokens a
+// sample unless said otherwise, texts of up to 64 | of up to 14 (16 queries):
+//   rows of 2 KB, 8 heads of 128: 6 samples 15.9 / 15.7, 10 22.9 / 26.5, 15 25.3 / 35.3 | 10 18.9 / 26.3
+//   rows of 4 KB, 16 heads of 128: 16 of 228 tokens 21.5 / 20.8, 16 46.6 / 50.5, with 4 key heads 32.3 / 38.6 | 26 of 228 22.6 / 27.9, 15 40.8 / 46.0
+//                 32 heads of 64: 12 39.8 / 39.6, 16 with 8 key heads 43.5 / 42.8 | 15 42.0 / 46.1, with 8 key heads 29.6 / 37.0
+//   rows of 6 KB, 32 heads of 96: | 15 59.6 / 62.2, with 8 key heads, 10 29.8 / 32.8
+//   rows of 8 KB, 32 heads of 128: 4 24.0 / 23.1, 16 83.0 / 81.5, e4m3 67.3 / 62.4 | 10 48.5 / 42.4
+//                 16 heads of 256: 16 81.3 / 80.3, 16 of 228 33.8 / 27.6, e4m3 with 8 key heads 54.2 / 52.4 | e4m3, 26 of 228 33.3 / 31.9
+//   rows of 10 KB, 40 heads of 128: 6 49.1 / 43.7 | 15 88.0 / 99.2; 20 heads: 6 28.0 / 33.5
+//   rows of 16 KB, 16 heads of 128: 6 45.6 / 38.4, 10 66.8 / 61.2 | 6 45.8 / 37.6
+// Above 88 tokens a multiprocessor inside loses whatever the texts (32 heads of 128: 18 samples 90.4 / 92.6, 32 153 / 163), and samples of more
+// than 16 key tiles go either way (2 x 3426 77.4 / 73.3, 7 x 2584 115.4 / 119).  Rows of eight times the keys' bytes, where the scores of few jobs end early:
+// e4m3, 16 heads of 256, 4 key heads, 12 x 435 (192 jobs) 26.5 / 27.3, 20 x 350 (320 jobs) 37.8 / 34.8.
+constexpr uint32_t kNormPiece = 8192;        // bytes of a row that a norm warp fetches at once
+struct NormsInsideSizes {
+    int64_t rows;               // visual tokens of the launch
+    int padded_text, max_tiles; // longest text rounded up to 16, key tiles of the largest sample
+    int jobs;                   // samples x heads
+    int n_heads;
+    int64_t row_bytes, key_bytes;   // of a token: its hidden row, its keys
+    int sm_count;
+};
+inline bool norms_inside_pays(const NormsInsideSizes& c)
+{
+    if (c.max_tiles > 16 || c.rows > 88 * c.sm_count) return false;
+    if (c.row_bytes >= 8 * c.key_bytes && c.jobs < 2 * c.sm_count) return false;
+    const int64_t pieces = (c.row_bytes + kNormPiece - 1) / kNormPiece;
+    return c.rows * (2048 * pieces - 15 * c.row_bytes / 64 - static_cast<int64_t>(c.n_heads) * c.padded_text) < 300000;
+}
+
+// The same of patch-by-patch batches, whose norms otherwise come from the indicators.  The scoring kernel writes the attention copy there, which
+// takes as long as (heads x text) does, whatever the heads' size.  Indicators / inside, samples of 256 patches unless said otherwise:
+//   640 and more: 32 heads x 32 queries, heads of 64, 8 samples 35.2 / 33.2, 16 64.0 / 57.4; of 128, 8 39.8 / 36.4, 16 68.4 / 67.9; 16 x 48, 12 of
+//     600 patches 97.4 / 84.9 (rows of 4 KB 87.9 / 80.7);
+//   512: 32 x 16, 16 of 500 patches 93.5 / 94.8; 16 x 32, 16 52.0 / 49.6, 8 41.2 / 43.0, rows of 4 KB 43.2 / 45.2; 16 of 100 27.2 / 29.1;
+//   256: 8 x 32, 16 42.7 / 45.0, rows of 4 KB 35.2 / 44.4; 16 x 16, 16 of 500 patches, rows of 4 KB 70.6 / 78.8.
+inline bool patch_norms_inside_pays(int n_heads, int padded_text) { return n_heads * padded_text >= 640; }
+
+}  // namespace mvla

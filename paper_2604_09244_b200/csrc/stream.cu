@@ -20,6 +20,7 @@
 // 16 requests 94.9 -> 93.7, 16 of 228 tokens 39.9 -> 35.6, 16 patch-by-patch steps 82.9 -> 78.7.
 // More softmax warps (12, 16), two tiles per warp at once and prefetching the next tile's columns were all slower.
 #include "common.cuh"
+#include "rules.h"
 #include "device_utils.cuh"
 #include "select_impl.cuh"
 #include "tmem_plan.h"
@@ -34,7 +35,6 @@ constexpr int kSoftThreads = kSoftWarps * 32;
 constexpr int kStreamThreads = kSoftThreads + 64;     // + the loading warp and the MMA warp
 constexpr int kNormWarps = 2;                         // + these, in launches that take the feature norms
 constexpr int kNormStages = 3;                        // pieces of rows in flight per norm warp
-constexpr uint32_t kNormPiece = 8192;
 constexpr int kStreamRegs = 168;                      // registers a thread, see the kernel
 constexpr int kMaxStages = 12;
 constexpr uint32_t kStageBytes = 16384;               // 128 keys x 128 bytes: one swizzled box of a key tile

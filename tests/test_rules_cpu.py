@@ -1,0 +1,52 @@
+"""The rules by which the host chooses between two ways of the same work (csrc/rules.h), at sizes on both sides of their lines
+where both ways were timed.  Checked by a small C++ program built from the header itself (no GPU needed)."""
+import os
+import subprocess
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def run_program(tmp_path, text):
+    src, exe = tmp_path / "rules.cpp", tmp_path / "rules"
+    src.write_text(text)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2604_09244_b200", "csrc"),
+                    "-o", str(exe), str(src)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout
+
+
+NORMS = r"""
+#include <cstdio>
+#include "rules.h"
+using namespace mvla;
+// (bytes of an element of k, heads, head dim, key heads, bytes of a hidden row, padded text, samples, tokens and key tiles of a sample)
+struct Point { int esize, heads, dim, kv, row, text, batch, tokens, tiles; bool inside; };
+static const Point points[] = {
+    {2, 8, 128, 8, 2048, 64, 10, 768, 6, false}, {2, 8, 128, 8, 2048, 16, 10, 768, 6, false},
+    {2, 16, 128, 16, 4096, 64, 16, 228, 3, true}, {2, 16, 128, 16, 4096, 64, 16, 768, 6, false}, {2, 16, 128, 4, 4096, 64, 16, 768, 6, false},
+    {1, 16, 128, 16, 4096, 64, 8, 768, 6, false}, {2, 16, 128, 16, 4096, 16, 26, 228, 3, false},
+    {2, 32, 64, 8, 4096, 64, 16, 768, 6, true}, {2, 32, 64, 8, 4096, 16, 15, 768, 6, false}, {1, 32, 64, 8, 4096, 32, 15, 768, 6, false},
+    {2, 32, 96, 32, 6144, 16, 15, 768, 6, false}, {2, 32, 96, 8, 6144, 16, 10, 768, 6, false}, {2, 32, 96, 32, 6144, 64, 15, 768, 6, true},
+    {2, 32, 128, 32, 8192, 64, 16, 768, 6, true}, {2, 32, 128, 32, 8192, 64, 18, 768, 6, false}, {2, 32, 128, 8, 8192, 64, 16, 768, 6, true},
+    {1, 32, 128, 32, 8192, 64, 16, 768, 6, true}, {2, 32, 128, 32, 8192, 16, 10, 768, 6, true}, {2, 16, 256, 16, 8192, 64, 16, 768, 6, true},
+    {1, 16, 256, 8, 8192, 64, 16, 768, 6, true}, {1, 16, 256, 16, 8192, 16, 26, 228, 3, true}, {1, 16, 256, 4, 8192, 64, 12, 435, 5, false},
+    {2, 40, 128, 40, 10240, 64, 6, 768, 6, true}, {2, 40, 128, 40, 10240, 16, 15, 768, 6, false}, {2, 20, 128, 20, 10240, 64, 6, 768, 6, false},
+    {2, 16, 128, 16, 16384, 64, 10, 768, 6, true}, {2, 16, 128, 16, 16384, 16, 6, 768, 6, true}, {2, 32, 128, 32, 8192, 64, 5, 2224, 18, false},
+};
+int main()
+{
+    for (const Point& p : points) {
+        const NormsInsideSizes c = {static_cast<int64_t>(p.batch) * p.tokens, p.text, p.tiles, p.batch * p.heads, p.heads, p.row,
+                                   static_cast<int64_t>(p.kv) * p.dim * p.esize, 148};
+        if (norms_inside_pays(c) != p.inside) { std::printf("%d heads of %d, %d x %d, text %d\n", p.heads, p.dim, p.batch, p.tokens, p.text); return 1; }
+    }
+    if (!patch_norms_inside_pays(32, 32) || !patch_norms_inside_pays(16, 48) || patch_norms_inside_pays(32, 16) || patch_norms_inside_pays(16, 32) ||
+        patch_norms_inside_pays(8, 32)) { std::printf("patch by patch\n"); return 1; }
+    std::printf("ok\n");
+    return 0;
+}
+"""
+
+
+def test_norms_are_taken_by_the_scoring_kernel_only_where_the_scores_hide_them(tmp_path):
+    run_program(tmp_path, NORMS)
