@@ -20,15 +20,6 @@ namespace {
 constexpr int kMaxBatch = 64;       // samples per call (mvla_prune_create refuses more)
 constexpr int kMapSlots = 16;       // tensor maps a context remembers
 constexpr int kSets = 6;            // scratch sets = prune steps that may be in flight at once
-// Steps of one sample with stable inputs, one key tile per scoring CTA, that move no more than this (keys, feature rows, text
-// queries, surviving rows in and out) are chained on the caller's stream, with the scores of a step taken beside the selection and
-// row copy of the one before: two or three launches, where the fork to a side stream is three or four launches and four event
-// calls, 10 to 14 us of host time on different hosts.  Per request of eight in a row, fork / chain in us, 32 heads: 630 tokens, heads of 64
-// (9 MB), adaptive 18.7 / 10.2, fixed 11.2 / 7.6; 750 of 128 (20 MB) 13.5 / 10.3, 9.5 to 14.4 / 10.0; 1010 of 96 (20 MB) 14.0 / 11.8, 11.5 / 11.1.
-// Above, the GPU is the limit, and a fork overlaps more: 1010 of 128 (27 MB), fixed, 11.3 / 15.1; two tiles per CTA: 1280 of
-// 64 (17 MB) 11.3 / 12.1, of 96 (26 MB) 11.4 / 14.3, adaptive 14.0 / 18.5.  (In a CUDA graph launches cost nothing: always the fork.)
-constexpr size_t kChainBytes = 20u << 20;
-
 // Tracing and logging, both on the host and off the device's path: every public call is an NVTX range (a profiler
 // shows the call and, inside mvla_prune_step, its phases around the kernels they enqueue; without a profiler
 // attached a range costs a few nanoseconds), and with MVLA_LOG=1 in the environment every call prints one line
@@ -1264,7 +1255,8 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         if (cudaStreamIsCapturing(st, &cst) != cudaSuccess) return fail_cuda(ctx, cudaGetLastError());
         const SampleDev& one = plan.s[0];
         const size_t moved = nvis_b * (kb + (adaptive ? hb : 0)) + static_cast<size_t>(one.n_txt) * qb + 2 * nout_b * (hb + 2 * kb);
-        if (batch == 1 && moved <= kChainBytes && cst == cudaStreamCaptureStatusNone && tiles_per_cta_of(tiles_of(one)) == 1) {
+        if (batch == 1 && cst == cudaStreamCaptureStatusNone && tiles_per_cta_of(tiles_of(one)) == 1 &&
+            chain_pays(static_cast<int64_t>(moved), ctx->cfg.n_heads * tiles_of(one), adaptive, ctx->sm_count)) {
             forked = false;
             chained = true;
             // (the first step of a chain, and its selection and row copy in any case, wait for all earlier work of the stream)

@@ -50,3 +50,30 @@ int main()
 
 def test_norms_are_taken_by_the_scoring_kernel_only_where_the_scores_hide_them(tmp_path):
     run_program(tmp_path, NORMS)
+
+
+CHAIN = r"""
+#include <cstdio>
+#include "rules.h"
+using namespace mvla;
+struct Point { double mb; int ctas; bool adaptive, chained; };
+static const Point points[] = {
+    {5.5, 64, false, true}, {14.8, 192, false, true}, {19.8, 192, false, true}, {24.0, 128, false, false},
+    {12.0, 256, false, true}, {15.4, 256, false, true}, {17.1, 256, false, false}, {18.0, 256, false, false}, {21.7, 256, false, false},
+    {15.0, 256, true, true}, {19.1, 256, true, true}, {19.6, 192, true, true}, {22.5, 192, true, false}, {27.0, 256, true, false},
+};
+int main()
+{
+    for (const Point& p : points)
+        if (chain_pays(static_cast<int64_t>(p.mb * (1 << 20)), p.ctas, p.adaptive, 148) != p.chained) {
+            std::printf("%.1f MB, %d CTAs, adaptive %d\n", p.mb, p.ctas, p.adaptive);
+            return 1;
+        }
+    std::printf("ok\n");
+    return 0;
+}
+"""
+
+
+def test_small_stable_steps_are_chained_only_where_the_gpu_keeps_up(tmp_path):
+    run_program(tmp_path, CHAIN)
