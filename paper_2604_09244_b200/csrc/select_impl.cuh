@@ -15,8 +15,8 @@
 //      (Sec. 4.2), fusion (Sec. 4.4), budget split                                      [barrier B]
 //   3. the number of keys in higher bins tells every thread what becomes of its keys: kept, dropped, or, in the bin where
 //      the budget runs out, listed                                                      [barrier C]
-//      The few listed keys are ranked by (key, lower index first) by the threads that own them.  A crowded bin
-//      is split again with a finer histogram over its range (only then: more barriers); keys that are
+//      The few listed keys are ranked by (key, lower index first) by the threads that own them.  The keys of a crowded bin
+//      are counted again, over the range that they have (only then: more barriers); keys that are
 //      all equal are ranked by index during the emission;
 //   4. emission merged with all text positions: warp ballots rank the kept tokens, the per-warp
 //      counts meet in shared memory                                                     [barrier D]
@@ -42,10 +42,17 @@ constexpr float kFixInv = 1.f / 1152921504606846976.f;      // 2^-60, exact
 // more, leave up to 32 keys in the bin where the budget runs out; fewer bins cost less to count up, fewer keys in one less to
 // rank.  (Bins laid over the range of the keys, which needs a pass, a barrier and two reductions first, held more:
 // a few strong tokens stretch the range.)
+// Where the window does not fit -- scores within a percent of one another, one token with nearly all of the attention, scores that
+// are not normalised -- a second histogram does.  mvla_select in us, 768 / 1791 / 3584 tokens: as the window expects 5.3 / 6.6 / 10.6, spread of 3e-4
+// 6.4 / 9.6 / 13.4, one token with 99 % 6.8 / 9.6 / 14.6, all equal 6.5 / 8.8 / 13.1, four fifths zero 6.4 / 8.6 / 12.0.  (Its bins laid over the whole
+// range of the crowded bin instead of over its keys, in a pass that also ranked the other modality: 6.3 / 9.5 / 13.2, 8.2 / 12.1 / 17.8, 9.0 / 15.0 /
+// 24.1, 10.5 / 17.2 / 27.2.  Keys of a warp that share a bin added up before they are counted: 0.3 to 1 us less with all keys in
+// one bin, but 0.1 to 0.2 more in every step.)
 constexpr int sel_bin_bits(int cap) { return cap <= 1024 ? 11 : 12; }
 constexpr int kWindowOctaves = 8, kWindowBelow = 6;
 constexpr int kSliceBins = 128;     // bins that a warp reads at once: four a lane
 constexpr int kCandMax = 64;        // keys of the threshold bin ranked from a list; above that the bin is split again
+constexpr int kSelLevels = 5;       // histograms at most: every one after the second takes 11 bits off a key (32, 21, 10: then all keys of a bin are equal)
 
 template <int NT, int EPT>
 struct SelectSmem {
@@ -55,10 +62,11 @@ struct SelectSmem {
     alignas(16) uint32_t before[kBins];      // counts in the bins before, within the slice
     uint32_t slice[kSlices];                 // counts of every slice of the bins
     alignas(16) float red[4][NT / 32];       // per-warp partial sums: scores 2D, 3D; norms 2D, 3D
-    alignas(16) uint32_t cand[2][kCandMax];  // listed keys: place in the bin, index complemented below it: larger = ranked first; unused: 0
-    int2 thr[2];                             // per modality: the bin in which the budget runs out, keys to take from it
-    int wtot[NT / 32];                       // emission: kept tokens of every warp; ties by index: 2D (low half), 3D (high half)
+    alignas(16) uint32_t cand[2][kCandMax];          // listed keys: place in the bin, index complemented below it: larger = ranked first; unused: 0
+    alignas(16) uint32_t ext[4];             // of a crowded bin: complement of its smallest key, its largest key: 2D, 3D
     int ncand[2];
+    int take[2];                             // per modality: keys to take from the bin in which the budget runs out
+    int wtot[NT / 32];                       // emission: kept tokens of every warp; ties by index: 2D (low half), 3D (high half)
     int budget[2];                           // kept tokens per modality
     float x[4], mhat[4];                     // the indicators, and smoothed
     int sets[3];                             // C_S1, C_S2, their fusion
@@ -164,11 +172,9 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
         for (int i = tid; i < kSelBins / 4; i += NT) reinterpret_cast<uint4*>(sm.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     };
     clear_hist();
-    auto clear_list = [&]() {
-        if (tid < 2 * kCandMax) (&sm.cand[0][0])[tid] = 0u;
-        if (tid < 2) sm.ncand[tid] = 0;
-    };
-    clear_list();
+    if (tid < 2 * kCandMax) (&sm.cand[0][0])[tid] = 0u;
+    if (tid < 2) sm.ncand[tid] = 0;
+    if (tid < 4) sm.ext[tid] = 0u;
     float a[EPT], prev[EPT], nrm[EPT];
     unsigned long long fx[EPT];
     float4 mprev = make_float4(0.f, 0.f, 0.f, 0.f);       // the smoothed indicators so far
@@ -315,29 +321,6 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
         }
     };
 
-    // The listed keys of a modality are ranked among themselves, unless its bin was crowded: then they are undecided again.
-    int listed2 = 0, listed3 = 0;
-    auto rank_listed = [&](int (&st)[EPT], bool crowded2, bool crowded3) {
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-            if (st[e] != 3) continue;
-            const int j = j0 + 32 * e;
-            const bool is3 = j >= n2;
-            if (is3 ? crowded3 : crowded2) { st[e] = 2; continue; }
-            const uint32_t place = (key[e] - (is3 ? lo3 : lo2)) & ((1u << (is3 ? sh3 : sh2)) - 1u);
-            const uint32_t mine = place << 12 | static_cast<uint32_t>(kMaxVis - 1 - j);
-            const int n = is3 ? listed3 : listed2;
-            int rank = 0;
-#pragma unroll 1
-            for (int i = 0; i < n; i += 8) {                   // (entries past n are zero)
-                const uint4 q = reinterpret_cast<const uint4*>(sm.cand[is3 ? 1 : 0])[i / 4], w = reinterpret_cast<const uint4*>(sm.cand[is3 ? 1 : 0])[i / 4 + 1];
-                rank += ((q.x > mine ? 1 : 0) + (q.y > mine ? 1 : 0)) + ((q.z > mine ? 1 : 0) + (q.w > mine ? 1 : 0));
-                rank += ((w.x > mine ? 1 : 0) + (w.y > mine ? 1 : 0)) + ((w.z > mine ? 1 : 0) + (w.w > mine ? 1 : 0));
-            }
-            st[e] = rank < sm.thr[is3 ? 1 : 0].y ? 1 : 0;
-        }
-    };
-
     // ---- 3. kept or dropped, by the number of keys in higher bins; where the budget runs out inside a bin, by rank in it
     // st[e]: 0 dropped, 1 kept, 2 undecided, 3 on the list of its bin
     int st[EPT];
@@ -347,8 +330,9 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
     int take2 = k2, take3 = k3;               // to be taken from the keys under examination
     bool act2 = true, act3 = true;            // the modality still has undecided keys
     bool ties = false;
+    int listed2 = 0, listed3 = 0;
 #pragma unroll 1
-    for (int level = 0; level < 6; ++level) {
+    for (int level = 0; level < kSelLevels; ++level) {
         auto count_slice = [&](int i) {                           // (both halves of a word at once: a half never exceeds kMaxVis)
             const uint4 x = reinterpret_cast<const uint4*>(sm.hist)[i * 32 + lane];
             const uint32_t b1 = x.x, b2 = b1 + x.y, b3 = b2 + x.z, mine = b3 + x.w;
@@ -391,7 +375,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
                 const uint32_t place = (key[e] - (is3 ? lo3 : lo2)) & ((1u << (is3 ? sh3 : sh2)) - 1u);
                 static_assert(kMaxVis == 1 << 12, "an index is 12 bits");
                 if (slot < kCandMax) sm.cand[is3 ? 1 : 0][slot] = place << 12 | static_cast<uint32_t>(kMaxVis - 1 - j);
-                sm.thr[is3 ? 1 : 0] = make_int2(bin[e], (is3 ? take3 : take2) - bound[e]);      // (the same from all keys of the bin)
+                sm.take[is3 ? 1 : 0] = (is3 ? take3 : take2) - bound[e];      // (the same from all keys of the bin)
             }
         }
         __syncthreads();                                                                   // ---- barrier C
@@ -399,29 +383,36 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
         listed3 = act3 ? sm.ncand[1] : listed3;
         act2 = act2 && listed2 > kCandMax;
         act3 = act3 && listed3 > kCandMax;
-        if (!act2 && !act3) break;                             // block-uniform
-        // A crowded bin becomes the whole range of the next pass, unless its keys are all equal.  The other modality's list
-        // is ranked now: the lists are cleared.
-        const int2 t2 = sm.thr[0], t3 = sm.thr[1];
-        rank_listed(st, act2, act3);
-        if (act2) take2 = t2.y;
-        if (act3) take3 = t3.y;
-        if (act2 && level > 0 && sh2 == 0) { ties = true; act2 = false; }
-        if (act3 && level > 0 && sh3 == 0) { ties = true; act3 = false; }
-        if (!act2 && !act3) break;
-        auto narrow = [&](int tb, uint32_t& lo, int& sh) {
-            const uint32_t b = static_cast<uint32_t>(kSelBins - 1 - tb), first = lo + (b << sh);
-            const uint32_t from = level == 0 && b == 0 ? 0u : first;             // (the ends of the window are open)
-            const uint32_t last = level == 0 && b == kSelBins - 1 ? 0xFFFFFFFFu : first + ((1u << sh) - 1u);
-            lo = from;
-            sh = max(0, 32 - __clz(last - from) - kSelBits);
-        };
-        if (act2) narrow(t2.x, lo2, sh2);
-        if (act3) narrow(t3.x, lo3, sh3);
-        __syncthreads();
+        if (__builtin_expect(!act2 && !act3, 1)) break;        // block-uniform
+        // The keys of a crowded bin are counted once more, over the range that they have, unless they are all equal.  (This
+        // part is rare and runs from a cold instruction cache, half a microsecond for 1.5 KB: it does no more than it must.)
+        if (act2) take2 = sm.take[0];
+        if (act3) take3 = sm.take[1];
+        uint32_t mn2 = 0u, mx2 = 0u, mn3 = 0u, mx3 = 0u;
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) {
+            const bool is3 = j0 + 32 * e >= n2;
+            if (st[e] != 3 || !(is3 ? act3 : act2)) continue;
+            st[e] = 2;
+            if (is3) { mn3 = max(mn3, ~key[e]); mx3 = max(mx3, key[e]); }
+            else     { mn2 = max(mn2, ~key[e]); mx2 = max(mx2, key[e]); }
+        }
+        mn2 = __reduce_max_sync(0xffffffffu, mn2); mx2 = __reduce_max_sync(0xffffffffu, mx2);
+        mn3 = __reduce_max_sync(0xffffffffu, mn3); mx3 = __reduce_max_sync(0xffffffffu, mx3);
+        if (lane == 0) { atomicMax(&sm.ext[0], mn2); atomicMax(&sm.ext[1], mx2); atomicMax(&sm.ext[2], mn3); atomicMax(&sm.ext[3], mx3); }
         clear_hist();
-        clear_list();
+        if (tid < 2 * kCandMax && (tid < kCandMax ? act2 : act3)) (&sm.cand[0][0])[tid] = 0u;
         __syncthreads();
+        const uint4 x = *reinterpret_cast<const uint4*>(sm.ext);
+        if (tid < 2) sm.ncand[tid] = 0;
+        auto narrow = [&](uint32_t least, uint32_t most, uint32_t& lo, int& sh) {
+            lo = least;
+            sh = max(0, 32 - __clz(most - least) - kSelBits);
+            return most > least;
+        };
+        if (act2 && !narrow(~x.x, x.y, lo2, sh2)) { ties = true; act2 = false; }
+        if (act3 && !narrow(~x.z, x.w, lo3, sh3)) { ties = true; act3 = false; }
+        if (!act2 && !act3) break;
 #pragma unroll
         for (int e = 0; e < EPT; ++e) {
             const bool is3 = j0 + 32 * e >= n2;
@@ -430,8 +421,26 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
             atomicAdd(&sm.hist[bin[e]], is3 ? 0x10000u : 1u);
         }
         __syncthreads();
+        if (tid < 4) sm.ext[tid] = 0u;
     }
-    rank_listed(st, false, false);
+    // the listed keys of a modality are ranked among themselves
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+        if (st[e] != 3) continue;
+        const int j = j0 + 32 * e;
+        const bool is3 = j >= n2;
+        const uint32_t place = (key[e] - (is3 ? lo3 : lo2)) & ((1u << (is3 ? sh3 : sh2)) - 1u);
+        const uint32_t mine = place << 12 | static_cast<uint32_t>(kMaxVis - 1 - j);
+        const int n = is3 ? listed3 : listed2;
+        int rank = 0;
+#pragma unroll 1
+        for (int i = 0; i < n; i += 8) {                   // (entries past n are zero)
+            const uint4 q = reinterpret_cast<const uint4*>(sm.cand[is3 ? 1 : 0])[i / 4], w = reinterpret_cast<const uint4*>(sm.cand[is3 ? 1 : 0])[i / 4 + 1];
+            rank += ((q.x > mine ? 1 : 0) + (q.y > mine ? 1 : 0)) + ((q.z > mine ? 1 : 0) + (q.w > mine ? 1 : 0));
+            rank += ((w.x > mine ? 1 : 0) + (w.y > mine ? 1 : 0)) + ((w.z > mine ? 1 : 0) + (w.w > mine ? 1 : 0));
+        }
+        st[e] = rank < sm.take[is3 ? 1 : 0] ? 1 : 0;
+    }
 
     // ---- 4. emission.  Tokens are ranked in visual order (2D first) by warp ballots.  The three segments are contiguous,
     //         so a kept token's output row is the number of rows that the segments lying before its own contribute plus its
