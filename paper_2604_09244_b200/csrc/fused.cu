@@ -357,7 +357,9 @@ salience_fast_kernel(const __grid_constant__ BD bd, const __grid_constant__ CUte
             for (int c = 0; c < nq; ++c)
                 if (one) tma_load_3d(q_smem + static_cast<uint32_t>(kh * npad * 128 + c * 2048), &tmap_q, kh * box_elems, h, qrow + c * 16, bar_full);
         // Whatever the kernel before this one wrote is complete: the next kernel may become resident now and may read
-        // such data in its prologue.
+        // such data in its prologue.  Not with `early`: the kernel behind it (the norms, or the tail of a chained step) reads
+        // promised inputs before its own wait, or nothing, and writes the norms into this step's scratch set, which the
+        // step six calls back left complete: the kernel before this one could start only after that.
         pdl_trigger();
         if (stamps && one) {                  // measurement aid: when this CTA was free to start its loads
             const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
@@ -622,10 +624,15 @@ cudaError_t with_fast_variant(const BatchDesc& bd, int npad, int tiles_per_cta, 
 #define MVLA_FAST1(TC, NTL, SP, KD)                                                                             \
     if (tcol == TC && tiles_per_cta == NTL && split == SP && kind == KD)                                        \
         return with_desc(bd, [&](const auto& d) { return use(FastVariant<TC, NTL, SP, KD, std::decay_t<decltype(d)>>{}, d); });
-#define MVLA_FAST(TC, NTL, SP) MVLA_FAST1(TC, NTL, SP, kPlain) MVLA_FAST1(TC, NTL, SP, kWithCache) MVLA_FAST1(TC, NTL, SP, kForPatches) MVLA_FAST1(TC, NTL, SP, kEarly)
+#define MVLA_FAST(TC, NTL, SP) MVLA_FAST1(TC, NTL, SP, kPlain) MVLA_FAST1(TC, NTL, SP, kWithCache) MVLA_FAST1(TC, NTL, SP, kForPatches)
     MVLA_FAST(16, 1, 1) MVLA_FAST(16, 2, 1) MVLA_FAST(32, 1, 2) MVLA_FAST(64, 1, 2) MVLA_FAST(32, 2, 2) MVLA_FAST(64, 2, 2)
 #undef MVLA_FAST1
 #undef MVLA_FAST
+    if (kind != kEarly || bd.n != 1 || tiles_per_cta != 1) return cudaErrorInvalidConfiguration;
+    const OneDesc one = {{bd.s[0]}, 1};       // a chained step has one sample and one tile per CTA (mvla_prune_step)
+    if (tcol == 16) return use(FastVariant<16, 1, 1, kEarly, OneDesc>{}, one);
+    if (tcol == 32) return use(FastVariant<32, 1, 2, kEarly, OneDesc>{}, one);
+    if (tcol == 64) return use(FastVariant<64, 1, 2, kEarly, OneDesc>{}, one);
     return cudaErrorInvalidConfiguration;
 }
 
