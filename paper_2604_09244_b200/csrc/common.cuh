@@ -206,8 +206,9 @@ cudaError_t launch_head_reduce(const float* part, int64_t part_stride, int n_hea
                                float* attn, cudaStream_t stream);
 
 // L1 feature norms of the visual rows.  `beside_predecessor`: the kernel is launched right after a scoring
-// kernel that releases its dependents only once ITS predecessor is complete (launch_salience_fast): it then
-// runs beside the scoring kernel and completes after it.  With `acc64` (and beside_predecessor) it also does what
+// kernel, runs beside it and completes after it.  That kernel releases its dependents only once ITS predecessor is
+// complete, so that `hidden` may come from there; with `early` (launch_salience_fast) at once, `hidden` being promised stable and
+// `l1` of a scratch set that no step in flight uses.  With `acc64` (and beside_predecessor) it also does what
 // launch_take_scores does, for the samples of the launch.
 cudaError_t launch_l1norm(const BatchDesc& bd, int dtype, int d_model, const void* hidden,
                           float* l1, bool beside_predecessor, unsigned long long* acc64, float* attn, cudaStream_t stream);
