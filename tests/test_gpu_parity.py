@@ -558,6 +558,104 @@ def test_chained_requests_match_serial_steps(text_first):
             assert len(got[t]) == len(ref[t]) and all(torch.equal(x, y) for x, y in zip(got[t], ref[t])), t
 
 
+@pytest.mark.parametrize("mode", [mvla.MODE_FIXED, mvla.MODE_ADAPTIVE])
+@pytest.mark.parametrize("shape", [
+    dict(H=4, d=128, n_txt=(5,)),                                   # 16, 32 and 64 tensor-memory columns
+    dict(H=4, d=128, n_txt=(32,)),
+    dict(H=4, d=128, n_txt=(64,)),
+    dict(H=8, d=64, n_txt=(33,), n_kv_heads=2),
+    dict(H=4, d=96, n_txt=(17,), dtype="fp8"),
+    dict(H=64, d=64, n_txt=(21,), n_2d=(500,), n_3d=(400,)),        # 512 scoring CTAs: the streaming kernel, in a chained step
+], ids=lambda s: f"{s['H']}x{s['d']}_text{s['n_txt'][0]}_{s.get('dtype', 'bf16')}_kv{s.get('n_kv_heads', 0)}")
+def test_chained_steps_of_one_episode_match_serial_steps(shape, mode):
+    # every step carries over the state of the step directly before it, whose tail its scores are taken beside
+    wl = W.small_workload(67, **{**dict(batch=1, D=256, dtype="bf16", n_2d=(129,), n_3d=(383,), keep=(0.2,), keep_fixed=(0.25, 0.15),
+                                        steps=14, cold_start=1), **shape})
+    devs = [device_tensors(wl, t) for t in range(14)]
+
+    def run(flag):
+        ctx = mvla.context_for(wl)
+        outs = [ctx.alloc_outputs(wl.samples, extras=True) for _ in range(14)]
+        torch.cuda.synchronize()
+        if flag:
+            torch.cuda._sleep(2_000_000)          # the host runs ahead: the steps follow one another on the GPU
+        for t, (d, o) in enumerate(zip(devs, outs)):
+            ctx.prune_step(0, wl.samples, mode, d["q"], d["k"], d["v"], d["hidden"], flags=flag | (mvla.FLAG_RESET_STATE if t == 0 else 0), out=o)
+            if not flag:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        ctx.close()
+        as_bytes = lambda x: x.contiguous().view(torch.uint8)
+        return [(o.attn, o.ahat, o.z, o.budgets, o.diag, o.kept_idx[:o.total_kept]) +
+                tuple(as_bytes(x[:o.total_kept]) for x in (o.out_hidden, o.out_k, o.out_v)) for o in outs]
+
+    ref, got = run(0), run(mvla.FLAG_INPUTS_STABLE)
+    for t in range(14):
+        assert all(torch.equal(x, y) for x, y in zip(got[t], ref[t])), t
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_chained_forked_and_unpromised_calls_in_one_context_match_serial_calls(seed):
+    # One sample (chained on the caller's stream), two samples (forked to the side streams), steps without the promise, dry
+    # runs and mvla_select in an order drawn at random, on shared state slots, through every scratch set several times, with
+    # inputs that one of the last eight calls has written and output buffers used again: the same bits as one at a time.
+    import dataclasses
+    wl = W.small_workload(71, batch=2, D=256, H=4, d=128, dtype="bf16", n_txt=(21, 9), n_2d=(130,), n_3d=(190,), keep=(0.4, 0.3), steps=6)
+    devs = [device_tensors(wl, t) for t in range(6)]
+    n_calls, n_out = 64, 16
+    rng = np.random.default_rng(seed)
+    calls = []
+    for t in range(n_calls):
+        kind = ("chain", "fork", "plain", "dry", "select")[rng.choice(5, p=[0.4, 0.35, 0.1, 0.08, 0.07])]
+        slots = [int(x) for x in rng.permutation(4)[:1 if kind in ("chain", "select") else 2]]
+        back = t - int(rng.integers(1, 9))
+        source = back if back >= 0 and kind != "select" and calls[back][0] != "select" and rng.random() < 0.4 else -1
+        if source < 0:
+            samples = [dataclasses.replace(wl.samples[i], state_slot=slot) for i, slot in enumerate(slots)]
+        else:                                                 # in the first 100 rows of an earlier call's outputs, states of their own
+            samples = [W.layout_2d_3d_txt(50 * i, 10, 15, 25, keep_2d=0.5, keep_3d=0.3, keep_total=0.4, state_slot=4 + slot)
+                       for i, slot in enumerate(slots)]
+        calls.append((kind, samples, source, mvla.MODE_FIXED if rng.random() < 0.5 else mvla.MODE_ADAPTIVE, rng.random() < 0.3))
+    scores = torch.from_numpy(rng.random(320).astype(np.float32)).cuda()
+
+    def run(flag):
+        ctx = mvla.context_for(wl, n_state_slots=8)
+        bufs = [ctx.alloc_outputs(wl.samples, extras=True) for _ in range(n_out)]
+        for o in bufs:
+            for x in (o.out_hidden, o.out_k, o.out_v):
+                x.zero_()
+        torch.cuda.synchronize()
+        for t, (kind, samples, source, mode, busy) in enumerate(calls):
+            d, o = devs[t % 6], bufs[t % n_out]
+            if flag and busy:
+                torch.cuda._sleep(200_000)                    # touches none of the calls' buffers
+            if kind == "select":
+                ctx.select(0, samples, mvla.MODE_FIXED, scores, out=o)
+                o.total_kept = 0                              # (no rows)
+            else:
+                p = bufs[source % n_out]
+                q, k, v, h = ((d["q"], d["k"], d["v"], d["hidden"]) if source < 0 else
+                              (d["q"][:100], p.out_k[:100], p.out_v[:100], p.out_hidden[:100]))
+                ctx.prune_step(0, samples, mode, q, k, v, h, out=o,
+                               flags=mvla.FLAG_NO_STATE_UPDATE if kind == "dry" else flag if kind in ("chain", "fork") else 0)
+            if not flag:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        ctx.close()
+        return bufs
+
+    ref, got = run(0), run(mvla.FLAG_INPUTS_STABLE)
+    for t in range(n_calls - n_out, n_calls):
+        kind, samples = calls[t][:2]
+        a, b = ref[t % n_out], got[t % n_out]
+        n_vis, n, m = sum(s.n_2d + s.n_3d for s in samples), len(samples), a.total_kept
+        listed = int(a.out_offsets[n])
+        for x, y in ((a.ahat[:n_vis], b.ahat[:n_vis]), (a.out_offsets[:n + 1], b.out_offsets[:n + 1]), (a.budgets[:n], b.budgets[:n]),
+                     (a.kept_idx[:listed], b.kept_idx[:listed]), (a.out_hidden[:m], b.out_hidden[:m]), (a.out_k[:m], b.out_k[:m]),
+                     (a.out_v[:m], b.out_v[:m])):
+            assert torch.equal(x, y), (t, kind)
+
+
 @pytest.mark.parametrize("reads", ["state", "rows"])
 def test_stable_steps_are_ordered_after_a_call_without_the_promise(reads):
     # Six stable batches, so that every scratch set has events of its own; a call without the promise, kept from running for 10 ms; a
