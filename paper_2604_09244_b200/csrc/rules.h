@@ -21,8 +21,8 @@ namespace mvla {
 //   rows of 10 KB, 40 heads of 128: 6 49.1 / 43.7 | 15 88.0 / 99.2; 20 heads: 6 28.0 / 33.5
 //   rows of 16 KB, 16 heads of 128: 6 45.6 / 38.4, 10 66.8 / 61.2 | 6 45.8 / 37.6
 // Above 88 tokens a multiprocessor inside loses whatever the texts (32 heads of 128: 18 samples 90.4 / 92.6, 32 153 / 163), and samples of more
-// than 16 key tiles go either way (2 x 3426 77.4 / 73.3, 7 x 2584 115.4 / 119).  Rows of eight times the keys' bytes, where the scores of few jobs end early:
-// e4m3, 16 heads of 256, 4 key heads, 12 x 435 (192 jobs) 26.5 / 27.3, 20 x 350 (320 jobs) 37.8 / 34.8.
+// than 16 key tiles go either way (2 x 3426 77.4 / 73.3, 7 x 2584 115.4 / 119).  Rows of eight times the keys' bytes, where the
+// scores of few jobs end early: e4m3, 16 heads of 256, 4 key heads, 12 x 435 (192 jobs) 26.5 / 27.3, 20 x 350 (320 jobs) 37.8 / 34.8.
 constexpr uint32_t kNormPiece = 8192;        // bytes of a row that a norm warp fetches at once
 struct NormsInsideSizes {
     int64_t rows;               // visual tokens of the launch
@@ -51,7 +51,8 @@ inline bool patch_norms_inside_pays(int n_heads, int padded_text) { return n_hea
 // Whether a step of one sample with stable inputs and one key tile per scoring CTA is chained on the caller's stream, with its
 // scores taken beside the selection and row copy of the step before, or forked to a side stream: two or three launches against three or four
 // and four event calls (10 to 14 us of host time).  `moved`: bytes of keys, feature rows, text queries and surviving rows in and out.
-// Per request of eight in a row, fork / chain in us, on a fast host (fork at the host's 9.6 to 10 us with fixed budgets, 11.5 to 12 adaptive, at any size):
+// Per request of eight in a row, fork / chain in us, on a fast host (fork at the host's 9.6 to 10 us with fixed budgets, 11.5 to
+// 12 adaptive, at any size):
 //   fixed, up to 1.5 scoring CTAs a multiprocessor: 160 tokens 9.8 / 6.5, 32 heads of 64, 768 tokens 9.7 / 7.9; of 96 (15 MB) 9.7 / 9.4; of 128, 640
 //     (17 MB) 9.7 / 9.9, 768 (20 MB) 9.6 / 9.9; 16 heads of 256, 768 (20 MB) 9.9 / 9.3, 850 (22 MB) 10.0 / 9.9, 950 (24 MB) 10.0 / 10.3;
 //   fixed, more CTAs: 32 heads of 64, 950 tokens (12 MB) 9.8 / 9.1; of 96, 800 (15.4 MB) 9.9 / 10.3, 900 (17.1 MB) 10.0 / 10.5,
@@ -59,8 +60,8 @@ inline bool patch_norms_inside_pays(int n_heads, int padded_text) { return n_hea
 //   adaptive: 32 heads of 64, 950 (15 MB) 11.8 / 9.8; of 96, 800 (19 MB) 11.7 / 12.0; of 128, 600 (20 MB) 11.9 / 10.6, 700 (22.5 MB) 12.0 / 12.3, 768
 //     (24.5 MB) 11.8 / 12.7, 850 (27 MB) 12.0 / 13.4;
 // on a slow host 768 of 128 fixed 13.4 / 9.8, 1010 of 96 adaptive 14.0 / 11.8.  The first pass of a new context gains more, eight requests of 768
-// tokens 167 / 106 us, of 800 tokens and heads of 96 165 / 106: a step that loses 3 % later is left chained.  Two tiles per CTA: 1280 tokens of 64 (17 MB) 11.3 / 12.1, of 96 11.4 / 14.3, adaptive 14.0 / 18.5.  (In a CUDA
-// graph launches cost nothing: always the fork.)
+// tokens 167 / 106 us, of 800 tokens and heads of 96 165 / 106: a step that loses 3 % later is left chained.  Two tiles per CTA:
+// 1280 tokens of 64 (17 MB) 11.3 / 12.1, of 96 11.4 / 14.3, adaptive 14.0 / 18.5.  (In a CUDA graph launches cost nothing: always the fork.)
 inline bool chain_pays(int64_t moved, int ctas, bool adaptive, int sm_count)
 {
     const bool all_at_once = 2 * ctas <= 3 * sm_count;      // scoring CTAs that run beside the tail before it
