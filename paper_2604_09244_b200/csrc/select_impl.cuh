@@ -43,16 +43,19 @@ constexpr float kFixInv = 1.f / 1152921504606846976.f;      // 2^-60, exact
 // rank.  (Bins laid over the range of the keys, which needs a pass, a barrier and two reductions first, held more:
 // a few strong tokens stretch the range.)
 // Where the window does not fit -- scores within a percent of one another, one token with nearly all of the attention, scores that
-// are not normalised -- a second histogram does.  mvla_select in us, 768 / 1791 / 3584 tokens: as the window expects 5.3 / 6.6 / 10.6, spread of 3e-4
-// 6.4 / 9.6 / 13.4, one token with 99 % 6.8 / 9.6 / 14.6, all equal 6.5 / 8.8 / 13.1, four fifths zero 6.4 / 8.6 / 12.0.  (Its bins laid over the whole
-// range of the crowded bin instead of over its keys, in a pass that also ranked the other modality: 6.3 / 9.5 / 13.2, 8.2 / 12.1 / 17.8, 9.0 / 15.0 /
-// 24.1, 10.5 / 17.2 / 27.2.  Keys of a warp that share a bin added up before they are counted: 0.3 to 1 us less with all keys in
-// one bin, but 0.1 to 0.2 more in every step.)
+// are not normalised -- a second histogram does.  mvla_select in us, 768 / 1791 / 3584 tokens, and in parentheses with bins laid
+// over the whole range of the crowded bin instead of over its keys, in a pass that also ranked the other modality:
+//   as the window expects 5.3 / 6.6 / 10.6; spread of 3e-4 6.4 / 9.6 / 13.4 (6.3 / 9.5 / 13.2);
+//   one token with 99 % 6.8 / 9.6 / 14.6 (8.2 / 12.1 / 17.8); all equal 6.5 / 8.8 / 13.1 (9.0 / 15.0 / 24.1);
+//   four fifths zero 6.4 / 8.6 / 12.0 (10.5 / 17.2 / 27.2).
+// Keys of a warp that share a bin added up before they are counted: 0.3 to 1 us less with all keys in one bin, but 0.1 to 0.2
+// more in every step.
 constexpr int sel_bin_bits(int cap) { return cap <= 1024 ? 11 : 12; }
 constexpr int kWindowOctaves = 8, kWindowBelow = 6;
 constexpr int kSliceBins = 128;     // bins that a warp reads at once: four a lane
 constexpr int kCandMax = 64;        // keys of the threshold bin ranked from a list; above that the bin is split again
-constexpr int kSelLevels = 5;       // histograms at most: every one after the second takes 11 bits off a key (32, 21, 10: then all keys of a bin are equal)
+// Histograms at most: every one after the second takes 11 bits off a key (32, 21, 10: then all keys of a bin are equal).
+constexpr int kSelLevels = 5;
 
 template <int NT, int EPT>
 struct SelectSmem {
