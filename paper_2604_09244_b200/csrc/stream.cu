@@ -446,11 +446,13 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
 }
 
 // grid = clusters x cluster size (1-D), one CTA per multiprocessor.
-// ROOM: the feature norms are to run beside this kernel (they do not fit its own two norm warps; figures from before there were these).  Its ten warps put three on two of a multiprocessor's four
-// register files (16384 registers each): at the 168 registers a thread that the compiler takes these are full, no CTA of
-// the norms fits, and they start when the scores are done.  144 leave room for two warps of 32 registers in each (adaptive
-// steps, 10 requests of 190 tokens 31.2 -> 24.1 us, 4 of 768 33.6 -> 27.1) at the price of 8 bytes a thread stored and 24
-// loaded; with 128 these are 68 and 144 (16 requests of 768 tokens 97 -> 106).  Without norms the registers are worth more (16 patch-by-patch steps 96.3 us, 99.1 with 144).
+// ROOM: the feature norms are to run beside this kernel (norms_inside_pays says no).  Its ten warps put three on two of a
+// multiprocessor's four register files (16384 registers each): at the 168 registers a thread that the compiler takes these are
+// full, no CTA of the norms fits, and they start when the scores are done.  144 leave room for two warps of 32 registers in
+// each, at the price of 8 bytes a thread stored and 24 loaded (with 128 these are 68 and 144: 16 requests of 768 tokens 97 ->
+// 106 us when their norms ran beside).  8 requests of 3584 tokens, 64 queries, take 161.7 us with 144 and 162.0 with 168.
+// Where no norms run beside, the registers are worth more to the attention copy: 16 patch-by-patch steps 76.5 us with 168, 78.6
+// with 144; 16 adaptive requests 93.7 and 93.0.
 template <bool ROOM>
 __global__ void __maxnreg__(ROOM ? 144 : kStreamRegs)
 salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,
