@@ -70,6 +70,7 @@ struct mvla_ctx {
                                  // the selections of the steps before it)
     int32_t* tail_list;          // [kSets][rows_all] kept list as the copying CTAs read it (-1 between launches)
     unsigned int* tail_ticket;   // [kSets] ticket counters of the patch-by-patch tail (zero between launches)
+    int32_t* hand;               // [kSets][chunks of a batch][kHandStride] counters of tails beside the scoring kernel (zero between launches)
     unsigned long long* patch_rec;   // [kSets][vis_all / 2][3] hand-over words of the patch-by-patch tail (all ones between launches)
     size_t rows_all;             // max_batch * (kHandWords + kListStride (max_text + max_vis))
     int sm_count;                // multiprocessors of the device
@@ -373,6 +374,12 @@ cudaError_t stream_pays(const mvla_ctx* ctx, const BatchDesc& bd, int tiles_per_
     return e;
 }
 
+// A tail that may run beside the scoring kernel: its counters in; whether it does, and how, out.
+struct BesideTail {
+    int32_t* hand;
+    int parts, free_sms;         // see stream_beside_tail; free_sms 0: behind it, as ever
+};
+
 // Salience of one chunk (+ L1 norms into `l1` when asked; + the scores as fp32 into `attn_out` when asked).  The per-head
 // contributions are added into the fixed-point accumulators `acc64` (*used_acc64 = true) where a kernel that does so covers the
 // shape, else they land in ctx->part.
@@ -381,7 +388,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
                            cudaStream_t st, AlphaOut alpha = AlphaOut{nullptr, 0, 0},
                            int32_t* rearm = nullptr, bool norms_beside = false, unsigned long long* stamps = nullptr,
                            bool with_cache = false, unsigned long long* rearm_rec = nullptr, float* attn_out = nullptr,
-                           bool* norms_inside = nullptr, bool early = false)
+                           bool* norms_inside = nullptr, bool early = false, BesideTail* tail = nullptr)
 {
     if (used_acc64) *used_acc64 = false;
     const mvla_config& c = ctx->cfg;
@@ -414,7 +421,14 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     // With `norms_inside`: norms only if the scoring kernel takes them itself, and whether it did.
     const NormsInsideSizes sizes = {visual_tokens(bd), npad, max_tiles, bd.n * c.n_heads, c.n_heads, static_cast<int64_t>(c.d_model * ctx->elem),
                                    static_cast<int64_t>(ctx->kv_heads * c.head_dim * ctx->qk_elem), ctx->sm_count};
-    const bool inside = streaming && hidden && l1 && (norms_inside ? patch_norms_inside_pays(c.n_heads, npad) : norms_beside && norms_inside_pays(sizes));
+    if (tail) {
+        tail->free_sms = 0;
+        if (streaming && (e = stream_beside_tail(bd, c.n_heads, static_cast<int64_t>(c.head_dim * ctx->qk_elem), sizes.key_bytes, hidden ? sizes.row_bytes : 0,
+                                               &tail->free_sms, &tail->parts)) != cudaSuccess)
+            return e == cudaErrorInvalidConfiguration ? MVLA_ERR_UNSUPPORTED : fail_cuda(ctx, e);
+    }
+    const bool beside = tail && tail->free_sms > 0;
+    const bool inside = streaming && hidden && l1 && (beside || (norms_inside ? patch_norms_inside_pays(c.n_heads, npad) : norms_beside && norms_inside_pays(sizes)));
     if (norms_inside) {
         *norms_inside = inside;
         if (!inside) hidden = nullptr;
@@ -430,7 +444,7 @@ int32_t run_salience_chunk(mvla_ctx* ctx, const BatchDesc& bd, const void* q, co
     if (streaming) {
         e = launch_salience_stream(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, static_cast<int>(ctx->qk_elem), tq, tk, acc64,
                                    ctx->status_dev, alpha, rearm, rearm_rec, stamps, hidden && l1 && norms_beside, inside ? hidden : nullptr,
-                                   static_cast<int>(c.d_model * ctx->elem), l1, st);
+                                   static_cast<int>(c.d_model * ctx->elem), l1, beside ? tail->hand : nullptr, st);
         if (used_acc64) *used_acc64 = acc64 != nullptr;
     } else if (f32) {
         e = launch_salience_f32(bd, c.n_heads, c.n_heads / ctx->kv_heads, c.head_dim, tq, tk, tiles_per_cta, cluster, npad, acc64, ctx->status_dev, rearm, stamps, st);
@@ -846,6 +860,7 @@ static int32_t mvla_prune_create_impl(const mvla_config* cfg, mvla_ctx** out)
     ctx->acc64 = nullptr;
     ctx->tail_list = nullptr;
     ctx->tail_ticket = nullptr;
+    ctx->hand = nullptr;
     ctx->patch_rec = nullptr;
     ctx->sm_count = sm_count;
     ctx->stage_event = nullptr;
@@ -894,8 +909,11 @@ static int32_t mvla_prune_create_impl(const mvla_config* cfg, mvla_ctx** out)
     // (+ 1: a word that no launch ever writes, for mvla_selftest_wait_timeout)
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->tail_list), (kSets * ctx->rows_all + 1) * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(ctx->tail_list, 0xFF, (kSets * ctx->rows_all + 1) * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->tail_ticket), kSets * sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMemset(ctx->tail_ticket, 0, kSets * sizeof(unsigned int));
+    // (one allocation: the ticket counters, then the counters of tails beside the scoring kernel)
+    const size_t n_hand = kSets * static_cast<size_t>((c.max_batch + kMaxChunk - 1) / kMaxChunk) * kHandStride;
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->tail_ticket), (kHandStride + n_hand) * sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMemset(ctx->tail_ticket, 0, (kHandStride + n_hand) * sizeof(unsigned int));
+    ctx->hand = reinterpret_cast<int32_t*>(ctx->tail_ticket) + kHandStride;
     if (c.logit_cache) {
         ctx->cache_sig.assign(n_state, mvla_ctx::CacheSig{false, 0, 0, 0});
         alloc(&ctx->lcache, n_state * static_cast<size_t>(c.n_heads) * ctx->max_vis * ctx->cache_cols);
@@ -1277,11 +1295,12 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         bool used_acc64 = false;
         // the fused selection + copy kernel (below) wants its list words re-armed by the scoring kernel
         const bool tail = !forked;
+        BesideTail beside = {ctx->hand + (par * static_cast<size_t>((ctx->cfg.max_batch + kMaxChunk - 1) / kMaxChunk) + first / kMaxChunk) * kHandStride, 0, 0};
         ph.mark("mvla: scoring");
         rc = run_salience_chunk(ctx, bd, in->q, in->k, in->rows, adaptive ? in->hidden : nullptr, l1_ws, acc64,
                                 &used_acc64, forked ? ctx->aux[par] : st, AlphaOut{nullptr, 0, 0},
                                 tail ? ctx->tail_list + par * ctx->rows_all : nullptr, tail, tail && !chained ? ctx->stamps : nullptr,
-                                cache_on, nullptr, nullptr, nullptr, early);
+                                cache_on, nullptr, nullptr, nullptr, early, tail && !chained ? &beside : nullptr);
         if (rc != MVLA_OK) return rc;
         if (ctx->stage_event && !forked && !chained) {
             // under stream capture the record must become an event-record node of the graph (an "external"
@@ -1312,11 +1331,14 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
             // one kernel: a CTA per sample selects, the others copy rows as the kept list becomes known
             ctx->sel_valid[par] = false;             // this set was used outside the event chain
             ph.mark("mvla: selection + row copy");
-            const cudaError_t e2 = launch_select_copy(bd, gp, io, job, ctx->tail_list + par * ctx->rows_all,
-                                                      ctx->status_dev, chained,
-                                                      ctx->stamps && !chained ? ctx->stamps + 2 * kStampSlots : nullptr, st);
+            int32_t* const list = ctx->tail_list + par * ctx->rows_all;
+            unsigned long long* const stamps = ctx->stamps && !chained ? ctx->stamps + 2 * kStampSlots : nullptr;
+            const cudaError_t e2 = beside.free_sms > 0
+                ? launch_select_copy_beside(bd, gp, io, job, list, beside.hand, beside.parts, beside.free_sms, ctx->status_dev, stamps, st)
+                : launch_select_copy(bd, gp, io, job, list, ctx->status_dev, chained, stamps, st);
             if (e2 != cudaSuccess) {
                 clear_accumulators(acc64, bd, st);
+                if (beside.free_sms > 0) cudaMemsetAsync(beside.hand, 0, kHandStride * sizeof(int32_t), st);
                 return fail_cuda(ctx, e2);
             }
             continue;

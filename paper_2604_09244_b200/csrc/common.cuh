@@ -24,6 +24,10 @@ constexpr int kHandWords = kHandLines * 32;
 // many warps as move its segments (a dozen); side by side, 32 words shared a line of the L2 and its pollers were served
 // one after another: eight words a line shorten a step by 2 to 3 % (four a line: no more).
 constexpr int kListStride = 4;
+// Counters through which the streaming scoring kernel and a tail beside it meet: finished (head, part)s of every sample (from word 0 on),
+// tickets of the tail's CTAs, lots of its row copy given out, copying CTAs that are done.  Zero between launches: the tail sees to that.
+constexpr int kHandTicket = 32, kHandLots = 33, kHandLeft = 34, kHandStride = 64;
+constexpr uint32_t kNoNorm = 0xFFFFFFFFu;    // a feature norm that is not there yet (no result of arithmetic has these bits)
 constexpr int kMaxChunk = 32;        // samples carried by one launch (descriptors travel as kernel parameters)
 constexpr int kKeyTile = 128;        // visual keys per tile = rows of one MMA
 constexpr int kMaxCluster = 8;       // portable cluster size
@@ -189,7 +193,11 @@ cudaError_t launch_salience_f32(const BatchDesc& bd, int n_heads, int kv_group, 
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
                                    AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
-                                   unsigned long long* stamps, bool norms_beside, const void* hidden, int row_bytes, float* l1, cudaStream_t stream);
+                                   unsigned long long* stamps, bool norms_beside, const void* hidden, int row_bytes, float* l1, int32_t* hand,
+                                   cudaStream_t stream);
+// Whether the tail of a step runs beside the streaming kernel that scores it (tail_beside_pays; bytes as there).  free_sms: multiprocessors
+// that the kernel then leaves to it (0: no); parts: what a sample's counter of finished jobs counts up to.
+cudaError_t stream_beside_tail(const BatchDesc& bd, int n_heads, int64_t head_bytes, int64_t key_bytes, int64_t row_bytes, int* free_sms, int* parts);
 
 // Salience: per-head partial scores part[h][vis] (already scaled by 1/(H n_t)).
 // `use_umma`: tensor-core path (bf16 only).  tmaps: device-usable tensor maps (passed by value).
@@ -266,6 +274,13 @@ cudaError_t launch_compact(const BatchDesc& bd, const CompactJob& job, const int
 // (start: past the wait for the kernel before; the selecting CTA's end is when the list is written).
 cudaError_t launch_select_copy(const BatchDesc& bd, const GateParams& gp, const SelectIO& io, const CompactJob& job,
                                int32_t* list, int* status, bool stable, unsigned long long* stamps, cudaStream_t stream);
+
+// The same beside the streaming kernel that scores the step: a sample is selected when its scores are complete (`hand`:
+// counters, zero before and after; and its norms as words that are kNoNorm until they are known), and its rows are copied while others are scored.
+// `parts`, `free_sms`: see stream_beside_tail.
+cudaError_t launch_select_copy_beside(const BatchDesc& bd, const GateParams& gp, const SelectIO& io, const CompactJob& job,
+                                      int32_t* list, int32_t* hand, int parts, int free_sms, int* status, unsigned long long* stamps,
+                                      cudaStream_t stream);
 
 // One warp runs the copying CTAs' bounded wait on `never_set` (a word that holds -1 and stays so) with the
 // given limit and reports MVLA_ERR_TIMEOUT into `status` when it runs out.

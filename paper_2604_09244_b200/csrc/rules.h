@@ -68,4 +68,34 @@ inline bool chain_pays(int64_t moved, int ctas, bool adaptive, int sm_count)
     return moved <= (all_at_once || adaptive ? 20 : 17) * (int64_t(1) << 20);
 }
 
+// Whether the tail of a batch runs beside the streaming kernel that scores it (launch_select_copy_beside): where the jobs fill more than two rounds, so that
+// some samples are scored well before the others; where a job is long enough that the multiprocessors given to the tail and the words that pass between
+// the kernels cost less than the idle memory between them; and where the scoring kernel's two norm warps, which take the feature norms then,
+// keep up with its scores.  Whole steps in us, behind / beside, 32 heads of 128, texts of 16 to 64, unless said otherwise:
+//   768 tokens (196 KB of keys a job): 10 samples 62.0 / 59.0, 16 93.4 / 87.9, 20 116.8 / 111.6, 28 156.8 / 152.8, fixed budgets 71.9 / 70.0, short
+//     texts 92.5 / 87.3; 3000 tokens: 3 samples 68.3 / 62.6, 5 105.1 / 99.7, 7 137.8 / 133.6; 3584: 8 161.5 / 155.8; 1700, short texts: 6 68.5 / 68.5;
+//     16 heads of 256, 24 samples 134.2 / 132.0;
+//   98 KB: e4m3 with 8 key heads 53.7 / 54.9, 32 heads of 64 56.9 / 57.8; 58 KB (228 tokens): 11 samples 31.1 / 38.4, 32 68.0 / 75.9;
+//   16 heads of 128 (4 KB of keys a token), 24 samples 74.0 / 78.3: the norms take longer than the scores.
+struct TailBesideSizes {
+    int64_t tokens;             // visual tokens of the launch
+    int samples, jobs;          // jobs: samples x heads
+    int at_once;                // clusters that run at once
+    int64_t head_bytes, key_bytes, row_bytes;   // of a token: its keys of one head, of all, its hidden row (0: no norms)
+};
+inline bool tail_beside_pays(const TailBesideSizes& c)
+{
+    if (c.samples < 2 || c.jobs <= 2 * c.at_once || c.tokens * c.head_bytes < (int64_t(160) << 10) * c.samples) return false;
+    return c.key_bytes >= 6144 * ((c.row_bytes + kNormPiece - 1) / kNormPiece);
+}
+
+// Clusters of the streaming scoring kernel when the tail of the step runs beside it: no more than its rounds of jobs need (what a last round
+// leaves idle is the tail's), and at least kTailSms multiprocessors for the tail.
+constexpr int kTailSms = 12;
+inline int clusters_beside_tail(int jobs, int at_once, int cluster, int sm_count)
+{
+    const int rounds = (jobs + at_once - 1) / at_once, used = (jobs + rounds - 1) / rounds, most = (sm_count - kTailSms) / cluster;
+    return used < most ? used : (most > 1 ? most : 1);
+}
+
 }  // namespace mvla

@@ -28,6 +28,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "copy_impl.cuh"
 
 #include <math_constants.h>
 
@@ -141,10 +142,14 @@ __device__ __forceinline__ int block_exscan(int x, int* warp_tot, int* total)
 //              is released only after the list.
 //   stable   : the next kernel may become resident as soon as the kernel before this one is complete, and the previous state is
 //              loaded after the wait.
+//   beside   : the scoring kernel is still running; the caller has seen that this sample's scores are complete.  Norms are waited
+//              for one by one, and nothing is waited for or released on behalf of the next kernel.
 struct SelectRole {
     int32_t* list = nullptr;
     bool late_pdl = false;
     bool stable = false;
+    bool beside = false;
+    int* status = nullptr;       // beside: receives MVLA_ERR_TIMEOUT
 };
 struct NoHook {
     __device__ void operator()() const {}
@@ -199,8 +204,34 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
                  "r"(s.off_txt), "r"(s.off_2d), "r"(s.off_3d), "r"(s.n_txt), "r"(s.budget), "r"(s.kmin_2d), "r"(s.kmin_3d), "f"(s.c_new),
                  "r"(gp.has_l1), "f"(gp.tau_2d), "f"(gp.tau_3d), "f"(gp.eps_3d), "l"(io.z_out));
     __syncthreads();                                       // the histogram is clear
-    asm volatile("griddepcontrol.wait;" ::: "memory");      // scores come from the kernel before this one
+    if (!role.beside) asm volatile("griddepcontrol.wait;" ::: "memory");      // scores come from the kernel before this one
     if (role.stable) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    // norms of this thread's tokens
+    auto load_norms = [&]() {
+        const int* const words = reinterpret_cast<const int*>(io.l1) + s.vis_off;
+        bool there = true;
+#pragma unroll
+        for (int e = 0; e < EPT; ++e)
+            if (j0 + 32 * e < j_end) {
+                nrm[e] = role.beside ? __int_as_float(ld_relaxed_gpu(words + j0 + 32 * e)) : io.l1[s.vis_off + j0 + 32 * e];
+                there &= __float_as_uint(nrm[e]) != kNoNorm;
+            }
+        if (!role.beside || there) return;
+        const uint64_t t0 = global_ns();
+#pragma unroll 1
+        for (int j = j0; j < j_end; j += 32)
+            for (uint32_t it = 0; static_cast<uint32_t>(ld_relaxed_gpu(words + j)) == kNoNorm; ++it) {
+                if (it >= kSpinLimit || ((it & 63u) == 63u && global_ns() - t0 > 1000000000ull)) {
+                    *reinterpret_cast<volatile int*>(role.status) = MVLA_ERR_TIMEOUT;
+                    break;
+                }
+                __nanosleep(40);
+            }
+#pragma unroll
+        for (int e = 0; e < EPT; ++e)
+            if (j0 + 32 * e < j_end) nrm[e] = __int_as_float(ld_relaxed_gpu(words + j0 + 32 * e));
+    };
 
     // ---- 1. all loads first
     // (Loops over a thread's tokens have no early exits: the chains of its tokens then run beside one another.)
@@ -213,11 +244,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
         for (int e = 0; e < EPT; ++e)
             if (j0 + 32 * e < j_end) a[e] = io.attn[s.vis_off + j0 + 32 * e];
     }
-    if (gp.has_l1 && !k_fixed) {
-#pragma unroll
-        for (int e = 0; e < EPT; ++e)
-            if (j0 + 32 * e < j_end) nrm[e] = io.l1[s.vis_off + j0 + 32 * e];
-    }
+    if (gp.has_l1 && !k_fixed) load_norms();
     if (!role.late_pdl) load_state();
     if (io.part && !io.acc64) {                            // per-head fp32 partials, summed in head order
 #pragma unroll
@@ -503,7 +530,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
         kept_idx[baset + i] = s.off_txt + i;
     }
     after_list();
-    if (role.late_pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (role.late_pdl && !role.beside) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // ---- 5. what nobody downstream waits for
 #pragma unroll
@@ -517,11 +544,7 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
         }
     }
     if (k_fixed) {                                            // host-decided budgets: the indicators come now
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-            const int j = j0 + 32 * e;
-            nrm[e] = gp.has_l1 && j < j_end ? io.l1[s.vis_off + j] : 0.f;
-        }
+        if (gp.has_l1) load_norms();
         partial_sums(a, nrm);
         __syncthreads();
         if (warp == NW - 1) indicators();

@@ -137,6 +137,179 @@ cudaError_t launch_t(const BD& bd, const TailPlan& tp, const GateParams& gp, con
     return cudaLaunchKernelEx(&cfg, select_copy_kernel<NT, CAP, STABLE, BD>, bd, tp, gp, io, ca, list, status, stamps);
 }
 
+// ------------------------------------------------------------------ beside the scoring kernel
+constexpr int kPieceSegs = 4;         // segments of rows that a warp takes at a time
+constexpr int kLotPieces = 16;        // pieces that a CTA takes at a time
+
+// Work of the row copy, in segments (kSegBytes): the text rows of every sample whose place the host knows, then every sample's other rows.
+struct BesidePlan {
+    int32_t begin[2 * kMaxChunk + 1];
+    int32_t baset[kMaxChunk];         // first output row of a sample's text rows inside the sample; -1: not known yet
+    int32_t n, selectors, parts;
+    int32_t lots;
+};
+
+// The tail of a batch scored by the streaming kernel, beside that kernel: it lives on the multiprocessors that the scoring kernel leaves free
+// and, as that kernel's CTAs end, on all of them.  CTAs take their roles by ticket: the first ones select, sample after sample, as the
+// samples' counters say that their scores are complete; all others copy rows, whose words the selecting CTAs write (select_copy_kernel).
+// Scoring is then bound by the memory for all of its time and the row copy for its own, where in turn a batch left the memory
+// idle from the drain of the one to the first list of the other.  Rows are given out piece by piece from one counter, samples in
+// order, because CTAs join while it runs.  A CTA waits only for the scoring kernel, all of whose CTAs run when this one starts, and for the selecting
+// CTAs, which have the lower tickets.
+template <int NT, int CAP>
+__global__ void __launch_bounds__(NT, 1024 / NT)
+select_copy_beside_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ BesidePlan bp, const GateParams gp, const SelectIO io,
+                          const __grid_constant__ CompactArgs ca, int32_t* __restrict__ list, int32_t* hand, int* status,
+                          unsigned long long* __restrict__ stamps)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int cta = cta_ticket(reinterpret_cast<unsigned int*>(hand + kHandTicket));
+    const uint64_t t0 = global_ns();
+    if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta] = t0;
+    if (cta < bp.selectors) {
+        __shared__ SelectSmem<NT, CAP / NT> sm;
+        for (int b = cta; b < bp.n; b += bp.selectors) {
+            if (tid == 0) {
+                int done = 0;
+                for (uint32_t it = 0; it < kSpinLimit; ++it) {
+                    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(done) : "l"(hand + b) : "memory");
+                    if (done == bp.parts || ((it & 63u) == 63u && global_ns() - t0 > 1000000000ull)) break;
+                    __nanosleep(100);
+                }
+                if (done != bp.parts) *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
+                hand[b] = 0;                                // for the next launch
+            }
+            __syncthreads();                                // (and the sample before is done with the shared memory)
+            SelectRole role;
+            role.late_pdl = true;
+            role.beside = true;
+            role.status = status;
+            if (bp.lots > 0) role.list = list + bd.s[b].out_off * kListStride;
+            select_sample<NT, CAP / NT>(bd.s[b], b, gp, io, sm, role, [&]() {
+                if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
+            });
+            __syncthreads();
+        }
+        // "This kernel is complete" implies that the scoring kernel is.
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        return;
+    }
+    // ---- row copy.  What a warp knows of the span of segments it is in stays in registers (an index into the parameters costs some hundred cycles).
+    const int per_row = ca.seg_begin[3], n = bp.n;
+    unsigned int* const counter = reinterpret_cast<unsigned int*>(hand + kHandLots);
+    // Pieces come in lots from one counter (11000 pieces of six segments straight from it, by 4700 warps, made that counter the limit:
+    // the rows of 16 requests moved at 4.8 instead of 6.8 TB/s).  s_lot: number of the lot << 12 | pieces given out; the warp that
+    // finds it used up puts the next one there, which was asked for one lot ago.
+    __shared__ unsigned int s_lot;
+    __shared__ volatile int s_next;
+    if (tid == 0) {
+        s_lot = atomicAdd(counter, 1u) << 12;
+        s_next = static_cast<int>(atomicAdd(counter, 1u));
+    }
+    __syncthreads();
+    auto take = [&]() {
+        unsigned int piece = 0;
+        if (lane == 0) {
+            uint32_t it = 0;
+            for (;;) {
+                const unsigned int got = atomicAdd(&s_lot, 1u), used = got & 0xFFFu;
+                if (used < kLotPieces) { piece = (got >> 12) * kLotPieces + used; break; }
+                if (used == kLotPieces) {
+                    int lot = s_next;
+                    for (; lot < 0 && it < kSpinLimit; ++it) lot = s_next;      // (the warp that has asked for it waits for nobody)
+                    if (lot < 0) lot = bp.lots;
+                    s_next = -1;
+                    __threadfence_block();
+                    atomicExch(&s_lot, static_cast<unsigned int>(lot) << 12 | 1u);
+                    piece = static_cast<unsigned int>(lot) * kLotPieces;
+                    s_next = lot < bp.lots ? static_cast<int>(atomicAdd(counter, 1u)) : lot;
+                    break;
+                }
+                while ((*reinterpret_cast<volatile unsigned int*>(&s_lot) & 0xFFFu) >= kLotPieces && it < kSpinLimit) ++it;
+                if (it >= kSpinLimit) { piece = static_cast<unsigned int>(bp.lots) * kLotPieces; break; }
+            }
+            if (it >= kSpinLimit) *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
+        }
+        return static_cast<int>(__shfl_sync(0xffffffffu, piece, 0));
+    };
+    int span = -1, begin = 0, end = 0, src0 = 0, dst0 = 0, skip_at = 0, skip = 0, row = -1, from = 0;
+    bool polled = false, released = false;
+    const int32_t* words = nullptr;
+    const int all = bp.begin[2 * n];
+    for (;;) {
+        const int first = take() * kPieceSegs;
+        if (first >= all) break;
+        const int u1 = min(first + kPieceSegs, all);
+        for (int u0 = first; u0 < u1; u0 += 2) {
+            uint4 v[2][4];
+            const uint4* sp[2];
+            uint4* dp[2];
+            int nvec[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int u = u0 + k;
+                nvec[k] = 0;
+                sp[k] = nullptr;
+                dp[k] = nullptr;
+                if (u >= u1) continue;
+                if (u >= end) {                             // the span that holds the segment (spans may be empty)
+                    do ++span; while (u >= bp.begin[span + 1]);
+                    begin = bp.begin[span];
+                    end = bp.begin[span + 1];
+                    row = -1;
+                    polled = span >= n;
+                    const int b = polled ? span - n : span, baset = bp.baset[b];
+                    const SampleDev& s = bd.s[b];
+                    dst0 = s.out_off + (polled ? 0 : baset);
+                    src0 = s.seq_off + (polled ? 0 : s.off_txt);
+                    skip_at = baset >= 0 ? baset : s.n_out;
+                    skip = baset >= 0 ? s.n_txt : 0;
+                    words = list + s.out_off * kListStride;
+                }
+                const int r = (u - begin) / per_row, g = u - begin - r * per_row;
+                int drow = r;
+                if (polled) {
+                    drow = r >= skip_at ? r + skip : r;     // the text rows have a span of their own
+                    if (r != row) {
+                        row = r;
+                        from = poll_word(words + drow * kListStride, t0, 1000000000ull);
+                        if (from < 0) *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
+                    }
+                    if (from < 0) continue;                 // gave up: leave the row alone
+                } else {
+                    from = r;
+                }
+                const int tsel = g >= ca.seg_begin[2] ? 2 : (g >= ca.seg_begin[1] ? 1 : 0);
+                const int seg = g - ca.seg_begin[tsel], rb = ca.row_bytes[tsel];
+                sp[k] = reinterpret_cast<const uint4*>(ca.src[tsel] + static_cast<int64_t>(src0 + from) * rb + static_cast<int64_t>(seg) * kSegBytes);
+                dp[k] = reinterpret_cast<uint4*>(ca.dst[tsel] + static_cast<int64_t>(dst0 + drow) * rb + static_cast<int64_t>(seg) * kSegBytes);
+                nvec[k] = min(kSegBytes, rb - seg * kSegBytes) >> 4;
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (lane + i * 32 < nvec[k]) v[k][i] = ld_row(sp[k] + lane + i * 32);
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (lane + i * 32 < nvec[k]) st_row(dp[k] + lane + i * 32, v[k][i]);
+        }
+        if (!released && span == 2 * n - 1) {               // the last sample's list is there: the scoring kernel is about done
+            released = true;
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        }
+    }
+    __syncthreads();                                        // no warp of this CTA asks for a lot any more
+    if (tid == 0) {
+        if (atomicInc(reinterpret_cast<unsigned int*>(hand + kHandLeft), gridDim.x - bp.selectors - 1) == gridDim.x - bp.selectors - 1) *counter = 0u;
+        if (stamps && cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
+    }
+}
+
 int max_vis_of(const BatchDesc& bd)
 {
     int m = 0;
@@ -144,7 +317,56 @@ int max_vis_of(const BatchDesc& bd)
     return m;
 }
 
+template <int NT, int CAP>
+cudaError_t launch_beside_t(const BatchDesc& bd, const BesidePlan& bp, const GateParams& gp, const SelectIO& io, const CompactArgs& ca, int32_t* list,
+                            int32_t* hand, int ctas, int* status, unsigned long long* stamps, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(ctas));
+    cfg.blockDim = dim3(NT);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1] = {pdl_attribute()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, select_copy_beside_kernel<NT, CAP>, bd, bp, gp, io, ca, list, hand, status, stamps);
+}
+
+// First output row of a sample's text rows inside the sample, where the host knows it (see select_copy_kernel); else -1.
+int text_base(const SampleDev& s)
+{
+    const bool b2 = s.n_2d > 0 && s.off_2d < s.off_txt, b3 = s.n_3d > 0 && s.off_3d < s.off_txt;
+    if (s.k_2d_fixed >= 0) return (b2 ? s.k_2d_fixed : 0) + (b3 ? s.budget - s.k_2d_fixed : 0);
+    return b2 == b3 ? (b2 ? s.budget : 0) : -1;
+}
+
 }  // namespace
+
+cudaError_t launch_select_copy_beside(const BatchDesc& bd, const GateParams& gp, const SelectIO& io, const CompactJob& job, int32_t* list,
+                                      int32_t* hand, int parts, int free_sms, int* status, unsigned long long* stamps, cudaStream_t stream)
+{
+    const CompactArgs ca = compact_args(job);
+    const int nv = max_vis_of(bd), per_sm = nv > 2048 ? 1 : 2, per_row = ca.seg_begin[3];
+    BesidePlan bp;
+    bp.n = bd.n;
+    bp.parts = parts;
+    int at = 0;
+    for (int b = 0; b < bd.n; ++b) {
+        bp.baset[b] = text_base(bd.s[b]);
+        bp.begin[b] = at;
+        if (bp.baset[b] >= 0) at += bd.s[b].n_txt * per_row;
+    }
+    for (int b = 0; b < bd.n; ++b) {
+        bp.begin[bd.n + b] = at;
+        at += (bd.s[b].n_out - (bp.baset[b] >= 0 ? bd.s[b].n_txt : 0)) * per_row;
+    }
+    bp.begin[2 * bd.n] = at;
+    bp.lots = (at + kPieceSegs * kLotPieces - 1) / (kPieceSegs * kLotPieces);
+    bp.selectors = std::min(bd.n, std::max(1, std::min(8, free_sms * per_sm / 4)));
+    const int ctas = at > 0 ? std::max(sm_count_of_current_device() * per_sm, bp.selectors + 1) : bp.selectors;
+    if (nv <= 1024) return launch_beside_t<512, 1024>(bd, bp, gp, io, ca, list, hand, ctas, status, stamps, stream);
+    if (nv <= 2048) return launch_beside_t<512, 2048>(bd, bp, gp, io, ca, list, hand, ctas, status, stamps, stream);
+    return launch_beside_t<1024, kMaxVis>(bd, bp, gp, io, ca, list, hand, ctas, status, stamps, stream);
+}
 
 cudaError_t launch_wait_probe(const int32_t* never_set, uint64_t limit_ns, int* status, cudaStream_t stream)
 {

@@ -54,6 +54,7 @@ struct StreamArgs {
     int32_t* rearm;               // see launch_salience_fast
     unsigned long long* rearm_rec;
     unsigned long long* stamps;
+    int32_t* hand;                // the tail runs beside this kernel: its counters (kDone...), or null
     // feature norms (null: none): bf16 rows of `row_bytes` bytes, their L1 norms, where the pieces in flight lie in dynamic shared memory
     const uint8_t* hidden;
     float* l1;
@@ -370,14 +371,18 @@ __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, in
 // or a CTA of their own.  What bounds it is a piece's fixed cost and the adds of its sums, not the bytes in flight (adaptive steps of
 // 16 requests of 768 tokens: two pieces in flight 99.9 us, three 98.4; pieces of 4 KB 110.8; a run of rows instead of every n_w-th, whose
 // sample has to be looked up each time, 97.8 instead of 98.4; four sums beside one another instead of one chain 94.8; eight loads at once 93.7).
+template <bool HAND>
 __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs& a, StreamSmem& sm, uint32_t buf, int nw, int lane)
 {
     const bool one = elect_one();
     int rows = 0;                                        // of all samples
     for (int b = 0; b < a.n_samples; ++b) rows += bd.s[b].n_2d + bd.s[b].n_3d;
     const int w = static_cast<int>(blockIdx.x) * kNormWarps + nw, n_w = static_cast<int>(gridDim.x) * kNormWarps;
-    const int first = static_cast<int>(static_cast<int64_t>(rows) * w / n_w), last = static_cast<int>(static_cast<int64_t>(rows) * (w + 1) / n_w);
-    const int pieces = (a.row_bytes + static_cast<int>(kNormPiece) - 1) / static_cast<int>(kNormPiece), n = (last - first) * pieces;
+    // a run of rows; every n_w-th where somebody waits for one sample after another
+    const int step = HAND ? n_w : 1;
+    const int first = HAND ? w : static_cast<int>(static_cast<int64_t>(rows) * w / n_w);
+    const int count = HAND ? (rows - w + n_w - 1) / n_w : static_cast<int>(static_cast<int64_t>(rows) * (w + 1) / n_w) - first;
+    const int pieces = (a.row_bytes + static_cast<int>(kNormPiece) - 1) / static_cast<int>(kNormPiece), n = max(count, 0) * pieces;
     // The row next to be fetched: visual index fv of sample fb, whose geometry stays in registers (a run-time index into the
     // kernel's parameters costs some hundred cycles); and the one next to be summed goes to *out.
     int fb = 0, fv = first, n_2d = 0, n_vis = 0, row_2d = 0, row_3d = 0;
@@ -402,7 +407,10 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
         }
         if (++fp == pieces) {
             fp = 0;
-            if (++fv == n_vis && fb < a.n_samples - 1) { fv = 0; ++fb; sample(); }
+            if constexpr (HAND) {
+                fv += step;
+                while (fv >= n_vis && fb < a.n_samples - 1) { fv -= n_vis; ++fb; sample(); }
+            } else if (++fv == n_vis && fb < a.n_samples - 1) { fv = 0; ++fb; sample(); }
         }
     };
     pdl_wait();                                          // the rows may come from the kernel before this one
@@ -438,7 +446,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
 #pragma unroll
             for (int off = 16; off >= 1; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
             if (lane == 0) *out = r;
-            ++out;
+            out += step;
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[e] = 0.f;
         }
@@ -453,7 +461,9 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
 // 106 us when their norms ran beside).  8 requests of 3584 tokens, 64 queries, take 161.7 us with 144 and 162.0 with 168.
 // Where no norms run beside, the registers are worth more to the attention copy: 16 patch-by-patch steps 76.5 us with 168, 78.6
 // with 144; 16 adaptive requests 93.7 and 93.0.
-template <bool ROOM>
+// HAND: the tail of the step runs beside this kernel (launch_select_copy_beside); a variant of its own, because in the others the skipped code
+// cost steps of 20 to 40 us 1 to 2 %.
+template <bool ROOM, bool HAND>
 __global__ void __maxnreg__(ROOM ? 144 : kStreamRegs)
 salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,
                        const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ StreamArgs a)
@@ -491,6 +501,19 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sm.aborted = 0;
     }
+    if constexpr (HAND) {
+        // The tail may start as soon as every CTA of this kernel has let it (below): its hand-over words, and the norms, which are
+        // words of that kind then, are re-armed before.  Their last users finished long ago; the first to write one of them is the
+        // tail, or the norm warp that re-arms it (a CTA may start when others have written norms already).
+        const SampleDev &s0 = bd.s[0], &sn = bd.s[a.n_samples - 1];
+        const int at = static_cast<int>(blockIdx.x * blockDim.x) + tid, all = static_cast<int>(gridDim.x * blockDim.x);
+        for (int i = s0.out_off + at; i < sn.out_off + sn.n_out; i += all) a.rearm[i * kListStride] = -1;
+        if (!ROOM && a.hidden && warp > kSoftWarps + 1) {
+            const int w = static_cast<int>(blockIdx.x) * kNormWarps + warp - kSoftWarps - 2, n_w = static_cast<int>(gridDim.x) * kNormWarps;
+            const int end = sn.vis_off + sn.n_2d + sn.n_3d;
+            for (int i = s0.vis_off + w + lane * n_w; i < end; i += 32 * n_w) a.l1[i] = __uint_as_float(kNoNorm);
+        }
+    }
     // all 512 columns: the launcher's shared-memory footprint keeps every other user of tensor memory off this multiprocessor
     if (warp == kSoftWarps + 1) tmem_alloc(smem_u32(&sm.tmem), kTmemColsPerSm);
     tc_fence_before();
@@ -513,6 +536,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             prefetch_tensormap(&tmap_q);
             prefetch_tensormap(&tmap_k);
         }
+        if constexpr (HAND) __threadfence();          // the CTA's re-armed words (behind the block barrier) before the trigger
         pdl_wait();
         if (a.stamps && one && blockIdx.x < kStampSlots) a.stamps[2 * blockIdx.x] = global_ns();
         pdl_trigger();                        // whatever the kernel before this one wrote is complete
@@ -595,7 +619,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
     } else if (!ROOM && warp > kSoftWarps + 1) {
         // ---------------------------------------------------------------- feature norms
         const int nw = warp - kSoftWarps - 2;
-        if (a.hidden) norm_warp(bd, a, sm, smem_u32(dyn) + a.norm_off + static_cast<uint32_t>(nw * kNormStages) * kNormPiece, nw, lane);
+        if (a.hidden) norm_warp<HAND>(bd, a, sm, smem_u32(dyn) + a.norm_off + static_cast<uint32_t>(nw * kNormStages) * kNormPiece, nw, lane);
     } else {
         // ---------------------------------------------------------------- softmax
         SoftJob j;
@@ -605,7 +629,16 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
         j.cscale = 1.4426950408889634f * rsqrtf(static_cast<float>(a.head_dim));   // log2 domain
         float* const my_w = sm.w[warp];
         bool waited = false;
-        int jn = 0;
+        int jn = 0, scored = -1;                         // sample of the job before
+        // A job's scores are in the accumulators when every softmax warp has passed the next barrier: one thread that has no part
+        // in the exchange tells (its fence takes about as long as that does; behind a barrier of its own at the end of every job
+        // 8 requests of 3584 tokens took 164.4 us instead of 155.4).
+        auto tell = [&]() {
+            if (HAND && scored >= 0 && tid == kSoftThreads - 1) {
+                __threadfence();
+                atomicAdd(a.hand + scored, 1);
+            }
+        };
         for (int job = first_job, b = b_first, h = h_first; job < a.n_jobs; job += job_step, ++jn, advance(b, h)) {
             const SampleDev& s = bd.s[b];
             j.tr = JobTiles(s, crank, lg);
@@ -614,7 +647,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             j.n_txt = n_txt;
             j.hn = static_cast<float>(a.n_heads) * static_cast<float>(n_txt);
             if (!ROOM && a.alpha.ptr) j.alpha = a.alpha.ptr + static_cast<int64_t>(h) * a.alpha.stride_h + static_cast<int64_t>(s.vis_off) * 4;
-            if (a.rearm && h == 0 && crank == 0) {    // the tail kernel's hand-over words; their last users finished long ago
+            if (!HAND && a.rearm && h == 0 && crank == 0) {    // the tail kernel's hand-over words; their last users finished long ago
                 if (!a.rearm_rec) {
                     for (int i = tid; i < s.n_out; i += kSoftThreads) a.rearm[(s.out_off + i) * kListStride] = -1;
                 } else {                              // the patch-by-patch tail: its list words, and three words per patch
@@ -632,6 +665,8 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
                 tmem_wait_st();
             }
             soft_barrier();
+            tell();
+            scored = b;
             // ---- one thread per query: the pairs of the warps, then those of the cluster's CTAs
             if (tid < npad) {
                 float mk[kSoftWarps], mx = -CUDART_INF_F, z = 0.f;
@@ -670,6 +705,10 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
             j.slot0 += j.tr.count;
             if (j.slot0 >= a.slots) { j.slot0 -= a.slots; j.parity0 ^= 1u; }
         }
+        if constexpr (HAND) {
+            soft_barrier();
+            tell();
+        }
     }
     __syncwarp();
     tc_fence_before();
@@ -699,24 +738,41 @@ int max_tiles(const BatchDesc& bd)
     return t;
 }
 
-template <bool ROOM>
-cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUtensorMap* tk, StreamArgs& a, int cluster,
-                            size_t smem, cudaStream_t stream)
+// The smallest cluster whose CTAs hold their share of a job's logits in tensor memory; a larger one while jobs are
+// fewer than multiprocessors and the tiles can still be shared out.  0: none holds them.
+int stream_cluster(int n_jobs, int tiles, int slots, int sms)
 {
-    auto kern = salience_stream_kernel<ROOM>;
+    int cluster = 1;
+    while (cluster < kMaxCluster && ((tiles + cluster - 1) / cluster > slots || (n_jobs * cluster * 2 <= sms && cluster * 2 <= tiles)))
+        cluster *= 2;
+    return (tiles + cluster - 1) / cluster > slots ? 0 : cluster;
+}
+
+// Clusters that run at once (a second wave of a persistent grid would double its time), with the kernel set up.
+template <bool ROOM, bool HAND>
+cudaError_t launch_size(int threads, int cluster, int* n)
+{
+    const void* kern = reinterpret_cast<const void*>(salience_stream_kernel<ROOM, HAND>);
     static KernelSetup ks;
-    cudaError_t e = setup_kernel(ks, reinterpret_cast<const void*>(kern), smem, kTmemColsPerSm);
-    if (e != cudaSuccess) return e;
-    // a second wave of a persistent grid would double its time
+    cudaError_t e = setup_kernel(ks, kern, kStreamSmem, kTmemColsPerSm);
+    if (e == cudaSuccess) e = clusters_at_once(ks, kern, threads, kStreamSmem, cluster, n);
+    return e == cudaSuccess && *n < 1 ? cudaErrorInvalidConfiguration : e;
+}
+
+template <bool ROOM, bool HAND>
+cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUtensorMap* tk, StreamArgs& a, int cluster, cudaStream_t stream)
+{
+    auto kern = salience_stream_kernel<ROOM, HAND>;
     int n = 0;
     const int threads = kStreamThreads + (a.hidden ? 32 * kNormWarps : 0);
-    e = clusters_at_once(ks, reinterpret_cast<const void*>(kern), threads, smem, cluster, &n);
+    const cudaError_t e = launch_size<ROOM, HAND>(threads, cluster, &n);
     if (e != cudaSuccess) return e;
-    if (n < 1) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>((a.hidden ? n : std::min(a.n_jobs, n)) * cluster));      // (norms are shared out over all CTAs)
+    int clusters = a.hidden ? n : std::min(a.n_jobs, n);       // (norms are shared out over all CTAs)
+    if (HAND) clusters = clusters_beside_tail(a.n_jobs, n, cluster, sm_count_of_current_device());
+    cfg.gridDim = dim3(static_cast<unsigned>(clusters * cluster));
     cfg.blockDim = dim3(static_cast<unsigned>(threads));
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = kStreamSmem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -736,10 +792,31 @@ static_assert(kSmemPerSm - static_cast<int>(kStreamSmem + sizeof(StreamSmem)) - 
               "the streaming kernel must be alone with the tensor memory of its multiprocessor");
 static_assert((kStreamThreads + 32 * kNormWarps) * kStreamRegs <= 65536, "the norm warps must fit the register file beside the others");
 
+cudaError_t stream_beside_tail(const BatchDesc& bd, int n_heads, int64_t head_bytes, int64_t key_bytes, int64_t row_bytes, int* free_sms, int* parts)
+{
+    *free_sms = *parts = 0;
+    const int sms = sm_count_of_current_device(), npad = padded_text(bd), jobs = bd.n * n_heads;
+    const int cluster = stream_cluster(jobs, max_tiles(bd), std::min(kMaxSlots, kTmemColsPerSm / npad), sms);
+    int64_t tokens = 0;
+    for (int b = 0; b < bd.n; ++b) tokens += bd.s[b].n_2d + bd.s[b].n_3d;
+    int n = cluster > 1 ? 1 : sms;
+    const auto pays = [&]() { return tail_beside_pays({tokens, bd.n, jobs, n, head_bytes, key_bytes, row_bytes}); };
+    if (cluster == 0 || !pays()) return cudaSuccess;         // (clusters: the runtime is asked only where the rest says yes)
+    if (cluster > 1) {
+        const cudaError_t e = launch_size<false, true>(kStreamThreads + 32 * kNormWarps, cluster, &n);
+        if (e != cudaSuccess) return e;
+        if (!pays()) return cudaSuccess;
+    }
+    *free_sms = sms - clusters_beside_tail(jobs, n, cluster, sms) * cluster;
+    *parts = n_heads * cluster;
+    return cudaSuccess;
+}
+
 cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
                                    AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
-                                   unsigned long long* stamps, bool norms_beside, const void* hidden, int row_bytes, float* l1, cudaStream_t stream)
+                                   unsigned long long* stamps, bool norms_beside, const void* hidden, int row_bytes, float* l1, int32_t* hand,
+                                   cudaStream_t stream)
 {
     const int sms = sm_count_of_current_device();
     const int npad = padded_text(bd), tiles = max_tiles(bd);
@@ -749,13 +826,9 @@ cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_grou
     a.slots = std::min(kMaxSlots, kTmemColsPerSm / npad);
     a.n_jobs = bd.n * n_heads;
     a.acc64 = acc64; a.status = status; a.alpha = alpha; a.rearm = rearm;
-    a.rearm_rec = rearm_rec; a.stamps = stamps;
-    // The smallest cluster whose CTAs hold their share of a job's logits in tensor memory; a larger one while jobs are
-    // fewer than multiprocessors and the tiles can still be shared out.
-    int cluster = 1;
-    while (cluster < kMaxCluster && ((tiles + cluster - 1) / cluster > a.slots || (a.n_jobs * cluster * 2 <= sms && cluster * 2 <= tiles)))
-        cluster *= 2;
-    if ((tiles + cluster - 1) / cluster > a.slots) return cudaErrorInvalidConfiguration;
+    a.rearm_rec = rearm_rec; a.stamps = stamps; a.hand = hand;
+    const int cluster = stream_cluster(a.n_jobs, tiles, a.slots, sms);
+    if (cluster == 0) return cudaErrorInvalidConfiguration;
     const size_t q_bytes = 2 * static_cast<size_t>((head_dim * esize + 127) / 128) * npad * 128;
     // shared memory: the ring of key boxes, two buffers of queries, the norm warps' pieces of rows
     const size_t norm_bytes = hidden ? static_cast<size_t>(kNormWarps * kNormStages) * kNormPiece : 0;
@@ -764,8 +837,9 @@ cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_grou
     a.hidden = static_cast<const uint8_t*>(hidden);
     a.l1 = l1; a.row_bytes = row_bytes; a.n_samples = bd.n;
     a.norm_off = static_cast<uint32_t>(a.stages * kStageBytes + q_bytes);
-    if (norms_beside && !alpha.ptr) return launch_stream<true>(bd, tmap_q, tmap_k, a, cluster, kStreamSmem, stream);
-    return launch_stream<false>(bd, tmap_q, tmap_k, a, cluster, kStreamSmem, stream);
+    if (norms_beside && !alpha.ptr) return launch_stream<true, false>(bd, tmap_q, tmap_k, a, cluster, stream);
+    if (hand) return launch_stream<false, true>(bd, tmap_q, tmap_k, a, cluster, stream);
+    return launch_stream<false, false>(bd, tmap_q, tmap_k, a, cluster, stream);
 }
 
 }  // namespace mvla

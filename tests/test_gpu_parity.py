@@ -1149,6 +1149,44 @@ def test_scoring_kernel_goes_by_what_fits_on_the_device(batch, d, n_txt, n_2d, n
     ctx.close()
 
 
+@pytest.mark.parametrize("batch,H,n_txt,n_2d,n_3d,kw,beside", [
+    (13, 24, (33, 16, 64), (256, 300, 1), (400, 384, 700), {}, True),                       # one tile of one token; three rounds of jobs
+    (13, 24, (33, 16, 64), (256, 300, 1), (400, 384, 700), {"text": "middle"}, True),       # rows of the text known with the list only
+    (13, 24, (5, 17), (300, 0), (400, 700), {"mode": W.MODE_FIXED, "text_first": True}, True),   # no norms; a modality without tokens
+    (13, 24, (33, 64), (256, 300), (400, 384), {"cold_start": 1}, True),                     # all kept first: norms after the list
+    (13, 24, (33, 64), (200, 160), (380, 440), {}, False),                                   # keys of a job below the line
+    (12, 24, (33, 64), (256, 300), (400, 384), {}, False),                                   # two rounds
+    (36, 24, (3, 20), (256, 300), (400, 384), {}, False),                                    # a launch of 32 samples beside, one of 4 behind
+    (7, 24, (64, 50), (600, 300), (500, 1024), {}, True),                                    # clusters of two, up to 1324 tokens
+    (3, 24, (64, 50), (1500, 900), (700, 1300), {}, True)])                                  # clusters of four, 2200 tokens
+def test_tail_beside_the_streaming_scoring_kernel(batch, H, n_txt, n_2d, n_3d, kw, beside):
+    """Batches whose samples are selected and copied while others are scored, told by the multiprocessors that the scoring kernel leaves
+    free; two action steps, the same bits when they are run again."""
+    kw = dict(kw)
+    text = kw.pop("text", "")
+    wl = W.small_workload(76, batch=batch, H=H, D=128, d=128, n_txt=n_txt, n_2d=n_2d, n_3d=n_3d, keep=(0.3, 0.5), steps=2, **kw)
+    if text == "middle":
+        wl.samples[:] = [W.Sample(**{**vars(s), "off_2d": 0, "off_txt": s.n_2d, "off_3d": s.n_2d + s.n_txt}) for s in wl.samples]
+    ctx, states = mvla.context_for(wl), [oracle.State(s.n_vis) for s in wl.samples]
+    for step in range(2):
+        stamps = torch.zeros(2, ctx.STAMP_SLOTS, 2, dtype=torch.int64, device="cuda")
+        ctx.set_kernel_stamps(stamps)
+        run_and_check_step(ctx, wl, step, states)
+        if batch <= 32:
+            sms = torch.cuda.get_device_properties(0).multi_processor_count
+            assert (int((stamps[0, :, 1] != 0).sum()) <= sms - 12 and int((stamps[1, :, 0] != 0).sum()) >= sms) == beside
+    ctx.set_kernel_stamps(None)
+    dev, runs = device_tensors(wl), []
+    for _ in range(8):
+        out = ctx.alloc_outputs(wl.samples, extras=True)
+        ctx.prune_step(0, wl.samples, wl.mode, dev["q"], dev["k"], dev["v"], dev["hidden"], flags=mvla.FLAG_RESET_STATE, out=out)
+        n = int(out.out_offsets[-1])
+        runs.append([out.budgets, out.ahat] + [t[:n] for t in (out.kept_idx, out.out_hidden, out.out_k, out.out_v)])
+    for r in runs[1:]:
+        assert all(torch.equal(x.contiguous().view(torch.uint8), y.contiguous().view(torch.uint8)) for x, y in zip(runs[0], r))
+    ctx.close()
+
+
 @pytest.mark.parametrize("gain", [30.0, 300.0])
 def test_streaming_scoring_kernel_moves_its_references_when_exponents_would_overflow(gain):
     """Keys whose logits grow from tile to tile by far more than an fp32 exponent holds."""
