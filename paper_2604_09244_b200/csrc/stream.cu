@@ -384,7 +384,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
     const int count = HAND ? (rows - w + n_w - 1) / n_w : static_cast<int>(static_cast<int64_t>(rows) * (w + 1) / n_w) - first;
     const int pieces = (a.row_bytes + static_cast<int>(kNormPiece) - 1) / static_cast<int>(kNormPiece), n = max(count, 0) * pieces;
     // The row next to be fetched: visual index fv of sample fb, whose geometry stays in registers (a run-time index into the
-    // kernel's parameters costs some hundred cycles); and the one next to be summed goes to *out.
+    // kernel's parameters costs some hundred cycles).
     int fb = 0, fv = first, n_2d = 0, n_vis = 0, row_2d = 0, row_3d = 0;
     auto sample = [&]() {
         const SampleDev& s = bd.s[fb];
@@ -395,7 +395,8 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
     };
     sample();
     while (fv >= n_vis && fb < a.n_samples - 1) { fv -= n_vis; ++fb; sample(); }
-    float* out = a.l1 + bd.s[0].vis_off + first;         // (visual arrays are packed over the samples of the launch)
+    int sb = fb, sv = fv, s_vis = n_vis;                 // the row next to be summed (HAND: the samples lie one behind another)
+    float* out = HAND ? a.l1 + bd.s[0].vis_off + first : a.l1 + bd.s[sb].vis_off + sv;
     int fp = 0;
     auto fetch = [&](int st) {
         const int row = (fv < n_2d ? row_2d : row_3d) + fv;
@@ -447,6 +448,12 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
             for (int off = 16; off >= 1; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
             if (lane == 0) *out = r;
             out += step;
+            if (!HAND && ++sv == s_vis && sb < a.n_samples - 1) {
+                ++sb;
+                sv = 0;
+                s_vis = bd.s[sb].n_2d + bd.s[sb].n_3d;
+                out = a.l1 + bd.s[sb].vis_off;
+            }
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[e] = 0.f;
         }
@@ -748,6 +755,26 @@ int stream_cluster(int n_jobs, int tiles, int slots, int sms)
     return (tiles + cluster - 1) / cluster > slots ? 0 : cluster;
 }
 
+// The samples whose jobs take longest come first: some CTAs have a job more than the others, their last one, which should be a short one.
+// A job's softmax takes as long as its tiles and padded text queries say, its keys as long as its tiles (as much as 32 queries more).
+// 16 patch-by-patch requests of 512 tokens with texts of 16 to 64: 76.9 -> 74.7 us; texts of one length: the order given.
+BatchDesc costly_first(const BatchDesc& given)
+{
+    BatchDesc bd = given;
+    auto cost = [](const SampleDev& s) {
+        const int tiles = (s.n_2d + kKeyTile - 1) / kKeyTile + (s.n_3d + kKeyTile - 1) / kKeyTile;
+        return tiles * (((s.n_txt + 15) & ~15) + 32);
+    };
+    for (int i = 1; i < bd.n; ++i) {                     // (insertion: at most kMaxChunk, often in order)
+        if (cost(bd.s[i - 1]) >= cost(bd.s[i])) continue;
+        const SampleDev s = bd.s[i];
+        int at = i;
+        for (; at > 0 && cost(bd.s[at - 1]) < cost(s); --at) bd.s[at] = bd.s[at - 1];
+        bd.s[at] = s;
+    }
+    return bd;
+}
+
 // Clusters that run at once (a second wave of a persistent grid would double its time), with the kernel set up.
 template <bool ROOM, bool HAND>
 cudaError_t launch_size(int threads, int cluster, int* n)
@@ -812,13 +839,14 @@ cudaError_t stream_beside_tail(const BatchDesc& bd, int n_heads, int64_t head_by
     return cudaSuccess;
 }
 
-cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
+cudaError_t launch_salience_stream(const BatchDesc& given, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
                                    AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
                                    unsigned long long* stamps, bool norms_beside, const void* hidden, int row_bytes, float* l1, int32_t* hand,
                                    cudaStream_t stream)
 {
     const int sms = sm_count_of_current_device();
+    const BatchDesc bd = hand ? given : costly_first(given);      // (a tail beside takes the samples as they are)
     const int npad = padded_text(bd), tiles = max_tiles(bd);
     StreamArgs a;
     a.n_heads = n_heads; a.kv_group = kv_group; a.head_dim = head_dim; a.esize = esize;
