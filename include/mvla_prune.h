@@ -279,7 +279,8 @@ int32_t mvla_prune_step(mvla_ctx *ctx, int32_t prune_point, int32_t batch,
  * (no MVLA_FLAG_INPUTS_STABLE) records it on the call's stream between its scoring kernel(s) and its
  * selection + row-copy kernel.  With events of the caller's own around the call this gives the duration of
  * each of the step's kernels as the step runs them.  The record sits between two kernels that otherwise
- * overlap at their edges, so the step is slightly slower while it is on; leave it off otherwise.  For
+ * overlap at their edges (large batches: for most of their time; while the event is set, the second follows the
+ * first there too), so the step is slower while it is on; leave it off otherwise.  For
  * batches of more than 32 samples the event is recorded once per launch of 32.  The library never destroys it.
  */
 int32_t mvla_set_stage_event(mvla_ctx *ctx, void *event);

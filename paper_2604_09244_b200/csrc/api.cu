@@ -1296,11 +1296,12 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         // the fused selection + copy kernel (below) wants its list words re-armed by the scoring kernel
         const bool tail = !forked;
         BesideTail beside = {ctx->hand + (par * static_cast<size_t>((ctx->cfg.max_batch + kMaxChunk - 1) / kMaxChunk) + first / kMaxChunk) * kHandStride, 0, 0};
+        const bool may_beside = tail && !chained && !ctx->stage_event;     // (an event between the two kernels is to lie between them)
         ph.mark("mvla: scoring");
         rc = run_salience_chunk(ctx, bd, in->q, in->k, in->rows, adaptive ? in->hidden : nullptr, l1_ws, acc64,
                                 &used_acc64, forked ? ctx->aux[par] : st, AlphaOut{nullptr, 0, 0},
                                 tail ? ctx->tail_list + par * ctx->rows_all : nullptr, tail, tail && !chained ? ctx->stamps : nullptr,
-                                cache_on, nullptr, nullptr, nullptr, early, tail && !chained ? &beside : nullptr);
+                                cache_on, nullptr, nullptr, nullptr, early, may_beside ? &beside : nullptr);
         if (rc != MVLA_OK) return rc;
         if (ctx->stage_event && !forked && !chained) {
             // under stream capture the record must become an event-record node of the graph (an "external"

@@ -1187,6 +1187,24 @@ def test_tail_beside_the_streaming_scoring_kernel(batch, H, n_txt, n_2d, n_3d, k
     ctx.close()
 
 
+def test_an_event_between_the_kernels_keeps_the_tail_behind_the_scoring_kernel():
+    """With a stage event set, a batch whose tail would run beside its scoring kernel is scored on all multiprocessors, and no copying
+    CTA starts before the last scoring CTA has ended."""
+    wl = W.small_workload(77, batch=13, H=24, D=128, d=128, n_txt=(33, 16, 64), n_2d=(256, 300), n_3d=(400, 384), keep=(0.3, 0.5), steps=2)
+    ctx, states = mvla.context_for(wl), [oracle.State(s.n_vis) for s in wl.samples]
+    event = torch.cuda.Event(enable_timing=True)
+    event.record()
+    ctx.set_stage_event(event)
+    for step in range(2):
+        stamps = torch.zeros(2, ctx.STAMP_SLOTS, 2, dtype=torch.int64, device="cuda")
+        ctx.set_kernel_stamps(stamps)
+        run_and_check_step(ctx, wl, step, states)
+        scored, copied = stamps[0, :, 1], stamps[1, len(wl.samples):, 0]
+        assert int((scored != 0).sum()) == torch.cuda.get_device_properties(0).multi_processor_count
+        assert int(copied[copied != 0].min()) >= int(scored.max())
+    ctx.close()
+
+
 @pytest.mark.parametrize("gain", [30.0, 300.0])
 def test_streaming_scoring_kernel_moves_its_references_when_exponents_would_overflow(gain):
     """Keys whose logits grow from tile to tile by far more than an fp32 exponent holds."""
