@@ -18,6 +18,7 @@
 #include "common.cuh"
 #include "device_utils.cuh"
 #include "copy_impl.cuh"
+#include "lots.h"
 #include "select_impl.cuh"
 
 #include <algorithm>
@@ -208,28 +209,22 @@ select_copy_beside_kernel(const __grid_constant__ BatchDesc bd, const __grid_con
         s_next = static_cast<int>(atomicAdd(counter, 1u));
     }
     __syncthreads();
+    struct Cell {
+        unsigned int *word, *counter;
+        volatile int* ahead;
+        __device__ __forceinline__ uint32_t add() { return atomicAdd(word, 1u); }
+        __device__ __forceinline__ void swap(uint32_t x) { __threadfence_block(); atomicExch(word, x); }
+        __device__ __forceinline__ uint32_t peek() { return *reinterpret_cast<volatile unsigned int*>(word); }
+        __device__ __forceinline__ int32_t next() { return *ahead; }
+        __device__ __forceinline__ void put(int32_t x) { *ahead = x; }
+        __device__ __forceinline__ int32_t ask() { return static_cast<int32_t>(atomicAdd(counter, 1u)); }
+    } cell = {&s_lot, counter, &s_next};
     auto take = [&]() {
-        unsigned int piece = 0;
+        uint32_t piece = 0;
         if (lane == 0) {
-            uint32_t it = 0;
-            for (;;) {
-                const unsigned int got = atomicAdd(&s_lot, 1u), used = got & 0xFFFu;
-                if (used < kLotPieces) { piece = (got >> 12) * kLotPieces + used; break; }
-                if (used == kLotPieces) {
-                    int lot = s_next;
-                    for (; lot < 0 && it < kSpinLimit; ++it) lot = s_next;      // (the warp that has asked for it waits for nobody)
-                    if (lot < 0) lot = bp.lots;
-                    s_next = -1;
-                    __threadfence_block();
-                    atomicExch(&s_lot, static_cast<unsigned int>(lot) << 12 | 1u);
-                    piece = static_cast<unsigned int>(lot) * kLotPieces;
-                    s_next = lot < bp.lots ? static_cast<int>(atomicAdd(counter, 1u)) : lot;
-                    break;
-                }
-                while ((*reinterpret_cast<volatile unsigned int*>(&s_lot) & 0xFFFu) >= kLotPieces && it < kSpinLimit) ++it;
-                if (it >= kSpinLimit) { piece = static_cast<unsigned int>(bp.lots) * kLotPieces; break; }
-            }
-            if (it >= kSpinLimit) *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
+            bool gave_up = false;
+            piece = take_piece(cell, kLotPieces, static_cast<uint32_t>(bp.lots), kSpinLimit, &gave_up);
+            if (gave_up) *reinterpret_cast<volatile int*>(status) = MVLA_ERR_TIMEOUT;
         }
         return static_cast<int>(__shfl_sync(0xffffffffu, piece, 0));
     };
