@@ -511,15 +511,19 @@ struct ForkPlan {
     unsigned long long cap_id = 0;       // stream capture the events of this step belong to (0: none)
 };
 
+bool overlap(const mvla_ctx::Range* a, int n, const mvla_ctx::Range* b, int m)
+{
+    for (int i = 0; i < n; ++i)
+        for (int j = 0; j < m; ++j)
+            if (a[i].lo && a[i].lo < b[j].hi && b[j].lo < a[i].hi) return true;
+    return false;
+}
+
 // A buffer that a step in flight beside the others (those remembered) writes, among `r`.
 bool clashes(const mvla_ctx* ctx, unsigned par, const mvla_ctx::Range* r, int n)
 {
-    for (unsigned s = 0; s < kSets; ++s) {
-        if (s == par) continue;
-        for (int i = 0; i < n; ++i)
-            for (int j = 0; j < ctx->n_hist[s]; ++j)
-                if (r[i].lo && r[i].lo < ctx->hist[s][j].hi && ctx->hist[s][j].lo < r[i].hi) return true;
-    }
+    for (unsigned s = 0; s < kSets; ++s)
+        if (s != par && overlap(r, n, ctx->hist[s], ctx->n_hist[s])) return true;
     return false;
 }
 
@@ -1257,18 +1261,18 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
     const size_t nvis_b = static_cast<size_t>(plan.total_vis), nout_b = static_cast<size_t>(plan.total_out);
     const size_t hb = static_cast<size_t>(ctx->cfg.d_model) * ctx->elem, kb = static_cast<size_t>(kv_bytes);
     const size_t qb = static_cast<size_t>(ctx->cfg.n_heads) * ctx->cfg.head_dim * ctx->qk_elem;
+    // buffers that selection and scoring touch: selection outputs (the first 7), and the inputs of scoring; and what the row copy writes
+    const size_t in_rows = static_cast<size_t>(in->rows);
+    const mvla_ctx::Range side[10] = {
+        range_of(out->kept_idx, nout_b * 4), range_of(out->out_offsets, (batch + 1) * 4u),
+        range_of(out->budgets, batch * 8u), range_of(out->attn, nvis_b * 4), range_of(out->ahat, nvis_b * 4),
+        range_of(out->z, nvis_b * 4), range_of(out->diag, batch * sizeof(mvla_diag)),
+        range_of(in->q, in_rows * qb), range_of(in->k, in_rows * kb),
+        range_of(adaptive ? in->hidden : nullptr, in_rows * hb)};
+    const mvla_ctx::Range copied[3] = {range_of(out->out_hidden, nout_b * hb), range_of(out->out_k, nout_b * kb),
+                                       range_of(out->out_v, nout_b * kb)};
     if ((flags & MVLA_FLAG_INPUTS_STABLE) && batch <= kMaxChunk && ctx->use_umma) {
         forked = true;
-        // buffers the side-stream work touches: selection outputs, and the inputs of scoring
-        const size_t in_rows = static_cast<size_t>(in->rows);
-        const mvla_ctx::Range side[10] = {
-            range_of(out->kept_idx, nout_b * 4), range_of(out->out_offsets, (batch + 1) * 4u),
-            range_of(out->budgets, batch * 8u), range_of(out->attn, nvis_b * 4), range_of(out->ahat, nvis_b * 4),
-            range_of(out->z, nvis_b * 4), range_of(out->diag, batch * sizeof(mvla_diag)),
-            range_of(in->q, in_rows * qb), range_of(in->k, in_rows * kb),
-            range_of(adaptive ? in->hidden : nullptr, in_rows * hb)};
-        const mvla_ctx::Range copied[3] = {range_of(out->out_hidden, nout_b * hb), range_of(out->out_k, nout_b * kb),
-                                           range_of(out->out_v, nout_b * kb)};
         cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &cst) != cudaSuccess) return fail_cuda(ctx, cudaGetLastError());
         const SampleDev& one = plan.s[0];
@@ -1296,7 +1300,8 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         // the fused selection + copy kernel (below) wants its list words re-armed by the scoring kernel
         const bool tail = !forked;
         BesideTail beside = {ctx->hand + (par * static_cast<size_t>((ctx->cfg.max_batch + kMaxChunk - 1) / kMaxChunk) + first / kMaxChunk) * kHandStride, 0, 0};
-        const bool may_beside = tail && !chained && !ctx->stage_event;     // (an event between the two kernels is to lie between them)
+        // (an event between the two kernels is to lie between them; and what scoring still reads may not be written yet)
+        const bool may_beside = tail && !chained && batch > 1 && !ctx->stage_event && !overlap(side, 7, side + 7, 3) && !overlap(copied, 3, side + 7, 3);
         ph.mark("mvla: scoring");
         rc = run_salience_chunk(ctx, bd, in->q, in->k, in->rows, adaptive ? in->hidden : nullptr, l1_ws, acc64,
                                 &used_acc64, forked ? ctx->aux[par] : st, AlphaOut{nullptr, 0, 0},

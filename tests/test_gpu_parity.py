@@ -1205,6 +1205,31 @@ def test_an_event_between_the_kernels_keeps_the_tail_behind_the_scoring_kernel()
     ctx.close()
 
 
+def test_outputs_in_the_memory_of_the_queries_are_written_when_all_samples_are_scored():
+    """Positions and smoothed scores that a caller has written over its queries: the same as in buffers of their own, from a tail that starts
+    behind the scoring kernel."""
+    wl = W.small_workload(78, batch=13, H=24, D=128, d=128, n_txt=(33, 16, 64), n_2d=(256, 300), n_3d=(400, 384), keep=(0.3, 0.5), cold_start=0)
+    ctx, dev = mvla.context_for(wl), device_tensors(wl)
+    call = lambda out: ctx.prune_step(0, wl.samples, wl.mode, dev["q"], dev["k"], dev["v"], dev["hidden"], flags=mvla.FLAG_RESET_STATE, out=out)
+    ref = call(ctx.alloc_outputs(wl.samples, extras=True))
+    torch.cuda.synchronize()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for name in ("kept_idx", "ahat"):
+        out = ctx.alloc_outputs(wl.samples, extras=True)
+        keep = dev["q"].clone()
+        own = getattr(out, name)
+        setattr(out, name, dev["q"].view(-1)[-2 * own.numel():].view(own.dtype))     # the queries of the last samples
+        stamps = torch.zeros(2, ctx.STAMP_SLOTS, 2, dtype=torch.int64, device="cuda")
+        ctx.set_kernel_stamps(stamps)
+        call(out)
+        torch.cuda.synchronize()
+        n = int(ref.out_offsets[-1])
+        assert int((stamps[0, :, 1] != 0).sum()) == sms
+        assert torch.equal(out.kept_idx[:n], ref.kept_idx[:n]) and torch.equal(out.ahat, ref.ahat) and torch.equal(out.out_v[:n], ref.out_v[:n])
+        dev["q"].copy_(keep)
+    ctx.close()
+
+
 @pytest.mark.parametrize("gain", [30.0, 300.0])
 def test_streaming_scoring_kernel_moves_its_references_when_exponents_would_overflow(gain):
     """Keys whose logits grow from tile to tile by far more than an fp32 exponent holds."""
