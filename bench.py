@@ -597,7 +597,9 @@ def run_ours(args, rank, local, world):
                        "stamps the kernels take themselves (mvla_set_kernel_stamps): from the moment the kernel's first CTA "
                        "is free to start (the kernel before it complete) to the end of its last CTA.  CUDA events cannot "
                        "bracket a kernel inside the step: a record between the two programmatically chained kernels removes "
-                       "their overlap and costs several microseconds in a graph.  The dominant kernel is the longer one"}
+                       "their overlap and costs several microseconds in a graph.  The dominant kernel is the longer one.  (Where "
+                       "the two spans add up to more than first_load_to_last_store the batch is large enough for the tail to run "
+                       "beside the scoring kernel: its span then starts while that one runs)"}
     else:
         # the patch-by-patch step: its two kernels take no stamps; the figure is the whole step's
         achieved = ab["total"] / (ms_per_step * 1e-3) / 1e9

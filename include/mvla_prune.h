@@ -305,6 +305,10 @@ int32_t mvla_logit_cache_stats(mvla_ctx *ctx, int64_t *tiles_computed, int64_t *
  * first, report the time the kept list was written as both).  Entries of CTAs that do not exist stay as they
  * were.  The pointer is read when the step is enqueued (or captured), so every captured step can have a buffer
  * of its own.  For batches of more than 32 samples the launches of 32 share the buffer.
+ * Large batches run the two kernels beside one another: the scoring kernel then leaves some multiprocessors to the other
+ * one, whose CTAs are numbered in the order in which they start, whose copying CTAs have the time they started as
+ * their start (they copy what is selected while other samples are scored) and whose first CTAs, eight at most, select one
+ * sample after another and report the time of their last list.  The spans of the two kernels overlap: they do not add up.
  */
 int32_t mvla_set_kernel_stamps(mvla_ctx *ctx, uint64_t *device_buffer);
 

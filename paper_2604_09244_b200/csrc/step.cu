@@ -166,7 +166,6 @@ select_copy_beside_kernel(const __grid_constant__ BatchDesc bd, const __grid_con
     const int tid = threadIdx.x, lane = tid & 31;
     const int cta = cta_ticket(reinterpret_cast<unsigned int*>(hand + kHandTicket));
     const uint64_t t0 = global_ns();
-    if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta] = t0;
     if (cta < bp.selectors) {
         __shared__ SelectSmem<NT, CAP / NT> sm;
         for (int b = cta; b < bp.n; b += bp.selectors) {
@@ -191,11 +190,13 @@ select_copy_beside_kernel(const __grid_constant__ BatchDesc bd, const __grid_con
             });
             __syncthreads();
         }
+        if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta] = stamps[2 * cta + 1];   // of its last list, as in select_copy_kernel
         // "This kernel is complete" implies that the scoring kernel is.
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         return;
     }
+    if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta] = t0;
     // ---- row copy.  What a warp knows of the span of segments it is in stays in registers (an index into the parameters costs some hundred cycles).
     const int per_row = ca.seg_begin[3], n = bp.n;
     unsigned int* const counter = reinterpret_cast<unsigned int*>(hand + kHandLots);

@@ -1205,6 +1205,21 @@ def test_an_event_between_the_kernels_keeps_the_tail_behind_the_scoring_kernel()
     ctx.close()
 
 
+def test_stamps_of_a_tail_beside_the_scoring_kernel():
+    """Selecting CTAs report the time of their last list as start and end; copying CTAs start before the scoring kernel has ended."""
+    wl = W.small_workload(79, batch=13, H=24, D=128, d=128, n_txt=(33, 16, 64), n_2d=(256, 300), n_3d=(400, 384), keep=(0.3, 0.5), cold_start=0)
+    ctx, stamps = mvla.context_for(wl), torch.zeros(2, mvla.PruneContext.STAMP_SLOTS, 2, dtype=torch.int64, device="cuda")
+    ctx.set_kernel_stamps(stamps)
+    run_and_check_step(ctx, wl, 0, [oracle.State(s.n_vis) for s in wl.samples])
+    scored, tail = stamps[0].cpu(), stamps[1].cpu()
+    tail = tail[tail[:, 1] != 0]
+    selecting = tail[:, 0] == tail[:, 1]
+    n = int(selecting.sum())
+    assert 1 <= n <= 8 and selecting[:n].all() and (tail[n:, 0] < tail[n:, 1]).all() and (tail[:, 0] > 0).all()
+    assert tail[n:, 0].min() < scored[:, 1].max() < tail[:n, 1].max()
+    ctx.close()
+
+
 def test_outputs_in_the_memory_of_the_queries_are_written_when_all_samples_are_scored():
     """Positions and smoothed scores that a caller has written over its queries: the same as in buffers of their own, from a tail that starts
     behind the scoring kernel."""
