@@ -149,7 +149,8 @@ struct SelectRole {
     bool late_pdl = false;
     bool stable = false;
     bool beside = false;
-    int* status = nullptr;       // beside: receives MVLA_ERR_TIMEOUT
+    int* status = nullptr;       // beside: receives MVLA_ERR_TIMEOUT ...
+    uint64_t t0 = 0;             // ... a second after this time (the CTA's start), whichever of its waits that falls in
 };
 struct NoHook {
     __device__ void operator()() const {}
@@ -218,12 +219,13 @@ __device__ __forceinline__ void select_sample(const SampleDev& s, int b_local, c
                 there &= __float_as_uint(nrm[e]) != kNoNorm;
             }
         if (!role.beside || there) return;
-        const uint64_t t0 = global_ns();
+        bool late = false;
 #pragma unroll 1
-        for (int j = j0; j < j_end; j += 32)
+        for (int j = j0; j < j_end && !late; j += 32)
             for (uint32_t it = 0; static_cast<uint32_t>(ld_relaxed_gpu(words + j)) == kNoNorm; ++it) {
-                if (it >= kSpinLimit || ((it & 63u) == 63u && global_ns() - t0 > 1000000000ull)) {
+                if (it >= kSpinLimit || ((it & 63u) == 63u && global_ns() - role.t0 > 1000000000ull)) {
                     *reinterpret_cast<volatile int*>(role.status) = MVLA_ERR_TIMEOUT;
+                    late = true;
                     break;
                 }
                 __nanosleep(40);

@@ -184,6 +184,7 @@ select_copy_beside_kernel(const __grid_constant__ BatchDesc bd, const __grid_con
             role.late_pdl = true;
             role.beside = true;
             role.status = status;
+            role.t0 = t0;
             if (bp.lots > 0) role.list = list + bd.s[b].out_off * kListStride;
             select_sample<NT, CAP / NT>(bd.s[b], b, gp, io, sm, role, [&]() {
                 if (stamps && tid == 0 && cta < kStampSlots) stamps[2 * cta + 1] = global_ns();
