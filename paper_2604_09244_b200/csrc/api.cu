@@ -2,6 +2,7 @@
 // tensor-map construction, launch sequencing.  No stream synchronisation anywhere.
 #include "common.cuh"
 #include "rules.h"
+#include "sets.h"
 
 #include <cudaTypedefs.h>
 
@@ -19,7 +20,6 @@ using namespace mvla;
 namespace {
 constexpr int kMaxBatch = 64;       // samples per call (mvla_prune_create refuses more)
 constexpr int kMapSlots = 16;       // tensor maps a context remembers
-constexpr int kSets = 6;            // scratch sets = prune steps that may be in flight at once
 // Tracing and logging, both on the host and off the device's path: every public call is an NVTX range (a profiler
 // shows the call and, inside mvla_prune_step, its phases around the kernels they enqueue; without a profiler
 // attached a range costs a few nanoseconds), and with MVLA_LOG=1 in the environment every call prints one line
@@ -92,7 +92,7 @@ struct mvla_ctx {
     int patch_sets;              // kSets when the attention copies fit a modest budget, else 1 (then no overlap)
     int32_t* nout_ws;            // [max_batch] kept rows, [max_batch] ready flags, [1] finished-CTA counter
     int max_patch;
-    unsigned step_parity;        // index of the scratch set of the current step
+    SetRing sets;
     // Scoring and selection of a step whose inputs are promised stable run on the side stream of the
     // step's scratch set, beside the selection and row copy of the steps before; the row copy stays
     // on the caller's stream and waits for ev_sel of the step.
@@ -379,6 +379,20 @@ struct BesideTail {
     int32_t* hand;
     int parts, free_sms;         // see stream_beside_tail; free_sms 0: behind it, as ever
 };
+
+// The scratch set of a call on `st` (SetRing).  Where it has to wait for all earlier work, a memset of the word that no launch ever writes, to what it
+// holds, keeps the next kernel from starting beside the one in front of it.
+int32_t take_set(mvla_ctx* ctx, cudaStream_t st, unsigned* set)
+{
+    cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(st, &cst, &id) != cudaSuccess) return fail_cuda(ctx, cudaGetLastError());
+    const SetRing::Turn turn = ctx->sets.take(cst == cudaStreamCaptureStatusActive ? id : 0);
+    *set = turn.set;
+    if (turn.wait && cudaMemsetAsync(ctx->tail_list + kSets * ctx->rows_all, 0xFF, sizeof(int32_t), st) != cudaSuccess)
+        return fail_cuda(ctx, cudaGetLastError());
+    return MVLA_OK;
+}
 
 // Salience of one chunk (+ L1 norms into `l1` when asked; + the scores as fp32 into `attn_out` when asked).  The per-head
 // contributions are added into the fixed-point accumulators `acc64` (*used_acc64 = true) where a kernel that does so covers the
@@ -717,8 +731,9 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
 
     // Scratch set of this step; with stable inputs its scoring, indicators and selection run on that set's
     // side stream beside the steps before (plan_fork), the row copy stays on the caller's stream.
-    ctx->step_parity = (ctx->step_parity + 1u) % kSets;
-    const unsigned par = ctx->step_parity;
+    unsigned par = 0;
+    rc = take_set(ctx, st, &par);
+    if (rc != MVLA_OK) return rc;
     bool forked = false;
     ForkPlan fp;
     if ((flags & MVLA_FLAG_INPUTS_STABLE) && ctx->patch_sets == kSets && batch <= kMaxChunk && ctx->use_umma) {
@@ -775,6 +790,7 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
                                                 l1_taken ? l1 : nullptr, x, attn, rec, pp, io, job, list, ctx->sm_count, ctx->tail_ticket + par, st);
         if (e != cudaSuccess) return fail_cuda(ctx, e);
         commit_steps(ctx, prune_point, plan, samples);
+        ctx->sets.done();
         if (total_kept_out) *total_kept_out = static_cast<int32_t>(cap);
         return MVLA_OK;
     }
@@ -801,6 +817,7 @@ int32_t prune_step_patch(mvla_ctx* ctx, int32_t prune_point, int32_t batch, cons
     }
     if (forked && cudaEventRecord(ctx->ev_copy[par], st) != cudaSuccess) return fail_cuda(ctx, cudaGetLastError());
     commit_steps(ctx, prune_point, plan, samples);
+    ctx->sets.done();
     if (total_kept_out) *total_kept_out = static_cast<int32_t>(cap);
     return MVLA_OK;
 }
@@ -904,7 +921,6 @@ static int32_t mvla_prune_create_impl(const mvla_config* cfg, mvla_ctx** out)
     alloc(&ctx->part, vis_all * c.n_heads);
     alloc(&ctx->l1_ws, kSets * vis_all);
     ctx->vis_all = vis_all;
-    ctx->step_parity = 0;
     alloc(&ctx->ahat_state, 2 * n_state * ctx->max_vis);
     alloc(&ctx->mhat_state, 2 * n_state * 4);
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->acc64), kSets * vis_all * sizeof(unsigned long long));
@@ -1015,9 +1031,11 @@ static int32_t mvla_salience_impl(mvla_ctx* ctx, int32_t batch, const mvla_sampl
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const bool want_l1 = hidden && l1_out;
     // the kernels of the fused step, into a scratch set of this call's own
-    ctx->step_parity = (ctx->step_parity + 1u) % kSets;
-    ctx->sel_valid[ctx->step_parity] = false;        // this set is used outside the event chain
-    unsigned long long* acc64 = ctx->acc64 + ctx->step_parity * ctx->vis_all;
+    unsigned par = 0;
+    rc = take_set(ctx, st, &par);
+    if (rc != MVLA_OK) return rc;
+    ctx->sel_valid[par] = false;                     // this set is used outside the event chain
+    unsigned long long* acc64 = ctx->acc64 + par * ctx->vis_all;
     for (int first = 0; first < batch; first += kMaxChunk) {
         const BatchDesc bd = chunk_of(plan, first, std::min(kMaxChunk, batch - first));
         bool used_acc64 = false;
@@ -1025,6 +1043,7 @@ static int32_t mvla_salience_impl(mvla_ctx* ctx, int32_t batch, const mvla_sampl
                                 AlphaOut{nullptr, 0, 0}, nullptr, true, nullptr, false, nullptr, attn_out);
         if (rc != MVLA_OK) return rc;
     }
+    ctx->sets.done();
     return MVLA_OK;
 }
 
@@ -1250,14 +1269,15 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
     }
 
     // scratch set of this step
-    ctx->step_parity = (ctx->step_parity + 1u) % kSets;
-    unsigned long long* acc64 = ctx->acc64 + ctx->step_parity * ctx->vis_all;
-    float* l1_ws = ctx->l1_ws + ctx->step_parity * ctx->vis_all;
+    unsigned par = 0;
+    rc = take_set(ctx, st, &par);
+    if (rc != MVLA_OK) return rc;
+    unsigned long long* acc64 = ctx->acc64 + par * ctx->vis_all;
+    float* l1_ws = ctx->l1_ws + par * ctx->vis_all;
     // With stable inputs (and the fast scoring kernel, whose scratch rotates over kSets sets) scoring and
     // selection go to the side stream of this step's scratch set (see plan_fork).
     bool forked = false, chained = false, early = false;
     ForkPlan fp;
-    const unsigned par = ctx->step_parity;
     const size_t nvis_b = static_cast<size_t>(plan.total_vis), nout_b = static_cast<size_t>(plan.total_out);
     const size_t hb = static_cast<size_t>(ctx->cfg.d_model) * ctx->elem, kb = static_cast<size_t>(kv_bytes);
     const size_t qb = static_cast<size_t>(ctx->cfg.n_heads) * ctx->cfg.head_dim * ctx->qk_elem;
@@ -1369,6 +1389,7 @@ static int32_t mvla_prune_step_impl(mvla_ctx* ctx, int32_t prune_point, int32_t 
         if (forked && cudaEventRecord(ctx->ev_copy[par], st) != cudaSuccess) return fail_cuda(ctx, cudaGetLastError());
     }
     commit_steps(ctx, prune_point, plan, samples);
+    ctx->sets.done();
     if (total_kept_out) *total_kept_out = plan.total_out;
     return MVLA_OK;
 }

@@ -1205,6 +1205,40 @@ def test_an_event_between_the_kernels_keeps_the_tail_behind_the_scoring_kernel()
     ctx.close()
 
 
+@pytest.mark.parametrize("batch,n_txt,n_2d,n_3d", [(13, (33, 16, 64), (256, 300), (400, 384)), (2, (12, 30), (100, 256), (300, 140))])
+def test_live_steps_with_captured_steps_between_them_in_the_rotation_of_scratch_sets(batch, n_txt, n_2d, n_3d):
+    """Two steps queued behind other work of their stream, and five that are captured in between: the second one comes round to the scratch
+    set of the first."""
+    wl = W.small_workload(80, batch=batch, H=24, D=128, d=128, n_txt=n_txt, n_2d=n_2d, n_3d=n_3d, keep=(0.3, 0.5), cold_start=0)
+    ctx, dev = mvla.context_for(wl), device_tensors(wl)
+    outs = [ctx.alloc_outputs(wl.samples, extras=True) for _ in range(4)]
+    call = lambda out: ctx.prune_step(0, wl.samples, wl.mode, dev["q"], dev["k"], dev["v"], dev["hidden"], flags=mvla.FLAG_RESET_STATE, out=out)
+    live, side, graph = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    call(outs[0])
+    torch.cuda.synchronize()
+    with torch.cuda.stream(live):
+        torch.cuda._sleep(20_000_000)                     # some 10 ms: the steps below wait in line, one behind the other
+        call(outs[1])
+    with torch.cuda.stream(side):
+        graph.capture_begin(capture_error_mode="relaxed")
+        for _ in range(5):
+            call(outs[2])
+        graph.capture_end()
+    with torch.cuda.stream(live):
+        call(outs[3])
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    n = int(outs[0].out_offsets[-1])
+    for out in outs[1:]:
+        assert torch.equal(out.budgets, outs[0].budgets) and torch.equal(out.ahat, outs[0].ahat)
+        for name in ("kept_idx", "out_hidden", "out_k", "out_v"):
+            assert torch.equal(getattr(out, name)[:n], getattr(outs[0], name)[:n]), name
+    call(outs[1])                                         # no wait ran out
+    torch.cuda.synchronize()
+    ctx.close()
+
+
 def test_stamps_of_a_tail_beside_the_scoring_kernel():
     """Selecting CTAs report the time of their last list as start and end; copying CTAs start before the scoring kernel has ended."""
     wl = W.small_workload(79, batch=13, H=24, D=128, d=128, n_txt=(33, 16, 64), n_2d=(256, 300), n_3d=(400, 384), keep=(0.3, 0.5), cold_start=0)
