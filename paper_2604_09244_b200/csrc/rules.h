@@ -89,13 +89,17 @@ inline bool tail_beside_pays(const TailBesideSizes& c)
     return c.key_bytes >= 6144 * ((c.row_bytes + kNormPiece - 1) / kNormPiece);
 }
 
-// Clusters of the streaming scoring kernel when the tail of the step runs beside it: no more than its rounds of jobs need (what a last round
-// leaves idle is the tail's), and at least kTailSms multiprocessors for the tail.
+// Clusters of the streaming scoring kernel when the tail of the step runs beside it: at least kTailSms multiprocessors are the tail's, and of the others no
+// more are taken than the rounds of jobs on them need (what a last round leaves idle is the tail's, too).  Counting the rounds on all multiprocessors and
+// leaving kTailSms out afterwards, 32 heads, fixed budgets, us a step: 18 samples (576 jobs: five rounds on 136) 77.9, five rounds on 116 75.2, four on 144 with
+// four left for the tail 80.3 (behind the scoring kernel 77.2); 27 samples 112.6 / 109.8 / 114.2; adaptive, 13 samples 74.1 / 72.5 / 74.5, 22 124.1 / 120.2 / 125.0,
+// 32 174.1 / 172.7; 13 of 1280 tokens (clusters of two) 127.7 / 125.1 / 128.2.
 constexpr int kTailSms = 12;
 inline int clusters_beside_tail(int jobs, int at_once, int cluster, int sm_count)
 {
-    const int rounds = (jobs + at_once - 1) / at_once, used = (jobs + rounds - 1) / rounds, most = (sm_count - kTailSms) / cluster;
-    return used < most ? used : (most > 1 ? most : 1);
+    const int left = (sm_count - kTailSms) / cluster, most = left < 1 ? 1 : (left < at_once ? left : at_once);
+    const int rounds = (jobs + most - 1) / most;
+    return (jobs + rounds - 1) / rounds;
 }
 
 }  // namespace mvla

@@ -77,3 +77,32 @@ int main()
 
 def test_small_stable_steps_are_chained_only_where_the_gpu_keeps_up(tmp_path):
     run_program(tmp_path, CHAIN)
+
+
+CLUSTERS = r"""
+#include <cstdio>
+#include "rules.h"
+using namespace mvla;
+int main()
+{
+    const int sizes[] = {1, 2, 4, 8}, at_once[] = {148, 74, 35, 16}, left[] = {136, 68, 34, 17};
+    for (int s = 0; s < 4; ++s)
+        for (int jobs = 1; jobs <= 2048; ++jobs) {
+            const int most = at_once[s] < left[s] ? at_once[s] : left[s], n = clusters_beside_tail(jobs, at_once[s], sizes[s], 148);
+            // no more than run at once beside the tail, as many rounds as on all of those, and no fewer clusters do
+            const int rounds = (jobs + most - 1) / most;
+            if (n < 1 || n > most || (jobs + n - 1) / n != rounds || (n > 1 && (jobs + n - 2) / (n - 1) == rounds)) {
+                std::printf("%d jobs, clusters of %d: %d\n", jobs, sizes[s], n);
+                return 1;
+            }
+        }
+    if (clusters_beside_tail(512, 148, 1, 148) != 128 || clusters_beside_tail(576, 148, 1, 148) != 116 || clusters_beside_tail(256, 35, 4, 148) != 32 ||
+        clusters_beside_tail(64, 4, 4, 16) != 1) { std::printf("points\n"); return 1; }
+    std::printf("ok\n");
+    return 0;
+}
+"""
+
+
+def test_clusters_beside_a_tail_are_those_that_their_rounds_need(tmp_path):
+    run_program(tmp_path, CLUSTERS)
