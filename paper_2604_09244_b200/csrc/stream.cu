@@ -756,24 +756,19 @@ int stream_cluster(int n_jobs, int tiles, int slots, int sms)
     return (tiles + cluster - 1) / cluster > slots ? 0 : cluster;
 }
 
-// The samples whose jobs take longest come first: some CTAs have a job more than the others, their last one, which should be a short one.
-// A job's softmax takes as long as its tiles and padded text queries say, its keys as long as its tiles (as much as 32 queries more).
-// 16 patch-by-patch requests of 512 tokens with texts of 16 to 64: 76.9 -> 74.7 us; texts of one length: the order given.
-BatchDesc costly_first(const BatchDesc& given)
+// The launch's samples in the order in which their jobs are taken (longest_first_pays); `room` for them where that is not the order given.
+const BatchDesc& in_order(const BatchDesc& given, int n_heads, int clusters, BatchDesc& room)
 {
-    BatchDesc bd = given;
-    auto cost = [](const SampleDev& s) {
-        const int tiles = (s.n_2d + kKeyTile - 1) / kKeyTile + (s.n_3d + kKeyTile - 1) / kKeyTile;
-        return tiles * (((s.n_txt + 15) & ~15) + 32);
-    };
-    for (int i = 1; i < bd.n; ++i) {                     // (insertion: at most kMaxChunk, often in order)
-        if (cost(bd.s[i - 1]) >= cost(bd.s[i])) continue;
-        const SampleDev s = bd.s[i];
-        int at = i;
-        for (; at > 0 && cost(bd.s[at - 1]) < cost(s); --at) bd.s[at] = bd.s[at - 1];
-        bd.s[at] = s;
+    int cost[kMaxChunk];
+    uint8_t order[kMaxChunk];
+    for (int b = 0; b < given.n; ++b) {
+        const SampleDev& s = given.s[b];
+        cost[b] = job_cost((s.n_2d + kKeyTile - 1) / kKeyTile + (s.n_3d + kKeyTile - 1) / kKeyTile, (s.n_txt + 15) & ~15);
     }
-    return bd;
+    if (!longest_first_pays(cost, given.n, n_heads, clusters, order)) return given;
+    room = given;
+    for (int b = 0; b < given.n; ++b) room.s[b] = given.s[order[b]];
+    return room;
 }
 
 // Clusters that run at once (a second wave of a persistent grid would double its time), with the kernel set up.
@@ -788,7 +783,7 @@ cudaError_t launch_size(int threads, int cluster, int* n)
 }
 
 template <bool ROOM, bool HAND>
-cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUtensorMap* tk, StreamArgs& a, int cluster, cudaStream_t stream)
+cudaError_t launch_stream(const BatchDesc& given, const CUtensorMap* tq, const CUtensorMap* tk, StreamArgs& a, int cluster, cudaStream_t stream)
 {
     auto kern = salience_stream_kernel<ROOM, HAND>;
     int n = 0;
@@ -798,6 +793,8 @@ cudaError_t launch_stream(const BatchDesc& bd, const CUtensorMap* tq, const CUte
     cudaLaunchConfig_t cfg = {};
     int clusters = a.hidden ? n : std::min(a.n_jobs, n);       // (norms are shared out over all CTAs)
     if (HAND) clusters = clusters_beside_tail(a.n_jobs, n, cluster, sm_count_of_current_device());
+    BatchDesc room;
+    const BatchDesc& bd = HAND ? given : in_order(given, a.n_heads, clusters, room);       // (a tail beside takes the samples as they are)
     cfg.gridDim = dim3(static_cast<unsigned>(clusters * cluster));
     cfg.blockDim = dim3(static_cast<unsigned>(threads));
     cfg.dynamicSmemBytes = kStreamSmem;
@@ -840,14 +837,13 @@ cudaError_t stream_beside_tail(const BatchDesc& bd, int n_heads, int64_t head_by
     return cudaSuccess;
 }
 
-cudaError_t launch_salience_stream(const BatchDesc& given, int n_heads, int kv_group, int head_dim, int esize,
+cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_group, int head_dim, int esize,
                                    const CUtensorMap* tmap_q, const CUtensorMap* tmap_k, unsigned long long* acc64, int* status,
                                    AlphaOut alpha, int32_t* rearm, unsigned long long* rearm_rec,
                                    unsigned long long* stamps, bool norms_beside, const void* hidden, int row_bytes, float* l1, int32_t* hand,
                                    cudaStream_t stream)
 {
     const int sms = sm_count_of_current_device();
-    const BatchDesc bd = hand ? given : costly_first(given);      // (a tail beside takes the samples as they are)
     const int npad = padded_text(bd), tiles = max_tiles(bd);
     StreamArgs a;
     a.n_heads = n_heads; a.kv_group = kv_group; a.head_dim = head_dim; a.esize = esize;

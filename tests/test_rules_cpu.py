@@ -106,3 +106,55 @@ int main()
 
 def test_clusters_beside_a_tail_are_those_that_their_rounds_need(tmp_path):
     run_program(tmp_path, CLUSTERS)
+
+
+ORDER = r"""
+#include <cstdio>
+#include <algorithm>
+#include <random>
+#include <vector>
+#include "rules.h"
+using namespace mvla;
+struct Point { int clusters; bool first; std::vector<int> cost; };      // 32 heads; costs of a sample's jobs (tiles x (padded text + 32))
+static const Point points[] = {
+    {148, true, {160, 160, 160, 160, 160, 128, 160, 128, 128, 192, 192, 160, 128, 192, 192, 160}},
+    {148, true, {160, 400, 160, 560, 160, 320, 160, 448, 128, 480, 192, 560, 128, 480, 192, 560}},
+    {74, true, {192, 192, 192, 192, 192, 1248, 192, 192, 192, 192, 192, 1248}},
+    {148, true, {480, 480, 480, 480, 480, 384, 480, 384, 384, 576}},
+    {148, true, {320, 160, 640, 160, 320, 128, 640, 128, 256, 192, 768, 160, 256, 192, 768, 160}},
+    {33, false, {288, 288, 288, 288, 288, 288, 288, 288, 288, 288, 288, 3072}},
+    {33, false, {192, 192, 192, 192, 192, 2688}},
+    {148, false, {160, 160, 160, 160, 160, 128, 160, 640}},
+    {148, false, {640, 640, 640, 640, 640, 512, 640, 512}}, {148, false, {480, 480, 480}},
+};
+int main()
+{
+    uint8_t order[32];
+    for (const Point& p : points)
+        if (longest_first_pays(p.cost.data(), static_cast<int>(p.cost.size()), 32, p.clusters, order) != p.first) {
+            std::printf("%d samples on %d clusters\n", static_cast<int>(p.cost.size()), p.clusters);
+            return 1;
+        }
+    std::mt19937 rng(5);
+    for (int k = 0; k < 4000; ++k) {                     // the sum against jobs dealt out one by one; the order a falling one, and stable
+        const int n = 1 + rng() % 32, heads = 1 + rng() % 64, clusters = 1 + rng() % 160;
+        std::vector<int> cost(n);
+        std::vector<int64_t> load(clusters, 0);
+        for (int& c : cost) c = 1 + rng() % 5 * 100;
+        for (int j = 0; j < n * heads; ++j) load[j % clusters] += cost[j / heads];
+        const int64_t most = *std::max_element(load.begin(), load.end());
+        if (fullest_cluster(cost.data(), n, heads, clusters) != most) { std::printf("%d x %d jobs on %d clusters\n", n, heads, clusters); return 1; }
+        longest_first_pays(cost.data(), n, heads, clusters, order);
+        std::vector<int> by(n);
+        for (int b = 0; b < n; ++b) by[b] = b;
+        std::stable_sort(by.begin(), by.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+        if (!std::equal(by.begin(), by.end(), order)) { std::printf("order\n"); return 1; }
+    }
+    std::printf("ok\n");
+    return 0;
+}
+"""
+
+
+def test_samples_with_long_jobs_come_first_only_where_the_fullest_cluster_gets_less(tmp_path):
+    run_program(tmp_path, ORDER)
