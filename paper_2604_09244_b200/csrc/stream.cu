@@ -62,6 +62,8 @@ struct StreamArgs {
     int row_bytes;
     uint32_t norm_off;
     int n_samples;
+    int vis0;                     // first visual token of the launch
+    uint8_t by_row[kMaxChunk];    // samples in the order of their visual tokens: a norm warp's run of rows crosses them without a look at whose sum it takes
 };
 
 struct StreamSmem {
@@ -388,7 +390,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
     // kernel's parameters costs some hundred cycles).
     int fb = 0, fv = first, n_2d = 0, n_vis = 0, row_2d = 0, row_3d = 0;
     auto sample = [&]() {
-        const SampleDev& s = bd.s[fb];
+        const SampleDev& s = bd.s[HAND ? fb : a.by_row[fb]];
         n_2d = s.n_2d;
         n_vis = s.n_2d + s.n_3d;
         row_2d = s.seq_off + s.off_2d;
@@ -396,8 +398,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
     };
     sample();
     while (fv >= n_vis && fb < a.n_samples - 1) { fv -= n_vis; ++fb; sample(); }
-    int sb = fb, sv = fv, s_vis = n_vis;                 // the row next to be summed (HAND: the samples lie one behind another)
-    float* out = HAND ? a.l1 + bd.s[0].vis_off + first : a.l1 + bd.s[sb].vis_off + sv;
+    float* out = a.l1 + a.vis0 + first;                  // the one next to be summed
     int fp = 0;
     auto fetch = [&](int st) {
         const int row = (fv < n_2d ? row_2d : row_3d) + fv;
@@ -449,12 +450,6 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
             for (int off = 16; off >= 1; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
             if (lane == 0) *out = r;
             out += step;
-            if (!HAND && ++sv == s_vis && sb < a.n_samples - 1) {
-                ++sb;
-                sv = 0;
-                s_vis = bd.s[sb].n_2d + bd.s[sb].n_3d;
-                out = a.l1 + bd.s[sb].vis_off;
-            }
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[e] = 0.f;
         }
@@ -756,8 +751,9 @@ int stream_cluster(int n_jobs, int tiles, int slots, int sms)
     return (tiles + cluster - 1) / cluster > slots ? 0 : cluster;
 }
 
-// The launch's samples in the order in which their jobs are taken (longest_first_pays); `room` for them where that is not the order given.
-const BatchDesc& in_order(const BatchDesc& given, int n_heads, int clusters, BatchDesc& room)
+// The launch's samples in the order in which their jobs are taken (longest_first_pays), `room` for them where that is not the order given; and which of them
+// comes where by its rows.
+const BatchDesc& in_order(const BatchDesc& given, int n_heads, int clusters, BatchDesc& room, uint8_t* by_row)
 {
     int cost[kMaxChunk];
     uint8_t order[kMaxChunk];
@@ -765,9 +761,13 @@ const BatchDesc& in_order(const BatchDesc& given, int n_heads, int clusters, Bat
         const SampleDev& s = given.s[b];
         cost[b] = job_cost((s.n_2d + kKeyTile - 1) / kKeyTile + (s.n_3d + kKeyTile - 1) / kKeyTile, (s.n_txt + 15) & ~15);
     }
+    for (int b = 0; b < given.n; ++b) by_row[b] = static_cast<uint8_t>(b);
     if (!longest_first_pays(cost, given.n, n_heads, clusters, order)) return given;
     room = given;
-    for (int b = 0; b < given.n; ++b) room.s[b] = given.s[order[b]];
+    for (int b = 0; b < given.n; ++b) {
+        room.s[b] = given.s[order[b]];
+        by_row[order[b]] = static_cast<uint8_t>(b);
+    }
     return room;
 }
 
@@ -794,7 +794,7 @@ cudaError_t launch_stream(const BatchDesc& given, const CUtensorMap* tq, const C
     int clusters = a.hidden ? n : std::min(a.n_jobs, n);       // (norms are shared out over all CTAs)
     if (HAND) clusters = clusters_beside_tail(a.n_jobs, n, cluster, sm_count_of_current_device());
     BatchDesc room;
-    const BatchDesc& bd = HAND ? given : in_order(given, a.n_heads, clusters, room);       // (a tail beside takes the samples as they are)
+    const BatchDesc& bd = HAND ? given : in_order(given, a.n_heads, clusters, room, a.by_row);       // (a tail beside takes the samples as they are)
     cfg.gridDim = dim3(static_cast<unsigned>(clusters * cluster));
     cfg.blockDim = dim3(static_cast<unsigned>(threads));
     cfg.dynamicSmemBytes = kStreamSmem;
@@ -860,7 +860,7 @@ cudaError_t launch_salience_stream(const BatchDesc& bd, int n_heads, int kv_grou
     a.stages = static_cast<int>(std::min<size_t>(hand ? kStagesBesideTail : kMaxStages, (kStreamSmem - 1024 - q_bytes - norm_bytes) / kStageBytes));
     if (a.stages < 4 || (hidden && norms_beside)) return cudaErrorInvalidConfiguration;
     a.hidden = static_cast<const uint8_t*>(hidden);
-    a.l1 = l1; a.row_bytes = row_bytes; a.n_samples = bd.n;
+    a.l1 = l1; a.row_bytes = row_bytes; a.n_samples = bd.n; a.vis0 = bd.s[0].vis_off;
     a.norm_off = static_cast<uint32_t>(a.stages * kStageBytes + q_bytes);
     if (norms_beside && !alpha.ptr) return launch_stream<true, false>(bd, tmap_q, tmap_k, a, cluster, stream);
     if (hand) return launch_stream<false, true>(bd, tmap_q, tmap_k, a, cluster, stream);
