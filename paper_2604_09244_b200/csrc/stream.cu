@@ -374,7 +374,7 @@ __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, in
 // or a CTA of their own.  What bounds it is a piece's fixed cost and the adds of its sums, not the bytes in flight (adaptive steps of
 // 16 requests of 768 tokens: two pieces in flight 99.9 us, three 98.4; pieces of 4 KB 110.8; a run of rows instead of every n_w-th, whose
 // sample has to be looked up each time, 97.8 instead of 98.4; four sums beside one another instead of one chain 94.8; eight loads at once 93.7).
-template <bool HAND>
+template <bool HAND, bool MIXED>
 __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs& a, StreamSmem& sm, uint32_t buf, int nw, int lane)
 {
     const bool one = elect_one();
@@ -390,7 +390,7 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
     // kernel's parameters costs some hundred cycles).
     int fb = 0, fv = first, n_2d = 0, n_vis = 0, row_2d = 0, row_3d = 0;
     auto sample = [&]() {
-        const SampleDev& s = bd.s[HAND ? fb : a.by_row[fb]];
+        const SampleDev& s = bd.s[MIXED ? a.by_row[fb] : fb];
         n_2d = s.n_2d;
         n_vis = s.n_2d + s.n_3d;
         row_2d = s.seq_off + s.off_2d;
@@ -466,7 +466,8 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
 // with 144; 16 adaptive requests 93.7 and 93.0.
 // HAND: the tail of the step runs beside this kernel (launch_select_copy_beside); a variant of its own, because in the others the skipped code
 // cost steps of 20 to 40 us 1 to 2 %.
-template <bool ROOM, bool HAND>
+// MIXED: the samples are not in the order of their rows, and the norm warps take them by by_row; a variant of its own for the same reason.
+template <bool ROOM, bool HAND, bool MIXED>
 __global__ void __maxnreg__(ROOM ? 144 : kStreamRegs)
 salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_constant__ CUtensorMap tmap_q,
                        const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ StreamArgs a)
@@ -622,7 +623,7 @@ salience_stream_kernel(const __grid_constant__ BatchDesc bd, const __grid_consta
     } else if (!ROOM && warp > kSoftWarps + 1) {
         // ---------------------------------------------------------------- feature norms
         const int nw = warp - kSoftWarps - 2;
-        if (a.hidden) norm_warp<HAND>(bd, a, sm, smem_u32(dyn) + a.norm_off + static_cast<uint32_t>(nw * kNormStages) * kNormPiece, nw, lane);
+        if (a.hidden) norm_warp<HAND, MIXED>(bd, a, sm, smem_u32(dyn) + a.norm_off + static_cast<uint32_t>(nw * kNormStages) * kNormPiece, nw, lane);
     } else {
         // ---------------------------------------------------------------- softmax
         SoftJob j;
@@ -771,32 +772,25 @@ const BatchDesc& in_order(const BatchDesc& given, int n_heads, int clusters, Bat
     return room;
 }
 
+int stream_threads(const StreamArgs& a) { return kStreamThreads + (a.hidden ? 32 * kNormWarps : 0); }
+
 // Clusters that run at once (a second wave of a persistent grid would double its time), with the kernel set up.
-template <bool ROOM, bool HAND>
+template <bool ROOM, bool HAND, bool MIXED>
 cudaError_t launch_size(int threads, int cluster, int* n)
 {
-    const void* kern = reinterpret_cast<const void*>(salience_stream_kernel<ROOM, HAND>);
+    const void* kern = reinterpret_cast<const void*>(salience_stream_kernel<ROOM, HAND, MIXED>);
     static KernelSetup ks;
     cudaError_t e = setup_kernel(ks, kern, kStreamSmem, kTmemColsPerSm);
     if (e == cudaSuccess) e = clusters_at_once(ks, kern, threads, kStreamSmem, cluster, n);
     return e == cudaSuccess && *n < 1 ? cudaErrorInvalidConfiguration : e;
 }
 
-template <bool ROOM, bool HAND>
-cudaError_t launch_stream(const BatchDesc& given, const CUtensorMap* tq, const CUtensorMap* tk, StreamArgs& a, int cluster, cudaStream_t stream)
+template <bool ROOM, bool HAND, bool MIXED>
+cudaError_t launch_variant(const BatchDesc& bd, const CUtensorMap* tq, const CUtensorMap* tk, const StreamArgs& a, int cluster, int clusters, cudaStream_t stream)
 {
-    auto kern = salience_stream_kernel<ROOM, HAND>;
-    int n = 0;
-    const int threads = kStreamThreads + (a.hidden ? 32 * kNormWarps : 0);
-    const cudaError_t e = launch_size<ROOM, HAND>(threads, cluster, &n);
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    int clusters = a.hidden ? n : std::min(a.n_jobs, n);       // (norms are shared out over all CTAs)
-    if (HAND) clusters = clusters_beside_tail(a.n_jobs, n, cluster, sm_count_of_current_device());
-    BatchDesc room;
-    const BatchDesc& bd = HAND ? given : in_order(given, a.n_heads, clusters, room, a.by_row);       // (a tail beside takes the samples as they are)
     cfg.gridDim = dim3(static_cast<unsigned>(clusters * cluster));
-    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.blockDim = dim3(static_cast<unsigned>(stream_threads(a)));
     cfg.dynamicSmemBytes = kStreamSmem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -807,7 +801,26 @@ cudaError_t launch_stream(const BatchDesc& given, const CUtensorMap* tq, const C
     attr[1] = pdl_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, bd, *tq, *tk, a);
+    return cudaLaunchKernelEx(&cfg, salience_stream_kernel<ROOM, HAND, MIXED>, bd, *tq, *tk, a);
+}
+
+template <bool ROOM, bool HAND>
+cudaError_t launch_stream(const BatchDesc& given, const CUtensorMap* tq, const CUtensorMap* tk, StreamArgs& a, int cluster, cudaStream_t stream)
+{
+    int n = 0;
+    cudaError_t e = launch_size<ROOM, HAND, false>(stream_threads(a), cluster, &n);
+    if (e != cudaSuccess) return e;
+    if constexpr (HAND)                  // (the samples as they are: the tail takes them in that order)
+        return launch_variant<ROOM, true, false>(given, tq, tk, a, cluster, clusters_beside_tail(a.n_jobs, n, cluster, sm_count_of_current_device()), stream);
+    const int clusters = a.hidden ? n : std::min(a.n_jobs, n);       // (norms are shared out over all CTAs)
+    BatchDesc room;
+    const BatchDesc& bd = in_order(given, a.n_heads, clusters, room, a.by_row);
+    if constexpr (!ROOM)
+        if (a.hidden && &bd != &given) {
+            e = launch_size<ROOM, HAND, true>(stream_threads(a), cluster, &n);       // (sets the variant up)
+            return e == cudaSuccess ? launch_variant<ROOM, HAND, true>(bd, tq, tk, a, cluster, clusters, stream) : e;
+        }
+    return launch_variant<ROOM, HAND, false>(bd, tq, tk, a, cluster, clusters, stream);
 }
 
 }  // namespace
@@ -828,7 +841,7 @@ cudaError_t stream_beside_tail(const BatchDesc& bd, int n_heads, int64_t head_by
     const auto pays = [&]() { return tail_beside_pays({tokens, bd.n, jobs, n, head_bytes, key_bytes, row_bytes}); };
     if (cluster == 0 || !pays()) return cudaSuccess;         // (clusters: the runtime is asked only where the rest says yes)
     if (cluster > 1) {
-        const cudaError_t e = launch_size<false, true>(kStreamThreads + 32 * kNormWarps, cluster, &n);
+        const cudaError_t e = launch_size<false, true, false>(kStreamThreads + 32 * kNormWarps, cluster, &n);
         if (e != cudaSuccess) return e;
         if (!pays()) return cudaSuccess;
     }
