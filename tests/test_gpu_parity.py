@@ -1156,7 +1156,7 @@ def test_scoring_kernel_goes_by_what_fits_on_the_device(batch, d, n_txt, n_2d, n
     (13, 24, (33, 64), (256, 300), (400, 384), {"cold_start": 1}, True),                     # all kept first: norms after the list
     (13, 24, (33, 64), (200, 160), (380, 440), {}, False),                                   # keys of a job below the line
     (12, 24, (33, 64), (256, 300), (400, 384), {}, False),                                   # two rounds
-    (36, 24, (3, 20), (256, 300), (400, 384), {}, False),                                    # a launch of 32 samples beside, one of 4 behind
+    (36, 24, (3, 20), (256, 300), (400, 384), {}, True),                                     # a launch of 32 samples beside, one of 4 (96 CTAs) behind
     (7, 24, (64, 50), (600, 300), (500, 1024), {}, True),                                    # clusters of two, up to 1324 tokens
     (3, 24, (64, 50), (1500, 900), (700, 1300), {}, True)])                                  # clusters of four, 2200 tokens
 def test_tail_beside_the_streaming_scoring_kernel(batch, H, n_txt, n_2d, n_3d, kw, beside):
@@ -1172,9 +1172,8 @@ def test_tail_beside_the_streaming_scoring_kernel(batch, H, n_txt, n_2d, n_3d, k
         stamps = torch.zeros(2, ctx.STAMP_SLOTS, 2, dtype=torch.int64, device="cuda")
         ctx.set_kernel_stamps(stamps)
         run_and_check_step(ctx, wl, step, states)
-        if batch <= 32:
-            sms = torch.cuda.get_device_properties(0).multi_processor_count
-            assert (int((stamps[0, :, 1] != 0).sum()) <= sms - 12 and int((stamps[1, :, 0] != 0).sum()) >= sms) == beside
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        assert (int((stamps[0, :, 1] != 0).sum()) <= sms - 12 and int((stamps[1, :, 0] != 0).sum()) >= sms) == beside
     ctx.set_kernel_stamps(None)
     dev, runs = device_tensors(wl), []
     for _ in range(8):
@@ -1184,6 +1183,73 @@ def test_tail_beside_the_streaming_scoring_kernel(batch, H, n_txt, n_2d, n_3d, k
         runs.append([out.budgets, out.ahat] + [t[:n] for t in (out.kept_idx, out.out_hidden, out.out_k, out.out_v)])
     for r in runs[1:]:
         assert all(torch.equal(x.contiguous().view(torch.uint8), y.contiguous().view(torch.uint8)) for x, y in zip(runs[0], r))
+    ctx.close()
+
+
+FORMS = {                     # heads, head dim, key heads, dtype, hidden width, samples, text, 2D, 3D, mode
+    "rows_of_two_pieces": (48, 128, 0, torch.bfloat16, 4104, 7, (33, 16, 64), (256, 300), (400, 384), mvla.MODE_ADAPTIVE),
+    "heads_of_256": (16, 256, 0, torch.bfloat16, 512, 20, (64, 5), (120, 130), (210, 200), mvla.MODE_ADAPTIVE),       # a ring of five stages
+    "e4m3": (48, 128, 0, torch.float8_e4m3fn, 264, 7, (16, 48), (600, 640), (700, 760), mvla.MODE_ADAPTIVE),
+    "e4m3_grouped": (32, 128, 8, torch.float8_e4m3fn, 256, 10, (7, 16), (600, 640), (700, 760), mvla.MODE_FIXED),
+    "grouped": (32, 128, 8, torch.bfloat16, 256, 10, (33, 64), (256, 300), (400, 384), mvla.MODE_FIXED),
+    "one_key_head": (32, 128, 1, torch.bfloat16, 64, 10, (1, 64), (0, 300), (700, 384), mvla.MODE_FIXED),
+    "above_2048_tokens": (24, 128, 0, torch.bfloat16, 128, 4, (48, 64), (100, 1500), (700, 1300), mvla.MODE_ADAPTIVE),   # CTAs of 32 warps; the last sample the longest
+}
+
+
+@pytest.mark.parametrize("outputs", ["all", "hidden", "none", "dry"])
+@pytest.mark.parametrize("form", FORMS)
+def test_tail_beside_gives_what_the_tail_behind_gives(form, outputs):
+    """The same batches from a tail beside the scoring kernel, from one behind it (an event set between the kernels) and from a graph that is replayed:
+    the same bits; the indicators, whose norms other warps have summed, to the last few bits of fp32."""
+    H, d, hkv, dtype, D, batch, n_txt, n_2d, n_3d, mode = FORMS[form]
+    samples, off = [], 0
+    for b in range(batch):
+        s = W.layout_2d_3d_txt(off, n_txt[b % len(n_txt)], n_2d[b % len(n_2d)], n_3d[b % len(n_3d)], keep_2d=0.3, keep_3d=0.4, keep_total=(0.2, 0.5)[b % 2], state_slot=b)
+        samples.append(s)
+        off += s.seq_len
+    gen = torch.Generator(device="cuda").manual_seed(81)
+    draw = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+    q, k, v = (draw(off, h, d).to(dtype) for h in (H, hkv or H, hkv or H))
+    hidden = draw(off, D).to(torch.bfloat16)
+    ctx = mvla.PruneContext(dtype=dtype, n_heads=H, head_dim=d, d_model=D, max_batch=batch, max_text=64, max_2d=max(n_2d), max_3d=max(n_3d), n_kv_heads=hkv,
+                            cold_start_full_keep=0, tau_2d=0.35, tau_3d=0.65)
+    flags = mvla.FLAG_RESET_STATE | (mvla.FLAG_NO_STATE_UPDATE if outputs == "dry" else 0)
+
+    def fresh():
+        out = ctx.alloc_outputs(samples, hidden=outputs != "none", kv=outputs in ("all", "dry"), extras=True)
+        for t in vars(out).values():
+            if torch.is_tensor(t):
+                t.view(torch.uint8).zero_()
+        return out
+    call = lambda out: ctx.prune_step(0, samples, mode, q, k, v if out.out_v is not None else None, hidden, flags=flags, out=out)
+    stamps = torch.zeros(2, ctx.STAMP_SLOTS, 2, dtype=torch.int64, device="cuda")
+    ctx.set_kernel_stamps(stamps)
+    sms, event = torch.cuda.get_device_properties(0).multi_processor_count, torch.cuda.Event()
+    beside, behind = fresh(), fresh()
+    call(beside)
+    assert int((stamps[0, :, 1] != 0).sum()) <= sms - 12 and int((stamps[1, :, 0] != 0).sum()) >= (sms if outputs != "none" else 1)
+    event.record()
+    ctx.set_stage_event(event)
+    call(behind)
+    ctx.set_stage_event(None)
+    ctx.set_kernel_stamps(None)
+    captured, graph = fresh(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(7):                                # the rotation of scratch sets comes round
+            call(captured)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    for out in (behind, captured):
+        for name, t in vars(beside).items():
+            other = getattr(out, name)
+            if name == "diag":
+                a, b = t.cpu().numpy(), other.cpu().numpy()
+                assert np.array_equal(a[:, :7], b[:, :7])
+                np.testing.assert_allclose(b[:, 8:].copy().view(np.float32), a[:, 8:].copy().view(np.float32), rtol=2e-6)
+            elif torch.is_tensor(t):
+                assert torch.equal(t.view(torch.uint8), other.view(torch.uint8)), name
     ctx.close()
 
 

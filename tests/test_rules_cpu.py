@@ -158,3 +158,40 @@ int main()
 
 def test_samples_with_long_jobs_come_first_only_where_the_fullest_cluster_gets_less(tmp_path):
     run_program(tmp_path, ORDER)
+
+
+BESIDE = r"""
+#include <cstdio>
+#include "rules.h"
+using namespace mvla;
+// (bytes of an element of k, heads, head dim, key heads, bytes of a hidden row, samples, tokens of a sample, clusters at once; norms: adaptive budgets)
+struct Point { int esize, heads, dim, kv, row, batch, tokens, at_once; bool norms, beside; };
+static const Point points[] = {
+    {2, 32, 128, 32, 8192, 10, 768, 148, true, true}, {2, 32, 128, 32, 8192, 16, 768, 148, true, true}, {2, 32, 128, 32, 8192, 32, 768, 148, true, true},
+    {2, 32, 128, 32, 8192, 9, 768, 148, true, false},          // 288 jobs: two rounds
+    {2, 32, 128, 32, 8192, 16, 640, 148, true, true}, {2, 32, 128, 32, 8192, 16, 639, 148, true, false},       // keys of a job on both sides of 160 KB
+    {2, 32, 128, 32, 8192, 16, 228, 148, true, false}, {2, 32, 128, 32, 8192, 32, 228, 148, false, false},
+    {2, 32, 128, 32, 8192, 5, 1280, 74, true, true}, {2, 32, 128, 32, 8192, 4, 1280, 74, true, false}, {2, 32, 128, 32, 8192, 3, 3000, 33, true, true},
+    {2, 32, 128, 32, 8192, 2, 3000, 33, true, false}, {2, 32, 128, 32, 8192, 1, 4096, 8, true, false},
+    {2, 16, 256, 16, 8192, 24, 768, 148, true, true}, {2, 32, 96, 32, 6144, 12, 900, 148, true, true},
+    {1, 32, 128, 32, 8192, 12, 1300, 148, false, true}, {1, 32, 128, 32, 8192, 12, 1300, 148, true, false}, {1, 32, 128, 8, 8192, 16, 768, 148, false, false},
+    {2, 32, 64, 32, 4096, 16, 768, 148, true, false}, {2, 32, 64, 32, 4096, 12, 1500, 148, false, true},
+    {2, 16, 128, 16, 4096, 24, 768, 148, true, false}, {2, 16, 128, 16, 4096, 24, 768, 148, false, true},      // the norms would take longer than the scores
+    {2, 32, 128, 8, 8192, 10, 768, 148, false, true}, {2, 32, 128, 8, 8192, 16, 768, 148, true, false},
+    {2, 48, 128, 48, 8208, 7, 700, 148, true, true}, {2, 40, 128, 40, 10240, 8, 768, 148, true, false},        // rows of two pieces
+};
+int main()
+{
+    for (const Point& p : points) {
+        const TailBesideSizes c = {static_cast<int64_t>(p.batch) * p.tokens, p.batch, p.batch * p.heads, p.at_once, p.dim * p.esize,
+                                   static_cast<int64_t>(p.kv) * p.dim * p.esize, p.norms ? p.row : 0};
+        if (tail_beside_pays(c) != p.beside) { std::printf("%d heads of %d, %d x %d, norms %d\n", p.heads, p.dim, p.batch, p.tokens, p.norms); return 1; }
+    }
+    std::printf("ok\n");
+    return 0;
+}
+"""
+
+
+def test_the_tail_runs_beside_the_scoring_kernel_only_where_jobs_are_long_and_many(tmp_path):
+    run_program(tmp_path, BESIDE)
