@@ -21,7 +21,8 @@ namespace mvla {
 //   rows of 10 KB, 40 heads of 128: 6 49.1 / 43.7 | 15 88.0 / 99.2; 20 heads: 6 28.0 / 33.5
 //   rows of 16 KB, 16 heads of 128: 6 45.6 / 38.4, 10 66.8 / 61.2 | 6 45.8 / 37.6
 // Above 88 tokens a multiprocessor inside loses whatever the texts (32 heads of 128: 18 samples 90.4 / 92.6, 32 153 / 163), and samples of more
-// than 16 key tiles go either way (2 x 3426 77.4 / 73.3, 7 x 2584 115.4 / 119).  Rows of eight times the keys' bytes, where the
+// than 16 key tiles go either way (2 x 3426 77.4 / 73.3, 7 x 2584 115.4 / 119); with the tail behind the kernel, that is: where it runs beside (tail_beside_pays, as
+// for most of these now) the norms are inside whatever this rule says.  Rows of eight times the keys' bytes, where the
 // scores of few jobs end early: e4m3, 16 heads of 256, 4 key heads, 12 x 435 (192 jobs) 26.5 / 27.3, 20 x 350 (320 jobs) 37.8 / 34.8.
 constexpr uint32_t kNormPiece = 8192;        // bytes of a row that a norm warp fetches at once
 struct NormsInsideSizes {
@@ -118,11 +119,15 @@ inline bool longest_first_pays(const int* cost, int samples, int heads, int clus
 // some samples are scored well before the others; where a job is long enough that the multiprocessors given to the tail and the words that pass between
 // the kernels cost less than the idle memory between them; and where the scoring kernel's two norm warps, which take the feature norms then,
 // keep up with its scores.  Whole steps in us, behind / beside, 32 heads of 128, texts of 16 to 64, unless said otherwise:
-//   768 tokens (196 KB of keys a job): 10 samples 62.0 / 59.0, 16 93.4 / 87.9, 20 116.8 / 111.6, 28 156.8 / 152.8, fixed budgets 71.9 / 70.0, short
-//     texts 92.5 / 87.3; 3000 tokens: 3 samples 68.3 / 62.6, 5 105.1 / 99.7, 7 137.8 / 133.6; 3584: 8 161.5 / 155.8; 1700, short texts: 6 68.5 / 68.5;
-//     16 heads of 256, 24 samples 134.2 / 132.0;
+//   768 tokens (196 KB of keys a job): 10 samples 62.4 / 56.6, 16 93.7 / 88.4, 24 139.8 / 133.2; fixed budgets 12 56.0 / 51.9, 16 72.1 / 67.1; with 8 key heads, fixed, 10
+//     39.0 / 37.3, 16 53.1 / 48.9, 32 90.6 / 86.1, short texts 42.0 / 41.4; 16 heads, fixed, short texts, 24 50.4 / 49.1; 640 tokens (160 KB), few kept, 16 55.0 / 54.5;
+//   3000 tokens: 5 samples 105.0 / 99.0; 3584: 8 163.6 / 156.0; e4m3, fixed, short texts, 12 of 1300 57.7 / 54.5, with 8 key heads 44.7 / 43.8; 32 heads of 64, fixed, short texts, 12 of 1500
+//     55.6 / 52.2, with 8 key heads 40.3 / 39.6;
+//   long and short samples: 5 of 228 and one of 3584 55.4 / 55.1, the long one first 61.1 / 55.4, 5 of 768 and one of 3584 67.5 / 65.5, 10 of 500 and two of 1800 82.8 / 76.2.
+// Of the other side of the lines, with rows copied in larger lots than now (kLotPieces in step.cu; between 98 and 160 KB nothing has been timed):
 //   98 KB: e4m3 with 8 key heads 53.7 / 54.9, 32 heads of 64 56.9 / 57.8; 58 KB (228 tokens): 11 samples 31.1 / 38.4, 32 68.0 / 75.9;
-//   16 heads of 128 (4 KB of keys a token), 24 samples 74.0 / 78.3: the norms take longer than the scores.
+//   16 heads of 128 (4 KB of keys a token), 24 samples 74.0 / 78.3: the norms take longer than the scores; two rounds and a bit of clusters of two, 6 of 1700 tokens with short
+//   texts 68.5 / 68.5.
 struct TailBesideSizes {
     int64_t tokens;             // visual tokens of the launch
     int samples, jobs;          // jobs: samples x heads

@@ -158,7 +158,7 @@ struct BesidePlan {
 // and, as that kernel's CTAs end, on all of them.  CTAs take their roles by ticket: the first ones select, sample after sample, as the
 // samples' counters say that their scores are complete; all others copy rows, whose words the selecting CTAs write (select_copy_kernel).
 // Scoring is then bound by the memory for all of its time and the row copy for its own, where in turn a batch left the memory
-// idle from the drain of the one to the first list of the other.  Rows are given out piece by piece from one counter, samples in
+// idle from the drain of the one to the first list of the other.  Rows are given out in lots from one counter, samples in
 // order, because CTAs join while it runs.  A CTA waits only for the scoring kernel, all of whose CTAs run when this one starts, and for the selecting
 // CTAs, which have the lower tickets.
 template <int NT, int CAP>
@@ -205,9 +205,8 @@ select_copy_beside_kernel(const __grid_constant__ BatchDesc bd, const __grid_con
     // ---- row copy.  What a warp knows of the span of segments it is in stays in registers (an index into the parameters costs some hundred cycles).
     const int per_row = ca.seg_begin[3], n = bp.n;
     unsigned int* const counter = reinterpret_cast<unsigned int*>(hand + kHandLots);
-    // Pieces come in lots from one counter (11000 pieces of six segments straight from it, by 4700 warps, made that counter the limit:
-    // the rows of 16 requests moved at 4.8 instead of 6.8 TB/s).  s_lot: number of the lot << 12 | pieces given out; the warp that
-    // finds it used up puts the next one there, which was asked for one lot ago.
+    // Pieces come in lots (lots.h): 11000 pieces of six segments straight from one counter, by 4700 warps, made that counter the limit (the rows of 16 requests moved
+    // at 4.8 instead of 6.8 TB/s).
     __shared__ unsigned int s_lot;
     __shared__ volatile int s_next;
     if (tid == 0) {

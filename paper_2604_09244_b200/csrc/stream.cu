@@ -37,7 +37,7 @@ constexpr int kNormWarps = 2;                         // + these, in launches th
 constexpr int kNormStages = 3;                        // pieces of rows in flight per norm warp
 constexpr int kStreamRegs = 168;                      // registers a thread, see the kernel
 constexpr int kMaxStages = 12;
-constexpr int kStagesBesideTail = 6;                  // deeper rings make the tail's copies wait: 16 requests 88.0 -> 87.2 us, 8 of 3584 tokens 155.2 -> 154.3
+constexpr int kStagesBesideTail = 6;                  // deeper rings make the tail's copies wait: 12 / 6, 16 requests 88.0 / 87.2 us, 8 of 3584 tokens 155.2 / 154.3
 constexpr uint32_t kStageBytes = 16384;               // 128 keys x 128 bytes: one swizzled box of a key tile
 constexpr int kMaxSlots = 32;
 // Pairs of job n go to buffer n mod 2: a CTA sends those of job n + 2 only after it has the pairs of job n + 1 of every
@@ -55,7 +55,7 @@ struct StreamArgs {
     int32_t* rearm;               // see launch_salience_fast
     unsigned long long* rearm_rec;
     unsigned long long* stamps;
-    int32_t* hand;                // the tail runs beside this kernel: its counters (kDone...), or null
+    int32_t* hand;                // the tail runs beside this kernel: its counters (kHandTicket and so on), or null
     // feature norms (null: none): bf16 rows of `row_bytes` bytes, their L1 norms, where the pieces in flight lie in dynamic shared memory
     const uint8_t* hidden;
     float* l1;
@@ -369,7 +369,8 @@ __device__ __forceinline__ void soft_scores(const SoftJob& j, StreamSmem& sm, in
     __syncwarp();
 }
 
-// One norm warp: L1 norms of its share of the visual rows of all samples, a run of them.  Rows come by bulk
+// One norm warp: L1 norms of its share of the visual rows of all samples: a run of them; with a tail beside the kernel (HAND) every n_w-th, so that the
+// samples' norms are complete in the samples' order.  Rows come by bulk
 // copies, kNormStages pieces in flight per warp, so that they take their part of the memory bandwidth without registers
 // or a CTA of their own.  What bounds it is a piece's fixed cost and the adds of its sums, not the bytes in flight (adaptive steps of
 // 16 requests of 768 tokens: two pieces in flight 99.9 us, three 98.4; pieces of 4 KB 110.8; a run of rows instead of every n_w-th, whose
@@ -461,7 +462,8 @@ __device__ __forceinline__ void norm_warp(const BatchDesc& bd, const StreamArgs&
 // multiprocessor's four register files (16384 registers each): at the 168 registers a thread that the compiler takes these are
 // full, no CTA of the norms fits, and they start when the scores are done.  144 leave room for two warps of 32 registers in
 // each, at the price of 8 bytes a thread stored and 24 loaded (with 128 these are 68 and 144: 16 requests of 768 tokens 97 ->
-// 106 us when their norms ran beside).  8 requests of 3584 tokens, 64 queries, take 161.7 us with 144 and 162.0 with 168.
+// 106 us when their norms ran beside).  8 requests of 3584 tokens, 64 queries, took 161.7 us with 144 and 162.0 with 168 (they have the tail
+// beside this kernel since, and their norms in it).
 // Where no norms run beside, the registers are worth more to the attention copy: 16 patch-by-patch steps 76.5 us with 168, 78.6
 // with 144; 16 adaptive requests 93.7 and 93.0.
 // HAND: the tail of the step runs beside this kernel (launch_select_copy_beside); a variant of its own, because in the others the skipped code
