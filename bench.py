@@ -52,22 +52,22 @@ def measured_peaks():
 # the source files it is compiled from.
 NCU_SOURCES = {
     "scoring": ("fused.cu", "device_utils.cuh", "tmem_ld.cuh", "tmem_plan.h", "select_impl.cuh", "common.cuh"),
-    "tail": ("step.cu", "copy_impl.cuh", "select_impl.cuh", "device_utils.cuh", "common.cuh"),
+    "tail": ("step.cu", "copy_impl.cuh", "lots.h", "select_impl.cuh", "device_utils.cuh", "common.cuh"),
     # the patch-by-patch step: scoring kernel + its tail kernel, counters of both added up
     "step": ("fused.cu", "patch_step.cu", "patch_impl.cuh", "copy_impl.cuh", "device_utils.cuh", "tmem_ld.cuh", "tmem_plan.h",
              "select_impl.cuh", "common.cuh"),
 }
 NCU_DIGEST = {             # kernel -> sha256 of its sources when the counters were taken
-    "scoring": "c3c60d1cd8e8e1d963f02f35d62f3bfd7bf1eb5e9018ff23c69e058481b83fb5",
-    "tail": "1e8d043a93807339bd58e6a93da5314d7ac659fab0708b5194f115d0f92abb16",
-    "step": "e9822b075fa7e9bad74dbc90f7c4225d5f83062b4ee4917ba49e3843b54ff066",
+    "scoring": "6677f63d46e38246bb3203c0cfd315129ce701c4e78462357d42e5addf94a3e1",
+    "tail": "1d418a561758f856001b3739b9e265b1e2d0adaec462f10cf5f9cdafa729653e",
+    "step": "19a64c18015fcf79227f181a9c73ae90f1030d6c33641e8248b6e5401fd9002e",
 }
 NCU_TRAFFIC = {             # (workload, kernel) -> dram__bytes_read.sum + dram__bytes_write.sum per launch
     ("config2", "scoring"): 6598912,       # salience_fast_kernel<32,1,2>
-    ("config2", "tail"): 7135488,          # select_copy_kernel<512,1024>: the written half is still in L2 when the kernel ends
+    ("config2", "tail"): 7136640,          # select_copy_kernel<512,1024>: the written half is still in L2 when the kernel ends
     # salience_fast_kernel<32,1,2> 4.498 MB + patch_tail_kernel<bf16,2> 8.104 MB.  ncu flushes the caches before each
     # kernel, so the 2.10 MB attention copy that the tail finds in L2 in a normal run is counted here as DRAM reads.
-    ("patch_mla", "step"): 12602368,
+    ("patch_mla", "step"): 12602496,
 }
 
 
@@ -588,6 +588,11 @@ def run_ours(args, rank, local, world):
                              (" + l1norm_kernel beside it" if wl.mode == 1 else ""),
                   "tail": "select_copy_kernel (selection + row copy)"}
         dom = max(("scoring", "tail"), key=lambda k: kt[k])
+        if kt["scoring"] + kt["tail"] > kt["first_load_to_last_store"]:
+            # a large batch: the tail runs beside the scoring kernel, and the bytes of the one cannot be held against its span alone
+            dom, kt["both"] = "both", kt["first_load_to_last_store"]
+            kbytes["both"] = kbytes["scoring"] + kbytes["tail"]
+            knames["both"] = "salience_stream_kernel (+ feature norms) with select_copy_beside_kernel beside it"
         achieved = kbytes[dom] / (kt[dom] * 1e-6) / 1e9
         roof = {"bound": "hbm", "kernel": knames[dom], "achieved": achieved, "peak": peaks["hbm_gbs"],
                 "peak_kind": f"of {peak_kind}", "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"],
@@ -597,9 +602,9 @@ def run_ours(args, rank, local, world):
                        "stamps the kernels take themselves (mvla_set_kernel_stamps): from the moment the kernel's first CTA "
                        "is free to start (the kernel before it complete) to the end of its last CTA.  CUDA events cannot "
                        "bracket a kernel inside the step: a record between the two programmatically chained kernels removes "
-                       "their overlap and costs several microseconds in a graph.  The dominant kernel is the longer one.  (Where "
-                       "the two spans add up to more than first_load_to_last_store the batch is large enough for the tail to run "
-                       "beside the scoring kernel: its span then starts while that one runs)"}
+                       "their overlap and costs several microseconds in a graph.  The dominant kernel is the longer one; where "
+                       "the tail runs beside the scoring kernel (large batches: the two spans add up to more than "
+                       "first_load_to_last_store) the figure is that of both over the span of both"}
     else:
         # the patch-by-patch step: its two kernels take no stamps; the figure is the whole step's
         achieved = ab["total"] / (ms_per_step * 1e-3) / 1e9
