@@ -59,7 +59,7 @@ NCU_SOURCES = {
 }
 NCU_DIGEST = {             # kernel -> sha256 of its sources when the counters were taken
     "scoring": "6677f63d46e38246bb3203c0cfd315129ce701c4e78462357d42e5addf94a3e1",
-    "tail": "1d418a561758f856001b3739b9e265b1e2d0adaec462f10cf5f9cdafa729653e",
+    "tail": "037653be1e7b1896f45d5fdf9dc1ad73a0e0787ea1c56071ae366aa187847061",
     "step": "19a64c18015fcf79227f181a9c73ae90f1030d6c33641e8248b6e5401fd9002e",
 }
 NCU_TRAFFIC = {             # (workload, kernel) -> dram__bytes_read.sum + dram__bytes_write.sum per launch

@@ -73,7 +73,8 @@ inline bool chain_pays(int64_t moved, int ctas, bool adaptive, int sm_count)
 // sample b: what the samples' order can make larger than it has to be, when clusters with a job more than others get one of the long ones last.
 // The samples whose jobs take longest come first where that makes it smaller.  Elsewhere the order given stays: a long job
 // behind short ones has its keys loaded while those are worked on.  Whole steps in us, order given / longest first, batches of 32 heads:
-//   smaller: 16 of 228 tokens, texts of 16 to 64, 38.8 / 37.3, of 128 to 768 59.4 / 57.8, e4m3 45.6 / 44.4; five of 228 and one of 1500, twice, 64.6 / 60.6; patch by patch
+//   smaller: 16 of 228 tokens, texts of 16 to 64, 38.8 / 37.3, of 128 to 768 59.4 / 57.8, e4m3 45.6 / 44.4; five of 228 and one of 1500, twice, 64.6
+//   / 60.6; patch by patch
 //     16 of 512 77.6 / 74.6, 10 of 600 65.8 / 62.1, 16 of 128 to 800 74.4 / 70.4;
 //   the same: eleven of 300 and one of 4048 87.5 / 90.8, fixed budgets 78.5 / 81.3; patch by patch seven of 128 and one of 1200 39.9 / 41.4, 8 of 1000 71.3 / 71.5.
 // The cost is that of the softmax, by tiles and padded text queries, and of the keys, by tiles (with 0, 16, 32 or 64 queries' worth the choice is
@@ -119,14 +120,19 @@ inline bool longest_first_pays(const int* cost, int samples, int heads, int clus
 // some samples are scored well before the others; where a job is long enough that the multiprocessors given to the tail and the words that pass between
 // the kernels cost less than the idle memory between them; and where the scoring kernel's two norm warps, which take the feature norms then,
 // keep up with its scores.  Whole steps in us, behind / beside, 32 heads of 128, texts of 16 to 64, unless said otherwise:
-//   768 tokens (196 KB of keys a job): 10 samples 62.4 / 56.6, 16 93.7 / 88.4, 24 139.8 / 133.2; fixed budgets 12 56.0 / 51.9, 16 72.1 / 67.1; with 8 key heads, fixed, 10
-//     39.0 / 37.3, 16 53.1 / 48.9, 32 90.6 / 86.1, short texts 42.0 / 41.4; 16 heads, fixed, short texts, 24 50.4 / 49.1; 640 tokens (160 KB), few kept, 16 55.0 / 54.5;
-//   3000 tokens: 5 samples 105.0 / 99.0; 3584: 8 163.6 / 156.0; e4m3, fixed, short texts, 12 of 1300 57.7 / 54.5, with 8 key heads 44.7 / 43.8; 32 heads of 64, fixed, short texts, 12 of 1500
+//   768 tokens (196 KB of keys a job): 10 samples 62.4 / 56.6, 16 93.7 / 88.4, 24 139.8 / 133.2; fixed budgets 12 56.0 / 51.9, 16 72.1 / 67.1; with 8
+//   key heads, fixed, 10
+//     39.0 / 37.3, 16 53.1 / 48.9, 32 90.6 / 86.1, short texts 42.0 / 41.4; 16 heads, fixed, short texts, 24 50.4 / 49.1; 640 tokens (160 KB), few
+//     kept, 16 55.0 / 54.5;
+//   3000 tokens: 5 samples 105.0 / 99.0; 3584: 8 163.6 / 156.0; e4m3, fixed, short texts, 12 of 1300 57.7 / 54.5, with 8 key heads 44.7 / 43.8; 32
+//   heads of 64, fixed, short texts, 12 of 1500
 //     55.6 / 52.2, with 8 key heads 40.3 / 39.6;
-//   long and short samples: 5 of 228 and one of 3584 55.4 / 55.1, the long one first 61.1 / 55.4, 5 of 768 and one of 3584 67.5 / 65.5, 10 of 500 and two of 1800 82.8 / 76.2.
+//   long and short samples: 5 of 228 and one of 3584 55.4 / 55.1, the long one first 61.1 / 55.4, 5 of 768 and one of 3584 67.5 / 65.5, 10 of 500 and
+//   two of 1800 82.8 / 76.2.
 // Of the other side of the lines, with rows copied in larger lots than now (kLotPieces in step.cu; between 98 and 160 KB nothing has been timed):
 //   98 KB: e4m3 with 8 key heads 53.7 / 54.9, 32 heads of 64 56.9 / 57.8; 58 KB (228 tokens): 11 samples 31.1 / 38.4, 32 68.0 / 75.9;
-//   16 heads of 128 (4 KB of keys a token), 24 samples 74.0 / 78.3: the norms take longer than the scores; two rounds and a bit of clusters of two, 6 of 1700 tokens with short
+//   16 heads of 128 (4 KB of keys a token), 24 samples 74.0 / 78.3: the norms take longer than the scores; two rounds and a bit of clusters of two, 6
+//   of 1700 tokens with short
 //   texts 68.5 / 68.5.
 struct TailBesideSizes {
     int64_t tokens;             // visual tokens of the launch

@@ -140,9 +140,12 @@ cudaError_t launch_t(const BD& bd, const TailPlan& tp, const GateParams& gp, con
 
 // ------------------------------------------------------------------ beside the scoring kernel
 constexpr int kPieceSegs = 2;         // segments of rows that a warp takes at a time
-// Pieces that a CTA takes at a time.  Smaller lots end together: with 16 pieces of four segments the rows of a dozen samples were 333 lots for 288 CTAs, and some copied
-// two where most had one.  Whole steps in us, behind the scoring kernel / 16 of 4 / 8 of 4 / 16 of 2 / 8 of 2 / 4 of 2: fixed budgets, 768 tokens, 8 key heads, 10 samples 39.0 / 45.5 / 41.9 /
-// 38.7 / 37.3 / 36.0, 16 53.1 / 54.9 / 51.3 / 49.6 / 48.9 / 48.6; 32 key heads, 16 72.1 / 68.7 / 66.7 / 68.5 / 67.1 / 67.0; adaptive, 16 93.7 / 88.4 / 88.5 / 89.5 / 88.4 / 88.3, 5 of 228
+// Pieces that a CTA takes at a time.  Smaller lots end together: with 16 pieces of four segments the rows of a dozen samples were 333 lots for 288
+// CTAs, and some copied
+// two where most had one.  Whole steps in us, behind the scoring kernel / 16 of 4 / 8 of 4 / 16 of 2 / 8 of 2 / 4 of 2: fixed budgets, 768 tokens, 8
+// key heads, 10 samples 39.0 / 45.5 / 41.9 /
+// 38.7 / 37.3 / 36.0, 16 53.1 / 54.9 / 51.3 / 49.6 / 48.9 / 48.6; 32 key heads, 16 72.1 / 68.7 / 66.7 / 68.5 / 67.1 / 67.0; adaptive, 16 93.7 / 88.4
+// / 88.5 / 89.5 / 88.4 / 88.3, 5 of 228
 // and one of 3584 tokens 55.4 / 59.2 / 57.3 / 56.2 / 55.1 / 55.2; 8 of 3584 (CTAs of 32 warps) 163.6 / 157.0 / 156.1 / 156.8 / 156.0 / 158.8.
 constexpr int kLotPieces = 8;
 
@@ -205,7 +208,8 @@ select_copy_beside_kernel(const __grid_constant__ BatchDesc bd, const __grid_con
     // ---- row copy.  What a warp knows of the span of segments it is in stays in registers (an index into the parameters costs some hundred cycles).
     const int per_row = ca.seg_begin[3], n = bp.n;
     unsigned int* const counter = reinterpret_cast<unsigned int*>(hand + kHandLots);
-    // Pieces come in lots (lots.h): 11000 pieces of six segments straight from one counter, by 4700 warps, made that counter the limit (the rows of 16 requests moved
+    // Pieces come in lots (lots.h): 11000 pieces of six segments straight from one counter, by 4700 warps, made that counter the limit (the rows of
+    // 16 requests moved
     // at 4.8 instead of 6.8 TB/s).
     __shared__ unsigned int s_lot;
     __shared__ volatile int s_next;
